@@ -851,7 +851,8 @@ extern "C" int32_t ckks_rotate_sum(ckks_ctx *c, const ckks_ct *in, const ckks_ev
             }
             KsWorkspace wt = w;
             wt.ext = w.ext + (size_t)t0 * beta * nt * N;
-            ks_inner_terms(c, level, wt, (size_t)beta * nt * N, tm, nterm, 0, s, 1, i0 + t0 > 0);
+            wt.d = w.d + (size_t)t0 * ctl;
+            ks_inner_terms(c, level, wt, (size_t)beta * nt * N, ctl, tm, nterm, 0, s, 1, i0 + t0 > 0);
         }
     }
     ks_moddown(c, level, w, nullptr, nullptr, 1, (u64 *)out->data, s);
@@ -1073,7 +1074,7 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
                         tm.galois[t] = ge;
                         tm.c0[t] = ag + (size_t)t * S * ctl;
                     }
-                    ks_inner_terms(c, level, kx, (size_t)S * kbeta * knt * N, tm, nterm, ctl, s, S, u_live);
+                    ks_inner_terms(c, level, kx, (size_t)S * kbeta * knt * N, (size_t)S * ctl, tm, nterm, ctl, s, S, u_live);
                     u_live = true;
                     gl += nterm;
                 }

@@ -37,12 +37,10 @@ struct DevTables {
     const double2 *inv_scale_dn;   // [K][2]          ModDown: special limb
     // ModUp, per level l (1..L), digit j, source a < alpha:
     const ulonglong2 *up_hat_inv;  // [(L+1)][dnum][alpha]        {qhat^-1 mod q_src, Shoup}
-    const u64 *up_hat_mod;         // [(L+1)][dnum][alpha][T]     qhat mod target
-    const double2 *up_hat_mod_d;   // same shape, {c, c / target prime} as doubles
+    const double *up_hat_mod_d;    // [(L+1)][dnum][T][alpha]     centred qhat mod target
     // ModDown:
     const ulonglong2 *dn_hat_inv;  // [K]      {Phat_k^-1 mod p_k, Shoup}
-    const u64 *dn_hat_mod;         // [L][K]   Phat_k mod q_i
-    const double2 *dn_hat_mod_d;   // [L][K]   {c, c / q_i} as doubles
+    const double *dn_hat_mod_d;    // [L][K]   centred Phat_k mod q_i
     const ulonglong2 *dn_p_inv;    // [L]      {P^-1 mod q_i, Shoup}
     const double2 *dn_p_inv_d;     // [L]      {P^-1 mod q_i, that / q_i} as doubles
     const double *dn_p_mod_d;      // [L]      P mod q_i as a double
@@ -317,14 +315,20 @@ void launch_tensor_sum(const ckks_ctx *c, const u64 *const *a, const u64 *const 
                        cudaStream_t s);
 
 // Key switch pieces.  Sizes in limbs: d [level], ext [beta][level+K], u [2][level+K], conv [2][level].
-struct KsWorkspace { u64 *dcoef, *ext, *u, *conv; };
+// d, d_stride: the evaluation-domain input of the last ks_modup (batch entries d_stride words apart).  A digit's own limbs
+// are not copied into ext; the inner product reads them from d, which has to stay as it is until then.
+struct KsWorkspace {
+    u64 *dcoef, *ext, *u, *conv;
+    const u64 *d = nullptr;
+    size_t d_stride = 0;
+};
 size_t ks_workspace_limbs(const ckks_ctx *c, uint32_t level);
 KsWorkspace ks_carve(const ckks_ctx *c, uint32_t level, void *ws, uint32_t nb = 1);
 // nb key switches side by side (batch entry b reads d + b * d_stride words, d_stride a multiple of N):
 // d (evaluation domain, [level][N]) -> ext (evaluation domain, all digits).  A rotation applies its sigma_g to the
 // extended digits when the inner product reads them (ext_galois below): the centred conversion commutes with the
 // permutation and the sign flips of sigma_g, so this equals extending sigma_g(d), and d is never copied.
-void ks_modup(const ckks_ctx *c, const u64 *d, uint32_t level, const KsWorkspace &w, cudaStream_t s, uint32_t nb = 1, size_t d_stride = 0);
+void ks_modup(const ckks_ctx *c, const u64 *d, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb = 1, size_t d_stride = 0);
 // inner product with evk (digits read through sigma_{ext_galois}; 1 = identity), ModDown, and the final
 // combination out_c (+)= sigma_{add_galois}(add_c) + k_c.  add0/add1 may be null.
 void ks_inner_moddown(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w,
@@ -340,7 +344,8 @@ void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const u
                 TiledOut tiled = TiledOut(), const KsMulti *multi = nullptr);
 // A sum of up to IP_TERMS key-switched terms in one pass over the extended basis:
 //   u[b] (+)= sum_t ( <ext[t][b] read through sigma_{g_t}, evk_t>  +  P sigma_{g_t}(c0_t[b]) on component 0's q-limbs )
-// ext holds term t's digits of batch entry b at ext + t * term_stride + b * beta * (level + K) * N words; c0[t]
+// ext holds term t's digits of batch entry b at ext + t * term_stride + b * beta * (level + K) * N words, and the own limbs of
+// the digits lie at d + t * d_term_stride + b * w.d_stride; c0[t]
 // (may be null) points at term t's first-component limbs, entries c0_stride words apart.  Adding P c0 before the
 // ModDown equals adding c0 after it, exactly.
 constexpr uint32_t IP_TERMS = 4;
@@ -349,7 +354,7 @@ struct IpTerms {
     u64 galois[IP_TERMS];
     const u64 *c0[IP_TERMS];
 };
-void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, size_t term_stride, const IpTerms &terms, uint32_t nterm,
+void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, size_t term_stride, size_t d_term_stride, const IpTerms &terms, uint32_t nterm,
                     size_t c0_stride, cudaStream_t s, uint32_t nb, bool acc_u);
 // The basis conversions on the tensor cores (N = 2^16 layout rules: any N that is a multiple of 1024).  Return false if
 // the context has no byte matrices (more than 8 sources) and nothing was launched.

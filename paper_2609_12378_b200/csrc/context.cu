@@ -243,7 +243,8 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
     const uint32_t dn = prm->dnum;
     std::vector<ulonglong2> up_inv((size_t)(L + 1) * dn * alpha, make_ulonglong2(0, 0));
     std::vector<u64> up_mod((size_t)(L + 1) * dn * alpha * T, 0);
-    std::vector<double2> up_mod_d(up_mod.size(), make_double2(0.0, 0.0));
+    std::vector<double> up_mod_d(up_mod.size(), 0.0);
+    auto centred = [](u64 v, u64 m) { return v > m / 2 ? -(double)(m - v) : (double)v; };
     for (uint32_t lvl = 1; lvl <= L; lvl++)
         for (uint32_t j = 0; j * alpha < lvl; j++) {
             uint32_t lo = j * alpha, hi = std::min(lo + alpha, lvl);
@@ -258,7 +259,7 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
                     for (uint32_t b = lo; b < hi; b++)
                         if (b != a) v = h_mul(v, mod[b] % mt, mt);
                     up_mod[base * T + t] = v;
-                    up_mod_d[base * T + t] = make_double2((double)v, (double)v / (double)mt);
+                    up_mod_d[(((size_t)lvl * dn + j) * T + t) * alpha + (a - lo)] = centred(v, mt);
                 }
             }
         }
@@ -268,7 +269,7 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
     std::vector<double2> dn_pinv_d(L);
     std::vector<double> dn_pmod_d(L);
     std::vector<u64> dn_mod((size_t)L * K);
-    std::vector<double2> dn_mod_d((size_t)L * K);
+    std::vector<double> dn_mod_d((size_t)L * K);
     for (uint32_t a = 0; a < K; a++) {
         u64 pa = mod[L + a], h = 1;
         for (uint32_t b = 0; b < K; b++)
@@ -282,7 +283,7 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
             for (uint32_t b = 0; b < K; b++)
                 if (b != a) v = h_mul(v, mod[L + b] % q, q);
             dn_mod[(size_t)i * K + a] = v;
-            dn_mod_d[(size_t)i * K + a] = make_double2((double)v, (double)v / (double)q);
+            dn_mod_d[(size_t)i * K + a] = centred(v, q);
             Pm = h_mul(Pm, mod[L + a] % q, q);
         }
         dn_pinv[i] = h_pair(h_inv(Pm, q), q);
@@ -409,8 +410,8 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
     const int *flag_dev = nullptr;
     if ((rc = upload(c, mod, &d.mod)) || (rc = upload(c, mu, &d.mu)) || (rc = upload(c, mu64, &d.mu64)) || (rc = upload(c, modd, &d.modd)) || (rc = upload(c, twf, &d.tw_fwd)) ||
         (rc = upload(c, twi, &d.tw_inv)) || (rc = upload(c, twdf, &d.twd_fwd)) || (rc = upload(c, twdi, &d.twd_inv)) || (rc = upload(c, ninvd, &d.n_inv_d)) || (rc = upload(c, isc_up, &d.inv_scale_up)) || (rc = upload(c, isc_dn, &d.inv_scale_dn)) || (rc = upload(c, ninv, &d.n_inv)) || (rc = upload(c, up_inv, &d.up_hat_inv)) ||
-        (rc = upload(c, up_mod, &d.up_hat_mod)) || (rc = upload(c, up_mod_d, &d.up_hat_mod_d)) || (rc = upload(c, dn_mod_d, &d.dn_hat_mod_d)) || (rc = upload(c, dn_inv, &d.dn_hat_inv)) ||
-        (rc = upload(c, dn_mod, &d.dn_hat_mod)) || (rc = upload(c, dn_pinv, &d.dn_p_inv)) || (rc = upload(c, dn_pinv_d, &d.dn_p_inv_d)) || (rc = upload(c, dn_pmod_d, &d.dn_p_mod_d)) || (rc = upload(c, up_bmat, &d.up_bmat)) || (rc = upload(c, dn_bmat, &d.dn_bmat)) || (rc = upload(c, two52, &d.two52_d)) || (rc = upload(c, rs, &d.rs_inv)) ||
+        (rc = upload(c, up_mod_d, &d.up_hat_mod_d)) || (rc = upload(c, dn_mod_d, &d.dn_hat_mod_d)) || (rc = upload(c, dn_inv, &d.dn_hat_inv)) ||
+        (rc = upload(c, dn_pinv, &d.dn_p_inv)) || (rc = upload(c, dn_pinv_d, &d.dn_p_inv_d)) || (rc = upload(c, dn_pmod_d, &d.dn_p_mod_d)) || (rc = upload(c, up_bmat, &d.up_bmat)) || (rc = upload(c, dn_bmat, &d.dn_bmat)) || (rc = upload(c, two52, &d.two52_d)) || (rc = upload(c, rs, &d.rs_inv)) ||
         (rc = upload(c, enc_src, &d.enc_src)) || (rc = upload(c, om, &d.enc_omega)) || (rc = upload(c, om_st, &d.enc_omega_st)) || (rc = upload(c, om_st2, &d.enc_omega_st2)) || (rc = upload(c, ze, &d.enc_zeta)) ||
         (rc = upload(c, flag, &flag_dev))) {
         cudaSetDevice(prev);

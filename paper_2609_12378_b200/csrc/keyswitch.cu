@@ -23,100 +23,154 @@ __global__ void __launch_bounds__(THREADS) permute_kernel(DevTables c, const u64
     dst[blockIdx.z * dst_stride + row + p] = src[blockIdx.z * src_stride + row + galois_src(p, g, c.log_n, c.N)];
 }
 
-// targets per CTA row in the basis-conversion kernels: the source limbs are re-read once per chunk, so large batches
-// take all targets in one chunk and single ciphertexts split them for parallelism
-inline uint32_t conv_chunk(uint32_t nb) { return nb >= 4 ? 32 : 16; }
+// ---------------------------------------------------------------------------
+// Basis conversions: out[x] = sum_a y_a C[a][x] mod t_x with centred sources |y_a| <= q_a / 2 and centred constants
+// |C| <= t / 2 (a dense contraction, bound by the FP64 pipe).  The exact 100-bit products are summed as they are and
+// reduced once per eight sources:
+//   H' = fma(y, C, H) starting from H = 1.5 * 2^102 rounds the running sum to multiples of 2^50 (|sum| <= 8 * 2^98 =
+//   2^101 keeps H inside [2^102, 2^103)); h = H' - H is exact, l = fma(y, C, -h) is the exact rest, |l| <= 2^49,
+// so the sum is (H - 1.5 * 2^102) + sum l, four instructions per (source, target) pair where a reduction of every product
+// took seven.  The high part is below 2 q t, so its quotient by t is below 2^51 (nearest rounding) and leaves |r| <= 1.1 t;
+// with the low parts (<= 8 * 2^49, plus a reduced carry of the previous eight sources) the sum stays below 2^53.
+// A thread takes CPT adjacent coefficients, so that a pair of constants from shared memory serves 2 CPT pairs.
+// ---------------------------------------------------------------------------
+constexpr double CONV_SIGMA = 0x1.8p+102;
 
-// ext[j][x][k] for x over q_0..q_{level-1}, p_0..p_{K-1}.  dcoef: sigma_g(d) in the coefficient domain;
-// deval: d in the evaluation domain, read through sigma_g for the digit's own limbs.
-// A thread owns one coefficient of one digit: it forms the centred y_a of the digit's limbs once and then
-// walks a chunk of CHUNK target limbs (blockIdx.y), so the source limbs are read once per chunk.
+template <uint32_t NS, uint32_t CPT>
+__device__ __forceinline__ void conv_dot(const double (&y)[CPT][NS], const double *w, double t, double tinv, double (&out)[CPT]) {
+    double H[CPT], lo[CPT];
+#pragma unroll
+    for (uint32_t p = 0; p < CPT; p++) { H[p] = CONV_SIGMA; lo[p] = 0.0; }
+#pragma unroll
+    for (uint32_t a = 0; a < NS; a++) {
+        const double wa = w[a];
+#pragma unroll
+        for (uint32_t p = 0; p < CPT; p++) {
+            const double Hn = __fma_rn(y[p][a], wa, H[p]);
+            const double l = __fma_rn(y[p][a], wa, -__dsub_rn(Hn, H[p]));
+            lo[p] = a == 0 ? l : __dadd_rn(lo[p], l);
+            H[p] = Hn;
+            if ((a & 7) == 7 || a + 1 == NS) {
+                const double hs = __dsub_rn(H[p], CONV_SIGMA);
+                const double k = __dsub_rn(__fma_rn(hs, tinv, MAGIC0), MAGIC0);
+                lo[p] = reduce_d(__dadd_rn(lo[p], __fma_rn(-k, t, hs)), t, tinv);
+                H[p] = CONV_SIGMA;
+            }
+        }
+    }
+#pragma unroll
+    for (uint32_t p = 0; p < CPT; p++) out[p] = lo[p];
+}
+
+// centred source residues of CPT adjacent coefficients
+template <uint32_t CPT>
+__device__ __forceinline__ void conv_load(const u64 *p, u64 (&v)[CPT]) {
+    if (CPT == 2) {
+        const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(p);
+        v[0] = w.x; v[CPT - 1] = w.y;
+    } else {
+        v[0] = *p;
+    }
+}
+template <uint32_t CPT>
+__device__ __forceinline__ void conv_store(u64 *p, const double (&v)[CPT], double t) {
+    if (CPT == 2) *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(canonical_d(v[0], t), canonical_d(v[CPT - 1], t));
+    else *p = canonical_d(v[0], t);
+}
+__device__ __forceinline__ double centre_d(u64 v, u64 q) { return v > (q >> 1) ? __dsub_rn(u64_to_d(v), (double)q) : u64_to_d(v); }
+
+// coefficients per thread: two while their sources fit the registers and the buffers take 16-byte accesses
+inline uint32_t conv_cpt(uint32_t ns, const void *a, const void *b) { return ns <= 8 && (((uintptr_t)a | (uintptr_t)b) & 15) == 0 ? 2 : 1; }
+
+// targets per CTA (grid y) for `items` conversions of `targets` targets over gx CTAs: as many as leave the machine three
+// waves of CTAs (4 per SM), so that large batches read their sources once and single ciphertexts still fill the GPU
 constexpr uint32_t CONV_CHUNK_MAX = 32;
+inline uint32_t conv_chunk(uint32_t gx, uint32_t items, uint32_t targets) {
+    const uint32_t want = 3 * 148 * 4;
+    uint32_t chunks = (want + gx * items - 1) / (gx * items);
+    chunks = std::max(1u, std::min(chunks, (targets + 3) / 4));
+    return std::min(CONV_CHUNK_MAX, (targets + chunks - 1) / chunks);
+}
 
+// ext[j][x][k] for the limbs x of q_0..q_{level-1}, p_0..p_{K-1} outside digit j, from dcoef (coefficient domain).  A thread
+// owns CPT coefficients of one digit: it forms the centred y_a of the digit's limbs once and walks a chunk of CHUNK target
+// limbs (blockIdx.y), so the source limbs are read once per chunk.
 // PRE: dcoef already holds [d_a qhat_a^-1] (the inverse transform multiplied it in), so only the centring is left.
-template <uint32_t ALPHA, bool PRE>
-__global__ void __launch_bounds__(THREADS) modup_kernel(DevTables c, const u64 *dcoef, const u64 *deval, size_t deval_stride, u64 g,
-                                                        u64 *ext, uint32_t level, uint32_t CHUNK) {
-    // the CTA's conversion constants (qhat_a mod t and its quotient by t; t and 1/t), fetched once: as global loads
-    // inside the loop they kept the L1 busier than the arithmetic kept the FP64 pipe
-    __shared__ double2 s_w[CONV_CHUNK_MAX][ALPHA];
+template <uint32_t ALPHA, bool PRE, uint32_t CPT>
+__global__ void __launch_bounds__(THREADS) modup_kernel(DevTables c, const u64 *dcoef, u64 *ext, uint32_t level, uint32_t CHUNK) {
+    // the CTA's conversion constants (qhat_a mod t; t and 1/t), fetched once
+    __shared__ __align__(16) double s_w[CONV_CHUNK_MAX][ALPHA];
     __shared__ double2 s_m[CONV_CHUNK_MAX];
-    const uint32_t k = blockIdx.x * THREADS + threadIdx.x;
+    const uint32_t k = (blockIdx.x * THREADS + threadIdx.x) * CPT;
     const uint32_t beta = (level + c.alpha - 1) / c.alpha, j = blockIdx.z % beta, bz = blockIdx.z / beta;
     const uint32_t nt = level + c.K, lo = j * c.alpha, hi = min(lo + c.alpha, level), nd = hi - lo;
-    const uint32_t x0 = blockIdx.y * CHUNK, x1 = min(x0 + CHUNK, nt);
-    const size_t cb = ((size_t)level * c.dnum + j) * c.alpha;
+    const uint32_t x0 = blockIdx.y * CHUNK, x1 = min(x0 + CHUNK, nt - nd);       // targets, counted without the digit's own limbs
+    if (x0 >= x1) return;
+    const size_t cb = (size_t)level * c.dnum + j;
     for (uint32_t e = threadIdx.x; e < (x1 - x0) * ALPHA; e += THREADS) {
-        const uint32_t xi = e / ALPHA, a = e % ALPHA, x = x0 + xi, t = x < level ? x : c.L + (x - level);
-        s_w[xi][a] = a < nd ? c.up_hat_mod_d[(cb + a) * c.T + t] : make_double2(0.0, 0.0);
+        const uint32_t xi = e / ALPHA, a = e % ALPHA, xt = x0 + xi, x = xt < lo ? xt : xt + nd, t = x < level ? x : c.L + (x - level);
+        s_w[xi][a] = a < nd ? c.up_hat_mod_d[(cb * c.T + t) * c.alpha + a] : 0.0;
         if (a == 0) s_m[xi] = c.modd[t];
     }
-    dcoef += (size_t)bz * level * c.N;
-    deval += bz * deval_stride;
-    ext += (size_t)bz * beta * nt * c.N;
-    // centred y_a = [d_a qhat_a^-1] as signed doubles (integer Shoup product, then the lift)
-    double y[ALPHA];
+    dcoef += ((size_t)bz * level + lo) * c.N + k;
+    ext += ((size_t)bz * beta + j) * nt * c.N + k;
+    double y[CPT][ALPHA];
 #pragma unroll
     for (uint32_t a = 0; a < ALPHA; a++) {
-        y[a] = 0.0;
-        if (a < nd) {
-            const u64 qa = c.mod[lo + a];
-            u64 v = dcoef[(size_t)(lo + a) * c.N + k];
-            if (!PRE) {
-                const ulonglong2 hinv = c.up_hat_inv[cb + a];
-                v = mul_shoup(v, hinv.x, hinv.y, qa);
+        u64 v[CPT];
+        if (a < nd) conv_load<CPT>(dcoef + (size_t)a * c.N, v);
+#pragma unroll
+        for (uint32_t p = 0; p < CPT; p++) {
+            y[p][a] = 0.0;
+            if (a < nd) {
+                const u64 qa = c.mod[lo + a];
+                if (!PRE) {
+                    const ulonglong2 hinv = c.up_hat_inv[cb * c.alpha + a];
+                    v[p] = mul_shoup(v[p], hinv.x, hinv.y, qa);
+                }
+                y[p][a] = centre_d(v[p], qa);
             }
-            y[a] = v > (qa >> 1) ? __dsub_rn(u64_to_d(v), (double)qa) : u64_to_d(v);
         }
     }
     __syncthreads();
-    u64 *dst = ext + ((size_t)j * nt + x0) * c.N + k;
-    for (uint32_t x = x0; x < x1; x++, dst += c.N) {
-        if (x >= lo && x < hi) {
-            *dst = deval[(size_t)x * c.N + galois_src(k, g, c.log_n, c.N)];
-            continue;
-        }
-        const double2 md = s_m[x - x0];
-        const double mt = md.x, mtinv = md.y;
-        // each product is reduced to |r| <= 0.57 m_t on the FP64 pipe; eight of them stay far below 2^53 (a missing
-        // source has y = 0 and a zero constant)
-        double acc = 0.0;
-#pragma unroll
-        for (uint32_t a = 0; a < ALPHA; a++) {
-            acc = __dadd_rn(acc, mulmod_d<0>(y[a], s_w[x - x0][a], mt));
-            if ((a & 7) == 7 && a + 1 < ALPHA) acc = reduce_d(acc, mt, mtinv);
-        }
-        *dst = canonical_d(reduce_d(acc, mt, mtinv), mt);
+    for (uint32_t xt = x0; xt < x1; xt++) {
+        const double2 md = s_m[xt - x0];
+        double r[CPT];
+        conv_dot<ALPHA, CPT>(y, s_w[xt - x0], md.x, md.y, r);
+        conv_store<CPT>(ext + (size_t)(xt < lo ? xt : xt + nd) * c.N, r, md.x);
     }
 }
 
 template <uint32_t ALPHA>
-void launch_modup(const ckks_ctx *c, const u64 *dcoef, const u64 *deval, size_t deval_stride, u64 g, u64 *ext, uint32_t level,
-                  uint32_t nb, cudaStream_t s, bool pre) {
+void launch_modup(const ckks_ctx *c, const u64 *dcoef, u64 *ext, uint32_t level, uint32_t nb, cudaStream_t s, bool pre) {
     const uint32_t nt = level + c->K, beta = (level + c->alpha - 1) / c->alpha;
-    const uint32_t CHUNK = conv_chunk(nb);
-    const dim3 grid(c->N / THREADS, (nt + CHUNK - 1) / CHUNK, beta * nb);
-    if (pre) modup_kernel<ALPHA, true><<<grid, THREADS, 0, s>>>(c->dev, dcoef, deval, deval_stride, g, ext, level, CHUNK);
-    else modup_kernel<ALPHA, false><<<grid, THREADS, 0, s>>>(c->dev, dcoef, deval, deval_stride, g, ext, level, CHUNK);
+    const uint32_t cpt = conv_cpt(ALPHA, dcoef, ext), gx = c->N / (THREADS * cpt), targets = nt - (level - (beta - 1) * c->alpha);   // the last digit has the most targets
+    const uint32_t CHUNK = conv_chunk(gx, beta * nb, targets);
+    const dim3 grid(gx, (targets + CHUNK - 1) / CHUNK, beta * nb);
+    constexpr uint32_t WIDE = ALPHA <= 8 ? 2 : 1;
+    auto *kernel = cpt == WIDE ? (pre ? modup_kernel<ALPHA, true, WIDE> : modup_kernel<ALPHA, false, WIDE>)
+                               : (pre ? modup_kernel<ALPHA, true, 1> : modup_kernel<ALPHA, false, 1>);
+    kernel<<<grid, THREADS, 0, s>>>(c->dev, dcoef, ext, level, CHUNK);
     count_launches();
 }
 
 // u[comp][x][p] = sum_j ext[j][x][pi_g(p)] * evk[j][comp][kt(x)][p]          (any number of digits)
-__global__ void __launch_bounds__(THREADS) inner_product_generic_kernel(DevTables c, const u64 *ext, const u64 *evk, u64 g,
+__global__ void __launch_bounds__(THREADS) inner_product_generic_kernel(DevTables c, const u64 *ext, const u64 *d, size_t d_stride, const u64 *evk, u64 g,
                                                                         u64 *u, uint32_t level, int has_multi, KsMulti multi, int acc_u) {
     const uint32_t p = blockIdx.x * THREADS + threadIdx.x;
     const uint32_t x = blockIdx.z, bz = blockIdx.y;     // batch varies faster than the limb: a key limb is reused from L2
     const uint32_t nt = level + c.K, beta = (level + c.alpha - 1) / c.alpha;
     const uint32_t kt = x < level ? x : c.L + (x - level);
     if (has_multi) { evk = multi.evk[bz]; g = multi.galois[bz]; }     // shared digits, per-entry key and permutation
-    else ext += (size_t)bz * beta * nt * c.N;
+    else { ext += (size_t)bz * beta * nt * c.N; d += bz * d_stride; }
+    const uint32_t own = x < level ? x / c.alpha : beta;        // the digit that has x among its own limbs
     const uint32_t src = galois_src(p, g, c.log_n, c.N);
     u += (size_t)bz * 2 * nt * c.N;
     // products on the FP64 pipe: each is reduced to |r| <= 0.75 m as it is formed, the few digits are summed exactly
     const double2 md = c.modd[kt];
     double a0 = 0.0, a1 = 0.0;
     for (uint32_t j = 0; j < beta; j++) {
-        const double e = u64_to_d(ext[((size_t)j * nt + x) * c.N + src]);
+        const double e = u64_to_d((j == own ? d + (size_t)x * c.N : ext + ((size_t)j * nt + x) * c.N)[src]);
         a0 = __dadd_rn(a0, mulmod_dd(e, u64_to_d(evk[(((size_t)j * 2 + 0) * c.T + kt) * c.N + p]), md.x, md.y));
         a1 = __dadd_rn(a1, mulmod_dd(e, u64_to_d(evk[(((size_t)j * 2 + 1) * c.T + kt) * c.N + p]), md.x, md.y));
         if ((j & 7) == 7) { a0 = reduce_d(a0, md.x, md.y); a1 = reduce_d(a1, md.x, md.y); }
@@ -137,7 +191,7 @@ __global__ void __launch_bounds__(THREADS) inner_product_generic_kernel(DevTable
 // of up to KS_MULTI keys applied to the same digits.
 constexpr uint32_t IP_MAX_BETA = 4;
 template <uint32_t BETA>
-__global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, const u64 *ext, const u64 *evk, u64 g, u64 *u,
+__global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, const u64 *ext, const u64 *d, size_t d_stride, const u64 *evk, u64 g, u64 *u,
                                                                 uint32_t level, uint32_t nb, uint32_t bch, int has_multi, KsMulti multi,
                                                                 int acc_u) {
     const uint32_t p = (blockIdx.x * THREADS + threadIdx.x) * 2;
@@ -165,13 +219,16 @@ __global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, con
             k[j][cm][0] = u64_to_d(v.x);
             k[j][cm][1] = u64_to_d(v.y);
         }
-    const u64 *e = ext + e0 * BETA * js + (size_t)x * c.N + (src & ~1u);
+    const uint32_t own = x < level ? x / c.alpha : BETA;       // the digit that has x among its own limbs: it lies in d
+    const uint32_t so = src & ~1u;
     u64 *o = u + b0 * 2 * js + (size_t)x * c.N + p;
-    for (uint32_t b = b0; b < b1; b++, e += BETA * js, o += 2 * js) {
+    for (uint32_t b = b0; b < b1; b++, o += 2 * js) {
+        const uint32_t be = b - b0 + e0;
         double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
         for (uint32_t j = 0; j < BETA; j++) {
-            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(e + j * js);
+            const u64 *ej = (j == own ? d + be * d_stride : ext + ((size_t)be * BETA + j) * js) + (size_t)x * c.N;
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(ej + so);
             const double d0 = u64_to_d(odd ? v.y : v.x), d1 = u64_to_d(odd ? v.x : v.y);
 #pragma unroll
             for (uint32_t cm = 0; cm < 2; cm++) {
@@ -200,7 +257,7 @@ __global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, con
 // registers over the terms.
 constexpr uint32_t IP_BCH = 4;
 template <uint32_t BETA>
-__global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTables c, const u64 *ext, size_t term_stride,
+__global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTables c, const u64 *ext, size_t term_stride, const u64 *d, size_t d_term_stride, size_t d_stride,
                                                                          const __grid_constant__ IpTerms tm, uint32_t nterm, size_t c0_stride,
                                                                          u64 *u, uint32_t level, uint32_t nb, int acc_u) {
     const uint32_t p = (blockIdx.x * THREADS + threadIdx.x) * 2;
@@ -210,6 +267,7 @@ __global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTabl
     const double2 md = c.modd[kt];
     const size_t js = (size_t)nt * c.N, ks = (size_t)c.T * c.N;
     const double pq = x < level ? c.dn_p_mod_d[x] : 0.0;
+    const uint32_t own = x < level ? x / c.alpha : BETA;       // the digit that has x among its own limbs: it lies in d
     double acc[IP_BCH][2][2];
 #pragma unroll
     for (uint32_t bi = 0; bi < IP_BCH; bi++) acc[bi][0][0] = acc[bi][0][1] = acc[bi][1][0] = acc[bi][1][1] = 0.0;
@@ -226,8 +284,8 @@ __global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTabl
                 k[j][cm][0] = u64_to_d(v.x);
                 k[j][cm][1] = u64_to_d(v.y);
             }
-        const u64 *e = ext + t * term_stride + (size_t)b0 * BETA * js + (size_t)x * c.N + (src & ~1u);
-        const u64 *z = (x < level && tm.c0[t]) ? tm.c0[t] + b0 * c0_stride + (size_t)x * c.N + (src & ~1u) : nullptr;
+        const uint32_t so = src & ~1u;
+        const u64 *z = (x < level && tm.c0[t]) ? tm.c0[t] + b0 * c0_stride + (size_t)x * c.N : nullptr;
         // no branch in here, so that the loads of all entries of the chunk are in flight together: an entry past the end
         // of the batch repeats the last one and is not stored
 #pragma unroll
@@ -236,7 +294,9 @@ __global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTabl
             double sum[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
             for (uint32_t j = 0; j < BETA; j++) {
-                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(e + ((size_t)bc * BETA + j) * js);
+                const u64 *ej = (j == own ? d + t * d_term_stride + (b0 + bc) * d_stride
+                                          : ext + t * term_stride + ((size_t)(b0 + bc) * BETA + j) * js) + (size_t)x * c.N;
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(ej + so);
                 const double d0 = u64_to_d(odd ? v.y : v.x), d1 = u64_to_d(odd ? v.x : v.y);
 #pragma unroll
                 for (uint32_t cm = 0; cm < 2; cm++) {
@@ -245,7 +305,7 @@ __global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTabl
                 }
             }
             if (z) {
-                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(z + bc * c0_stride);
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(z + bc * c0_stride + so);
                 sum[0][0] = __dadd_rn(sum[0][0], mulmod_dd(u64_to_d(odd ? v.y : v.x), pq, md.x, md.y));
                 sum[0][1] = __dadd_rn(sum[0][1], mulmod_dd(u64_to_d(odd ? v.x : v.y), pq, md.x, md.y));
             }
@@ -279,56 +339,56 @@ __global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTabl
 
 // conv[comp][i][k] = sum_a centre([u_{p_a} Phat_a^-1]) (Phat_a mod q_i)  mod q_i   (coefficient domain)
 // Same shape as ModUp: the K centred special residues are formed once per thread, then a chunk of targets is walked.
-template <uint32_t KK, bool PRE>
-__global__ void __launch_bounds__(THREADS, 6) moddown_conv_kernel(DevTables c, const u64 *u, u64 *conv, uint32_t level, uint32_t CHUNK) {
-    __shared__ double2 s_w[CONV_CHUNK_MAX][KK];     // Phat_a mod q_i and its quotient by q_i
-    __shared__ double2 s_m[CONV_CHUNK_MAX];         // q_i, 1 / q_i
-    const uint32_t k = blockIdx.x * THREADS + threadIdx.x;
+template <uint32_t KK, bool PRE, uint32_t CPT>
+__global__ void __launch_bounds__(THREADS) moddown_conv_kernel(DevTables c, const u64 *u, u64 *conv, uint32_t level, uint32_t CHUNK) {
+    __shared__ __align__(16) double s_w[CONV_CHUNK_MAX][KK];     // Phat_a mod q_i
+    __shared__ double2 s_m[CONV_CHUNK_MAX];                      // q_i, 1 / q_i
+    const uint32_t k = (blockIdx.x * THREADS + threadIdx.x) * CPT;
     const uint32_t comp = blockIdx.z & 1, bz = blockIdx.z >> 1;
     const uint32_t nt = level + c.K;
     const uint32_t i0 = blockIdx.y * CHUNK, i1 = min(i0 + CHUNK, level);
     for (uint32_t e = threadIdx.x; e < (i1 - i0) * KK; e += THREADS) {
         const uint32_t ii = e / KK, a = e % KK;
-        s_w[ii][a] = a < c.K ? c.dn_hat_mod_d[(size_t)(i0 + ii) * c.K + a] : make_double2(0.0, 0.0);
+        s_w[ii][a] = a < c.K ? c.dn_hat_mod_d[(size_t)(i0 + ii) * c.K + a] : 0.0;
         if (a == 0) s_m[ii] = c.modd[i0 + ii];
     }
-    u += (size_t)bz * 2 * nt * c.N;
-    conv += (size_t)bz * 2 * level * c.N;
-    double y[KK];
+    u += (((size_t)bz * 2 + comp) * nt + level) * c.N + k;
+    conv += ((size_t)bz * 2 + comp) * level * c.N + k;
+    double y[CPT][KK];
 #pragma unroll
     for (uint32_t a = 0; a < KK; a++) {
-        y[a] = 0.0;
-        if (a < c.K) {
-            const u64 pa = c.mod[c.L + a];
-            u64 v = u[((size_t)comp * nt + level + a) * c.N + k];
-            if (!PRE) {
-                const ulonglong2 hinv = c.dn_hat_inv[a];
-                v = mul_shoup(v, hinv.x, hinv.y, pa);
+        u64 v[CPT];
+        if (a < c.K) conv_load<CPT>(u + (size_t)a * c.N, v);
+#pragma unroll
+        for (uint32_t p = 0; p < CPT; p++) {
+            y[p][a] = 0.0;
+            if (a < c.K) {
+                const u64 pa = c.mod[c.L + a];
+                if (!PRE) {
+                    const ulonglong2 hinv = c.dn_hat_inv[a];
+                    v[p] = mul_shoup(v[p], hinv.x, hinv.y, pa);
+                }
+                y[p][a] = centre_d(v[p], pa);
             }
-            y[a] = v > (pa >> 1) ? __dsub_rn(u64_to_d(v), (double)pa) : u64_to_d(v);
         }
     }
     __syncthreads();
-    u64 *dst = conv + ((size_t)comp * level + i0) * c.N + k;
-    for (uint32_t i = i0; i < i1; i++, dst += c.N) {
+    for (uint32_t i = i0; i < i1; i++) {
         const double2 md = s_m[i - i0];
-        const double q = md.x, qinv = md.y;
-        double acc = 0.0;
-#pragma unroll
-        for (uint32_t a = 0; a < KK; a++) {
-            acc = __dadd_rn(acc, mulmod_d<0>(y[a], s_w[i - i0][a], q));
-            if ((a & 7) == 7 && a + 1 < KK) acc = reduce_d(acc, q, qinv);
-        }
-        *dst = canonical_d(reduce_d(acc, q, qinv), q);
+        double r[CPT];
+        conv_dot<KK, CPT>(y, s_w[i - i0], md.x, md.y, r);
+        conv_store<CPT>(conv + (size_t)i * c.N, r, md.x);
     }
 }
 
 template <uint32_t KK>
 void launch_moddown_conv(const ckks_ctx *c, const u64 *u, u64 *conv, uint32_t level, uint32_t nb, cudaStream_t s, bool pre) {
-    const uint32_t CHUNK = conv_chunk(nb);
-    const dim3 grid(c->N / THREADS, (level + CHUNK - 1) / CHUNK, 2 * nb);
-    if (pre) moddown_conv_kernel<KK, true><<<grid, THREADS, 0, s>>>(c->dev, u, conv, level, CHUNK);
-    else moddown_conv_kernel<KK, false><<<grid, THREADS, 0, s>>>(c->dev, u, conv, level, CHUNK);
+    const uint32_t cpt = conv_cpt(KK, u, conv), gx = c->N / (THREADS * cpt), CHUNK = conv_chunk(gx, 2 * nb, level);
+    const dim3 grid(gx, (level + CHUNK - 1) / CHUNK, 2 * nb);
+    constexpr uint32_t WIDE = KK <= 8 ? 2 : 1;
+    auto *kernel = cpt == WIDE ? (pre ? moddown_conv_kernel<KK, true, WIDE> : moddown_conv_kernel<KK, false, WIDE>)
+                               : (pre ? moddown_conv_kernel<KK, true, 1> : moddown_conv_kernel<KK, false, 1>);
+    kernel<<<grid, THREADS, 0, s>>>(c->dev, u, conv, level, CHUNK);
     count_launches();
 }
 
@@ -416,7 +476,8 @@ KsWorkspace ks_carve(const ckks_ctx *c, uint32_t level, void *ws, uint32_t nb) {
     return w;
 }
 
-void ks_modup(const ckks_ctx *c, const u64 *d, uint32_t level, const KsWorkspace &w, cudaStream_t s, uint32_t nb, size_t d_stride) {
+void ks_modup(const ckks_ctx *c, const u64 *d, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb, size_t d_stride) {
+    w.d = d; w.d_stride = d_stride;
     const uint32_t N = c->N, beta = (level + c->alpha - 1) / c->alpha, nt = level + c->K;
     // N = 2^16 with the FP64 transform and conversion: the inverse transform's last stage multiplies qhat^-1 in
     const bool pre = c->log_n == 16 && c->ntt_fp_share >= 8 && c->conv_kernel != CKKS_CONV_TENSOR;
@@ -429,7 +490,7 @@ void ks_modup(const ckks_ctx *c, const u64 *d, uint32_t level, const KsWorkspace
     }
     // the context option CKKS_CONV_TENSOR takes the tensor-core conversion of conv_mma.cu: bit-identical, 2 % slower on B200
     if (c->conv_kernel != CKKS_CONV_TENSOR || !launch_modup_mma(c, w.dcoef, d, d_stride, w.ext, level, nb, s)) {
-#define CALL_UP(A) launch_modup<A>(c, w.dcoef, d, d_stride, 1, w.ext, level, nb, s, pre)
+#define CALL_UP(A) launch_modup<A>(c, w.dcoef, w.ext, level, nb, s, pre)
         DISPATCH_POW2(c->alpha, CALL_UP);
 #undef CALL_UP
     }
@@ -441,7 +502,7 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
     const uint32_t N = c->N, nt = level + c->K;
     const uint32_t beta = (level + c->alpha - 1) / c->alpha;
     const int au = acc_u ? 1 : 0;
-    bool aligned = ((uintptr_t)w.ext & 15) == 0 && ((uintptr_t)w.u & 15) == 0 && (multi || ((uintptr_t)evk & 15) == 0);
+    bool aligned = ((uintptr_t)w.ext & 15) == 0 && ((uintptr_t)w.u & 15) == 0 && ((uintptr_t)w.d & 15) == 0 && (w.d_stride & 1) == 0 && (multi || ((uintptr_t)evk & 15) == 0);
     const uint32_t nkeys = multi ? (multi->group ? nb / multi->group : nb) : 0;
     for (uint32_t b = 0; b < nkeys; b++) aligned = aligned && ((uintptr_t)multi->evk[b] & 15) == 0;
     const bool fast = beta <= IP_MAX_BETA && N >= 2 * THREADS && aligned;
@@ -460,13 +521,13 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
         const dim3 grid(N / (2 * THREADS), grp ? (nb / grp) * ((grp + bch - 1) / bch) : (nb + bch - 1) / bch, nt);
         const KsMulti m = multi ? *multi : KsMulti{};
         switch (beta) {
-        case 1: inner_product_kernel<1><<<grid, THREADS, 0, s>>>(c->dev, w.ext, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au); break;
-        case 2: inner_product_kernel<2><<<grid, THREADS, 0, s>>>(c->dev, w.ext, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au); break;
-        case 3: inner_product_kernel<3><<<grid, THREADS, 0, s>>>(c->dev, w.ext, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au); break;
-        default: inner_product_kernel<4><<<grid, THREADS, 0, s>>>(c->dev, w.ext, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au); break;
+        case 1: inner_product_kernel<1><<<grid, THREADS, 0, s>>>(c->dev, w.ext, w.d, w.d_stride, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au); break;
+        case 2: inner_product_kernel<2><<<grid, THREADS, 0, s>>>(c->dev, w.ext, w.d, w.d_stride, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au); break;
+        case 3: inner_product_kernel<3><<<grid, THREADS, 0, s>>>(c->dev, w.ext, w.d, w.d_stride, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au); break;
+        default: inner_product_kernel<4><<<grid, THREADS, 0, s>>>(c->dev, w.ext, w.d, w.d_stride, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au); break;
         }
     } else {
-        inner_product_generic_kernel<<<dim3(N / THREADS, nb, nt), THREADS, 0, s>>>(c->dev, w.ext, evk, ext_galois, w.u, level, multi ? 1 : 0,
+        inner_product_generic_kernel<<<dim3(N / THREADS, nb, nt), THREADS, 0, s>>>(c->dev, w.ext, w.d, w.d_stride, evk, ext_galois, w.u, level, multi ? 1 : 0,
                                                                                      multi ? *multi : KsMulti{}, au);
     }
     count_launches();
@@ -516,26 +577,27 @@ void ks_inner_moddown(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext
     ks_moddown(c, level, w, add0, add1, add_galois, out, s, nb, add_stride, out_stride, accumulate, tiled, multi);
 }
 
-void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, size_t term_stride, const IpTerms &terms, uint32_t nterm,
+void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, size_t term_stride, size_t d_term_stride, const IpTerms &terms, uint32_t nterm,
                     size_t c0_stride, cudaStream_t s, uint32_t nb, bool acc_u) {
     const uint32_t N = c->N, nt = level + c->K, beta = (level + c->alpha - 1) / c->alpha;
-    bool aligned = ((uintptr_t)w.ext & 15) == 0 && ((uintptr_t)w.u & 15) == 0 && (term_stride & 1) == 0 && (c0_stride & 1) == 0;
+    bool aligned = ((uintptr_t)w.ext & 15) == 0 && ((uintptr_t)w.u & 15) == 0 && (term_stride & 1) == 0 && (c0_stride & 1) == 0 &&
+                   ((uintptr_t)w.d & 15) == 0 && (w.d_stride & 1) == 0 && (d_term_stride & 1) == 0;
     for (uint32_t t = 0; t < nterm; t++) aligned = aligned && ((uintptr_t)terms.evk[t] & 15) == 0 && ((uintptr_t)terms.c0[t] & 15) == 0;
     if (beta <= IP_MAX_BETA && N >= 2 * THREADS && aligned) {
         const dim3 grid(N / (2 * THREADS), (nb + IP_BCH - 1) / IP_BCH, nt);
         const int au = acc_u ? 1 : 0;
         switch (beta) {
-        case 1: inner_product_terms_kernel<1><<<grid, THREADS, 0, s>>>(c->dev, w.ext, term_stride, terms, nterm, c0_stride, w.u, level, nb, au); break;
-        case 2: inner_product_terms_kernel<2><<<grid, THREADS, 0, s>>>(c->dev, w.ext, term_stride, terms, nterm, c0_stride, w.u, level, nb, au); break;
-        case 3: inner_product_terms_kernel<3><<<grid, THREADS, 0, s>>>(c->dev, w.ext, term_stride, terms, nterm, c0_stride, w.u, level, nb, au); break;
-        default: inner_product_terms_kernel<4><<<grid, THREADS, 0, s>>>(c->dev, w.ext, term_stride, terms, nterm, c0_stride, w.u, level, nb, au); break;
+        case 1: inner_product_terms_kernel<1><<<grid, THREADS, 0, s>>>(c->dev, w.ext, term_stride, w.d, d_term_stride, w.d_stride, terms, nterm, c0_stride, w.u, level, nb, au); break;
+        case 2: inner_product_terms_kernel<2><<<grid, THREADS, 0, s>>>(c->dev, w.ext, term_stride, w.d, d_term_stride, w.d_stride, terms, nterm, c0_stride, w.u, level, nb, au); break;
+        case 3: inner_product_terms_kernel<3><<<grid, THREADS, 0, s>>>(c->dev, w.ext, term_stride, w.d, d_term_stride, w.d_stride, terms, nterm, c0_stride, w.u, level, nb, au); break;
+        default: inner_product_terms_kernel<4><<<grid, THREADS, 0, s>>>(c->dev, w.ext, term_stride, w.d, d_term_stride, w.d_stride, terms, nterm, c0_stride, w.u, level, nb, au); break;
         }
         count_launches();
         return;
     }
     // any number of digits, any alignment: one term at a time through the generic kernel, then its P c0
     for (uint32_t t = 0; t < nterm; t++) {
-        inner_product_generic_kernel<<<dim3(N / THREADS, nb, nt), THREADS, 0, s>>>(c->dev, w.ext + t * term_stride, terms.evk[t], terms.galois[t],
+        inner_product_generic_kernel<<<dim3(N / THREADS, nb, nt), THREADS, 0, s>>>(c->dev, w.ext + t * term_stride, w.d + t * d_term_stride, w.d_stride, terms.evk[t], terms.galois[t],
                                                                                      w.u, level, 0, KsMulti{}, (acc_u || t > 0) ? 1 : 0);
         count_launches();
         if (terms.c0[t]) {
