@@ -133,10 +133,8 @@ const char *ckks_last_cuda_error(const ckks_ctx *ctx);
  *                           about a second).  A wait that runs out makes its kernel drain its copies and return, and
  *                           sets the sticky flag ckks_device_status reports; 0 makes every wait that is not already
  *                           satisfied give up at once (used to test that path).
- *   CKKS_OPT_NTT_BULK_STORE N = 2^16 transforms: 1 (default) = in the forward transform's last pass every thread stages its
- *                           16 results in shared memory and a 128-byte bulk copy writes them out, and in the inverse
- *                           transform's first pass every thread's 16 inputs arrive by a 128-byte bulk copy (a bounded wait
- *                           on an mbarrier, see CKKS_OPT_WAIT_CYCLES); 0 = 32-byte global stores and loads.
+ *   CKKS_OPT_NTT_BULK_STORE 0 or 1 (default), kept for programs that set it: it chose between 128-byte bulk copies and 32-byte
+ *                           accesses of the transforms' row passes, which now move 16 bytes per lane either way.
  *   CKKS_OPT_LANES          1..4 (default 4): streams over which the attention entry points spread their independent
  *                           single-ciphertext chains (per channel, per score group).  Lane 0 is the caller's stream, the
  *                           others belong to the context; they are forked from and joined to the caller's stream by events

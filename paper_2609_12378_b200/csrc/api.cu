@@ -81,7 +81,7 @@ int make_plan(const ckks_ctx *c, const ckks_proj_desc *d, ProjPlan &p) {
 
 struct ProjWs { size_t baby, xin, pts, ptt, slots, enc, acc, total, tmp, ks, ksx, rs, bytes; uint32_t gg, gacc, eg; bool per_block, ib_outer; };
 
-constexpr uint32_t BABY_ROTS = 4;            // baby-step rotations per key-switch pass (N = 2^16)
+constexpr uint32_t BABY_ROTS = 4;            // baby-step rotations per key-switch pass
 constexpr uint32_t MAC_GT = 4;               // giants per register tile of the fallback multiply-accumulate kernel
 constexpr uint32_t ENC_PTS = 128;            // plaintexts per encode call of the tensor-core path (its scratch is 13.25 MiB each)
 
@@ -197,9 +197,7 @@ extern "C" int32_t ckks_ntt_butterfly_probe(ckks_ctx *c, uint32_t iters, uint64_
     if (!c || !scratch || !iters || !butterflies) return CKKS_ERR_ARG;
     if (c->log_n != 16) return CKKS_ERR_UNSUPPORTED;
     DeviceGuard g(c->device);
-    int sms = 148;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    if (scratch_words < (size_t)sms * 4 * 256) return CKKS_ERR_WORKSPACE;
+    if (scratch_words < (size_t)c->sms * 4 * 256) return CKKS_ERR_WORKSPACE;
     *butterflies = launch_butterfly_probe(c, iters, (u64 *)scratch, (cudaStream_t)stream);
     return finish(c);
 }
@@ -272,6 +270,30 @@ extern "C" int32_t ckks_add(ckks_ctx *c, const ckks_ct *a, const ckks_ct *b, ckk
     return rc;
 }
 
+// o[2][level][N] += key switch of e2
+static void relinearise(const ckks_ctx *c, const u64 *rlk, const u64 *e2, u64 *o, uint32_t level, KsWorkspace &w, cudaStream_t s) {
+    ks_modup(c, Ptrs(e2, 0), level, w, s);
+    ks_inner(c, rlk, level, 1, w, s);
+    KsOut ko;
+    ko.add = ko.out = Ptrs(o, 0);
+    ko.add_comps = 3;
+    ks_moddown(c, level, w, ko, s);
+}
+// rotation of nb ciphertexts by one key: c0, c1 at in, in + level * N
+static void rotate_ks(const ckks_ctx *c, const ckks_evk *key, const Ptrs &in, const Ptrs &out, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb = 1,
+                      bool accumulate = false) {
+    Ptrs c1 = in;
+    const size_t ptl = (size_t)level * c->N;
+    if (in.n) for (uint32_t b = 0; b < in.n; b++) c1.p[b] += ptl;
+    else c1.base += ptl;
+    ks_modup(c, c1, level, w, s, nb);
+    ks_inner(c, (const u64 *)key->data, level, key->galois, w, s, nb);
+    KsOut ko;
+    ko.add = in; ko.out = out;
+    ko.add_comps = 1; ko.galois = key->galois; ko.accumulate = accumulate;
+    ks_moddown(c, level, w, ko, s, nb);
+}
+
 extern "C" int32_t ckks_mul_relin(ckks_ctx *c, const ckks_ct *a, const ckks_ct *b, const ckks_evk *rlk, ckks_ct *out, void *ws,
                                   size_t ws_bytes, void *stream) {
     if (!c || !ct_ok(a) || !ct_ok(b) || !ct_ok(out) || a->ncomp != 2 || b->ncomp != 2) return CKKS_ERR_ARG;
@@ -285,8 +307,7 @@ extern "C" int32_t ckks_mul_relin(ckks_ctx *c, const ckks_ct *a, const ckks_ct *
     KsWorkspace w = ks_carve(c, level, e2 + (size_t)level * c->N);
     u64 *o = (u64 *)out->data;
     launch_tensor(c, (const u64 *)a->data, (const u64 *)b->data, o, e2, level, s);
-    ks_modup(c, e2, level, w, s);
-    ks_inner_moddown(c, (const u64 *)rlk->data, level, 1, w, o, o + (size_t)level * c->N, 1, o, s);
+    relinearise(c, (const u64 *)rlk->data, e2, o, level, w, s);
     int rc = finish(c);
     if (rc == CKKS_OK) { out->level = level; out->ncomp = 2; out->scale = a->scale * b->scale; }
     return rc;
@@ -325,8 +346,12 @@ extern "C" int32_t ckks_mul_relin_batch(ckks_ctx *c, const ckks_ct *a, const ckk
         for (uint32_t i = 0; i < m; i++)
             launch_tensor(c, (const u64 *)a[i0 + i].data, (const u64 *)b[i0 + i].data, stage + (size_t)i * ctl, e2 + (size_t)i * ptl, level, s);
         // the m key switches run side by side: one ModUp, one inner product, one ModDown over the whole chunk
-        ks_modup(c, e2, level, w, s, m, ptl);
-        ks_inner_moddown(c, (const u64 *)rlk->data, level, 1, w, stage, stage + ptl, 1, stage, s, m, ctl, ctl, false);
+        ks_modup(c, Ptrs(e2, ptl), level, w, s, m);
+        ks_inner(c, (const u64 *)rlk->data, level, 1, w, s, m);
+        KsOut ko;
+        ko.add = ko.out = Ptrs(stage, ctl);
+        ko.add_comps = 3;
+        ks_moddown(c, level, w, ko, s, m);
         for (uint32_t i = 0; i < m; i++)
             cudaMemcpyAsync(out[i0 + i].data, stage + (size_t)i * ctl, ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
     }
@@ -358,8 +383,7 @@ extern "C" int32_t ckks_mul_relin_sum(ckks_ctx *c, const ckks_ct *a, const ckks_
     std::vector<const u64 *> pa(n), pb(n);
     for (uint32_t i = 0; i < n; i++) { pa[i] = (const u64 *)a[i].data; pb[i] = (const u64 *)b[i].data; }
     launch_tensor_sum(c, pa.data(), pb.data(), n, o, e2, level, s);
-    ks_modup(c, e2, level, w, s);
-    ks_inner_moddown(c, (const u64 *)rlk->data, level, 1, w, o, o + (size_t)level * c->N, 1, o, s);
+    relinearise(c, (const u64 *)rlk->data, e2, o, level, w, s);
     int rc = finish(c);
     if (rc == CKKS_OK) { out->level = level; out->ncomp = 2; out->scale = a[0].scale * b[0].scale; }
     return rc;
@@ -432,7 +456,7 @@ extern "C" int32_t ckks_poly_eval(ckks_ctx *c, const ckks_ct *x, const double *c
     const u64 *xd = (const u64 *)x->data;
     // r = x * c_d; rescale; + c_{d-1}
     launch_const(c, xd, vs[degree], true, ra, 2, level, s);
-    launch_rescale(c, ra, rb, 2, level, rsw, s);
+    launch_rescale(c, Ptrs(ra, 0), Ptrs(rb, 0), 2, level, rsw, s);
     uint32_t lvl = level - 1;
     launch_const(c, rb, vs[degree - 1], false, rb, 2, lvl, s);
     u64 *cur = rb, *other = ra;
@@ -442,9 +466,8 @@ extern "C" int32_t ckks_poly_eval(ckks_ctx *c, const ckks_ct *x, const double *c
             cudaMemcpyAsync(xt + (size_t)comp * lvl * N, xd + (size_t)comp * level * N, (size_t)lvl * N * sizeof(u64), cudaMemcpyDeviceToDevice, s);
         KsWorkspace w = ks_carve(c, lvl, ksw);
         launch_tensor(c, cur, xt, other, e2, lvl, s);
-        ks_modup(c, e2, lvl, w, s);
-        ks_inner_moddown(c, (const u64 *)rlk->data, lvl, 1, w, other, other + (size_t)lvl * N, 1, other, s);
-        launch_rescale(c, other, cur, 2, lvl, rsw, s);
+        relinearise(c, (const u64 *)rlk->data, e2, other, lvl, w, s);
+        launch_rescale(c, Ptrs(other, 0), Ptrs(cur, 0), 2, lvl, rsw, s);
         lvl--;
         launch_const(c, cur, vs[k], false, cur, 2, lvl, s);
     }
@@ -505,9 +528,8 @@ extern "C" int32_t ckks_poly_eval_tree(ckks_ctx *c, const ckks_ct *x, const doub
         if (lvl[b] != lv) { truncate(pb, lvl[b], lv, tb); pb = tb; }
         KsWorkspace w = ks_carve(c, lv, ksw);
         launch_tensor(c, pa, pb, prod, e2, lv, s);
-        ks_modup(c, e2, lv, w, s);
-        ks_inner_moddown(c, (const u64 *)rlk->data, lv, 1, w, prod, prod + (size_t)lv * N, 1, prod, s);
-        launch_rescale(c, prod, pw + (size_t)(k - 2) * ctw, 2, lv, rsw, s);
+        relinearise(c, (const u64 *)rlk->data, e2, prod, lv, w, s);
+        launch_rescale(c, Ptrs(prod, 0), Ptrs(pw + (size_t)(k - 2) * ctw, 0), 2, lv, rsw, s);
     }
     bool first = true;
     for (uint32_t k = 1; k <= degree; k++) {
@@ -518,7 +540,7 @@ extern "C" int32_t ckks_poly_eval_tree(ckks_ctx *c, const ckks_ct *x, const doub
         if (!first) launch_add(c, acc, term, acc, 2, Lt, s);
         first = false;
     }
-    launch_rescale(c, acc, (u64 *)out->data, 2, Lt, rsw, s);
+    launch_rescale(c, Ptrs(acc, 0), Ptrs((u64 *)out->data, 0), 2, Lt, rsw, s);
     launch_const(c, (const u64 *)out->data, vs[0], false, (u64 *)out->data, 2, Lt - 1, s);
     int rc = finish(c);
     if (rc == CKKS_OK) { out->level = Lt - 1; out->ncomp = 2; out->scale = so; }
@@ -775,9 +797,7 @@ extern "C" int32_t ckks_rotate(ckks_ctx *c, const ckks_ct *in, const ckks_evk *k
     cudaStream_t s = (cudaStream_t)stream;
     const uint32_t level = in->level;
     KsWorkspace w = ks_carve(c, level, ws);
-    const u64 *c0 = (const u64 *)in->data, *c1 = c0 + (size_t)level * c->N;
-    ks_modup(c, c1, level, w, s);
-    ks_inner_moddown(c, (const u64 *)key->data, level, key->galois, w, c0, nullptr, key->galois, (u64 *)out->data, s);
+    rotate_ks(c, key, Ptrs((const u64 *)in->data, 0), Ptrs((const u64 *)out->data, 0), level, w, s);
     rc = finish(c);
     if (rc == CKKS_OK) { out->level = level; out->ncomp = 2; out->scale = in->scale; }
     return rc;
@@ -803,8 +823,7 @@ extern "C" int32_t ckks_rotate_batch(ckks_ctx *c, const ckks_ct *in, uint32_t n,
         KsWorkspace w = ks_carve(c, level, xout + (size_t)m * ctl, m);
         for (uint32_t i = 0; i < m; i++)
             cudaMemcpyAsync(xin + (size_t)i * ctl, in[i0 + i].data, ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
-        ks_modup(c, xin + ptl, level, w, s, m, ctl);
-        ks_inner_moddown(c, (const u64 *)key->data, level, key->galois, w, xin, nullptr, key->galois, xout, s, m, ctl, ctl, false);
+        rotate_ks(c, key, Ptrs(xin, ctl), Ptrs(xout, ctl), level, w, s, m);
         for (uint32_t i = 0; i < m; i++)
             cudaMemcpyAsync(out[i0 + i].data, xout + (size_t)i * ctl, ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
     }
@@ -838,7 +857,7 @@ extern "C" int32_t ckks_rotate_sum(ckks_ctx *c, const ckks_ct *in, const ckks_ev
         const uint32_t m = std::min(MRB_CHUNK, n - i0);
         for (uint32_t i = 0; i < m; i++)
             cudaMemcpyAsync(xin + (size_t)i * ctl, in[i0 + i].data, ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
-        ks_modup(c, xin + ptl, level, w, s, m, ctl);
+        ks_modup(c, Ptrs(xin + ptl, ctl), level, w, s, m);
         // every term has its own digits, key and first component; all of them add into entry 0 of the inner-product
         // buffer, the first components multiplied by P so that the one ModDown returns them unchanged
         for (uint32_t t0 = 0; t0 < m; t0 += IP_TERMS) {
@@ -851,11 +870,13 @@ extern "C" int32_t ckks_rotate_sum(ckks_ctx *c, const ckks_ct *in, const ckks_ev
             }
             KsWorkspace wt = w;
             wt.ext = w.ext + (size_t)t0 * beta * nt * N;
-            wt.d = w.d + (size_t)t0 * ctl;
-            ks_inner_terms(c, level, wt, (size_t)beta * nt * N, ctl, tm, nterm, 0, s, 1, i0 + t0 > 0);
+            wt.d.base += (size_t)t0 * ctl;
+            ks_inner_terms(c, level, wt, (size_t)beta * nt * N, tm, nterm, 0, s, 1, i0 + t0 > 0);
         }
     }
-    ks_moddown(c, level, w, nullptr, nullptr, 1, (u64 *)out->data, s);
+    KsOut ko;
+    ko.out = Ptrs((const u64 *)out->data, 0);
+    ks_moddown(c, level, w, ko, s);
     int rc = finish(c);
     if (rc == CKKS_OK) { out->level = level; out->ncomp = 2; out->scale = in[0].scale; }
     return rc;
@@ -878,12 +899,16 @@ extern "C" int32_t ckks_rotate_hoisted(ckks_ctx *c, const ckks_ct *in, const ckk
     w.u = w.ext + beta * nt * N;
     w.conv = w.u + (size_t)nbh * 2 * nt * N;
     const u64 *c0 = (const u64 *)in->data, *c1 = c0 + (size_t)level * N;
-    ks_modup(c, c1, level, w, s);
+    ks_modup(c, Ptrs(c1, 0), level, w, s);
+    KsOut ko;
+    ko.add = Ptrs(c0, 0);
+    ko.add_comps = 1;
     for (uint32_t r0 = 0; r0 < nrot; r0 += nbh) {
         const uint32_t nb = std::min(nbh, nrot - r0);
         KsMulti m{};
         for (uint32_t b = 0; b < nb; b++) { m.evk[b] = (const u64 *)keys[r0 + b].data; m.galois[b] = keys[r0 + b].galois; m.out[b] = (u64 *)outs[r0 + b].data; }
-        ks_inner_moddown(c, nullptr, level, 1, w, c0, nullptr, 1, nullptr, s, nb, 0, 0, false, TiledOut(), &m);
+        ks_inner(c, nullptr, level, 1, w, s, nb, false, &m);
+        ks_moddown(c, level, w, ko, s, nb, &m);
     }
     rc = finish(c);
     if (rc == CKKS_OK)
@@ -897,7 +922,7 @@ extern "C" int32_t ckks_rescale(ckks_ctx *c, const ckks_ct *in, ckks_ct *out, vo
     if (!out->data || (in->ncomp > 1 && in->data == out->data)) return CKKS_ERR_ARG;
     if (!ws || ws_bytes < rescale_bytes(c, in->level, in->ncomp)) return CKKS_ERR_WORKSPACE;
     DeviceGuard g(c->device);
-    launch_rescale(c, (const u64 *)in->data, (u64 *)out->data, in->ncomp, in->level, (u64 *)ws, (cudaStream_t)stream);
+    launch_rescale(c, Ptrs((const u64 *)in->data, 0), Ptrs((u64 *)out->data, 0), in->ncomp, in->level, (u64 *)ws, (cudaStream_t)stream);
     int rc = finish(c);
     if (rc == CKKS_OK) {
         const double ql = (double)c->mod[in->level - 1];
@@ -997,30 +1022,26 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
         for (uint32_t comp = 0; comp < 2; comp++)
             launch_to_tiled(c, xb + comp * ptl, xs, nx, baby, Rx, comp, 2 * B, level, s);
         if (B <= 1) return;
-        ks_modup(c, xb + ptl, level, kw, s, nx, xs);
-        // N = 2^16: BABY_ROTS rotations of all inputs per pass (the digits of a limb are fetched once for all of them and
-        // the launches are four times larger); the inner-product and conversion buffers follow the digits
-        const uint32_t rots = c->log_n == 16 ? BABY_ROTS : 1;       // the grouped ModDown tail exists for N = 2^16 only
+        ks_modup(c, Ptrs(xb + ptl, xs), level, kw, s, nx);
+        // BABY_ROTS rotations of all inputs per pass (the digits of a limb are fetched once for all of them and the launches
+        // are four times larger); the inner-product and conversion buffers follow the digits
         KsWorkspace kb = kw;
         kb.u = kw.ext + (size_t)nx * kbeta * knt * N;
-        kb.conv = kb.u + (size_t)rots * nx * 2 * knt * N;
-        for (uint32_t b = 1; b < B; b += rots) {
-            const uint32_t nr = std::min(rots, B - b);
-            TiledOut to;
-            to.R = Rx; to.row0 = 2 * b; to.row_stride = 2 * B;
-            if (rots == 1) {
-                const u64 ge = ckks_galois_element(c, (int64_t)b * T);
-                ks_inner_moddown(c, (const u64 *)find_key(keys, nkeys, ge)->data, level, ge, kw, xb, nullptr, ge, baby, s, nx, xs, 0,
-                                 false, to);
-                continue;
-            }
+        kb.conv = kb.u + (size_t)BABY_ROTS * nx * 2 * knt * N;
+        for (uint32_t b = 1; b < B; b += BABY_ROTS) {
+            const uint32_t nr = std::min(BABY_ROTS, B - b);
+            KsOut ko;
+            ko.add = Ptrs(xb, xs); ko.out = Ptrs(baby, 0);
+            ko.add_comps = 1;
+            ko.tiled.R = Rx; ko.tiled.row0 = 2 * b; ko.tiled.row_stride = 2 * B;
             KsMulti m{};
             m.group = nx; m.rot_rows = 2;
             for (uint32_t r = 0; r < nr; r++) {
                 m.galois[r] = ckks_galois_element(c, (int64_t)(b + r) * T);
                 m.evk[r] = (const u64 *)find_key(keys, nkeys, m.galois[r])->data;
             }
-            ks_inner_moddown(c, nullptr, level, 1, kb, xb, nullptr, 1, baby, s, nr * nx, xs, 0, false, to, &m);
+            ks_inner(c, nullptr, level, 1, kb, s, nr * nx, false, &m);
+            ks_moddown(c, level, kb, ko, s, nr * nx, &m);
         }
     };
     if (!L.ib_outer) baby_steps(0);
@@ -1051,10 +1072,8 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
                         continue;
                     }
                     const u64 ge = ckks_galois_element(c, (int64_t)gi * B * T);
-                    const u64 *key = (const u64 *)find_key(keys, nkeys, ge)->data;
                     // total[sh] += rotate(acc_g[sh]) for all shards in one batch
-                    ks_modup(c, ag + ptl, level, kw, s, S, ctl);
-                    ks_inner_moddown(c, key, level, ge, kw, ag, nullptr, ge, total, s, S, ctl, ctl, true);
+                    rotate_ks(c, find_key(keys, nkeys, ge), Ptrs(ag, ctl), Ptrs(total, ctl), level, kw, s, S, true);
                 }
                 // lazy: the key-switched parts of up to IP_TERMS giant steps (all shards) are extended in one batch and
                 // added to the running sum in the key-switching basis in one pass, their first components with them
@@ -1066,7 +1085,7 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
                     }
                     const uint32_t nterm = std::min(IP_TERMS, ng - gl);
                     u64 *ag = acc + (size_t)gl * S * ctl;
-                    ks_modup(c, ag + ptl, level, kx, s, nterm * S, ctl);
+                    ks_modup(c, Ptrs(ag + ptl, ctl), level, kx, s, nterm * S);
                     IpTerms tm{};
                     for (uint32_t t = 0; t < nterm; t++) {
                         const u64 ge = ckks_galois_element(c, (int64_t)(g0 + gl + t) * B * T);
@@ -1074,7 +1093,7 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
                         tm.galois[t] = ge;
                         tm.c0[t] = ag + (size_t)t * S * ctl;
                     }
-                    ks_inner_terms(c, level, kx, (size_t)S * kbeta * knt * N, (size_t)S * ctl, tm, nterm, ctl, s, S, u_live);
+                    ks_inner_terms(c, level, kx, (size_t)S * kbeta * knt * N, tm, nterm, ctl, s, S, u_live);
                     u_live = true;
                     gl += nterm;
                 }
@@ -1157,18 +1176,21 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
                 }
                 giant_steps(acc, g0, ng);
             }
-            if (u_live) ks_moddown(c, level, kw, total, total + ptl, 1, total, s, S, ctl, ctl, false);
+            if (u_live) {
+                KsOut ko;
+                ko.add = ko.out = Ptrs(total, ctl);
+                ko.add_comps = 3;
+                ks_moddown(c, level, kw, ko, s, S);
+            }
             for (uint32_t f = o.size; fold > 1; f *= 2, fold /= 2) {
                 const u64 ge = ckks_galois_element(c, (int64_t)f * T);
-                const u64 *key = (const u64 *)find_key(keys, nkeys, ge)->data;
                 // total += rotate(total): the rotated copy goes to the (now free) accumulator buffer first
-                ks_modup(c, total + ptl, level, kw, s, S, ctl);
-                ks_inner_moddown(c, key, level, ge, kw, total, nullptr, ge, acc, s, S, ctl, ctl, false);
+                rotate_ks(c, find_key(keys, nkeys, ge), Ptrs(total, ctl), Ptrs(acc, ctl), level, kw, s, S);
                 for (uint32_t sh = 0; sh < S; sh++)
                     launch_add(c, total + (size_t)sh * ctl, acc + (size_t)sh * ctl, total + (size_t)sh * ctl, 2, level, s);
             }
             for (uint32_t sh = 0; sh < S; sh++)
-                launch_rescale(c, total + (size_t)sh * ctl, (u64 *)out_m[sh * nob + ob].data, 2, level, rsw, s);
+                launch_rescale(c, Ptrs(total + (size_t)sh * ctl, 0), Ptrs((u64 *)out_m[sh * nob + ob].data, 0), 2, level, rsw, s);
         }
         out_m += S * nob;
     }

@@ -24,14 +24,14 @@ struct DevTables {
     const u64 *mu;           // [T] floor(2^112 / prime)
     const u64 *mu64;         // [T] floor(2^64 / prime)
     const double2 *modd;     // [T] {prime, 1/prime} as doubles
-    const ulonglong2 *tw_fwd;  // [T][N] {psi^bitrev(i), Shoup companion}, index m+i
+    const ulonglong2 *tw_fwd;  // [T][N] {psi^bitrev(i), Shoup companion}, index m+i (integer transform: N = 2^16 only)
     const ulonglong2 *tw_inv;  // [T][N] inverses of the same
     const ulonglong2 *n_inv;   // [T] {N^-1, Shoup}
-    // fp64 copies for the double-precision NTT path (N = 2^16 only): the centred representative of w as a double, same
+    // fp64 tables of the transform: the centred representative of w as a double, same
     // indexing (the transform estimates a product's quotient from the rounded product and 1/q, so the table holds w alone)
     const double *twd_fwd, *twd_inv;    // [T][N]
     const double2 *n_inv_d;             // [T][2] {N^-1, N^-1/q}, {w N^-1, that/q} for the inverse's last twiddle w, all centred
-    // inverse-transform scalings that deliver the basis conversions' first factor y = [d qhat^-1] (N = 2^16 only), pairs
+    // inverse-transform scalings that deliver the basis conversions' first factor y = [d qhat^-1], pairs
     // {N^-1 qhat^-1, last inverse twiddle times that}, each {v, v / prime} centred
     const double2 *inv_scale_up;   // [(L+1)][L][2]   ModUp: level, limb
     const double2 *inv_scale_dn;   // [K][2]          ModDown: special limb
@@ -41,7 +41,6 @@ struct DevTables {
     // ModDown:
     const ulonglong2 *dn_hat_inv;  // [K]      {Phat_k^-1 mod p_k, Shoup}
     const double *dn_hat_mod_d;    // [L][K]   centred Phat_k mod q_i
-    const ulonglong2 *dn_p_inv;    // [L]      {P^-1 mod q_i, Shoup}
     const double2 *dn_p_inv_d;     // [L]      {P^-1 mod q_i, that / q_i} as doubles
     const double *dn_p_mod_d;      // [L]      P mod q_i as a double
     // Tensor-core basis conversion (conv_mma.cu; conv_groups = 0 when alpha or K exceeds 8 sources): byte matrices of
@@ -51,8 +50,8 @@ struct DevTables {
     const uint32_t *dn_bmat;       // [conv_groups][13][2][64]
     const double2 *two52_d;        // [T] {2^52 mod prime, that / prime}
     uint32_t conv_groups;
-    // Rescale: [L(last)][L(i)] {q_last^-1 mod q_i, Shoup}
-    const ulonglong2 *rs_inv;
+    // Rescale:
+    const double2 *rs_inv_d;       // [L(last)][L(i)] {q_last^-1 mod q_i, that / q_i} as doubles
     // Encode:
     const uint32_t *enc_src;       // [n] slot index feeding FFT input position pos (bit-reversed e_j)
     const double2 *enc_omega;      // [n] exp(2 pi i t / n)
@@ -64,7 +63,7 @@ struct DevTables {
 
 struct ckks_ctx {
     uint32_t log_n, N, n, L, K, dnum, alpha, T;
-    int device;
+    int device, sms;
     std::vector<u64> mod;        // host copy of the primes
     std::vector<u64> pow5;       // 5^j mod 2N, j < n (host)
     DevTables dev;               // pointers into `allocs`
@@ -72,7 +71,7 @@ struct ckks_ctx {
     std::string cuda_error;
     // options (ckks_context_set_option); host-side state read when a call is made
     uint32_t ntt_fp_share = 8;               // of every 8 limbs, how many take the double-precision NTT path
-    int ntt_bulk_store = 1;                  // forward row pass (N = 2^16): results leave as 128-byte bulk copies from shared memory
+    int ntt_bulk_store = 1;                  // kept for get and set; selects nothing
     int conv_kernel = 0;                     // basis conversions: 0 = FP64 pipe, 1 = tensor cores (conv_mma.cu)
     int mac_kernel = 82;                     // projection multiply-accumulate kernel (see launch_mac_mma)
     long long wait_cycles = 2000000000ll;    // clock bound of every device-side wait (about a second)
@@ -137,13 +136,15 @@ struct TiledOut { uint32_t R = 0, row0 = 0, row_stride = 0; };
 //           x < level, else p_{x-level}; with skip_own the digit's own limbs
 //           (which never leave the evaluation domain) are skipped.
 // ---------------------------------------------------------------------------
-struct LimbMap {
+struct LimbMap {      // kind 2: prime = first for every limb
     uint32_t kind, first, period, pitch, level, L, alpha, nbeta, skip_own;
 };
 // limbs [..][period][N] contiguous, limb x of every period under prime first + x
 inline LimbMap plain_map(uint32_t first, uint32_t period) { return LimbMap{0, first, period, period, 0, 0, 0, 1, 0}; }
 // same, but consecutive periods start `pitch` limbs apart (a sub-range of limbs of a larger array)
 inline LimbMap pitched_map(uint32_t first, uint32_t period, uint32_t pitch) { return LimbMap{0, first, period, pitch, 0, 0, 0, 1, 0}; }
+// limbs [..][period][N], all under one prime
+inline LimbMap same_map(uint32_t prime, uint32_t period) { return LimbMap{2, prime, period, period, 0, 0, 0, 1, 0}; }
 // extended digits [batch][beta][level + K]
 inline LimbMap ext_map(uint32_t level, uint32_t K, uint32_t L, uint32_t alpha, uint32_t beta) {
     return LimbMap{1, 0, level + K, level + K, level, L, alpha, beta, 1};
@@ -152,6 +153,7 @@ inline LimbMap ext_map(uint32_t level, uint32_t K, uint32_t L, uint32_t alpha, u
 __host__ __device__ inline int limb_prime(const LimbMap &m, uint32_t y) {
     uint32_t x = y % m.period;
     if (m.kind == 0) return (int)(m.first + x);
+    if (m.kind == 2) return (int)m.first;
     if (m.skip_own) {
         uint32_t j = (y / m.period) % m.nbeta, lo = j * m.alpha, hi = lo + m.alpha < m.level ? lo + m.alpha : m.level;
         if (x >= lo && x < hi) return -1;
@@ -243,25 +245,42 @@ __device__ __forceinline__ u64 d_to_u64(double v) { return (u64)__double_as_long
 __device__ __forceinline__ u64 canonical_d(double v, double q) { return d_to_u64(v < 0.0 ? __dadd_rn(v, q) : v); }
 
 __device__ __forceinline__ uint32_t bitrev_n(uint32_t x, uint32_t bits) { return __brev(x) >> (32 - bits); }
-// index p' with stored[p] of sigma_g(a) = stored[p'] of a (evaluation domain, bit-reversed); g = 1: identity
-__device__ __forceinline__ uint32_t galois_src(uint32_t p, u64 g, uint32_t log_n, uint32_t N) {
+// index p' with stored[p] of sigma_g(a) = stored[p'] of a (evaluation domain, bit-reversed); g = 1: identity.  The exponents
+// live modulo 2N <= 2^17, so 32-bit products do.
+__device__ __forceinline__ uint32_t galois_src(uint32_t p, uint32_t g, uint32_t log_n) {
     if (g == 1) return p;
-    const u64 e = (g * (2ull * bitrev_n(p, log_n) + 1)) & (2ull * N - 1);
-    return bitrev_n((uint32_t)((e - 1) >> 1), log_n);
+    const uint32_t e = g * (2 * bitrev_n(p, log_n) + 1);
+    return bitrev_n((e >> 1) & ((1u << log_n) - 1), log_n);
 }
+// centred representative of a canonical residue
+__device__ __forceinline__ double centre_d(u64 v, u64 q) { return v > (q >> 1) ? __dsub_rn(u64_to_d(v), (double)q) : u64_to_d(v); }
 
 // Kernel launches issued by this library since it was loaded (all contexts, all streams).
 extern unsigned long long g_kernel_launches;
 inline void count_launches(unsigned n = 1) { g_kernel_launches += n; }
 
+// Launches are programmatic dependent launches: a kernel's CTAs may become resident as soon as every CTA of the kernel before
+// it on the stream has exited, and grid_dep_sync waits until that kernel's writes are visible.  Until then a kernel may only
+// read the context's tables.  Between dependent kernels of a few microseconds this hides the launch latency and the table
+// fetches (a rotation of one ciphertext, 11 launches: 208 -> 186 us).  No kernel triggers its dependents earlier: CTAs that
+// wait for the last wave of a large launch take the slots and the issue cycles it needs (64 hoisted rotations 1 % slower,
+// the 4096 x 4096 projection 3 %).
+__device__ __forceinline__ void grid_dep_sync() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+template <class... P, class... A>
+inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    count_launches();
+}
+
 // ---------------------------------------------------------------------------
 // Internal launchers (each validates nothing; the C ABI layer does).
 // ---------------------------------------------------------------------------
-// Optional epilogue of the forward transform (N = 2^16 path): instead of storing NTT(conv) the last pass finishes the
-// ModDown: out[b][comp][i][p] (+)= (u[b][comp][i][p] - NTT(conv)[p]) P^-1 + sigma_g(add_comp)[b][i][p], for a buffer of
-// limbs laid out [b][comp][level]; `out` in the plain layout (out_stride words per b) or tiled (tl.R != 0).
-// mode 2: the transform's own result is stored, but into a tiled buffer: limb y = b * level + i becomes row
-// tl.row0 + b * tl.row_stride, limb i.
 // Up to KS_MULTI key switches that share one set of extended digits but differ in key, Galois element and output
 // buffer (hoisted rotations): batch entry b uses evk[b], galois[b], out[b].
 constexpr uint32_t KS_MULTI = 16;
@@ -269,40 +288,71 @@ struct KsMulti {
     const u64 *evk[KS_MULTI];
     u64 galois[KS_MULTI];
     u64 *out[KS_MULTI];
-    // group > 0 (N = 2^16 only): `group` ciphertexts with their own digits take every one of the keys; batch entry
-    // b = r * group + m is key r applied to member m's digits, added to member m's addend, and written to the tiled
-    // row  row0 + r * rot_rows + m * row_stride + component  (out[] is not used)
+    // group > 0: `group` ciphertexts with their own digits take every one of the keys; batch entry b = r * group + m is key r
+    // applied to member m's digits, added to member m's addend, and written to the tiled row
+    // row0 + r * rot_rows + m * row_stride + component, or (plain layout) to out + r * rot_stride + m * out_stride words
+    // (out[] is not used)
     uint32_t group, rot_rows;
+    size_t rot_stride;
 };
 
+// Batch entries of a buffer: entry b at base + b * stride words, or (n > 0) at p[b]
+struct Ptrs {
+    const u64 *base = nullptr;
+    size_t stride = 0;
+    uint32_t n = 0;
+    const u64 *p[KS_MULTI] = {};
+    Ptrs() = default;
+    __host__ __device__ Ptrs(const u64 *b, size_t s) : base(b), stride(s) {}
+    __host__ __device__ const u64 *at(uint32_t b) const { return n ? p[b] : base + b * stride; }
+};
+
+// Epilogue of the forward transform, for a buffer of limbs laid out [b][ncomp][level].
+//   mode 1: instead of storing NTT(conv) the last pass finishes a ModDown or a rescale:
+//           out[b][comp][i][p] (+)= (u[b][comp][i][p] - NTT(conv)[p]) pinv[i] + sigma_g(add[b][comp][i])[p]
+//           u: [ncomp][nt][N] words per entry; add: [..][level][N] words, taken for the components in the mask add_comps;
+//           out: plain ([ncomp][level][N] per entry) or tiled (tl.R != 0, component comp of entry b in row
+//           tl.row0 + b * tl.row_stride + comp)
+//   mode 2: the transform's own result is stored, but into a tiled buffer (out.base): limb y = b * level + i becomes row
+//           tl.row0 + b * tl.row_stride, limb i
 struct NttEpilogue {
-    int mode;      // 1 = ModDown tail, 2 = tiled store
-    const u64 *u, *add0, *add1;
-    u64 *out;
-    size_t add_stride, out_stride;
+    int mode;
+    Ptrs u, add, out;
+    const double2 *pinv;   // [level] {constant, constant / q_i}
+    uint32_t add_comps, ncomp, level, nt;
     u64 galois;
-    uint32_t level, nt;
     int accumulate;
     TiledOut tl;
-    int multi;             // mode 1: batch entry b adds through mgalois[b] and writes to mout[b]
+    int multi;             // batch entry b adds through mgalois[b]
     u64 mgalois[KS_MULTI];
-    u64 *mout[KS_MULTI];
-    uint32_t group, rot_rows;   // KsMulti's grouped form
+    // KsMulti's grouped form: entry b = r * group + m takes mgalois[r] and add.at(m) and goes to row
+    // tl.row0 + r * rot_rows + m * tl.row_stride + comp, or to out.base + r * rot_stride + m * out.stride
+    uint32_t group, rot_rows;
+    size_t rot_stride;
+    uint32_t y0;           // (filled in) first limb of the launch
 };
-// coef_src (forward, N = 2^16 path only): the first pass reads signed 64-bit coefficients [batch][N] (batch = limb
-// index / map.period) and reduces them modulo the limb's prime on the fly instead of reading `base`.
-// inv_src (inverse, N = 2^16 path only): the first pass reads its limbs from another buffer whose periods start
-// inv_src_pitch limbs apart, so the transform runs out of place and the input stays intact.
-// inv_scale (inverse, N = 2^16 path only): pairs [map.period][2] that replace {N^-1, last twiddle N^-1} for limb x of every
-// period (device pointer), so that the output is scaled by a per-limb constant.
+// Prologue of the forward transform: the first pass reads one buffer [batch][N] (batch = limb index / map.period) instead of
+// `base`: signed 64-bit coefficients, or (lift) residues modulo prime src_prime whose centred representatives are meant.
+struct NttPrologue {
+    const u64 *src;
+    bool lift;
+    uint32_t src_prime;
+};
+// Source of the inverse transform: the first pass reads limb x of entry b at ptr.at(b) + x * lpitch limbs, so the transform
+// runs out of place and the input stays as it is (b = limb index / map.period, x = limb index % map.period).
+struct NttSource {
+    Ptrs ptr;
+    uint32_t lpitch = 0;
+};
+// inv_scale (inverse): pairs [map.period][2] that replace {N^-1, last twiddle N^-1} for limb x of every period (device
+// pointer), so that the output is scaled by a per-limb constant.
 void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbMap &map, bool inverse, cudaStream_t s,
-                const NttEpilogue *ep = nullptr, const long long *coef_src = nullptr, const u64 *inv_src = nullptr,
-                uint32_t inv_src_pitch = 0, const double2 *inv_scale = nullptr);
+                const NttEpilogue *ep = nullptr, const NttPrologue *pro = nullptr, const NttSource *src = nullptr, const double2 *inv_scale = nullptr);
+void launch_ntt_int(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, bool inverse, const u64 *src, uint32_t src_pitch, cudaStream_t s);
 
 void launch_mul_plain_acc(const ckks_ctx *c, const u64 *const *cts, u64 *const *accs, uint32_t ncts, const u64 *pt,
                           uint32_t level, bool init, cudaStream_t s);
 void launch_add(const ckks_ctx *c, const u64 *a, const u64 *b, u64 *out, uint32_t ncomp, uint32_t level, cudaStream_t s);
-void launch_automorphism(const ckks_ctx *c, const u64 *in, u64 *out, uint32_t nlimbs, u64 galois, cudaStream_t s);
 void launch_tensor(const ckks_ctx *c, const u64 *a, const u64 *b, u64 *e01, u64 *e2, uint32_t level, cudaStream_t s);
 // slot values 1.0 on the slots x with lo <= x / B < hi and t0 <= x % Ti < t1, else 0.0 (n doubles on the device)
 void launch_slot_mask(const ckks_ctx *c, double *out, uint32_t B, uint32_t lo, uint32_t hi, uint32_t Ti, uint32_t t0, uint32_t t1, cudaStream_t s);
@@ -315,37 +365,36 @@ void launch_tensor_sum(const ckks_ctx *c, const u64 *const *a, const u64 *const 
                        cudaStream_t s);
 
 // Key switch pieces.  Sizes in limbs: d [level], ext [beta][level+K], u [2][level+K], conv [2][level].
-// d, d_stride: the evaluation-domain input of the last ks_modup (batch entries d_stride words apart).  A digit's own limbs
-// are not copied into ext; the inner product reads them from d, which has to stay as it is until then.
+// d: the evaluation-domain input of the last ks_modup.  A digit's own limbs are not copied into ext; the inner product reads
+// them from d, which has to stay as it is until then.
 struct KsWorkspace {
     u64 *dcoef, *ext, *u, *conv;
-    const u64 *d = nullptr;
-    size_t d_stride = 0;
+    Ptrs d;
 };
 size_t ks_workspace_limbs(const ckks_ctx *c, uint32_t level);
 KsWorkspace ks_carve(const ckks_ctx *c, uint32_t level, void *ws, uint32_t nb = 1);
-// nb key switches side by side (batch entry b reads d + b * d_stride words, d_stride a multiple of N):
-// d (evaluation domain, [level][N]) -> ext (evaluation domain, all digits).  A rotation applies its sigma_g to the
-// extended digits when the inner product reads them (ext_galois below): the centred conversion commutes with the
-// permutation and the sign flips of sigma_g, so this equals extending sigma_g(d), and d is never copied.
-void ks_modup(const ckks_ctx *c, const u64 *d, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb = 1, size_t d_stride = 0);
-// inner product with evk (digits read through sigma_{ext_galois}; 1 = identity), ModDown, and the final
-// combination out_c (+)= sigma_{add_galois}(add_c) + k_c.  add0/add1 may be null.
-void ks_inner_moddown(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w,
-                      const u64 *add0, const u64 *add1, u64 add_galois, u64 *out, cudaStream_t s, uint32_t nb = 1,
-                      size_t add_stride = 0, size_t out_stride = 0, bool accumulate = false, TiledOut tiled = TiledOut(),
-                      const KsMulti *multi = nullptr);
-// The two halves of ks_inner_moddown.  ks_inner leaves u = <digits, evk> in the extended basis (w.u, nb entries); with
-// acc_u it adds to what w.u holds, so that a sum of key-switched terms can share one ks_moddown.
+// nb key switches side by side: d (evaluation domain, [level][N] per entry) -> ext (evaluation domain, all digits without
+// their own limbs).  A rotation applies its sigma_g to the extended digits when the inner product reads them (ext_galois
+// below): the centred conversion commutes with the permutation and the sign flips of sigma_g, so this equals extending
+// sigma_g(d), and d is never copied.
+void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb = 1);
+// inner product with evk (digits read through sigma_{ext_galois}; 1 = identity): leaves u = <digits, evk> in the extended basis
+// (w.u, nb entries); with acc_u it adds to what w.u holds, so that a sum of key-switched terms can share one ks_moddown.
 void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w, cudaStream_t s, uint32_t nb = 1,
               bool acc_u = false, const KsMulti *multi = nullptr);
-void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const u64 *add0, const u64 *add1, u64 add_galois, u64 *out,
-                cudaStream_t s, uint32_t nb = 1, size_t add_stride = 0, size_t out_stride = 0, bool accumulate = false,
-                TiledOut tiled = TiledOut(), const KsMulti *multi = nullptr);
+// ModDown and the final combination out_c (+)= sigma_galois(add_c) + k_c (add taken for the components in add_comps)
+struct KsOut {
+    Ptrs add, out;
+    uint32_t add_comps = 0;
+    u64 galois = 1;
+    bool accumulate = false;
+    TiledOut tiled;
+};
+void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb = 1, const KsMulti *multi = nullptr);
 // A sum of up to IP_TERMS key-switched terms in one pass over the extended basis:
 //   u[b] (+)= sum_t ( <ext[t][b] read through sigma_{g_t}, evk_t>  +  P sigma_{g_t}(c0_t[b]) on component 0's q-limbs )
-// ext holds term t's digits of batch entry b at ext + t * term_stride + b * beta * (level + K) * N words, and the own limbs of
-// the digits lie at d + t * d_term_stride + b * w.d_stride; c0[t]
+// ext holds term t's digits of batch entry b at ext + t * term_stride + b * beta * (level + K) * N words, the own limbs of the
+// digits lie at w.d.at(t * nb + b); c0[t]
 // (may be null) points at term t's first-component limbs, entries c0_stride words apart.  Adding P c0 before the
 // ModDown equals adding c0 after it, exactly.
 constexpr uint32_t IP_TERMS = 4;
@@ -354,13 +403,11 @@ struct IpTerms {
     u64 galois[IP_TERMS];
     const u64 *c0[IP_TERMS];
 };
-void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, size_t term_stride, size_t d_term_stride, const IpTerms &terms, uint32_t nterm,
+void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, size_t term_stride, const IpTerms &terms, uint32_t nterm,
                     size_t c0_stride, cudaStream_t s, uint32_t nb, bool acc_u);
-// The basis conversions on the tensor cores (N = 2^16 layout rules: any N that is a multiple of 1024).  Return false if
-// the context has no byte matrices (more than 8 sources) and nothing was launched.
-bool launch_modup_mma(const ckks_ctx *c, const u64 *dcoef, const u64 *deval, size_t deval_stride, u64 *ext, uint32_t level, uint32_t nb,
-                      cudaStream_t s);
-bool launch_moddown_conv_mma(const ckks_ctx *c, const u64 *u, u64 *conv, uint32_t level, uint32_t nb, cudaStream_t s);
+// The basis conversions on the tensor cores (contexts with byte matrices: at most 8 sources)
+void launch_modup_mma(const ckks_ctx *c, const u64 *dcoef, u64 *ext, uint32_t level, uint32_t nb, cudaStream_t s);
+void launch_moddown_conv_mma(const ckks_ctx *c, const u64 *u, u64 *conv, uint32_t level, uint32_t nb, cudaStream_t s);
 // rows of [level][N] words, src_stride words apart, into rows row0, row0 + row_step, .. of a tiled buffer with R rows
 void launch_to_tiled(const ckks_ctx *c, const u64 *src, size_t src_stride, uint32_t nrows, u64 *dst, uint32_t R, uint32_t row0,
                      uint32_t row_step, uint32_t level, cudaStream_t s);
@@ -385,10 +432,11 @@ bool mac_umma_supported(const ckks_ctx *c, uint32_t J);
 bool launch_mac_umma(const ckks_ctx *c, const u64 *baby, const u64 *pts, u64 *acc, uint32_t J, uint32_t S, uint32_t G, uint32_t level,
                      cudaStream_t s, uint32_t Jx = 0, uint32_t j0 = 0, bool accumulate = false);
 
-void launch_rescale(const ckks_ctx *c, const u64 *in, u64 *out, uint32_t ncomp, uint32_t level, u64 *ws, cudaStream_t s);
+// nb ciphertexts (at most KS_MULTI when the pointers are scattered) of ncomp components; ws: nb * ncomp * level limbs
+void launch_rescale(const ckks_ctx *c, const Ptrs &in, const Ptrs &out, uint32_t ncomp, uint32_t level, u64 *ws, cudaStream_t s, uint32_t nb = 1);
 
 size_t encode_workspace_bytes(const ckks_ctx *c, uint32_t batch);
-// tiled.R != 0 (N = 2^16 only): plaintext b is written as row tiled.row0 + b * tiled.row_stride of the tiled buffer
+// tiled.R != 0: plaintext b is written as row tiled.row0 + b * tiled.row_stride of the tiled buffer
 // `tiled_out`; `out` is then only the scratch between the two NTT passes.
 void launch_encode(const ckks_ctx *c, const double *re, const double *im, uint32_t batch, double scale, uint32_t level,
                    u64 *out, void *ws, cudaStream_t s, TiledOut tiled = TiledOut(), u64 *tiled_out = nullptr);

@@ -195,6 +195,8 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
     ckks_ctx *c = new ckks_ctx();
     c->log_n = prm->log_n; c->N = N; c->n = n; c->L = L; c->K = K; c->dnum = prm->dnum; c->alpha = alpha; c->T = T;
     c->device = prm->device;
+    c->sms = 148;
+    cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, prm->device);
     c->mod = mod;
     c->pow5.resize(n);
     c->pow5[0] = 1;
@@ -207,9 +209,11 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
     // ---- per-prime scalars and twiddles
     std::vector<u64> mu(T), mu64(T);
     std::vector<double2> modd(T);
-    std::vector<ulonglong2> ninv(T), twf((size_t)T * N), twi((size_t)T * N);
-    const bool fp = prm->log_n == 16;
-    std::vector<double> twdf(fp ? (size_t)T * N : 0), twdi(fp ? (size_t)T * N : 0);
+    std::vector<ulonglong2> ninv(T), twf, twi;
+    const bool integer = prm->log_n == 16;          // the integer transform exists for N = 2^16
+    if (integer) { twf.resize((size_t)T * N); twi.resize((size_t)T * N); }
+    std::vector<double> twdf((size_t)T * N), twdi((size_t)T * N);
+    std::vector<u64> last_inv(T);                   // the inverse transform's last twiddle (index 1 of its table)
     std::vector<double2> ninvd((size_t)2 * T);
     for (uint32_t t = 0; t < T; t++) {
         u64 m = mod[t];
@@ -228,13 +232,16 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
         for (uint32_t j = 1; j < N; j++) { pw[j] = h_mul(pw[j - 1], psi, m); pwi[j] = h_mul(pwi[j - 1], psi_inv, m); }
         for (uint32_t i = 0; i < N; i++) {
             uint32_t r = h_bitrev(i, prm->log_n);
-            twf[(size_t)t * N + i] = h_pair(pw[r], m);
-            twi[(size_t)t * N + i] = h_pair(pwi[r], m);
-            if (fp) {
-                // centred representatives: |w| <= q/2 halves the quotient estimate's error and doubles the input range
-                twdf[(size_t)t * N + i] = pw[r] > m / 2 ? -(double)(m - pw[r]) : (double)pw[r];
-                twdi[(size_t)t * N + i] = pwi[r] > m / 2 ? -(double)(m - pwi[r]) : (double)pwi[r];
-                if (i == 1) ninvd[2 * t + 1] = centred_pair(h_mul(pwi[r], ninv[t].x, m));     // the inverse's last twiddle times N^-1
+            if (integer) {
+                twf[(size_t)t * N + i] = h_pair(pw[r], m);
+                twi[(size_t)t * N + i] = h_pair(pwi[r], m);
+            }
+            // centred representatives: |w| <= q/2 halves the quotient estimate's error and doubles the input range
+            twdf[(size_t)t * N + i] = pw[r] > m / 2 ? -(double)(m - pw[r]) : (double)pw[r];
+            twdi[(size_t)t * N + i] = pwi[r] > m / 2 ? -(double)(m - pwi[r]) : (double)pwi[r];
+            if (i == 1) {
+                last_inv[t] = pwi[r];
+                ninvd[2 * t + 1] = centred_pair(h_mul(pwi[r], ninv[t].x, m));     // the inverse's last twiddle times N^-1
             }
         }
     }
@@ -265,7 +272,7 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
         }
 
     // ---- ModDown constants
-    std::vector<ulonglong2> dn_inv(K), dn_pinv(L);
+    std::vector<ulonglong2> dn_inv(K);
     std::vector<double2> dn_pinv_d(L);
     std::vector<double> dn_pmod_d(L);
     std::vector<u64> dn_mod((size_t)L * K);
@@ -286,22 +293,19 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
             dn_mod_d[(size_t)i * K + a] = centred(v, q);
             Pm = h_mul(Pm, mod[L + a] % q, q);
         }
-        dn_pinv[i] = h_pair(h_inv(Pm, q), q);
-        dn_pinv_d[i] = make_double2((double)dn_pinv[i].x, (double)dn_pinv[i].x / (double)q);
+        const double pinv = (double)h_inv(Pm, q);
+        dn_pinv_d[i] = make_double2(pinv, pinv / (double)q);
         dn_pmod_d[i] = (double)Pm;
     }
 
     // ---- The inverse transform can deliver the conversions' first factor directly: its last stage multiplies by
     // N^-1 anyway, so with N^-1 qhat^-1 (and the last twiddle times that) in its place the coefficient-domain output is
     // y = [d qhat^-1] instead of d.  Pairs {constant, constant / prime}, centred; index [level][limb][2] and [k][2].
-    std::vector<double2> isc_up(fp ? (size_t)(L + 1) * L * 2 : 0), isc_dn(fp ? (size_t)K * 2 : 0);
-    if (fp) {
+    std::vector<double2> isc_up((size_t)(L + 1) * L * 2), isc_dn((size_t)K * 2);
+    {
         auto centred_pair_mod = [&](u64 v, u64 m) {
             const double dd = v > m / 2 ? -(double)(m - v) : (double)v;
             return make_double2(dd, dd * (1.0 / (double)m));
-        };
-        auto last_tw = [&](uint32_t t) {     // the inverse transform's last twiddle (index 1 of the inverse table)
-            return twi[(size_t)t * N + 1].x;
         };
         for (uint32_t l = 1; l <= L; l++)
             for (uint32_t x = 0; x < l; x++) {
@@ -309,12 +313,12 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
                 const u64 m = mod[x], h = up_inv[((size_t)l * dn + j) * alpha + a].x;
                 const u64 nh = h_mul(ninv[x].x, h, m);
                 isc_up[((size_t)l * L + x) * 2] = centred_pair_mod(nh, m);
-                isc_up[((size_t)l * L + x) * 2 + 1] = centred_pair_mod(h_mul(last_tw(x), nh, m), m);
+                isc_up[((size_t)l * L + x) * 2 + 1] = centred_pair_mod(h_mul(last_inv[x], nh, m), m);
             }
         for (uint32_t a = 0; a < K; a++) {
             const u64 m = mod[L + a], nh = h_mul(ninv[L + a].x, dn_inv[a].x, m);
             isc_dn[(size_t)a * 2] = centred_pair_mod(nh, m);
-            isc_dn[(size_t)a * 2 + 1] = centred_pair_mod(h_mul(last_tw(L + a), nh, m), m);
+            isc_dn[(size_t)a * 2 + 1] = centred_pair_mod(h_mul(last_inv[L + a], nh, m), m);
         }
     }
 
@@ -371,10 +375,13 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
     }
 
     // ---- Rescale constants
-    std::vector<ulonglong2> rs((size_t)L * L, make_ulonglong2(0, 0));
+    std::vector<double2> rs((size_t)L * L, make_double2(0.0, 0.0));
     for (uint32_t last = 0; last < L; last++)
         for (uint32_t i = 0; i < L; i++)
-            if (i != last) rs[(size_t)last * L + i] = h_pair(h_inv(mod[last] % mod[i], mod[i]), mod[i]);
+            if (i != last) {
+                const double inv = (double)h_inv(mod[last] % mod[i], mod[i]);
+                rs[(size_t)last * L + i] = make_double2(inv, inv / (double)mod[i]);
+            }
 
     // ---- Encode tables: input permutation and fp64 twiddles from the host libm
     std::vector<uint32_t> enc_src(n);
@@ -411,7 +418,7 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
     if ((rc = upload(c, mod, &d.mod)) || (rc = upload(c, mu, &d.mu)) || (rc = upload(c, mu64, &d.mu64)) || (rc = upload(c, modd, &d.modd)) || (rc = upload(c, twf, &d.tw_fwd)) ||
         (rc = upload(c, twi, &d.tw_inv)) || (rc = upload(c, twdf, &d.twd_fwd)) || (rc = upload(c, twdi, &d.twd_inv)) || (rc = upload(c, ninvd, &d.n_inv_d)) || (rc = upload(c, isc_up, &d.inv_scale_up)) || (rc = upload(c, isc_dn, &d.inv_scale_dn)) || (rc = upload(c, ninv, &d.n_inv)) || (rc = upload(c, up_inv, &d.up_hat_inv)) ||
         (rc = upload(c, up_mod_d, &d.up_hat_mod_d)) || (rc = upload(c, dn_mod_d, &d.dn_hat_mod_d)) || (rc = upload(c, dn_inv, &d.dn_hat_inv)) ||
-        (rc = upload(c, dn_pinv, &d.dn_p_inv)) || (rc = upload(c, dn_pinv_d, &d.dn_p_inv_d)) || (rc = upload(c, dn_pmod_d, &d.dn_p_mod_d)) || (rc = upload(c, up_bmat, &d.up_bmat)) || (rc = upload(c, dn_bmat, &d.dn_bmat)) || (rc = upload(c, two52, &d.two52_d)) || (rc = upload(c, rs, &d.rs_inv)) ||
+        (rc = upload(c, dn_pinv_d, &d.dn_p_inv_d)) || (rc = upload(c, dn_pmod_d, &d.dn_p_mod_d)) || (rc = upload(c, up_bmat, &d.up_bmat)) || (rc = upload(c, dn_bmat, &d.dn_bmat)) || (rc = upload(c, two52, &d.two52_d)) || (rc = upload(c, rs, &d.rs_inv_d)) ||
         (rc = upload(c, enc_src, &d.enc_src)) || (rc = upload(c, om, &d.enc_omega)) || (rc = upload(c, om_st, &d.enc_omega_st)) || (rc = upload(c, om_st2, &d.enc_omega_st2)) || (rc = upload(c, ze, &d.enc_zeta)) ||
         (rc = upload(c, flag, &flag_dev))) {
         cudaSetDevice(prev);

@@ -54,8 +54,8 @@ __device__ __forceinline__ void assemble7(const uint32_t (&E)[7], uint32_t &w0, 
 // MODE 0: ModUp.   item = (batch b, digit j); sources dcoef[b][lo + a]; targets the limbs of ext[b][j] outside the digit.
 // MODE 1: ModDown. item = (batch b, component); sources the special limbs of u; targets conv[b][comp][0 .. level).
 template <int MODE>
-__global__ void __launch_bounds__(CM_THREADS, 2) conv_mma_kernel(DevTables c, const u64 *src, const u64 *deval, size_t deval_stride, u64 *dst,
-                                                                 uint32_t level) {
+__global__ void __launch_bounds__(CM_THREADS, 2) conv_mma_kernel(DevTables c, const u64 *src, u64 *dst, uint32_t level) {
+    grid_dep_sync();
     extern __shared__ __align__(16) uint32_t bs[];
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
     const uint32_t nt = level + c.K, N = c.N;
@@ -73,7 +73,6 @@ __global__ void __launch_bounds__(CM_THREADS, 2) conv_mma_kernel(DevTables c, co
         dbase = dst + (size_t)(b * beta + j) * nt * N;
         bm = c.up_bmat + ((size_t)level * c.dnum + j) * c.conv_groups * CM_GWORDS;
         hinv = c.up_hat_inv + ((size_t)level * c.dnum + j) * c.alpha;
-        deval += b * deval_stride;
     } else {
         nsrc = c.K; ntgt = level; qbase = c.L;
         sbase = src + ((size_t)blockIdx.z * nt + level) * N;
@@ -102,11 +101,6 @@ __global__ void __launch_bounds__(CM_THREADS, 2) conv_mma_kernel(DevTables c, co
         }
     }
     const uint32_t kcta = blockIdx.x * (CM_TILES * 128);
-    if (MODE == 0)      // the digit's own limbs are copied as they are (evaluation domain)
-        for (uint32_t e = tid; e < nd * (CM_TILES * 128); e += CM_THREADS) {
-            const uint32_t a = e / (CM_TILES * 128), k = kcta + e % (CM_TILES * 128);
-            dbase[(size_t)(lo + a) * N + k] = deval[(size_t)(lo + a) * N + k];
-        }
     __syncthreads();
 
     // this thread prepares the words of sources t and 4 + t for rows g and g + 8 of its warp's 16 coefficients
@@ -194,22 +188,15 @@ size_t conv_smem(uint32_t ngroups) { return (size_t)ngroups * (CM_GWORDS * 4 + 8
 
 }  // namespace
 
-bool launch_modup_mma(const ckks_ctx *c, const u64 *dcoef, const u64 *deval, size_t deval_stride, u64 *ext, uint32_t level, uint32_t nb,
-                      cudaStream_t s) {
-    if (!c->dev.conv_groups || c->N % (CM_TILES * 128)) return false;
+void launch_modup_mma(const ckks_ctx *c, const u64 *dcoef, u64 *ext, uint32_t level, uint32_t nb, cudaStream_t s) {
     const uint32_t beta = (level + c->alpha - 1) / c->alpha, nt = level + c->K;
     const size_t smem = conv_smem((nt + 7) / 8);
-    if (cudaFuncSetAttribute(conv_mma_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
-    conv_mma_kernel<0><<<dim3(c->N / (CM_TILES * 128), 1, beta * nb), CM_THREADS, smem, s>>>(c->dev, dcoef, deval, deval_stride, ext, level);
-    count_launches();
-    return true;
+    cudaFuncSetAttribute(conv_mma_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    launch(conv_mma_kernel<0>, dim3(c->N / (CM_TILES * 128), 1, beta * nb), CM_THREADS, smem, s, c->dev, dcoef, ext, level);
 }
 
-bool launch_moddown_conv_mma(const ckks_ctx *c, const u64 *u, u64 *conv, uint32_t level, uint32_t nb, cudaStream_t s) {
-    if (!c->dev.conv_groups || c->N % (CM_TILES * 128)) return false;
+void launch_moddown_conv_mma(const ckks_ctx *c, const u64 *u, u64 *conv, uint32_t level, uint32_t nb, cudaStream_t s) {
     const size_t smem = conv_smem((level + 7) / 8);
-    if (cudaFuncSetAttribute(conv_mma_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
-    conv_mma_kernel<1><<<dim3(c->N / (CM_TILES * 128), 1, 2 * nb), CM_THREADS, smem, s>>>(c->dev, u, nullptr, 0, conv, level);
-    count_launches();
-    return true;
+    cudaFuncSetAttribute(conv_mma_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    launch(conv_mma_kernel<1>, dim3(c->N / (CM_TILES * 128), 1, 2 * nb), CM_THREADS, smem, s, c->dev, u, conv, level);
 }

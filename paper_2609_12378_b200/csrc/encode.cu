@@ -33,6 +33,7 @@ __global__ void __launch_bounds__(THREADS) fft_chunks(DevTables c, const double 
     __shared__ double2 sm[CH];
     __shared__ double2 tw[CH];
     const uint32_t b = blockIdx.y, base = blockIdx.x * ch;
+    grid_dep_sync();
     for (uint32_t x = threadIdx.x; x < ch; x += THREADS) {
         const uint32_t j = c.enc_src[base + x];
         sm[x] = make_double2(re[(size_t)b * n + j], im ? im[(size_t)b * n + j] : 0.0);
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(THREADS) fft_strips_round(DevTables c, const d
     extern __shared__ double2 sm2[];
     const uint32_t b = blockIdx.y, rows = n / ch, col0 = blockIdx.x * COLS;
     double2 *tw = sm2 + rows * COLS;          // the strip's twiddles, entry (hr + jr) * COLS + column (row 0 unused)
+    grid_dep_sync();
     for (uint32_t x = threadIdx.x; x < rows * COLS; x += THREADS) {
         sm2[x] = buf[(size_t)b * n + (size_t)(x / COLS) * ch + col0 + x % COLS];
         tw[x] = c.enc_omega_st2[(size_t)(x / COLS) * ch + col0 + x % COLS];
@@ -111,23 +113,13 @@ __global__ void __launch_bounds__(THREADS) fft_strips_round(DevTables c, const d
     }
 }
 
-// out[b][i][k] = canonical residue of coef[b][k] modulo q_i
-__global__ void __launch_bounds__(THREADS) reduce_coeffs(DevTables c, const long long *coef, u64 *out, uint32_t level) {
-    const uint32_t k = blockIdx.x * THREADS + threadIdx.x;
-    const uint32_t i = blockIdx.y, b = blockIdx.z;
-    const long long v = coef[(size_t)b * c.N + k];
-    const u64 q = c.mod[i];
-    const u64 mag = v < 0 ? (u64)(-v) : (u64)v;
-    const u64 r = barrett112(0, mag, q, c.mu[i]);
-    out[((size_t)b * level + i) * c.N + k] = (v < 0 && r) ? q - r : r;
-}
-
 // slots[kk][r*T + t] = d'_k[r],  k = k0 + kk,  d'_k[r] = d_k[(r - pre_rot) mod F],
 // d_k[r'] = W^T[out0 + r' mod m_out, in0 + (r' + k) mod m_in]
 __global__ void __launch_bounds__(THREADS) extract_diagonals(const double *W, uint32_t d_out_total, uint32_t in0, uint32_t m_in,
                                                              uint32_t out0, uint32_t m_out, uint32_t F, uint32_t T, uint32_t k0,
                                                              uint32_t pre_rot, double *slots, uint32_t n) {
     const uint32_t x = blockIdx.x * THREADS + threadIdx.x;
+    grid_dep_sync();
     if (x >= n) return;
     const uint32_t r = x / T, k = k0 + blockIdx.y;
     const uint32_t rp = (r + F - pre_rot % F) % F;
@@ -149,34 +141,18 @@ void launch_encode(const ckks_ctx *c, const double *re, const double *im, uint32
     const double sc = scale / (double)n;
     for (uint32_t b0 = 0; b0 < batch; b0 += 32768) {
         const uint32_t nb = batch - b0 < 32768 ? batch - b0 : 32768;
-        fft_chunks<<<dim3(n / ch, nb), THREADS, 0, s>>>(c->dev, re + (size_t)b0 * n, im ? im + (size_t)b0 * n : nullptr,
-                                                         buf + (size_t)b0 * n, n, ch); count_launches();
-        fft_strips_round<<<dim3(ch / COLS, nb), THREADS, (size_t)2 * (n / ch) * COLS * sizeof(double2), s>>>(
-            c->dev, buf + (size_t)b0 * n, coef + (size_t)b0 * N, n, ch, sc); count_launches();
+        launch(fft_chunks, dim3(n / ch, nb), THREADS, 0, s, c->dev, re + (size_t)b0 * n, im ? im + (size_t)b0 * n : nullptr, buf + (size_t)b0 * n, n, ch);
+        launch(fft_strips_round, dim3(ch / COLS, nb), THREADS, (size_t)2 * (n / ch) * COLS * sizeof(double2), s, c->dev, buf + (size_t)b0 * n, coef + (size_t)b0 * N, n, ch, sc);
     }
-    if (c->log_n == 16 && (uint64_t)batch * level <= 32768) {
-        // the first NTT pass reduces the signed coefficients itself; the last one can write the tiled layout
-        if (tiled.R) {
-            NttEpilogue ep{};
-            ep.mode = 2; ep.out = tiled_out; ep.level = level; ep.tl = tiled;
-            launch_ntt(c, out, batch * level, plain_map(0, level), false, s, &ep, coef);
-        } else {
-            launch_ntt(c, out, batch * level, plain_map(0, level), false, s, nullptr, coef);
-        }
-        return;
-    }
-    for (uint32_t b0 = 0; b0 < batch; b0 += 32768) {
-        const uint32_t nb = batch - b0 < 32768 ? batch - b0 : 32768;
-        reduce_coeffs<<<dim3(N / THREADS, level, nb), THREADS, 0, s>>>(c->dev, coef + (size_t)b0 * N, out + (size_t)b0 * level * N, level);
-        count_launches();
-    }
-    launch_ntt(c, out, batch * level, plain_map(0, level), false, s);
-    if (tiled.R) launch_to_tiled(c, out, (size_t)level * N, batch, tiled_out, tiled.R, tiled.row0, tiled.row_stride, level, s);
+    // the first NTT pass reduces the signed coefficients itself; the last one can write the tiled layout
+    const NttPrologue pro{(const u64 *)coef, false, 0};
+    NttEpilogue ep{};
+    ep.mode = 2; ep.out.base = tiled_out; ep.level = level; ep.tl = tiled;
+    launch_ntt(c, out, batch * level, plain_map(0, level), false, s, tiled.R ? &ep : nullptr, &pro);
 }
 
 void launch_extract_diagonals(const ckks_ctx *c, const double *W, uint32_t d_out_total, uint32_t in0, uint32_t m_in,
                               uint32_t out0, uint32_t m_out, uint32_t F, uint32_t T, uint32_t k0, uint32_t count,
                               uint32_t pre_rot, double *slots, cudaStream_t s) {
-    extract_diagonals<<<dim3((c->n + THREADS - 1) / THREADS, count), THREADS, 0, s>>>(W, d_out_total, in0, m_in, out0, m_out, F, T, k0,
-                                                                                       pre_rot, slots, c->n); count_launches();
+    launch(extract_diagonals, dim3((c->n + THREADS - 1) / THREADS, count), THREADS, 0, s, W, d_out_total, in0, m_in, out0, m_out, F, T, k0, pre_rot, slots, c->n);
 }

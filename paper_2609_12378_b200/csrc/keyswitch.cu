@@ -16,13 +16,6 @@ namespace {
 
 constexpr uint32_t THREADS = 256;
 
-// dst[b][i][p] = src[b][i][pi_g(p)]  (g = 1: copy); batch entries src_stride / dst_stride words apart
-__global__ void __launch_bounds__(THREADS) permute_kernel(DevTables c, const u64 *src, size_t src_stride, u64 *dst, size_t dst_stride, u64 g) {
-    const uint32_t p = blockIdx.x * THREADS + threadIdx.x;
-    const size_t row = (size_t)blockIdx.y * c.N;
-    dst[blockIdx.z * dst_stride + row + p] = src[blockIdx.z * src_stride + row + galois_src(p, g, c.log_n, c.N)];
-}
-
 // ---------------------------------------------------------------------------
 // Basis conversions: out[x] = sum_a y_a C[a][x] mod t_x with centred sources |y_a| <= q_a / 2 and centred constants
 // |C| <= t / 2 (a dense contraction, bound by the FP64 pipe).  The exact 100-bit products are summed as they are and
@@ -77,7 +70,6 @@ __device__ __forceinline__ void conv_store(u64 *p, const double (&v)[CPT], doubl
     if (CPT == 2) *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(canonical_d(v[0], t), canonical_d(v[CPT - 1], t));
     else *p = canonical_d(v[0], t);
 }
-__device__ __forceinline__ double centre_d(u64 v, u64 q) { return v > (q >> 1) ? __dsub_rn(u64_to_d(v), (double)q) : u64_to_d(v); }
 
 // coefficients per thread: two while their sources fit the registers and the buffers take 16-byte accesses
 inline uint32_t conv_cpt(uint32_t ns, const void *a, const void *b) { return ns <= 8 && (((uintptr_t)a | (uintptr_t)b) & 15) == 0 ? 2 : 1; }
@@ -95,8 +87,8 @@ inline uint32_t conv_chunk(uint32_t gx, uint32_t items, uint32_t targets) {
 // ext[j][x][k] for the limbs x of q_0..q_{level-1}, p_0..p_{K-1} outside digit j, from dcoef (coefficient domain).  A thread
 // owns CPT coefficients of one digit: it forms the centred y_a of the digit's limbs once and walks a chunk of CHUNK target
 // limbs (blockIdx.y), so the source limbs are read once per chunk.
-// PRE: dcoef already holds [d_a qhat_a^-1] (the inverse transform multiplied it in), so only the centring is left.
-template <uint32_t ALPHA, bool PRE, uint32_t CPT>
+// dcoef already holds [d_a qhat_a^-1] (the inverse transform multiplied it in), so only the centring is left.
+template <uint32_t ALPHA, uint32_t CPT>
 __global__ void __launch_bounds__(THREADS) modup_kernel(DevTables c, const u64 *dcoef, u64 *ext, uint32_t level, uint32_t CHUNK) {
     // the CTA's conversion constants (qhat_a mod t; t and 1/t), fetched once
     __shared__ __align__(16) double s_w[CONV_CHUNK_MAX][ALPHA];
@@ -115,6 +107,7 @@ __global__ void __launch_bounds__(THREADS) modup_kernel(DevTables c, const u64 *
     dcoef += ((size_t)bz * level + lo) * c.N + k;
     ext += ((size_t)bz * beta + j) * nt * c.N + k;
     double y[CPT][ALPHA];
+    grid_dep_sync();
 #pragma unroll
     for (uint32_t a = 0; a < ALPHA; a++) {
         u64 v[CPT];
@@ -124,10 +117,6 @@ __global__ void __launch_bounds__(THREADS) modup_kernel(DevTables c, const u64 *
             y[p][a] = 0.0;
             if (a < nd) {
                 const u64 qa = c.mod[lo + a];
-                if (!PRE) {
-                    const ulonglong2 hinv = c.up_hat_inv[cb * c.alpha + a];
-                    v[p] = mul_shoup(v[p], hinv.x, hinv.y, qa);
-                }
                 y[p][a] = centre_d(v[p], qa);
             }
         }
@@ -142,29 +131,28 @@ __global__ void __launch_bounds__(THREADS) modup_kernel(DevTables c, const u64 *
 }
 
 template <uint32_t ALPHA>
-void launch_modup(const ckks_ctx *c, const u64 *dcoef, u64 *ext, uint32_t level, uint32_t nb, cudaStream_t s, bool pre) {
+void launch_modup(const ckks_ctx *c, const u64 *dcoef, u64 *ext, uint32_t level, uint32_t nb, cudaStream_t s) {
     const uint32_t nt = level + c->K, beta = (level + c->alpha - 1) / c->alpha;
     const uint32_t cpt = conv_cpt(ALPHA, dcoef, ext), gx = c->N / (THREADS * cpt), targets = nt - (level - (beta - 1) * c->alpha);   // the last digit has the most targets
     const uint32_t CHUNK = conv_chunk(gx, beta * nb, targets);
     const dim3 grid(gx, (targets + CHUNK - 1) / CHUNK, beta * nb);
     constexpr uint32_t WIDE = ALPHA <= 8 ? 2 : 1;
-    auto *kernel = cpt == WIDE ? (pre ? modup_kernel<ALPHA, true, WIDE> : modup_kernel<ALPHA, false, WIDE>)
-                               : (pre ? modup_kernel<ALPHA, true, 1> : modup_kernel<ALPHA, false, 1>);
-    kernel<<<grid, THREADS, 0, s>>>(c->dev, dcoef, ext, level, CHUNK);
-    count_launches();
+    launch(cpt == WIDE ? modup_kernel<ALPHA, WIDE> : modup_kernel<ALPHA, 1>, grid, THREADS, 0, s, c->dev, dcoef, ext, level, CHUNK);
 }
 
 // u[comp][x][p] = sum_j ext[j][x][pi_g(p)] * evk[j][comp][kt(x)][p]          (any number of digits)
-__global__ void __launch_bounds__(THREADS) inner_product_generic_kernel(DevTables c, const u64 *ext, const u64 *d, size_t d_stride, const u64 *evk, u64 g,
-                                                                        u64 *u, uint32_t level, int has_multi, KsMulti multi, int acc_u) {
+__global__ void __launch_bounds__(THREADS) inner_product_generic_kernel(DevTables c, const u64 *ext, const __grid_constant__ Ptrs dp, uint32_t d0, const u64 *evk, u64 g,
+                                                                        u64 *u, uint32_t level, int has_multi, const __grid_constant__ KsMulti multi, int acc_u) {
     const uint32_t p = blockIdx.x * THREADS + threadIdx.x;
     const uint32_t x = blockIdx.z, bz = blockIdx.y;     // batch varies faster than the limb: a key limb is reused from L2
     const uint32_t nt = level + c.K, beta = (level + c.alpha - 1) / c.alpha;
     const uint32_t kt = x < level ? x : c.L + (x - level);
     if (has_multi) { evk = multi.evk[bz]; g = multi.galois[bz]; }     // shared digits, per-entry key and permutation
-    else { ext += (size_t)bz * beta * nt * c.N; d += bz * d_stride; }
+    else ext += (size_t)bz * beta * nt * c.N;
+    const u64 *d = dp.at(d0 + (has_multi ? 0 : bz));
+    grid_dep_sync();
     const uint32_t own = x < level ? x / c.alpha : beta;        // the digit that has x among its own limbs
-    const uint32_t src = galois_src(p, g, c.log_n, c.N);
+    const uint32_t src = galois_src(p, (uint32_t)g, c.log_n);
     u += (size_t)bz * 2 * nt * c.N;
     // products on the FP64 pipe: each is reduced to |r| <= 0.75 m as it is formed, the few digits are summed exactly
     const double2 md = c.modd[kt];
@@ -191,8 +179,8 @@ __global__ void __launch_bounds__(THREADS) inner_product_generic_kernel(DevTable
 // of up to KS_MULTI keys applied to the same digits.
 constexpr uint32_t IP_MAX_BETA = 4;
 template <uint32_t BETA>
-__global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, const u64 *ext, const u64 *d, size_t d_stride, const u64 *evk, u64 g, u64 *u,
-                                                                uint32_t level, uint32_t nb, uint32_t bch, int has_multi, KsMulti multi,
+__global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, const u64 *ext, const __grid_constant__ Ptrs d, const u64 *evk, u64 g, u64 *u,
+                                                                uint32_t level, uint32_t nb, uint32_t bch, int has_multi, const __grid_constant__ KsMulti multi,
                                                                 int acc_u) {
     const uint32_t p = (blockIdx.x * THREADS + threadIdx.x) * 2;
     const uint32_t x = blockIdx.z;     // chunks of a limb run together: its key words (and shared digits) come from L2
@@ -208,28 +196,39 @@ __global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, con
         b1 = min(b0 + bch, (r + 1) * multi.group);
         evk = multi.evk[r]; g = multi.galois[r];
     } else if (has_multi) { evk = multi.evk[b0]; g = multi.galois[b0]; }
-    const uint32_t src = galois_src(p, g, c.log_n, c.N);
+    const uint32_t src = galois_src(p, (uint32_t)g, c.log_n);
     const bool odd = src & 1;
-    double k[BETA][2][2];                         // [digit][component][coefficient of the pair]
+    grid_dep_sync();
+    // all loads of a step are issued before the first product (the barrier keeps the compiler from spreading them out): the
+    // kernel is bound by how many of its scattered 16-byte reads are in flight
+    ulonglong2 kv[BETA][2], ev[BETA];             // [digit][component]
 #pragma unroll
     for (uint32_t j = 0; j < BETA; j++)
 #pragma unroll
-        for (uint32_t cm = 0; cm < 2; cm++) {
-            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(evk + ((size_t)j * 2 + cm) * ks + (size_t)kt * c.N + p);
-            k[j][cm][0] = u64_to_d(v.x);
-            k[j][cm][1] = u64_to_d(v.y);
-        }
+        for (uint32_t cm = 0; cm < 2; cm++) kv[j][cm] = *reinterpret_cast<const ulonglong2 *>(evk + ((size_t)j * 2 + cm) * ks + (size_t)kt * c.N + p);
     const uint32_t own = x < level ? x / c.alpha : BETA;       // the digit that has x among its own limbs: it lies in d
-    const uint32_t so = src & ~1u;
+    const size_t off = (size_t)x * c.N + (src & ~1u);
     u64 *o = u + b0 * 2 * js + (size_t)x * c.N + p;
+    double k[BETA][2][2];                         // [digit][component][coefficient of the pair]
     for (uint32_t b = b0; b < b1; b++, o += 2 * js) {
         const uint32_t be = b - b0 + e0;
+#pragma unroll
+        for (uint32_t j = 0; j < BETA; j++)
+            ev[j] = *reinterpret_cast<const ulonglong2 *>((j == own ? d.at(be) : ext + ((size_t)be * BETA + j) * js) + off);
+        __syncwarp();
+        if (b == b0) {
+#pragma unroll
+            for (uint32_t j = 0; j < BETA; j++)
+#pragma unroll
+                for (uint32_t cm = 0; cm < 2; cm++) {
+                    k[j][cm][0] = u64_to_d(kv[j][cm].x);
+                    k[j][cm][1] = u64_to_d(kv[j][cm].y);
+                }
+        }
         double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
         for (uint32_t j = 0; j < BETA; j++) {
-            const u64 *ej = (j == own ? d + be * d_stride : ext + ((size_t)be * BETA + j) * js) + (size_t)x * c.N;
-            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(ej + so);
-            const double d0 = u64_to_d(odd ? v.y : v.x), d1 = u64_to_d(odd ? v.x : v.y);
+            const double d0 = u64_to_d(odd ? ev[j].y : ev[j].x), d1 = u64_to_d(odd ? ev[j].x : ev[j].y);
 #pragma unroll
             for (uint32_t cm = 0; cm < 2; cm++) {
                 acc[cm][0] = __dadd_rn(acc[cm][0], mulmod_dd(d0, k[j][cm][0], md.x, md.y));
@@ -257,7 +256,7 @@ __global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, con
 // registers over the terms.
 constexpr uint32_t IP_BCH = 4;
 template <uint32_t BETA>
-__global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTables c, const u64 *ext, size_t term_stride, const u64 *d, size_t d_term_stride, size_t d_stride,
+__global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTables c, const u64 *ext, size_t term_stride, const u64 *d, size_t d_stride,
                                                                          const __grid_constant__ IpTerms tm, uint32_t nterm, size_t c0_stride,
                                                                          u64 *u, uint32_t level, uint32_t nb, int acc_u) {
     const uint32_t p = (blockIdx.x * THREADS + threadIdx.x) * 2;
@@ -271,8 +270,9 @@ __global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTabl
     double acc[IP_BCH][2][2];
 #pragma unroll
     for (uint32_t bi = 0; bi < IP_BCH; bi++) acc[bi][0][0] = acc[bi][0][1] = acc[bi][1][0] = acc[bi][1][1] = 0.0;
+    grid_dep_sync();
     for (uint32_t t = 0; t < nterm; t++) {
-        const uint32_t src = galois_src(p, tm.galois[t], c.log_n, c.N);
+        const uint32_t src = galois_src(p, (uint32_t)tm.galois[t], c.log_n);
         const bool odd = src & 1;
         const u64 *evk = tm.evk[t];
         double k[BETA][2][2];
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTabl
             double sum[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
             for (uint32_t j = 0; j < BETA; j++) {
-                const u64 *ej = (j == own ? d + t * d_term_stride + (b0 + bc) * d_stride
+                const u64 *ej = (j == own ? d + (size_t)(t * nb + b0 + bc) * d_stride
                                           : ext + t * term_stride + ((size_t)(b0 + bc) * BETA + j) * js) + (size_t)x * c.N;
                 const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(ej + so);
                 const double d0 = u64_to_d(odd ? v.y : v.x), d1 = u64_to_d(odd ? v.x : v.y);
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTabl
 
 // conv[comp][i][k] = sum_a centre([u_{p_a} Phat_a^-1]) (Phat_a mod q_i)  mod q_i   (coefficient domain)
 // Same shape as ModUp: the K centred special residues are formed once per thread, then a chunk of targets is walked.
-template <uint32_t KK, bool PRE, uint32_t CPT>
+template <uint32_t KK, uint32_t CPT>
 __global__ void __launch_bounds__(THREADS) moddown_conv_kernel(DevTables c, const u64 *u, u64 *conv, uint32_t level, uint32_t CHUNK) {
     __shared__ __align__(16) double s_w[CONV_CHUNK_MAX][KK];     // Phat_a mod q_i
     __shared__ double2 s_m[CONV_CHUNK_MAX];                      // q_i, 1 / q_i
@@ -355,6 +355,7 @@ __global__ void __launch_bounds__(THREADS) moddown_conv_kernel(DevTables c, cons
     u += (((size_t)bz * 2 + comp) * nt + level) * c.N + k;
     conv += ((size_t)bz * 2 + comp) * level * c.N + k;
     double y[CPT][KK];
+    grid_dep_sync();
 #pragma unroll
     for (uint32_t a = 0; a < KK; a++) {
         u64 v[CPT];
@@ -364,10 +365,6 @@ __global__ void __launch_bounds__(THREADS) moddown_conv_kernel(DevTables c, cons
             y[p][a] = 0.0;
             if (a < c.K) {
                 const u64 pa = c.mod[c.L + a];
-                if (!PRE) {
-                    const ulonglong2 hinv = c.dn_hat_inv[a];
-                    v[p] = mul_shoup(v[p], hinv.x, hinv.y, pa);
-                }
                 y[p][a] = centre_d(v[p], pa);
             }
         }
@@ -382,14 +379,11 @@ __global__ void __launch_bounds__(THREADS) moddown_conv_kernel(DevTables c, cons
 }
 
 template <uint32_t KK>
-void launch_moddown_conv(const ckks_ctx *c, const u64 *u, u64 *conv, uint32_t level, uint32_t nb, cudaStream_t s, bool pre) {
+void launch_moddown_conv(const ckks_ctx *c, const u64 *u, u64 *conv, uint32_t level, uint32_t nb, cudaStream_t s) {
     const uint32_t cpt = conv_cpt(KK, u, conv), gx = c->N / (THREADS * cpt), CHUNK = conv_chunk(gx, 2 * nb, level);
     const dim3 grid(gx, (level + CHUNK - 1) / CHUNK, 2 * nb);
     constexpr uint32_t WIDE = KK <= 8 ? 2 : 1;
-    auto *kernel = cpt == WIDE ? (pre ? moddown_conv_kernel<KK, true, WIDE> : moddown_conv_kernel<KK, false, WIDE>)
-                               : (pre ? moddown_conv_kernel<KK, true, 1> : moddown_conv_kernel<KK, false, 1>);
-    kernel<<<grid, THREADS, 0, s>>>(c->dev, u, conv, level, CHUNK);
-    count_launches();
+    launch(cpt == WIDE ? moddown_conv_kernel<KK, WIDE> : moddown_conv_kernel<KK, 1>, grid, THREADS, 0, s, c->dev, u, conv, level, CHUNK);
 }
 
 // register-array size for a digit / special-prime count: next of 1, 2, 4, 8, 16, 32, 64
@@ -404,56 +398,22 @@ void launch_moddown_conv(const ckks_ctx *c, const u64 *u, u64 *conv, uint32_t le
         else { CALL(64); }                          \
     } while (0)
 
-// out[b][comp][i][p] (+)= (u[b][comp][i][p] - conv[b][comp][i][p]) P^-1 + add_comp[b][i][pi_g(p)]
-__global__ void __launch_bounds__(THREADS) moddown_final_kernel(DevTables c, const u64 *u, const u64 *conv, const u64 *add0,
-                                                                const u64 *add1, size_t add_stride, u64 g, u64 *out,
-                                                                size_t out_stride, int accumulate, uint32_t level, TiledOut tl) {
-    const uint32_t p = blockIdx.x * THREADS + threadIdx.x;
-    const uint32_t i = blockIdx.y, comp = blockIdx.z & 1, bz = blockIdx.z >> 1;
-    const uint32_t nt = level + c.K;
-    const u64 q = c.mod[i];
-    const ulonglong2 pinv = c.dn_p_inv[i];
-    u64 r = sub_mod(u[(((size_t)bz * 2 + comp) * nt + i) * c.N + p], conv[(((size_t)bz * 2 + comp) * level + i) * c.N + p], q);
-    r = mul_shoup(r, pinv.x, pinv.y, q);
-    const u64 *add = comp ? add1 : add0;
-    if (add) r = add_mod(r, add[bz * add_stride + (size_t)i * c.N + galois_src(p, g, c.log_n, c.N)], q);
-    u64 *dst = tl.R ? out + tiled_index(tl.R, c.N, tl.row0 + bz * tl.row_stride + comp, i, p)
-                    : out + bz * out_stride + ((size_t)comp * level + i) * c.N + p;
-    if (accumulate) r = add_mod(r, *dst, q);
-    *dst = r;
-}
-
 // dst row (row0 + r * row_step) of a tiled buffer <- src + r * src_stride ([level][N] words)
 __global__ void __launch_bounds__(THREADS) to_tiled_kernel(DevTables c, const u64 *src, size_t src_stride, u64 *dst, uint32_t R,
                                                            uint32_t row0, uint32_t row_step) {
+    grid_dep_sync();
     const uint32_t p = (blockIdx.x * THREADS + threadIdx.x) * 2, i = blockIdx.y, r = blockIdx.z;
     const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(src + r * src_stride + (size_t)i * c.N + p);
     *reinterpret_cast<ulonglong2 *>(dst + tiled_index(R, c.N, row0 + r * row_step, i, p)) = v;
 }
 
-// tmp[comp][i][k] = centred lift of last[comp][k] (mod q_last) taken mod q_i
-__global__ void __launch_bounds__(THREADS) rescale_lift_kernel(DevTables c, const u64 *last, u64 *tmp, uint32_t level) {
-    const uint32_t k = blockIdx.x * THREADS + threadIdx.x;
-    const uint32_t i = blockIdx.y, comp = blockIdx.z;
-    tmp[((size_t)comp * (level - 1) + i) * c.N + k] = centred_to(last[(size_t)comp * c.N + k], c.mod[level - 1], c.mod[i]);
-}
-
-// out[comp][i][p] = (in[comp][i][p] - tmp[comp][i][p]) q_last^-1
-__global__ void __launch_bounds__(THREADS) rescale_final_kernel(DevTables c, const u64 *in, const u64 *tmp, u64 *out, uint32_t level) {
-    const uint32_t p = blockIdx.x * THREADS + threadIdx.x;
-    const uint32_t i = blockIdx.y, comp = blockIdx.z;
-    const u64 q = c.mod[i];
-    const ulonglong2 inv = c.rs_inv[(size_t)(level - 1) * c.L + i];
-    const u64 r = sub_mod(in[((size_t)comp * level + i) * c.N + p], tmp[((size_t)comp * (level - 1) + i) * c.N + p], q);
-    out[((size_t)comp * (level - 1) + i) * c.N + p] = mul_shoup(r, inv.x, inv.y, q);
-}
-
 // u[b][0][i][p] += P sigma_g(c0[b][i])[p]   (first component's q-limbs of the extended-basis sum)
 __global__ void __launch_bounds__(THREADS) p_c0_acc_kernel(DevTables c, const u64 *c0, size_t c0_stride, u64 g, u64 *u, size_t u_stride) {
+    grid_dep_sync();
     const uint32_t p = blockIdx.x * THREADS + threadIdx.x, i = blockIdx.y, b = blockIdx.z;
     const double2 md = c.modd[i];
     u64 *d = u + b * u_stride + (size_t)i * c.N + p;
-    const double v = mulmod_dd(u64_to_d(c0[b * c0_stride + (size_t)i * c.N + galois_src(p, g, c.log_n, c.N)]), c.dn_p_mod_d[i], md.x, md.y);
+    const double v = mulmod_dd(u64_to_d(c0[b * c0_stride + (size_t)i * c.N + galois_src(p, (uint32_t)g, c.log_n)]), c.dn_p_mod_d[i], md.x, md.y);
     *d = add_mod(*d, canonical_d(reduce_d(v, md.x, md.y), md.x), c.mod[i]);
 }
 
@@ -476,25 +436,33 @@ KsWorkspace ks_carve(const ckks_ctx *c, uint32_t level, void *ws, uint32_t nb) {
     return w;
 }
 
-void ks_modup(const ckks_ctx *c, const u64 *d, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb, size_t d_stride) {
-    w.d = d; w.d_stride = d_stride;
-    const uint32_t N = c->N, beta = (level + c->alpha - 1) / c->alpha, nt = level + c->K;
-    // N = 2^16 with the FP64 transform and conversion: the inverse transform's last stage multiplies qhat^-1 in
-    const bool pre = c->log_n == 16 && c->ntt_fp_share >= 8 && c->conv_kernel != CKKS_CONV_TENSOR;
-    if (c->log_n == 16) {      // the inverse transform reads d and writes the coefficient copy
-        launch_ntt(c, w.dcoef, nb * level, plain_map(0, level), true, s, nullptr, nullptr, d, (uint32_t)(d_stride / N),
-                   pre ? c->dev.inv_scale_up + (size_t)level * c->L * 2 : nullptr);
+// whether the conversions run on the tensor cores (context option CKKS_CONV_TENSOR: bit-identical, slower on B200); they take
+// the inverse transform's plain output, the FP64 kernels one with qhat^-1 (Phat^-1) multiplied in
+static bool conv_tensor(const ckks_ctx *c) { return c->conv_kernel == CKKS_CONV_TENSOR && c->dev.conv_groups; }
+
+void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb) {
+    const uint32_t beta = (level + c->alpha - 1) / c->alpha, nt = level + c->K;
+    w.d = d;
+    NttSource src;
+    src.ptr = d; src.lpitch = 1;
+    launch_ntt(c, w.dcoef, nb * level, plain_map(0, level), true, s, nullptr, nullptr, &src,
+               conv_tensor(c) ? nullptr : c->dev.inv_scale_up + (size_t)level * c->L * 2);
+    if (conv_tensor(c)) {
+        launch_modup_mma(c, w.dcoef, w.ext, level, nb, s);
     } else {
-        permute_kernel<<<dim3(N / THREADS, level, nb), THREADS, 0, s>>>(c->dev, d, d_stride, w.dcoef, (size_t)level * N, 1); count_launches();
-        launch_ntt(c, w.dcoef, nb * level, plain_map(0, level), true, s);
-    }
-    // the context option CKKS_CONV_TENSOR takes the tensor-core conversion of conv_mma.cu: bit-identical, 2 % slower on B200
-    if (c->conv_kernel != CKKS_CONV_TENSOR || !launch_modup_mma(c, w.dcoef, d, d_stride, w.ext, level, nb, s)) {
-#define CALL_UP(A) launch_modup<A>(c, w.dcoef, w.ext, level, nb, s, pre)
+#define CALL_UP(A) launch_modup<A>(c, w.dcoef, w.ext, level, nb, s)
         DISPATCH_POW2(c->alpha, CALL_UP);
 #undef CALL_UP
     }
     launch_ntt(c, w.ext, nb * beta * nt, ext_map(level, c->K, c->L, c->alpha, beta), false, s);
+}
+
+static bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
+static bool aligned16(const Ptrs &p) {
+    if (!p.n) return aligned16(p.base) && (p.stride & 1) == 0;
+    for (uint32_t i = 0; i < p.n; i++)
+        if (!aligned16(p.p[i])) return false;
+    return true;
 }
 
 void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w, cudaStream_t s, uint32_t nb,
@@ -502,10 +470,10 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
     const uint32_t N = c->N, nt = level + c->K;
     const uint32_t beta = (level + c->alpha - 1) / c->alpha;
     const int au = acc_u ? 1 : 0;
-    bool aligned = ((uintptr_t)w.ext & 15) == 0 && ((uintptr_t)w.u & 15) == 0 && ((uintptr_t)w.d & 15) == 0 && (w.d_stride & 1) == 0 && (multi || ((uintptr_t)evk & 15) == 0);
+    bool aligned = aligned16(w.ext) && aligned16(w.u) && aligned16(w.d) && (multi || aligned16(evk));
     const uint32_t nkeys = multi ? (multi->group ? nb / multi->group : nb) : 0;
-    for (uint32_t b = 0; b < nkeys; b++) aligned = aligned && ((uintptr_t)multi->evk[b] & 15) == 0;
-    const bool fast = beta <= IP_MAX_BETA && N >= 2 * THREADS && aligned;
+    for (uint32_t b = 0; b < nkeys; b++) aligned = aligned && aligned16(multi->evk[b]);
+    const bool fast = beta <= IP_MAX_BETA && aligned;
     if (multi && multi->group && !fast) {       // grouped entries without the fast kernel: one key at a time
         for (uint32_t r = 0; r < nkeys; r++) {
             KsWorkspace wr = w;
@@ -514,96 +482,63 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
         }
         return;
     }
+    const KsMulti m = multi ? *multi : KsMulti{};
     if (fast) {
         // batch entries per thread: enough chunks left to fill the machine, key words reused across a chunk
         const uint32_t grp = multi ? multi->group : 0, per = grp ? grp : nb;
         const uint32_t bch = (multi && !grp) ? 1 : (per >= 8 ? 4 : (per >= 4 ? 2 : 1));
         const dim3 grid(N / (2 * THREADS), grp ? (nb / grp) * ((grp + bch - 1) / bch) : (nb + bch - 1) / bch, nt);
-        const KsMulti m = multi ? *multi : KsMulti{};
-        switch (beta) {
-        case 1: inner_product_kernel<1><<<grid, THREADS, 0, s>>>(c->dev, w.ext, w.d, w.d_stride, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au); break;
-        case 2: inner_product_kernel<2><<<grid, THREADS, 0, s>>>(c->dev, w.ext, w.d, w.d_stride, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au); break;
-        case 3: inner_product_kernel<3><<<grid, THREADS, 0, s>>>(c->dev, w.ext, w.d, w.d_stride, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au); break;
-        default: inner_product_kernel<4><<<grid, THREADS, 0, s>>>(c->dev, w.ext, w.d, w.d_stride, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au); break;
-        }
+        auto *k = beta == 1 ? inner_product_kernel<1> : beta == 2 ? inner_product_kernel<2> : beta == 3 ? inner_product_kernel<3> : inner_product_kernel<4>;
+        launch(k, grid, THREADS, 0, s, c->dev, w.ext, w.d, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au);
     } else {
-        inner_product_generic_kernel<<<dim3(N / THREADS, nb, nt), THREADS, 0, s>>>(c->dev, w.ext, w.d, w.d_stride, evk, ext_galois, w.u, level, multi ? 1 : 0,
-                                                                                     multi ? *multi : KsMulti{}, au);
+        launch(inner_product_generic_kernel, dim3(N / THREADS, nb, nt), THREADS, 0, s, c->dev, w.ext, w.d, 0u, evk, ext_galois, w.u, level, multi ? 1 : 0, m, au);
     }
-    count_launches();
 }
 
-void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const u64 *add0, const u64 *add1, u64 add_galois, u64 *out,
-                cudaStream_t s, uint32_t nb, size_t add_stride, size_t out_stride, bool accumulate, TiledOut tiled, const KsMulti *multi) {
+void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb, const KsMulti *multi) {
     const uint32_t N = c->N, nt = level + c->K, K = c->K;
-    // the K special limbs of every (batch, component): groups of K limbs, nt limbs apart; at N = 2^16 the inverse
-    // transform's last stage multiplies Phat^-1 in
-    const bool pre = c->log_n == 16 && c->ntt_fp_share >= 8 && c->conv_kernel != CKKS_CONV_TENSOR;
-    launch_ntt(c, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, nullptr, nullptr, nullptr, 0,
-               pre ? c->dev.inv_scale_dn : nullptr);
-    if (c->conv_kernel != CKKS_CONV_TENSOR || !launch_moddown_conv_mma(c, w.u, w.conv, level, nb, s)) {
-#define CALL_DN(A) launch_moddown_conv<A>(c, w.u, w.conv, level, nb, s, pre)
+    // the K special limbs of every (batch, component): groups of K limbs, nt limbs apart
+    launch_ntt(c, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, nullptr, nullptr, nullptr,
+               conv_tensor(c) ? nullptr : c->dev.inv_scale_dn);
+    if (conv_tensor(c)) {
+        launch_moddown_conv_mma(c, w.u, w.conv, level, nb, s);
+    } else {
+#define CALL_DN(A) launch_moddown_conv<A>(c, w.u, w.conv, level, nb, s)
         DISPATCH_POW2(K, CALL_DN);
 #undef CALL_DN
     }
-    if (c->log_n == 16) {      // the last NTT pass finishes the ModDown itself
-        NttEpilogue ep{1, w.u, add0, add1, out, add_stride, out_stride, add_galois, level, nt, accumulate ? 1 : 0, tiled};
-        ep.multi = multi ? 1 : 0;
-        ep.group = multi ? multi->group : 0;
-        ep.rot_rows = multi ? multi->rot_rows : 0;
-        if (multi)
-            for (uint32_t b = 0; b < KS_MULTI; b++) { ep.mgalois[b] = multi->galois[b]; ep.mout[b] = multi->out[b]; }
-        launch_ntt(c, w.conv, nb * 2 * level, plain_map(0, level), false, s, &ep);
-        return;
-    }
-    launch_ntt(c, w.conv, nb * 2 * level, plain_map(0, level), false, s);
+    NttEpilogue ep{};      // the last NTT pass finishes the ModDown itself
+    ep.mode = 1;
+    ep.u = Ptrs(w.u, (size_t)2 * nt * N);
+    ep.add = o.add; ep.out = o.out; ep.add_comps = o.add_comps;
+    ep.pinv = c->dev.dn_p_inv_d;
+    ep.ncomp = 2; ep.level = level; ep.nt = nt;
+    ep.galois = o.galois; ep.accumulate = o.accumulate ? 1 : 0; ep.tl = o.tiled;
     if (multi) {
-        for (uint32_t b = 0; b < nb; b++) {
-            moddown_final_kernel<<<dim3(N / THREADS, level, 2), THREADS, 0, s>>>(c->dev, w.u + (size_t)b * 2 * nt * N, w.conv + (size_t)b * 2 * level * N,
-                                                                                  add0, add1, 0, multi->galois[b], multi->out[b], 0, 0, level, TiledOut());
-            count_launches();
-        }
-        return;
+        ep.multi = 1; ep.group = multi->group; ep.rot_rows = multi->rot_rows; ep.rot_stride = multi->rot_stride;
+        for (uint32_t b = 0; b < KS_MULTI; b++) { ep.mgalois[b] = multi->galois[b]; ep.out.p[b] = multi->out[b]; }
+        if (!multi->group) ep.out.n = nb;
     }
-    moddown_final_kernel<<<dim3(N / THREADS, level, 2 * nb), THREADS, 0, s>>>(c->dev, w.u, w.conv, add0, add1, add_stride, add_galois, out,
-                                                                               out_stride, accumulate ? 1 : 0, level, tiled);
-    count_launches();
+    launch_ntt(c, w.conv, nb * 2 * level, plain_map(0, level), false, s, &ep);
 }
 
-void ks_inner_moddown(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w,
-                      const u64 *add0, const u64 *add1, u64 add_galois, u64 *out, cudaStream_t s, uint32_t nb,
-                      size_t add_stride, size_t out_stride, bool accumulate, TiledOut tiled, const KsMulti *multi) {
-    ks_inner(c, evk, level, ext_galois, w, s, nb, false, multi);
-    ks_moddown(c, level, w, add0, add1, add_galois, out, s, nb, add_stride, out_stride, accumulate, tiled, multi);
-}
-
-void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, size_t term_stride, size_t d_term_stride, const IpTerms &terms, uint32_t nterm,
+void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, size_t term_stride, const IpTerms &terms, uint32_t nterm,
                     size_t c0_stride, cudaStream_t s, uint32_t nb, bool acc_u) {
     const uint32_t N = c->N, nt = level + c->K, beta = (level + c->alpha - 1) / c->alpha;
-    bool aligned = ((uintptr_t)w.ext & 15) == 0 && ((uintptr_t)w.u & 15) == 0 && (term_stride & 1) == 0 && (c0_stride & 1) == 0 &&
-                   ((uintptr_t)w.d & 15) == 0 && (w.d_stride & 1) == 0 && (d_term_stride & 1) == 0;
-    for (uint32_t t = 0; t < nterm; t++) aligned = aligned && ((uintptr_t)terms.evk[t] & 15) == 0 && ((uintptr_t)terms.c0[t] & 15) == 0;
-    if (beta <= IP_MAX_BETA && N >= 2 * THREADS && aligned) {
+    bool aligned = aligned16(w.ext) && aligned16(w.u) && (term_stride & 1) == 0 && (c0_stride & 1) == 0 && aligned16(w.d);
+    for (uint32_t t = 0; t < nterm; t++) aligned = aligned && aligned16(terms.evk[t]) && aligned16(terms.c0[t]);
+    if (beta <= IP_MAX_BETA && aligned) {
         const dim3 grid(N / (2 * THREADS), (nb + IP_BCH - 1) / IP_BCH, nt);
-        const int au = acc_u ? 1 : 0;
-        switch (beta) {
-        case 1: inner_product_terms_kernel<1><<<grid, THREADS, 0, s>>>(c->dev, w.ext, term_stride, w.d, d_term_stride, w.d_stride, terms, nterm, c0_stride, w.u, level, nb, au); break;
-        case 2: inner_product_terms_kernel<2><<<grid, THREADS, 0, s>>>(c->dev, w.ext, term_stride, w.d, d_term_stride, w.d_stride, terms, nterm, c0_stride, w.u, level, nb, au); break;
-        case 3: inner_product_terms_kernel<3><<<grid, THREADS, 0, s>>>(c->dev, w.ext, term_stride, w.d, d_term_stride, w.d_stride, terms, nterm, c0_stride, w.u, level, nb, au); break;
-        default: inner_product_terms_kernel<4><<<grid, THREADS, 0, s>>>(c->dev, w.ext, term_stride, w.d, d_term_stride, w.d_stride, terms, nterm, c0_stride, w.u, level, nb, au); break;
-        }
-        count_launches();
+        auto *k = beta == 1 ? inner_product_terms_kernel<1> : beta == 2 ? inner_product_terms_kernel<2> : beta == 3 ? inner_product_terms_kernel<3> : inner_product_terms_kernel<4>;
+        launch(k, grid, THREADS, 0, s, c->dev, w.ext, term_stride, w.d.base, w.d.stride, terms, nterm, c0_stride, w.u, level, nb, acc_u ? 1 : 0);
         return;
     }
     // any number of digits, any alignment: one term at a time through the generic kernel, then its P c0
     for (uint32_t t = 0; t < nterm; t++) {
-        inner_product_generic_kernel<<<dim3(N / THREADS, nb, nt), THREADS, 0, s>>>(c->dev, w.ext + t * term_stride, w.d + t * d_term_stride, w.d_stride, terms.evk[t], terms.galois[t],
-                                                                                     w.u, level, 0, KsMulti{}, (acc_u || t > 0) ? 1 : 0);
-        count_launches();
-        if (terms.c0[t]) {
-            p_c0_acc_kernel<<<dim3(N / THREADS, level, nb), THREADS, 0, s>>>(c->dev, terms.c0[t], c0_stride, terms.galois[t], w.u, (size_t)2 * nt * N);
-            count_launches();
-        }
+        launch(inner_product_generic_kernel, dim3(N / THREADS, nb, nt), THREADS, 0, s, c->dev, w.ext + t * term_stride, w.d, t * nb, terms.evk[t], terms.galois[t],
+               w.u, level, 0, KsMulti{}, (acc_u || t > 0) ? 1 : 0);
+        if (terms.c0[t])
+            launch(p_c0_acc_kernel, dim3(N / THREADS, level, nb), THREADS, 0, s, c->dev, terms.c0[t], c0_stride, terms.galois[t], w.u, (size_t)2 * nt * N);
     }
 }
 
@@ -611,21 +546,29 @@ void launch_to_tiled(const ckks_ctx *c, const u64 *src, size_t src_stride, uint3
                      uint32_t row_step, uint32_t level, cudaStream_t s) {
     for (uint32_t r0 = 0; r0 < nrows; r0 += 32768) {
         const uint32_t nr = nrows - r0 < 32768 ? nrows - r0 : 32768;
-        to_tiled_kernel<<<dim3(c->N / (2 * THREADS), level, nr), THREADS, 0, s>>>(c->dev, src + r0 * src_stride, src_stride, dst, R,
-                                                                                   row0 + r0 * row_step, row_step);
-        count_launches();
+        launch(to_tiled_kernel, dim3(c->N / (2 * THREADS), level, nr), THREADS, 0, s, c->dev, src + r0 * src_stride, src_stride, dst, R,
+               row0 + r0 * row_step, row_step);
     }
 }
 
-// ws: [ncomp][N] last limbs + [ncomp][level-1][N]
-void launch_rescale(const ckks_ctx *c, const u64 *in, u64 *out, uint32_t ncomp, uint32_t level, u64 *ws, cudaStream_t s) {
-    const uint32_t N = c->N;
-    u64 *last = ws, *tmp = ws + (size_t)ncomp * N;
-    for (uint32_t comp = 0; comp < ncomp; comp++)
-        cudaMemcpyAsync(last + (size_t)comp * N, in + ((size_t)comp * level + level - 1) * N, (size_t)N * 8,
-                        cudaMemcpyDeviceToDevice, s);
-    launch_ntt(c, last, ncomp, plain_map(level - 1, 1), true, s);
-    rescale_lift_kernel<<<dim3(N / THREADS, level - 1, ncomp), THREADS, 0, s>>>(c->dev, last, tmp, level); count_launches();
-    launch_ntt(c, tmp, ncomp * (level - 1), plain_map(0, level - 1), false, s);
-    rescale_final_kernel<<<dim3(N / THREADS, level - 1, ncomp), THREADS, 0, s>>>(c->dev, in, tmp, out, level); count_launches();
+// Drops the last limb of every component: its inverse transform (out of place), then the forward transform whose first pass
+// lifts it to its centred representative modulo every remaining prime and whose last pass finishes (in - NTT(lift)) q_last^-1.
+// Four launches for the whole batch; copies of the last limbs, the lift and the final step were kernels of their own before
+// (10 operations, 63 -> 36 us for one ciphertext at N = 2^16, level 17).
+// ws: [nb][ncomp][N] last limbs + [nb][ncomp][level-1][N]
+void launch_rescale(const ckks_ctx *c, const Ptrs &in, const Ptrs &out, uint32_t ncomp, uint32_t level, u64 *ws, cudaStream_t s, uint32_t nb) {
+    const size_t N = c->N;
+    u64 *last = ws, *tmp = ws + (size_t)nb * ncomp * N;
+    NttSource src;
+    src.ptr = in; src.lpitch = level;
+    if (in.n) for (uint32_t b = 0; b < in.n; b++) src.ptr.p[b] += (size_t)(level - 1) * N;
+    else src.ptr.base += (size_t)(level - 1) * N;
+    launch_ntt(c, last, nb * ncomp, same_map(level - 1, ncomp), true, s, nullptr, nullptr, &src);
+    NttPrologue pro{last, true, level - 1};
+    NttEpilogue ep{};
+    ep.mode = 1;
+    ep.u = in; ep.out = out;
+    ep.pinv = c->dev.rs_inv_d + (size_t)(level - 1) * c->L;
+    ep.ncomp = ncomp; ep.level = level - 1; ep.nt = level; ep.galois = 1;
+    launch_ntt(c, tmp, nb * ncomp * (level - 1), plain_map(0, level - 1), false, s, &ep, &pro);
 }

@@ -95,6 +95,7 @@ __global__ void __launch_bounds__(COEF * 64 / NW, 8 / COEF) mac_mma_kernel(DevTa
                                                                            const u64 *__restrict__ pts, u64 *__restrict__ acc, uint32_t J,
                                                                            uint32_t S, uint32_t G, uint32_t level, uint32_t ntiles,
                                                                            uint32_t Jx, uint32_t j0, uint32_t accumulate) {
+    grid_dep_sync();
     using T = Geo<COEF>;
     constexpr uint32_t THREADS = COEF * 64 / NW, CH = T::CH;
     constexpr uint32_t AH = THREADS / (CH * MK);      // blocks a loaded side by side; a thread walks a = arow + AH it
@@ -311,6 +312,7 @@ __global__ void __launch_bounds__(COEF * 64 / NW, 8 / COEF) mac_mma_async_kernel
                                                                                  uint32_t J, uint32_t S, uint32_t G, uint32_t level,
                                                                                  uint32_t ntiles, uint32_t Jx, uint32_t j0, uint32_t accumulate,
                                                                                  long long wait_limit) {
+    grid_dep_sync();
     using T = Geo<COEF>;
     constexpr uint32_t THREADS = COEF * 64 / NW, CH = T::CH, NWARPS = THREADS / 32;
     constexpr uint32_t AH = THREADS / (CH * MK), NIT = MG / AH, XB64 = 64 / COEF;
@@ -512,16 +514,13 @@ bool launch_as(const ckks_ctx *c, const u64 *baby, const u64 *pts, u64 *acc, uin
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<COEF>::SMEM_BYTES) != cudaSuccess) return false;
     const uint32_t coltiles = (2 * S + MS - 1) / MS, gt = (G + MG - 1) / MG;
     const uint32_t ntiles = (c->N / COEF) * level * coltiles * gt;
-    int sms = 148;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    const uint32_t ctas = (uint32_t)sms * (8 / COEF), grid = ntiles < ctas ? ntiles : ctas;
+    const uint32_t ctas = (uint32_t)c->sms * (8 / COEF), grid = ntiles < ctas ? ntiles : ctas;
     if (ASYNC)
-        mac_mma_async_kernel<COEF, NW><<<grid, COEF * 64 / NW, Geo<COEF>::SMEM_BYTES, s>>>(c->dev, baby, pts, acc, J, S, G, level, ntiles, Jx, j0,
-                                                                                            accumulate ? 1u : 0u, c->wait_cycles);
+        launch(mac_mma_async_kernel<COEF, NW>, grid, COEF * 64 / NW, Geo<COEF>::SMEM_BYTES, s, c->dev, baby, pts, acc, J, S, G, level, ntiles, Jx, j0,
+               accumulate ? 1u : 0u, c->wait_cycles);
     else
-        mac_mma_kernel<COEF, NW><<<grid, COEF * 64 / NW, Geo<COEF>::SMEM_BYTES, s>>>(c->dev, baby, pts, acc, J, S, G, level, ntiles, Jx, j0,
-                                                                                      accumulate ? 1u : 0u);
-    count_launches();
+        launch(mac_mma_kernel<COEF, NW>, grid, COEF * 64 / NW, Geo<COEF>::SMEM_BYTES, s, c->dev, baby, pts, acc, J, S, G, level, ntiles, Jx, j0,
+               accumulate ? 1u : 0u);
     return true;
 }
 

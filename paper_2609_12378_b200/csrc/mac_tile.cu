@@ -40,6 +40,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // back the words it requested itself, so no block-wide barrier is needed.
 __global__ void __launch_bounds__(MAC_THREADS) mac_tile_kernel(DevTables c, const u64 *__restrict__ baby, const u64 *__restrict__ pts,
                                                                u64 *__restrict__ acc, uint32_t J, uint32_t S, uint32_t G, uint32_t level) {
+    grid_dep_sync();
     __shared__ u64 ring[MAC_DEPTH][MAC_WORDS][MAC_THREADS];
     const uint32_t stiles = (S + MAC_ST - 1) / MAC_ST;
     const uint32_t s0 = (blockIdx.x % stiles) * MAC_ST, g0 = (blockIdx.x / stiles) * MAC_GT;
@@ -113,6 +114,5 @@ __global__ void __launch_bounds__(MAC_THREADS) mac_tile_kernel(DevTables c, cons
 void launch_mac_tile(const ckks_ctx *c, const u64 *baby, const u64 *pts, u64 *acc, uint32_t J, uint32_t S, uint32_t G, uint32_t level,
                      cudaStream_t s) {
     const uint32_t stiles = (S + MAC_ST - 1) / MAC_ST, gtiles = (G + MAC_GT - 1) / MAC_GT;
-    mac_tile_kernel<<<dim3(stiles * gtiles, c->N / MAC_THREADS, level), MAC_THREADS, 0, s>>>(c->dev, baby, pts, acc, J, S, G, level);
-    count_launches();
+    launch(mac_tile_kernel, dim3(stiles * gtiles, c->N / MAC_THREADS, level), MAC_THREADS, 0, s, c->dev, baby, pts, acc, J, S, G, level);
 }

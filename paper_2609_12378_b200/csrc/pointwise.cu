@@ -1,5 +1,5 @@
 // Pointwise (coefficient-wise) kernels on evaluation-domain limbs: ciphertext x
-// plaintext multiply-accumulate, addition, tensor product, Galois automorphism.
+// plaintext multiply-accumulate, addition, tensor product.
 // All are streaming kernels bound by HBM bandwidth: 128-bit loads and stores,
 // one pass over each operand.
 #include "common.cuh"
@@ -17,6 +17,7 @@ struct MacArgs {
 // acc[s][c][i][k] (+)= ct[s][c][i][k] * pt[i][k]; one thread owns two adjacent coefficients of one (c, i).
 template <bool INIT>
 __global__ void __launch_bounds__(THREADS) mac_kernel(DevTables c, MacArgs a, uint32_t ncts, const u64 *pt, uint32_t level) {
+    grid_dep_sync();
     const uint32_t half = c.N / 2;
     const uint32_t x = blockIdx.x * THREADS + threadIdx.x;   // pair index inside the limb
     const uint32_t limb = blockIdx.y, comp = blockIdx.z;
@@ -40,6 +41,7 @@ __global__ void __launch_bounds__(THREADS) mac_kernel(DevTables c, MacArgs a, ui
 }
 
 __global__ void __launch_bounds__(THREADS) add_kernel(DevTables c, const u64 *a, const u64 *b, u64 *out, uint32_t level) {
+    grid_dep_sync();
     const uint32_t half = c.N / 2;
     const uint32_t x = blockIdx.x * THREADS + threadIdx.x;
     if (x >= half) return;
@@ -49,17 +51,9 @@ __global__ void __launch_bounds__(THREADS) add_kernel(DevTables c, const u64 *a,
     reinterpret_cast<ulonglong2 *>(out)[off] = make_ulonglong2(add_mod(u.x, v.x, q), add_mod(u.y, v.y, q));
 }
 
-// out[y][p] = in[y][pi(p)], 2 bitrev(pi(p)) + 1 = g (2 bitrev(p) + 1) mod 2N
-__global__ void __launch_bounds__(THREADS) automorphism_kernel(DevTables c, const u64 *in, u64 *out, u64 g) {
-    const uint32_t p = blockIdx.x * THREADS + threadIdx.x;
-    if (p >= c.N) return;
-    const u64 e = (g * (2ull * bitrev_n(p, c.log_n) + 1)) & (2ull * c.N - 1);
-    const uint32_t src = bitrev_n((uint32_t)((e - 1) >> 1), c.log_n);
-    out[(size_t)blockIdx.y * c.N + p] = in[(size_t)blockIdx.y * c.N + src];
-}
-
 // (a0 b0, a0 b1 + a1 b0) -> e01 [2][level][N];  a1 b1 -> e2 [level][N]
 __global__ void __launch_bounds__(THREADS) tensor_kernel(DevTables c, const u64 *a, const u64 *b, u64 *e01, u64 *e2, uint32_t level) {
+    grid_dep_sync();
     const uint32_t k = blockIdx.x * THREADS + threadIdx.x;
     if (k >= c.N) return;
     const uint32_t limb = blockIdx.y;
@@ -79,6 +73,7 @@ __global__ void __launch_bounds__(THREADS) tensor_kernel(DevTables c, const u64 
 // every position of the evaluation domain); blockIdx.y = component * level + limb
 template <bool MUL>
 __global__ void __launch_bounds__(THREADS) const_kernel(DevTables c, const u64 *in, long long v, u64 *out, uint32_t level) {
+    grid_dep_sync();
     const uint32_t half = c.N / 2;
     const uint32_t x = blockIdx.x * THREADS + threadIdx.x;
     if (x >= half) return;
@@ -97,6 +92,7 @@ __global__ void __launch_bounds__(THREADS) const_kernel(DevTables c, const u64 *
 // 2^112), one Barrett step per component, then the previous partial sum is added unless INIT
 template <bool INIT>
 __global__ void __launch_bounds__(THREADS) tensor_sum_kernel(DevTables c, TensorSumArgs args, uint32_t n, u64 *e01, u64 *e2, uint32_t level) {
+    grid_dep_sync();
     const uint32_t k = blockIdx.x * THREADS + threadIdx.x;
     if (k >= c.N) return;
     const uint32_t limb = blockIdx.y;
@@ -122,6 +118,7 @@ __global__ void __launch_bounds__(THREADS) tensor_sum_kernel(DevTables c, Tensor
 // out[x] = 1.0 where lo <= x / B < hi and t0 <= x % Ti < t1, else 0.0 (slot masks of the attention layout's conversions)
 __global__ void __launch_bounds__(THREADS) slot_mask_kernel(double *out, uint32_t n, uint32_t B, uint32_t lo, uint32_t hi, uint32_t Ti, uint32_t t0,
                                                             uint32_t t1) {
+    grid_dep_sync();
     const uint32_t x = blockIdx.x * THREADS + threadIdx.x;
     if (x >= n) return;
     const uint32_t blk = x / B, t = x % Ti;
@@ -129,15 +126,13 @@ __global__ void __launch_bounds__(THREADS) slot_mask_kernel(double *out, uint32_
 }
 
 void launch_slot_mask(const ckks_ctx *c, double *out, uint32_t B, uint32_t lo, uint32_t hi, uint32_t Ti, uint32_t t0, uint32_t t1, cudaStream_t s) {
-    slot_mask_kernel<<<(c->n + THREADS - 1) / THREADS, THREADS, 0, s>>>(out, c->n, B, lo, hi, Ti, t0, t1);
-    count_launches();
+    launch(slot_mask_kernel, (c->n + THREADS - 1) / THREADS, THREADS, 0, s, out, c->n, B, lo, hi, Ti, t0, t1);
 }
 
 void launch_const(const ckks_ctx *c, const u64 *in, long long v, bool mul, u64 *out, uint32_t ncomp, uint32_t level, cudaStream_t s) {
     dim3 grid((c->N / 2 + THREADS - 1) / THREADS, ncomp * level);
-    if (mul) const_kernel<true><<<grid, THREADS, 0, s>>>(c->dev, in, v, out, level);
-    else const_kernel<false><<<grid, THREADS, 0, s>>>(c->dev, in, v, out, level);
-    count_launches();
+    if (mul) launch(const_kernel<true>, grid, THREADS, 0, s, c->dev, in, v, out, level);
+    else launch(const_kernel<false>, grid, THREADS, 0, s, c->dev, in, v, out, level);
 }
 
 void launch_tensor_sum(const ckks_ctx *c, const u64 *const *a, const u64 *const *b, uint32_t n, u64 *e01, u64 *e2, uint32_t level,
@@ -147,9 +142,8 @@ void launch_tensor_sum(const ckks_ctx *c, const u64 *const *a, const u64 *const 
         TensorSumArgs args;
         const uint32_t m = n - i0 < TS_MAX ? n - i0 : TS_MAX;
         for (uint32_t i = 0; i < m; i++) { args.a[i] = a[i0 + i]; args.b[i] = b[i0 + i]; }
-        if (i0 == 0) tensor_sum_kernel<true><<<grid, THREADS, 0, s>>>(c->dev, args, m, e01, e2, level);
-        else tensor_sum_kernel<false><<<grid, THREADS, 0, s>>>(c->dev, args, m, e01, e2, level);
-        count_launches();
+        if (i0 == 0) launch(tensor_sum_kernel<true>, grid, THREADS, 0, s, c->dev, args, m, e01, e2, level);
+        else launch(tensor_sum_kernel<false>, grid, THREADS, 0, s, c->dev, args, m, e01, e2, level);
     }
 }
 
@@ -160,22 +154,16 @@ void launch_mul_plain_acc(const ckks_ctx *c, const u64 *const *cts, u64 *const *
         MacArgs a;
         uint32_t n = ncts - s0 < MAC_MAX ? ncts - s0 : MAC_MAX;
         for (uint32_t i = 0; i < n; i++) { a.ct[i] = cts[s0 + i]; a.acc[i] = accs[s0 + i]; }
-        if (init) { mac_kernel<true><<<grid, THREADS, 0, s>>>(c->dev, a, n, pt, level); count_launches(); }
-        else { mac_kernel<false><<<grid, THREADS, 0, s>>>(c->dev, a, n, pt, level); count_launches(); }
+        launch(init ? mac_kernel<true> : mac_kernel<false>, grid, THREADS, 0, s, c->dev, a, n, pt, level);
     }
 }
 
 void launch_add(const ckks_ctx *c, const u64 *a, const u64 *b, u64 *out, uint32_t ncomp, uint32_t level, cudaStream_t s) {
     dim3 grid((c->N / 2 + THREADS - 1) / THREADS, ncomp * level);
-    add_kernel<<<grid, THREADS, 0, s>>>(c->dev, a, b, out, level); count_launches();
-}
-
-void launch_automorphism(const ckks_ctx *c, const u64 *in, u64 *out, uint32_t nlimbs, u64 galois, cudaStream_t s) {
-    dim3 grid((c->N + THREADS - 1) / THREADS, nlimbs);
-    automorphism_kernel<<<grid, THREADS, 0, s>>>(c->dev, in, out, galois); count_launches();
+    launch(add_kernel, grid, THREADS, 0, s, c->dev, a, b, out, level);
 }
 
 void launch_tensor(const ckks_ctx *c, const u64 *a, const u64 *b, u64 *e01, u64 *e2, uint32_t level, cudaStream_t s) {
     dim3 grid((c->N + THREADS - 1) / THREADS, level);
-    tensor_kernel<<<grid, THREADS, 0, s>>>(c->dev, a, b, e01, e2, level); count_launches();
+    launch(tensor_kernel, grid, THREADS, 0, s, c->dev, a, b, e01, e2, level);
 }

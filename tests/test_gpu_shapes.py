@@ -31,3 +31,79 @@ def test_basis_conversion_at_the_ends_of_the_residues(L, K, dnum, level):
     gal = o.galois_element(3)
     out = ctx.rotate(ct_dev(ct, 1.0), key_dev(key, gal))
     assert np.array_equal(host(out.data), o.rotate(ct, key, gal))
+
+
+@pytest.mark.parametrize("log_n", range(10, 17))
+@pytest.mark.parametrize("batch,limbs", [(1, 1), (5, 3)])
+def test_transforms_of_every_ring_at_extreme_residues(log_n, batch, limbs):
+    """Both directions on constant, alternating and random limbs (the lazy ranges of the butterflies peak where every input
+    is 0 or q - 1), in a 16-byte aligned buffer and in one that is only 8-byte aligned."""
+    import torch
+    from tests.gpu_util import context, host
+    P, ctx = params(log_n, 3, 1, 3), context(log_n, 3, 1, 3)
+    o, g = P.oracle, inputs.rng(710, log_n)
+    x = inputs.uniform_residues(g, P.q[:limbs], P.N, batch)
+    for i in range(limbs):
+        q = int(P.q[i])
+        x[0, i] = q - 1
+        if batch > 1:
+            x[1, i] = np.where(np.arange(P.N) & 1, q - 1, 0)
+            x[2, i] = np.where(g.integers(0, 2, P.N), q - 1, 0)
+            x[3, i] = np.where(g.integers(0, 2, P.N), q // 2, q // 2 + 1)
+    fwd, inv = o.ntt(x), o.intt(x)
+    for offset in (0, 1):
+        buf = torch.zeros(x.size + 1, dtype=torch.int64, device="cuda").view(torch.uint64)
+        y = buf[offset:offset + x.size].view(batch, limbs, P.N)
+        y.copy_(torch.from_numpy(x))
+        assert np.array_equal(host(ctx.ntt(y)), fwd)
+        y.copy_(torch.from_numpy(x))
+        assert np.array_equal(host(ctx.intt(y)), inv)
+        assert int(buf[x.size if offset == 0 else 0]) == 0
+
+
+@pytest.mark.parametrize("log_n,level", [(10, 2), (13, 3), (15, 3), (16, 2)])
+@pytest.mark.parametrize("ncomp", [1, 2])
+def test_rescale_components_and_alignment(log_n, level, ncomp):
+    """One and two components; dropped residues at the ends of their centred range; one component in place; buffers that are
+    only 8-byte aligned."""
+    import torch
+    from tests.gpu_util import context, ct_dev, host
+    from paper_2609_12378_b200 import binding
+    P, ctx = params(log_n, 3, 1, 3), context(log_n, 3, 1, 3)
+    g = inputs.rng(720, log_n)
+    x = inputs.uniform_residues(g, P.q[:level], P.N, ncomp)
+    q = int(P.q[level - 1])
+    d = np.array([0, 1, q - 1, q // 2, q // 2 + 1], dtype=np.uint64)[g.integers(0, 5, P.N)]
+    full = np.zeros((1, 3, P.N), dtype=np.uint64)
+    full[0, level - 1] = d
+    x[0, level - 1] = P.oracle.ntt(full)[0, level - 1]
+    want = P.oracle.rescale(x)
+    out = ctx.rescale(ct_dev(x, 1.0))
+    assert np.array_equal(host(out.data), want)
+    buf = torch.zeros(x.size + 1, dtype=torch.int64, device="cuda").view(torch.uint64)
+    y = buf[1:].view(ncomp, level, P.N)
+    y.copy_(torch.from_numpy(x))
+    assert np.array_equal(host(ctx.rescale(binding.Ciphertext(y, 1.0)).data), want)
+    if ncomp == 1:
+        ct = ct_dev(x, 1.0)
+        short = binding.Ciphertext(ct.data.view(-1)[:(level - 1) * P.N].view(1, level - 1, P.N), 0.0)
+        ctx.rescale(ct, out=short)
+        assert np.array_equal(host(short.data), want)
+
+
+@pytest.mark.parametrize("log_n", [11, 14, 16])
+def test_encode_coefficients_of_every_size(log_n):
+    """Coefficients below 2^49 are taken as residues as they are, larger ones (here up to 2^61) are reduced; a batch mixes
+    both, and one plaintext has a single large coefficient's worth of slots."""
+    from tests.gpu_util import context, dev, host
+    P, ctx = params(log_n, 3, 1, 3), context(log_n, 3, 1, 3)
+    g = inputs.rng(730, log_n)
+    z = g.uniform(-1, 1, (4, P.n))
+    z[1] *= 2.0 ** 20
+    z[2] = 2.0 ** 9          # one coefficient of 2^59, the others zero
+    z[3, 1:] = 0.0
+    for scale in (2.0 ** 30, 2.0 ** 50):
+        zz = z if scale < 2.0 ** 40 else z * np.array([[1.0], [2.0 ** -10], [1.0], [1.0]])
+        got = host(ctx.encode(dev(zz), None, scale, 3))
+        for b in range(4):
+            assert np.array_equal(got[b], P.oracle.encode(zz[b], scale, 3)), (scale, b)
