@@ -135,13 +135,12 @@ const char *ckks_last_cuda_error(const ckks_ctx *ctx);
  *                           satisfied give up at once (used to test that path).
  *   CKKS_OPT_NTT_BULK_STORE 0 or 1 (default), kept for programs that set it: it chose between 128-byte bulk copies and 32-byte
  *                           accesses of the transforms' row passes, which now move 16 bytes per lane either way.
- *   CKKS_OPT_LANES          1..4 (default 4): streams over which the attention entry points spread their independent
- *                           single-ciphertext chains (per channel, per score group).  Lane 0 is the caller's stream, the
- *                           others belong to the context; they are forked from and joined to the caller's stream by events
- *                           inside the call, so the call still behaves as work on the caller's stream.  The workspace sizes
- *                           of those calls depend on it: set it before asking for them.  Results do not depend on it.
- *                           The lanes' streams and events belong to the context: two host threads must not run attention
- *                           entry points on the same context at the same time (use a context per thread).
+ *   CKKS_OPT_LANES          1..4 (default 4): streams over which ckks_attention_pack spreads its independent chains (one per
+ *                           channel).  Lane 0 is the caller's stream, the others belong to the context; they are forked from and
+ *                           joined to the caller's stream by events inside the call, so the call still behaves as work on the
+ *                           caller's stream.  Its workspace size depends on it: set it before asking.  Results do not depend on it.
+ *                           The lanes' streams and events belong to the context: two host threads must not run
+ *                           ckks_attention_pack on the same context at the same time (use a context per thread).
  *   CKKS_OPT_STATIC_SCRATCH_BYTES  (read only) CKKS_STATIC_SCRATCH_BYTES of the loaded library.
  * set returns CKKS_ERR_ARG for an unknown option or a value outside its range; get returns -1 for an unknown option. */
 enum { CKKS_OPT_NTT_FP_SHARE = 1, CKKS_OPT_CONV_KERNEL = 2, CKKS_OPT_MAC_KERNEL = 3, CKKS_OPT_WAIT_CYCLES = 4,
@@ -280,8 +279,7 @@ int32_t ckks_poly_eval_bsgs(ckks_ctx *ctx, const ckks_ct *x, const double *coeff
                             ckks_ct *out, void *ws, size_t ws_bytes, void *stream);
 size_t ckks_poly_eval_bsgs_workspace_bytes(const ckks_ctx *ctx, uint32_t level, uint32_t degree, uint32_t m);
 /* The same polynomial of n ciphertexts at one level (an activation function over a layer's ciphertexts): every out[i] is
- * bit-identical to ckks_poly_eval_bsgs(x[i]); the n independent chains are spread over the context's lanes
- * (CKKS_OPT_LANES), each with a workspace of its own.  Errors as ckks_poly_eval_bsgs. */
+ * bit-identical to ckks_poly_eval_bsgs(x[i]); up to four ciphertexts of one scale run side by side.  Errors as ckks_poly_eval_bsgs. */
 int32_t ckks_poly_eval_bsgs_batch(ckks_ctx *ctx, const ckks_ct *x, uint32_t n, const double *coeffs, uint32_t degree, uint32_t m,
                                   const ckks_evk *rlk, ckks_ct *out, void *ws, size_t ws_bytes, void *stream);
 size_t ckks_poly_eval_bsgs_batch_workspace_bytes(const ckks_ctx *ctx, uint32_t level, uint32_t degree, uint32_t m, uint32_t n);

@@ -8,22 +8,7 @@
 
 namespace {
 
-struct DeviceGuard {
-    int prev = 0;
-    explicit DeviceGuard(int dev) { cudaGetDevice(&prev); cudaSetDevice(dev); }
-    ~DeviceGuard() { cudaSetDevice(prev); }
-};
-
-int finish(ckks_ctx *c) {
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) { c->cuda_error = cudaGetErrorString(e); return CKKS_ERR_CUDA; }
-    return CKKS_OK;
-}
-
 bool scales_agree(double a, double b) { return fabs(a - b) <= ldexp(fmax(fabs(a), fabs(b)), -30); }
-bool level_ok(const ckks_ctx *c, uint32_t level) { return level >= 1 && level <= c->L; }
-bool ct_ok(const ckks_ct *ct) { return ct && ct->data; }
-size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 size_t ks_bytes(const ckks_ctx *c, uint32_t level) { return ks_workspace_limbs(c, level) * c->N * sizeof(u64); }
 // hoisted rotations: one set of digits, nbh rotations' worth of inner-product and ModDown buffers side by side
@@ -31,7 +16,7 @@ size_t hoisted_bytes(const ckks_ctx *c, uint32_t level, uint32_t nbh) {
     const size_t beta = (level + c->alpha - 1) / c->alpha, nt = level + c->K;
     return (level + beta * nt + (size_t)nbh * (2 * nt + 2 * level)) * c->N * sizeof(u64);
 }
-constexpr uint32_t MRB_CHUNK = 16;      // products key-switched side by side by ckks_mul_relin_batch
+constexpr uint32_t MRB_CHUNK = 16;      // products key-switched side by side (at most KS_MULTI)
 size_t rescale_bytes(const ckks_ctx *c, uint32_t level, uint32_t ncomp) { return (size_t)ncomp * level * c->N * sizeof(u64); }
 
 // ---- projection plan -------------------------------------------------------
@@ -120,7 +105,7 @@ ProjWs proj_layout(const ckks_ctx *c, const ProjPlan &p, uint32_t level, bool la
     w.acc = off;   off += align256(ct * p.S * w.gacc);
     w.total = off; off += align256(ct * p.S);
     w.tmp = off;   off += align256(ct);
-    w.rs = off;    off += align256(rescale_bytes(c, level, 2));
+    w.rs = off;    off += align256(rescale_bytes(c, level, 2) * std::min(p.S, KS_MULTI));
     const size_t shared = off;
     w.ptt = off;   off += align256(pt * npt);               // encoded plaintexts of a group, tiled: rows g * J + j
     w.pts = off;   off += align256(pt * nenc);              // plain layout: the encoder's words between its two NTT passes
@@ -159,19 +144,17 @@ extern "C" size_t ckks_workspace_bytes(const ckks_ctx *c, int32_t op, uint32_t l
         case CKKS_OP_ROTATE_HOISTED: return hoisted_bytes(c, level, std::min<uint32_t>(count ? count : 1, KS_MULTI));
         case CKKS_OP_RESCALE: return rescale_bytes(c, level, 2);
         // per product of a chunk (at most MRB_CHUNK): the staged result, e_2 and a key-switch workspace
-        // per ciphertext of a chunk: staged input, staged output and a key-switch workspace
+        // per ciphertext of a chunk: a staged input and a key-switch workspace
         case CKKS_OP_ROTATE_BATCH:
-            return (size_t)std::min<uint32_t>(count ? count : 1, MRB_CHUNK) * ((size_t)4 * level * limb + ks_bytes(c, level));
+            return (size_t)std::min<uint32_t>(count ? count : 1, MRB_CHUNK) * ((size_t)2 * level * limb + ks_bytes(c, level));
         // a chunk of staged inputs with their key-switch workspaces
         case CKKS_OP_ROTATE_SUM:
             return (size_t)std::min<uint32_t>(count ? count : 1, MRB_CHUNK) * ((size_t)2 * level * limb + ks_bytes(c, level));
         case CKKS_OP_MUL_RELIN_BATCH:
-            return (size_t)std::min<uint32_t>(count ? count : 1, MRB_CHUNK) * ((size_t)3 * level * limb + ks_bytes(c, level));
-        // two running ciphertexts, the truncated copy of x, then the Mult and rescale scratch
-        case CKKS_OP_POLY_EVAL: return 3 * (size_t)2 * level * limb + ks_bytes(c, level) + (size_t)level * limb + rescale_bytes(c, level, 2);
-        // the powers x^2..x^degree, two truncated operands, the product, the accumulator and a term, then the scratch
-        case CKKS_OP_POLY_EVAL_TREE:
-            return ((size_t)(count > 1 ? count - 1 : 1) + 5) * 2 * level * limb + ks_bytes(c, level) + (size_t)level * limb + rescale_bytes(c, level, 2);
+            return (size_t)std::min<uint32_t>(count ? count : 1, MRB_CHUNK) * product_bytes(c, level);
+        // two running ciphertexts, then the Mult and rescale scratch
+        case CKKS_OP_POLY_EVAL: return 2 * (size_t)2 * level * limb + ks_bytes(c, level) + (size_t)level * limb + rescale_bytes(c, level, 2);
+        case CKKS_OP_POLY_EVAL_TREE: return poly_tree_bytes(c, level, count, 1);
         default: return 0;
     }
 }
@@ -270,30 +253,6 @@ extern "C" int32_t ckks_add(ckks_ctx *c, const ckks_ct *a, const ckks_ct *b, ckk
     return rc;
 }
 
-// o[2][level][N] += key switch of e2
-static void relinearise(const ckks_ctx *c, const u64 *rlk, const u64 *e2, u64 *o, uint32_t level, KsWorkspace &w, cudaStream_t s) {
-    ks_modup(c, Ptrs(e2, 0), level, w, s);
-    ks_inner(c, rlk, level, 1, w, s);
-    KsOut ko;
-    ko.add = ko.out = Ptrs(o, 0);
-    ko.add_comps = 3;
-    ks_moddown(c, level, w, ko, s);
-}
-// rotation of nb ciphertexts by one key: c0, c1 at in, in + level * N
-static void rotate_ks(const ckks_ctx *c, const ckks_evk *key, const Ptrs &in, const Ptrs &out, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb = 1,
-                      bool accumulate = false) {
-    Ptrs c1 = in;
-    const size_t ptl = (size_t)level * c->N;
-    if (in.n) for (uint32_t b = 0; b < in.n; b++) c1.p[b] += ptl;
-    else c1.base += ptl;
-    ks_modup(c, c1, level, w, s, nb);
-    ks_inner(c, (const u64 *)key->data, level, key->galois, w, s, nb);
-    KsOut ko;
-    ko.add = in; ko.out = out;
-    ko.add_comps = 1; ko.galois = key->galois; ko.accumulate = accumulate;
-    ks_moddown(c, level, w, ko, s, nb);
-}
-
 extern "C" int32_t ckks_mul_relin(ckks_ctx *c, const ckks_ct *a, const ckks_ct *b, const ckks_evk *rlk, ckks_ct *out, void *ws,
                                   size_t ws_bytes, void *stream) {
     if (!c || !ct_ok(a) || !ct_ok(b) || !ct_ok(out) || a->ncomp != 2 || b->ncomp != 2) return CKKS_ERR_ARG;
@@ -306,8 +265,11 @@ extern "C" int32_t ckks_mul_relin(ckks_ctx *c, const ckks_ct *a, const ckks_ct *
     u64 *e2 = (u64 *)ws;
     KsWorkspace w = ks_carve(c, level, e2 + (size_t)level * c->N);
     u64 *o = (u64 *)out->data;
-    launch_tensor(c, (const u64 *)a->data, (const u64 *)b->data, o, e2, level, s);
-    relinearise(c, (const u64 *)rlk->data, e2, o, level, w, s);
+    auto view = [&](const ckks_ct *t) { return CtView{(const u64 *)t->data, (size_t)level * c->N}; };
+    TensorArgs ta;
+    ta.a[0] = view(a); ta.b[0] = view(b); ta.e01[0] = o; ta.e2[0] = e2;
+    launch_tensor(c, ta, 1, level, s);
+    relinearise(c, (const u64 *)rlk->data, Ptrs(e2, 0), Ptrs(o, 0), level, w, s);
     int rc = finish(c);
     if (rc == CKKS_OK) { out->level = level; out->ncomp = 2; out->scale = a->scale * b->scale; }
     return rc;
@@ -342,17 +304,25 @@ extern "C" int32_t ckks_mul_relin_batch(ckks_ctx *c, const ckks_ct *a, const ckk
     for (uint32_t i0 = 0; i0 < n; i0 += MRB_CHUNK) {
         const uint32_t m = std::min(MRB_CHUNK, n - i0);
         u64 *stage = (u64 *)ws, *e2 = stage + (size_t)m * ctl;
+        // results go straight to their place unless another product of the chunk still has to read what lies there
+        bool staged = false;
+        for (uint32_t i = 0; i < m; i++)
+            for (uint32_t j = 0; j < m; j++)
+                staged = staged || (i != j && (out[i0 + i].data == a[i0 + j].data || out[i0 + i].data == b[i0 + j].data || out[i0 + i].data == out[i0 + j].data));
+        TensorArgs ta;
+        Ptrs o(stage, ctl);
+        for (uint32_t i = 0; i < m; i++) {
+            ta.a[i] = CtView{(const u64 *)a[i0 + i].data, ptl}; ta.b[i] = CtView{(const u64 *)b[i0 + i].data, ptl};
+            ta.e01[i] = staged ? stage + (size_t)i * ctl : (u64 *)out[i0 + i].data;
+            ta.e2[i] = e2 + (size_t)i * ptl;
+            if (!staged) o.p[i] = (const u64 *)out[i0 + i].data;
+        }
+        if (!staged) o.n = m;
         KsWorkspace w = ks_carve(c, level, e2 + (size_t)m * ptl, m);
-        for (uint32_t i = 0; i < m; i++)
-            launch_tensor(c, (const u64 *)a[i0 + i].data, (const u64 *)b[i0 + i].data, stage + (size_t)i * ctl, e2 + (size_t)i * ptl, level, s);
+        launch_tensor(c, ta, m, level, s);
         // the m key switches run side by side: one ModUp, one inner product, one ModDown over the whole chunk
-        ks_modup(c, Ptrs(e2, ptl), level, w, s, m);
-        ks_inner(c, (const u64 *)rlk->data, level, 1, w, s, m);
-        KsOut ko;
-        ko.add = ko.out = Ptrs(stage, ctl);
-        ko.add_comps = 3;
-        ks_moddown(c, level, w, ko, s, m);
-        for (uint32_t i = 0; i < m; i++)
+        relinearise(c, (const u64 *)rlk->data, Ptrs(e2, ptl), o, level, w, s, m);
+        for (uint32_t i = 0; i < m && staged; i++)
             cudaMemcpyAsync(out[i0 + i].data, stage + (size_t)i * ctl, ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
     }
     int rc = finish(c);
@@ -380,16 +350,16 @@ extern "C" int32_t ckks_mul_relin_sum(ckks_ctx *c, const ckks_ct *a, const ckks_
     u64 *e2 = (u64 *)ws;
     KsWorkspace w = ks_carve(c, level, e2 + (size_t)level * c->N);
     u64 *o = (u64 *)out->data;
-    std::vector<const u64 *> pa(n), pb(n);
-    for (uint32_t i = 0; i < n; i++) { pa[i] = (const u64 *)a[i].data; pb[i] = (const u64 *)b[i].data; }
+    std::vector<CtView> pa(n), pb(n);
+    for (uint32_t i = 0; i < n; i++) { pa[i] = CtView{(const u64 *)a[i].data, (size_t)level * c->N}; pb[i] = CtView{(const u64 *)b[i].data, (size_t)level * c->N}; }
     launch_tensor_sum(c, pa.data(), pb.data(), n, o, e2, level, s);
-    relinearise(c, (const u64 *)rlk->data, e2, o, level, w, s);
+    relinearise(c, (const u64 *)rlk->data, Ptrs(e2, 0), Ptrs(o, 0), level, w, s);
     int rc = finish(c);
     if (rc == CKKS_OK) { out->level = level; out->ncomp = 2; out->scale = a[0].scale * b[0].scale; }
     return rc;
 }
 
-static bool const_value(double c, double scale, long long *v) {
+bool const_value(double c, double scale, long long *v) {
     const double x = c * scale;
     if (!(fabs(x) < 4611686018427387904.0)) return false;      // 2^62; also rejects NaN
     *v = llrint(x);                                            // round half to even in the default rounding mode
@@ -403,7 +373,7 @@ extern "C" int32_t ckks_mul_const(ckks_ctx *c, const ckks_ct *in, double cv, dou
     long long v;
     if (!const_value(cv, cs, &v)) return CKKS_ERR_RANGE;
     DeviceGuard g(c->device);
-    launch_const(c, (const u64 *)in->data, v, true, (u64 *)out->data, in->ncomp, in->level, (cudaStream_t)stream);
+    launch_const(c, Ptrs((const u64 *)in->data, 0), v, true, Ptrs((u64 *)out->data, 0), in->ncomp, in->level, (cudaStream_t)stream);
     int rc = finish(c);
     if (rc == CKKS_OK) { out->level = in->level; out->ncomp = in->ncomp; out->scale = in->scale * cs; }
     return rc;
@@ -415,7 +385,7 @@ extern "C" int32_t ckks_add_const(ckks_ctx *c, const ckks_ct *in, double cv, ckk
     long long v;
     if (!const_value(cv, in->scale, &v)) return CKKS_ERR_RANGE;
     DeviceGuard g(c->device);
-    launch_const(c, (const u64 *)in->data, v, false, (u64 *)out->data, in->ncomp, in->level, (cudaStream_t)stream);
+    launch_const(c, Ptrs((const u64 *)in->data, 0), v, false, Ptrs((u64 *)out->data, 0), in->ncomp, in->level, (cudaStream_t)stream);
     int rc = finish(c);
     if (rc == CKKS_OK) { out->level = in->level; out->ncomp = in->ncomp; out->scale = in->scale; }
     return rc;
@@ -450,26 +420,27 @@ extern "C" int32_t ckks_poly_eval(ckks_ctx *c, const ckks_ct *x, const double *c
     DeviceGuard g(c->device);
     cudaStream_t s = (cudaStream_t)stream;
     const size_t N = c->N, ctw = (size_t)2 * level * N;
-    u64 *ra = (u64 *)ws, *rb = ra + ctw, *xt = rb + ctw, *e2 = xt + ctw;
+    u64 *ra = (u64 *)ws, *rb = ra + ctw, *e2 = rb + ctw;
     u64 *ksw = e2 + (size_t)level * N;
     u64 *rsw = (u64 *)((char *)ksw + ks_bytes(c, level));
     const u64 *xd = (const u64 *)x->data;
     // r = x * c_d; rescale; + c_{d-1}
-    launch_const(c, xd, vs[degree], true, ra, 2, level, s);
+    launch_const(c, Ptrs(xd, 0), vs[degree], true, Ptrs(ra, 0), 2, level, s);
     launch_rescale(c, Ptrs(ra, 0), Ptrs(rb, 0), 2, level, rsw, s);
     uint32_t lvl = level - 1;
-    launch_const(c, rb, vs[degree - 1], false, rb, 2, lvl, s);
+    launch_const(c, Ptrs(rb, 0), vs[degree - 1], false, Ptrs(rb, 0), 2, lvl, s);
     u64 *cur = rb, *other = ra;
     for (uint32_t k = degree - 1; k-- > 0;) {
-        // x truncated to lvl limbs per component
-        for (uint32_t comp = 0; comp < 2; comp++)
-            cudaMemcpyAsync(xt + (size_t)comp * lvl * N, xd + (size_t)comp * level * N, (size_t)lvl * N * sizeof(u64), cudaMemcpyDeviceToDevice, s);
         KsWorkspace w = ks_carve(c, lvl, ksw);
-        launch_tensor(c, cur, xt, other, e2, lvl, s);
-        relinearise(c, (const u64 *)rlk->data, e2, other, lvl, w, s);
+        TensorArgs ta;
+        ta.a[0] = CtView{cur, (size_t)lvl * N};
+        ta.b[0] = CtView{xd, (size_t)level * N};         // x truncated to lvl limbs per component
+        ta.e01[0] = other; ta.e2[0] = e2;
+        launch_tensor(c, ta, 1, lvl, s);
+        relinearise(c, (const u64 *)rlk->data, Ptrs(e2, 0), Ptrs(other, 0), lvl, w, s);
         launch_rescale(c, Ptrs(other, 0), Ptrs(cur, 0), 2, lvl, rsw, s);
         lvl--;
-        launch_const(c, cur, vs[k], false, cur, 2, lvl, s);
+        launch_const(c, Ptrs(cur, 0), vs[k], false, Ptrs(cur, 0), 2, lvl, s);
     }
     cudaMemcpyAsync(out->data, cur, (size_t)2 * lvl * N * sizeof(u64), cudaMemcpyDeviceToDevice, s);
     int rc = finish(c);
@@ -477,250 +448,20 @@ extern "C" int32_t ckks_poly_eval(ckks_ctx *c, const ckks_ct *x, const double *c
     return rc;
 }
 
-extern "C" int32_t ckks_poly_eval_tree(ckks_ctx *c, const ckks_ct *x, const double *coeffs, uint32_t degree, const ckks_evk *rlk,
-                                       ckks_ct *out, void *ws, size_t ws_bytes, void *stream) {
-    if (!c || !ct_ok(x) || !ct_ok(out) || x->ncomp != 2 || !coeffs || degree < 2) return CKKS_ERR_ARG;
-    const uint32_t level = x->level;
-    uint32_t depth = 0;
-    while ((1u << depth) < degree) depth++;
-    if (!level_ok(c, level) || level < depth + 2) return CKKS_ERR_LEVEL;
-    if (!rlk || !rlk->data || rlk->galois != 0) return CKKS_ERR_NO_KEY;
-    if (!ws || ws_bytes < ckks_workspace_bytes(c, CKKS_OP_POLY_EVAL_TREE, level, degree)) return CKKS_ERR_WORKSPACE;
-    // levels and scales of the powers, the combination's constants: all fixed and range-checked before the first launch
-    std::vector<uint32_t> lvl(degree + 1);
-    std::vector<double> sc(degree + 1);
-    lvl[1] = level; sc[1] = x->scale;
-    for (uint32_t k = 2; k <= degree; k++) {
-        const uint32_t a = k / 2, b = k - a, lv = std::min(lvl[a], lvl[b]);
-        sc[k] = sc[a] * sc[b] / (double)c->mod[lv - 1];
-        lvl[k] = lv - 1;
-    }
-    const uint32_t Lt = lvl[degree];
-    const double T = x->scale * (double)c->mod[Lt - 1], so = T / (double)c->mod[Lt - 1];
-    std::vector<long long> vs(degree + 1, 0);
-    bool any = false;
-    for (uint32_t k = 1; k <= degree; k++) {
-        if (coeffs[k] == 0.0) continue;
-        any = true;
-        if (!const_value(coeffs[k], T / sc[k], &vs[k])) return CKKS_ERR_RANGE;
-    }
-    if (!any) return CKKS_ERR_ARG;
-    if (!const_value(coeffs[0], so, &vs[0])) return CKKS_ERR_RANGE;
-
-    DeviceGuard g(c->device);
-    cudaStream_t s = (cudaStream_t)stream;
-    const size_t N = c->N, ctw = (size_t)2 * level * N;
-    u64 *pw = (u64 *)ws;                                        // x^k at pw + (k - 2) * ctw, k >= 2
-    u64 *ta = pw + (size_t)(degree - 1) * ctw, *tb = ta + ctw, *prod = tb + ctw, *acc = prod + ctw, *term = acc + ctw;
-    u64 *e2 = term + ctw, *ksw = e2 + (size_t)level * N;
-    u64 *rsw = (u64 *)((char *)ksw + ks_bytes(c, level));
-    const u64 *xd = (const u64 *)x->data;
-    auto power = [&](uint32_t k) { return k == 1 ? xd : pw + (size_t)(k - 2) * ctw; };
-    // [2][from][N] -> [2][to][N], to <= from
-    auto truncate = [&](const u64 *src, uint32_t from, uint32_t to, u64 *dst) {
-        for (uint32_t comp = 0; comp < 2; comp++)
-            cudaMemcpyAsync(dst + (size_t)comp * to * N, src + (size_t)comp * from * N, (size_t)to * N * sizeof(u64), cudaMemcpyDeviceToDevice, s);
-    };
-    for (uint32_t k = 2; k <= degree; k++) {
-        const uint32_t a = k / 2, b = k - a, lv = std::min(lvl[a], lvl[b]);
-        const u64 *pa = power(a), *pb = power(b);
-        if (lvl[a] != lv) { truncate(pa, lvl[a], lv, ta); pa = ta; }
-        if (lvl[b] != lv) { truncate(pb, lvl[b], lv, tb); pb = tb; }
-        KsWorkspace w = ks_carve(c, lv, ksw);
-        launch_tensor(c, pa, pb, prod, e2, lv, s);
-        relinearise(c, (const u64 *)rlk->data, e2, prod, lv, w, s);
-        launch_rescale(c, Ptrs(prod, 0), Ptrs(pw + (size_t)(k - 2) * ctw, 0), 2, lv, rsw, s);
-    }
-    bool first = true;
-    for (uint32_t k = 1; k <= degree; k++) {
-        if (coeffs[k] == 0.0) continue;
-        const u64 *pk = power(k);
-        if (lvl[k] != Lt) { truncate(pk, lvl[k], Lt, ta); pk = ta; }
-        launch_const(c, pk, vs[k], true, first ? acc : term, 2, Lt, s);
-        if (!first) launch_add(c, acc, term, acc, 2, Lt, s);
-        first = false;
-    }
-    launch_rescale(c, Ptrs(acc, 0), Ptrs((u64 *)out->data, 0), 2, Lt, rsw, s);
-    launch_const(c, (const u64 *)out->data, vs[0], false, (u64 *)out->data, 2, Lt - 1, s);
-    int rc = finish(c);
-    if (rc == CKKS_OK) { out->level = Lt - 1; out->ncomp = 2; out->scale = so; }
-    return rc;
-}
-
-// ---- Baby-step / giant-step polynomial evaluation: a composition of the entry points above
-static bool bsgs_shape_ok(uint32_t degree, uint32_t m) { return m >= 2 && !(m & (m - 1)) && m <= degree; }
-static size_t bsgs_scratch_bytes(const ckks_ctx *c, uint32_t level) {
-    return align256(std::max(ckks_workspace_bytes(c, CKKS_OP_MUL_RELIN, level, 0), ckks_workspace_bytes(c, CKKS_OP_RESCALE, level, 0)));
-}
-static uint32_t bsgs_buffers(uint32_t degree, uint32_t m) {
-    const uint32_t G = degree / m + 1;
-    return (m - 1) + (G > 2 ? G - 2 : 0) + 2 * (G - 1) + 6;      // baby powers, giant powers, blocks and truncated giants, temporaries
-}
-
-extern "C" size_t ckks_poly_eval_bsgs_workspace_bytes(const ckks_ctx *c, uint32_t level, uint32_t degree, uint32_t m) {
-    if (!c || !level_ok(c, level) || !bsgs_shape_ok(degree, m)) return 0;
-    return (size_t)bsgs_buffers(degree, m) * align256((size_t)2 * level * c->N * sizeof(u64)) + bsgs_scratch_bytes(c, level);
-}
-
-extern "C" int32_t ckks_poly_eval_bsgs(ckks_ctx *c, const ckks_ct *x, const double *coeffs, uint32_t degree, uint32_t m, const ckks_evk *rlk,
-                                       ckks_ct *out, void *ws, size_t ws_bytes, void *stream) {
-    if (!c || !ct_ok(x) || !ct_ok(out) || x->ncomp != 2 || !coeffs || !bsgs_shape_ok(degree, m)) return CKKS_ERR_ARG;
-    const uint32_t level = x->level, G = degree / m + 1;
-    if (!level_ok(c, level)) return CKKS_ERR_LEVEL;
-    if (!rlk || !rlk->data || rlk->galois != 0) return CKKS_ERR_NO_KEY;
-    // levels of the powers (operands k / 2 and k - k / 2, one level per product)
-    std::vector<uint32_t> lb(m + 1), lg(G);
-    lb[1] = level;
-    for (uint32_t k = 2; k <= m; k++) {
-        const uint32_t lv = std::min(lb[k / 2], lb[k - k / 2]);
-        if (lv < 2) return CKKS_ERR_LEVEL;
-        lb[k] = lv - 1;
-    }
-    lg[1] = lb[m];
-    for (uint32_t i = 2; i < G; i++) {
-        const uint32_t lv = std::min(lg[i / 2], lg[i - i / 2]);
-        if (lv < 2) return CKKS_ERR_LEVEL;
-        lg[i] = lv - 1;
-    }
-    const uint32_t Lb = lb[m - 1], Lc = std::min(lg[G - 1], Lb - 1);
-    if (Lb < 2 || Lc < 2) return CKKS_ERR_LEVEL;
-    if (!ws || ws_bytes < ckks_poly_eval_bsgs_workspace_bytes(c, level, degree, m)) return CKKS_ERR_WORKSPACE;
-    auto coef = [&](uint32_t k) { return k <= degree ? coeffs[k] : 0.0; };
-    auto q = [&](uint32_t l) { return (double)c->mod[l - 1]; };
-
-    const size_t N = c->N, ctb = align256((size_t)2 * level * N * sizeof(u64)), scratch = bsgs_scratch_bytes(c, level);
-    char *base = (char *)ws;
-    uint32_t next = 0;
-    auto buffer = [&]() { return ckks_ct{(uint64_t *)(base + (size_t)(next++) * ctb), level, 2, 0.0}; };
-    std::vector<ckks_ct> pw(m + 1), gp(G);
-    pw[1] = *x;
-    for (uint32_t k = 2; k <= m; k++) pw[k] = buffer();
-    for (uint32_t i = 2; i < G; i++) gp[i] = buffer();
-    std::vector<ckks_ct> blk(G), gpt(G);
-    for (uint32_t i = 1; i < G; i++) { blk[i] = buffer(); gpt[i] = buffer(); }
-    ckks_ct ta = buffer(), tb = buffer(), prod = buffer(), acc = buffer(), term = buffer(), S = buffer();
-    void *sw = base + (size_t)bsgs_buffers(degree, m) * ctb;
-    cudaStream_t s = (cudaStream_t)stream;
-    DeviceGuard guard(c->device);
-    // src cut down to `to` limbs per component (a copy into dst), or src itself if it has that many
-    auto at_level = [&](const ckks_ct &src, uint32_t to, ckks_ct &dst) -> ckks_ct {
-        if (src.level == to) return src;
-        for (uint32_t comp = 0; comp < 2; comp++)
-            cudaMemcpyAsync(dst.data + (size_t)comp * to * N, src.data + (size_t)comp * src.level * N, (size_t)to * N * sizeof(u64),
-                            cudaMemcpyDeviceToDevice, s);
-        dst.level = to; dst.ncomp = 2; dst.scale = src.scale;
-        return dst;
-    };
-    int rc;
-    auto powers = [&](std::vector<ckks_ct> &p, uint32_t top) -> int {
-        for (uint32_t k = 2; k <= top; k++) {
-            const uint32_t a = k / 2, b = k - a, lv = std::min(p[a].level, p[b].level);
-            const ckks_ct pa = at_level(p[a], lv, ta), pb = at_level(p[b], lv, tb);
-            int r;
-            if ((r = ckks_mul_relin(c, &pa, &pb, rlk, &prod, sw, scratch, stream))) return r;
-            if ((r = ckks_rescale(c, &prod, &p[k], sw, scratch, stream))) return r;
-        }
-        return CKKS_OK;
-    };
-    if ((rc = powers(pw, m))) return rc;
-    gp[1] = pw[m];
-    if ((rc = powers(gp, G - 1))) return rc;
-    const double Tp = x->scale * q(Lc);
-    // the blocks B_i, i >= 1, encoded so that B_i y^i has scale Tp; constant-only blocks are kept for later
-    std::vector<ckks_ct> A, B;
-    std::vector<uint32_t> const_only;
-    for (uint32_t i = 1; i < G; i++) {
-        const double Ti = (Tp / gp[i].scale) * q(Lb);
-        bool first = true;
-        for (uint32_t j = 1; j < m; j++) {
-            if (coef(i * m + j) == 0.0) continue;
-            const ckks_ct pj = at_level(pw[j], Lb, ta);
-            ckks_ct &dst = first ? acc : term;
-            if ((rc = ckks_mul_const(c, &pj, coef(i * m + j), Ti / pw[j].scale, &dst, stream))) return rc;
-            if (!first && (rc = ckks_add(c, &acc, &term, &acc, stream))) return rc;
-            first = false;
-        }
-        if (first) {
-            if (coef(i * m) != 0.0) const_only.push_back(i);
-            continue;
-        }
-        acc.scale = Ti;
-        if ((rc = ckks_rescale(c, &acc, &prod, sw, scratch, stream))) return rc;
-        if ((rc = ckks_add_const(c, &prod, coef(i * m), &prod, stream))) return rc;
-        ckks_ct a = at_level(prod, Lc, blk[i]);
-        if (a.data == prod.data) {       // already at the common level: keep a copy, prod is reused
-            cudaMemcpyAsync(blk[i].data, prod.data, (size_t)2 * Lc * N * sizeof(u64), cudaMemcpyDeviceToDevice, s);
-            blk[i].level = Lc; blk[i].ncomp = 2;
-            a = blk[i];
-        }
-        ckks_ct b = at_level(gp[i], Lc, gpt[i]);
-        a.scale = 1.0; b.scale = Tp;      // the products agree in scale (Tp up to rounding); the factors need not
-        A.push_back(a); B.push_back(b);
-    }
-    bool have = false;
-    if (!A.empty()) {
-        if ((rc = ckks_mul_relin_sum(c, A.data(), B.data(), (uint32_t)A.size(), rlk, &S, sw, scratch, stream))) return rc;
-        have = true;
-    }
-    auto add_in = [&](const ckks_ct &src, double cv, double cs) -> int {
-        const ckks_ct p = at_level(src, Lc, ta);
-        ckks_ct &dst = have ? term : S;
-        int r;
-        if ((r = ckks_mul_const(c, &p, cv, cs, &dst, stream))) return r;
-        dst.scale = Tp;
-        if (have && (r = ckks_add(c, &S, &term, &S, stream))) return r;
-        have = true;
-        return CKKS_OK;
-    };
-    S.scale = Tp;
-    for (uint32_t j = 1; j < m; j++)
-        if (coef(j) != 0.0 && (rc = add_in(pw[j], coef(j), Tp / pw[j].scale))) return rc;
-    for (uint32_t i : const_only)
-        if ((rc = add_in(gp[i], coef(i * m), Tp / gp[i].scale))) return rc;
-    if (!have) return CKKS_ERR_ARG;
-    S.scale = Tp;
-    if ((rc = ckks_rescale(c, &S, out, sw, scratch, stream))) return rc;
-    return ckks_add_const(c, out, coef(0), out, stream);
-}
-
 // ---- Softmax by doubling (Algorithm 1): a composition of the entry points above on buffers carved from the workspace
 static uint32_t log2_ceil(uint32_t x) { uint32_t d = 0; while ((1u << d) < x) d++; return d; }
 static size_t softmax_scratch_bytes(const ckks_ctx *c, const ckks_softmax_desc *d, uint32_t level) {
     const uint32_t deg = std::max(d->exp_degree, d->rsqrt_degree);
     size_t b = std::max(ckks_workspace_bytes(c, CKKS_OP_POLY_EVAL_TREE, level, deg),
-                        std::max(ckks_workspace_bytes(c, CKKS_OP_MUL_RELIN, level, 0), ckks_workspace_bytes(c, CKKS_OP_RESCALE, level, 0)));
+                        product_bytes(c, level));
     if (d->exp_m) b = std::max(b, ckks_poly_eval_bsgs_workspace_bytes(c, level, d->exp_degree, d->exp_m));
     if (d->rsqrt_m && d->rounds) b = std::max(b, ckks_poly_eval_bsgs_workspace_bytes(c, level, d->rsqrt_degree, d->rsqrt_m));
     return align256(b);
 }
 static bool softmax_desc_ok(const ckks_ctx *c, const ckks_softmax_desc *d) {
     return d && d->exp_coeffs && d->exp_degree >= 2 && (d->rounds == 0 || (d->rsqrt_coeffs && d->rsqrt_degree >= 2)) && d->row_len >= 2 &&
-           !(d->row_len & (d->row_len - 1)) && c->n % d->row_len == 0 && (!d->exp_m || bsgs_shape_ok(d->exp_degree, d->exp_m)) &&
-           (!d->rsqrt_m || !d->rounds || bsgs_shape_ok(d->rsqrt_degree, d->rsqrt_m));
-}
-
-// The same polynomial of n ciphertexts: independent chains, spread over the context's lanes with a workspace each.
-extern "C" size_t ckks_poly_eval_bsgs_batch_workspace_bytes(const ckks_ctx *c, uint32_t level, uint32_t degree, uint32_t m, uint32_t n) {
-    const size_t one = ckks_poly_eval_bsgs_workspace_bytes(c, level, degree, m);
-    return one ? align256(one) * std::min<uint32_t>(std::max<uint32_t>(n, 1), lane_count(c)) : 0;
-}
-
-extern "C" int32_t ckks_poly_eval_bsgs_batch(ckks_ctx *c, const ckks_ct *x, uint32_t n, const double *coeffs, uint32_t degree, uint32_t m,
-                                             const ckks_evk *rlk, ckks_ct *out, void *ws, size_t ws_bytes, void *stream) {
-    if (!c || !x || !out || !n) return CKKS_ERR_ARG;
-    for (uint32_t i = 0; i < n; i++)
-        if (!ct_ok(&x[i]) || !ct_ok(&out[i]) || x[i].level != x[0].level) return x && ct_ok(&x[i]) && ct_ok(&out[i]) ? CKKS_ERR_LEVEL : CKKS_ERR_ARG;
-    const size_t one = align256(ckks_poly_eval_bsgs_workspace_bytes(c, x[0].level, degree, m));
-    if (!one) return CKKS_ERR_ARG;
-    const Lanes lanes(c, stream);
-    const uint32_t nl = std::min<uint32_t>(n, lanes.n);
-    if (!ws || ws_bytes < one * nl) return CKKS_ERR_WORKSPACE;
-    int rc = CKKS_OK;
-    lanes.fork();
-    for (uint32_t i = 0; i < n && !rc; i++)
-        rc = ckks_poly_eval_bsgs(c, &x[i], coeffs, degree, m, rlk, &out[i], (char *)ws + (size_t)(i % nl) * one, one, lanes.at(i % nl));
-    lanes.join();
-    return rc;
+           !(d->row_len & (d->row_len - 1)) && c->n % d->row_len == 0 && (!d->exp_m || poly_bsgs_shape_ok(d->exp_degree, d->exp_m)) &&
+           (!d->rsqrt_m || !d->rounds || poly_bsgs_shape_ok(d->rsqrt_degree, d->rsqrt_m));
 }
 
 extern "C" size_t ckks_softmax_workspace_bytes(const ckks_ctx *c, const ckks_softmax_desc *d, uint32_t level) {
@@ -758,32 +499,36 @@ extern "C" int32_t ckks_softmax(ckks_ctx *c, const ckks_softmax_desc *d, const c
         return bm ? ckks_poly_eval_bsgs(c, x, co, deg, bm, rlk, o, sw, scratch, stream) : ckks_poly_eval_tree(c, x, co, deg, rlk, o, sw, scratch, stream);
     };
     if ((rc = poly(&A, d->exp_coeffs, d->exp_degree, d->exp_m, &U))) return rc;
+    DeviceGuard guard(c->device);
+    const u64 *rk_data = (const u64 *)rlk->data;
+    auto view = [&](const ckks_ct &t) { return CtView{(const u64 *)t.data, (size_t)t.level * N}; };
+    // dst = rescale(relin(a b)) at a level both operands reach
+    auto mul = [&](const ckks_ct &a, const ckks_ct &b, ckks_ct &dst) {
+        const uint32_t lv = std::min(a.level, b.level);
+        const CtView va = view(a), vb = view(b);
+        u64 *o = (u64 *)dst.data;
+        const double sc = a.scale * b.scale / (double)c->mod[lv - 1];
+        mul_rescale(c, &va, &vb, &o, 1, rk_data, lv, sw, 1, s);
+        dst.level = lv - 1; dst.ncomp = 2; dst.scale = sc;
+    };
     for (uint32_t j = 0; j < d->rounds; j++) {
-        // s = row sums of u^2
-        if ((rc = ckks_mul_relin(c, &U, &U, rlk, &A, sw, scratch, stream))) return rc;
-        if ((rc = ckks_rescale(c, &A, &S, sw, scratch, stream))) return rc;
+        // s = row sums of u^2, the ladder going back and forth between two buffers
+        if (U.level < 2) return CKKS_ERR_LEVEL;
+        mul(U, U, S);
         for (const ckks_evk *k : rk) {
-            if ((rc = ckks_rotate(c, &S, k, &A, sw, scratch, stream))) return rc;
-            if ((rc = ckks_add(c, &S, &A, &S, stream))) return rc;
+            KsWorkspace w = ks_carve(c, S.level, sw);
+            const Ptrs from((const u64 *)S.data, 0);
+            rotate_ks(c, k, from, Ptrs((const u64 *)A.data, 0), S.level, w, s, 1, &from);
+            A.level = S.level; A.scale = S.scale;
+            std::swap(S, A);
         }
         // lambda = p_rsqrt_j(s);  u = (lambda u)^2
         if ((rc = poly(&S, d->rsqrt_coeffs + (size_t)j * (d->rsqrt_degree + 1), d->rsqrt_degree, d->rsqrt_m, &B))) return rc;
-        {
-            DeviceGuard g(c->device);       // u truncated to lambda's level
-            for (uint32_t comp = 0; comp < 2; comp++)
-                cudaMemcpyAsync((u64 *)A.data + (size_t)comp * B.level * N, (const u64 *)U.data + (size_t)comp * U.level * N,
-                                (size_t)B.level * N * sizeof(u64), cudaMemcpyDeviceToDevice, s);
-            A.level = B.level; A.ncomp = 2; A.scale = U.scale;
-        }
-        if ((rc = ckks_mul_relin(c, &B, &A, rlk, &S, sw, scratch, stream))) return rc;
-        if ((rc = ckks_rescale(c, &S, &A, sw, scratch, stream))) return rc;
-        if ((rc = ckks_mul_relin(c, &A, &A, rlk, &S, sw, scratch, stream))) return rc;
-        if ((rc = ckks_rescale(c, &S, &U, sw, scratch, stream))) return rc;
+        if (std::min(B.level, U.level) < 3) return CKKS_ERR_LEVEL;
+        mul(B, U, A);
+        mul(A, A, U);
     }
-    {
-        DeviceGuard g(c->device);
-        cudaMemcpyAsync(out->data, U.data, (size_t)2 * U.level * N * sizeof(u64), cudaMemcpyDeviceToDevice, s);
-    }
+    cudaMemcpyAsync(out->data, U.data, (size_t)2 * U.level * N * sizeof(u64), cudaMemcpyDeviceToDevice, s);
     rc = finish(c);
     if (rc == CKKS_OK) { out->level = U.level; out->ncomp = 2; out->scale = U.scale; }
     return rc;
@@ -819,13 +564,21 @@ extern "C" int32_t ckks_rotate_batch(ckks_ctx *c, const ckks_ct *in, uint32_t n,
     const size_t N = c->N, ctl = (size_t)2 * level * N, ptl = (size_t)level * N;
     for (uint32_t i0 = 0; i0 < n; i0 += MRB_CHUNK) {
         const uint32_t m = std::min(MRB_CHUNK, n - i0);
-        u64 *xin = (u64 *)ws, *xout = xin + (size_t)m * ctl;
-        KsWorkspace w = ks_carve(c, level, xout + (size_t)m * ctl, m);
-        for (uint32_t i = 0; i < m; i++)
-            cudaMemcpyAsync(xin + (size_t)i * ctl, in[i0 + i].data, ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
-        rotate_ks(c, key, Ptrs(xin, ctl), Ptrs(xout, ctl), level, w, s, m);
-        for (uint32_t i = 0; i < m; i++)
-            cudaMemcpyAsync(out[i0 + i].data, xout + (size_t)i * ctl, ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
+        // a result may lie where an input of the chunk does: such inputs are copied first
+        u64 *xin = (u64 *)ws;
+        KsWorkspace w = ks_carve(c, level, xin + (size_t)m * ctl, m);
+        Ptrs src, dst;
+        src.n = dst.n = m;
+        for (uint32_t i = 0; i < m; i++) {
+            src.p[i] = (const u64 *)in[i0 + i].data;
+            dst.p[i] = (const u64 *)out[i0 + i].data;
+            bool alias = false;
+            for (uint32_t j = 0; j < m; j++) alias = alias || out[i0 + j].data == in[i0 + i].data;
+            if (!alias) continue;
+            cudaMemcpyAsync(xin + (size_t)i * ctl, src.p[i], ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
+            src.p[i] = xin + (size_t)i * ctl;
+        }
+        rotate_ks(c, key, src, dst, level, w, s, m);
     }
     int rc = finish(c);
     if (rc == CKKS_OK)
@@ -1073,7 +826,8 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
                     }
                     const u64 ge = ckks_galois_element(c, (int64_t)gi * B * T);
                     // total[sh] += rotate(acc_g[sh]) for all shards in one batch
-                    rotate_ks(c, find_key(keys, nkeys, ge), Ptrs(ag, ctl), Ptrs(total, ctl), level, kw, s, S, true);
+                    const Ptrs tot(total, ctl);
+                    rotate_ks(c, find_key(keys, nkeys, ge), Ptrs(ag, ctl), tot, level, kw, s, S, &tot);
                 }
                 // lazy: the key-switched parts of up to IP_TERMS giant steps (all shards) are extended in one batch and
                 // added to the running sum in the key-switching basis in one pass, their first components with them
@@ -1182,15 +936,20 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
                 ko.add_comps = 3;
                 ks_moddown(c, level, kw, ko, s, S);
             }
+            u64 *folded = total;
             for (uint32_t f = o.size; fold > 1; f *= 2, fold /= 2) {
-                const u64 ge = ckks_galois_element(c, (int64_t)f * T);
-                // total += rotate(total): the rotated copy goes to the (now free) accumulator buffer first
-                rotate_ks(c, find_key(keys, nkeys, ge), Ptrs(total, ctl), Ptrs(acc, ctl), level, kw, s, S);
-                for (uint32_t sh = 0; sh < S; sh++)
-                    launch_add(c, total + (size_t)sh * ctl, acc + (size_t)sh * ctl, total + (size_t)sh * ctl, 2, level, s);
+                // folded + rotate(folded), back and forth between the total and the (now free) accumulator buffer
+                u64 *dst = folded == total ? acc : total;
+                const Ptrs from(folded, ctl);
+                rotate_ks(c, find_key(keys, nkeys, ckks_galois_element(c, (int64_t)f * T)), from, Ptrs(dst, ctl), level, kw, s, S, &from);
+                folded = dst;
             }
-            for (uint32_t sh = 0; sh < S; sh++)
-                launch_rescale(c, Ptrs(total + (size_t)sh * ctl, 0), Ptrs((u64 *)out_m[sh * nob + ob].data, 0), 2, level, rsw, s);
+            for (uint32_t s0 = 0; s0 < S; s0 += KS_MULTI) {
+                Ptrs po;
+                po.n = std::min(KS_MULTI, S - s0);
+                for (uint32_t k = 0; k < po.n; k++) po.p[k] = (const u64 *)out_m[(s0 + k) * nob + ob].data;
+                launch_rescale(c, Ptrs(folded + (size_t)s0 * ctl, ctl), po, 2, level, rsw, s, po.n);
+            }
         }
         out_m += S * nob;
     }

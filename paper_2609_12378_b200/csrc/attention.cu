@@ -52,24 +52,12 @@ const ckks_evk *find_key(const ckks_ctx *c, const ckks_evk *keys, uint32_t nkeys
     return nullptr;
 }
 
-size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 size_t ct_bytes(const ckks_ctx *c, uint32_t level) { return align256((size_t)2 * level * c->N * sizeof(uint64_t)); }
-size_t scratch_bytes(const ckks_ctx *c, uint32_t level, uint32_t nrot) {
-    return align256(std::max({ckks_workspace_bytes(c, CKKS_OP_MUL_RELIN, level, 0), ckks_workspace_bytes(c, CKKS_OP_RESCALE, level, 0),
-                              ckks_workspace_bytes(c, CKKS_OP_ROTATE_HOISTED, level, nrot ? nrot : 1),
-                              ckks_workspace_bytes(c, CKKS_OP_ROTATE, level, 0)}));
+// scratch of the steps over `n` ciphertexts: `nrot` rotations of each (side by side), sums of products and their rescale
+size_t scratch_bytes(const ckks_ctx *c, uint32_t level, uint32_t n, uint32_t nrot, uint32_t nsum) {
+    return align256(std::max(nrot ? rotate_grid_bytes(c, level, n, nrot) : 0, (size_t)std::min(nsum, KS_MULTI) * product_bytes(c, level)));
 }
-
-// s += rotate(s, r) for the ladder rotations in ascending order; tmp: a ciphertext buffer
-int block_ladder(ckks_ctx *c, const AttnPlan &p, const ckks_evk *keys, uint32_t nkeys, ckks_ct *s, ckks_ct *tmp, void *sw, size_t sw_bytes,
-                 void *stream) {
-    for (int64_t r : p.lad) {
-        int rc;
-        if ((rc = ckks_rotate(c, s, find_key(c, keys, nkeys, r), tmp, sw, sw_bytes, stream))) return rc;
-        if ((rc = ckks_add(c, s, tmp, s, stream))) return rc;
-    }
-    return CKKS_OK;
-}
+CtView view(const ckks_ctx *c, const ckks_ct &t) { return CtView{(const u64 *)t.data, (size_t)t.level * c->N}; }
 
 int check_cts(const ckks_ctx *c, const ckks_ct *cts, uint32_t n, uint32_t *level, bool same_scale) {
     if (!cts || !n) return CKKS_ERR_ARG;
@@ -104,60 +92,60 @@ extern "C" int32_t ckks_attention_rotations(const ckks_ctx *c, const ckks_attn_d
 }
 
 // ---- scores -------------------------------------------------------------------------------------------------------
-// workspace: [pass groups][dim] rotated key operands, one product, the scratch of the calls
+// workspace: [pass groups][dim] rotated key operands, the scratch of the steps
 extern "C" size_t ckks_attention_scores_workspace_bytes(const ckks_ctx *c, const ckks_attn_desc *d, uint32_t level, uint32_t dim) {
     AttnPlan p;
     if (!c || !dim || level < 2 || level > c->L || make_attn_plan(c, d, p)) return 0;
-    // the split holds Gb - 1 rotated key sets, G / Gb - 1 rotated query sets, a product and a rescaled product
+    // the split holds Gb - 1 rotated key sets, G / Gb - 1 rotated query sets and the rescaled sums of one giant step
     if (p.Gb > 1)
-        return (size_t)(p.Gb + p.G / p.Gb - 2) * dim * ct_bytes(c, level) + 2 * ct_bytes(c, level) + lane_count(c) * scratch_bytes(c, level, p.G - 1);
-    return (size_t)(p.G - 1) * dim * ct_bytes(c, level) + ct_bytes(c, level) + scratch_bytes(c, level, p.G - 1);
+        return (size_t)(p.Gb + p.G / p.Gb - 2) * dim * ct_bytes(c, level) + p.Gb * ct_bytes(c, level) +
+               scratch_bytes(c, level, dim, std::max(p.Gb, p.G / p.Gb) - 1, p.G);
+    return (size_t)(p.G - 1) * dim * ct_bytes(c, level) + scratch_bytes(c, level, dim, p.G - 1, p.G);
 }
 
 // scores with the groups split into Gb baby and G / Gb giant steps
 static int scores_split(ckks_ctx *c, const AttnPlan &p, const ckks_ct *q, const ckks_ct *k, uint32_t dim, uint32_t level, const ckks_evk *rlk,
-                        const ckks_evk *keys, uint32_t nkeys, ckks_ct *scores, void *ws, size_t ws_bytes, void *stream) {
+                        const ckks_evk *keys, uint32_t nkeys, ckks_ct *scores, void *ws, cudaStream_t s) {
     const uint32_t Gb = p.Gb, Gg = p.G / p.Gb;
-    const size_t ctb = ct_bytes(c, level);
-    char *base = (char *)ws;
-    char *kr = base, *qr = base + (size_t)(Gb - 1) * dim * ctb;         // [Gb - 1][dim], [Gg - 1][dim] ciphertexts
-    char *rest = qr + (size_t)(Gg - 1) * dim * ctb;
-    ckks_ct prod{(uint64_t *)rest, level, 2, 0.0}, resc{(uint64_t *)(rest + ctb), level - 1, 2, 0.0};
-    void *sw = rest + 2 * ctb;
-    const size_t sw_bytes = scratch_bytes(c, level, p.G - 1);
-    int rc = CKKS_OK;
+    const size_t ctw = ct_bytes(c, level) / sizeof(u64), N = c->N;
+    u64 *kr = (u64 *)ws, *qr = kr + (size_t)(Gb - 1) * dim * ctw;         // [Gb - 1][dim], [Gg - 1][dim] ciphertexts
+    u64 *resc = qr + (size_t)(Gg - 1) * dim * ctw;                        // [Gb] rescaled sums of a giant step
+    void *sw = resc + Gb * ctw;
     std::vector<ckks_evk> bk, gk;
     for (uint32_t g0 = 1; g0 < Gb; g0++) bk.push_back(*find_key(c, keys, nkeys, p.tok[g0 - 1]));
     for (int64_t r : p.neg) gk.push_back(*find_key(c, keys, nkeys, r));
-    std::vector<ckks_ct> outs(std::max(Gb, Gg));
-    // the channels' rotations are independent: spread over the lanes, each with its own scratch
-    const Lanes lanes(c, stream);
-    lanes.fork();
-    for (uint32_t dd = 0; dd < dim && !rc; dd++) {
-        void *lw = (char *)sw + (dd % lanes.n) * sw_bytes, *ls = lanes.at(dd);
-        for (uint32_t x = 0; x + 1 < Gb; x++) outs[x] = ckks_ct{(uint64_t *)(kr + ((size_t)x * dim + dd) * ctb), level, 2, 0.0};
-        if (Gb > 1) rc = ckks_rotate_hoisted(c, &k[dd], bk.data(), Gb - 1, outs.data(), lw, sw_bytes, ls);
-        for (uint32_t y = 0; y + 1 < Gg; y++) outs[y] = ckks_ct{(uint64_t *)(qr + ((size_t)y * dim + dd) * ctb), level, 2, 0.0};
-        if (!rc && Gg > 1) rc = ckks_rotate_hoisted(c, &q[dd], gk.data(), Gg - 1, outs.data(), lw, sw_bytes, ls);
-    }
-    lanes.join();
-    if (rc) return rc;
-    std::vector<ckks_ct> a(dim), b(dim);
-    for (uint32_t g = 0; g < p.G; g++) {
-        const uint32_t g1 = g / Gb, g0 = g % Gb;
-        for (uint32_t dd = 0; dd < dim; dd++) {
-            a[dd] = g1 ? ckks_ct{(uint64_t *)(qr + ((size_t)(g1 - 1) * dim + dd) * ctb), level, 2, q[dd].scale} : q[dd];
-            b[dd] = g0 ? ckks_ct{(uint64_t *)(kr + ((size_t)(g0 - 1) * dim + dd) * ctb), level, 2, k[dd].scale} : k[dd];
+    std::vector<CtView> vq, vk;
+    for (uint32_t dd = 0; dd < dim; dd++) { vq.push_back(view(c, q[dd])); vk.push_back(view(c, k[dd])); }
+    DeviceGuard guard(c->device);
+    rotate_grid(c, vk.data(), dim, bk.data(), Gb - 1, kr, dim * ctw, ctw, level, sw, s);
+    rotate_grid(c, vq.data(), dim, gk.data(), Gg - 1, qr, dim * ctw, ctw, level, sw, s);
+    auto set = [&](const u64 *base, uint32_t x) {
+        std::vector<CtView> v(dim);
+        for (uint32_t dd = 0; dd < dim; dd++) v[dd] = CtView{base + ((size_t)x * dim + dd) * ctw, (size_t)level * N};
+        return v;
+    };
+    // all groups of one giant step: their sums side by side, then their rotation by it
+    const double scale = q[0].scale * k[0].scale / (double)c->mod[level - 1];
+    for (uint32_t g1 = 0; g1 < Gg; g1++) {
+        std::vector<std::vector<CtView>> a, b;
+        std::vector<u64 *> out;
+        for (uint32_t g0 = 0; g0 < Gb; g0++) {
+            a.push_back(g1 ? set(qr, g1 - 1) : vq);
+            b.push_back(g0 ? set(kr, g0 - 1) : vk);
+            out.push_back(g1 ? resc + g0 * ctw : (u64 *)scores[g0].data);
         }
-        if ((rc = ckks_mul_relin_sum(c, a.data(), b.data(), dim, rlk, &prod, sw, sw_bytes, stream))) return rc;
-        if (!g1) {
-            if ((rc = ckks_rescale(c, &prod, &scores[g], sw, sw_bytes, stream))) return rc;
-            continue;
+        sum_rescale(c, a, b, out.data(), Gb, (const u64 *)rlk->data, level, sw, s);
+        for (uint32_t i0 = 0; i0 < Gb && g1; i0 += KS_MULTI) {
+            Ptrs po;
+            po.n = std::min(KS_MULTI, Gb - i0);
+            for (uint32_t i = 0; i < po.n; i++) po.p[i] = (const u64 *)scores[g1 * Gb + i0 + i].data;
+            KsWorkspace w = ks_carve(c, level - 1, sw, po.n);
+            rotate_ks(c, find_key(c, keys, nkeys, p.tok[g1 * Gb - 1]), Ptrs(resc + i0 * ctw, ctw), po, level - 1, w, s, po.n);
         }
-        if ((rc = ckks_rescale(c, &prod, &resc, sw, sw_bytes, stream))) return rc;
-        if ((rc = ckks_rotate(c, &resc, find_key(c, keys, nkeys, p.tok[g1 * Gb - 1]), &scores[g], sw, sw_bytes, stream))) return rc;
     }
-    return CKKS_OK;
+    const int rc = finish(c);
+    for (uint32_t g = 0; g < p.G && rc == CKKS_OK; g++) { scores[g].level = level - 1; scores[g].ncomp = 2; scores[g].scale = scale; }
+    return rc;
 }
 
 extern "C" int32_t ckks_attention_scores(ckks_ctx *c, const ckks_attn_desc *d, const ckks_ct *q, const ckks_ct *k, uint32_t dim,
@@ -179,55 +167,58 @@ extern "C" int32_t ckks_attention_scores(ckks_ctx *c, const ckks_attn_desc *d, c
         if (!scores[g].data) return CKKS_ERR_ARG;
     if (p.Gb > 1) {
         if (!ws || ws_bytes < ckks_attention_scores_workspace_bytes(c, d, level, dim)) return CKKS_ERR_WORKSPACE;
-        return scores_split(c, p, q, k, dim, level, rlk, keys, nkeys, scores, ws, ws_bytes, stream);
+        return scores_split(c, p, q, k, dim, level, rlk, keys, nkeys, scores, ws, (cudaStream_t)stream);
     }
     // as many groups per pass as the workspace holds (one at least)
-    const size_t ctb = ct_bytes(c, level), fixed = ctb + scratch_bytes(c, level, p.G - 1);
+    const size_t ctb = ct_bytes(c, level), ctw = ctb / sizeof(u64), N = c->N, fixed = scratch_bytes(c, level, dim, p.G - 1, p.G);
     uint32_t per_pass = p.G > 1 ? (uint32_t)std::min<size_t>(p.G - 1, ws_bytes > fixed ? (ws_bytes - fixed) / ((size_t)dim * ctb) : 0) : 0;
     if (!ws || ws_bytes < fixed || (p.G > 1 && per_pass == 0)) return CKKS_ERR_WORKSPACE;
-    char *base = (char *)ws;
-    char *rk = base;                                                     // [per_pass][dim] ciphertexts
-    ckks_ct prod{(uint64_t *)(base + (size_t)per_pass * dim * ctb), level, 2, 0.0};
-    void *sw = base + (size_t)per_pass * dim * ctb + ctb;
-    const size_t sw_bytes = ws_bytes - ((size_t)per_pass * dim * ctb + ctb);
-    // group 0: the key operands as they are
-    if ((rc = ckks_mul_relin_sum(c, q, k, dim, rlk, &prod, sw, sw_bytes, stream))) return rc;
-    if ((rc = ckks_rescale(c, &prod, &scores[0], sw, sw_bytes, stream))) return rc;
-    std::vector<ckks_evk> pk(per_pass);
-    std::vector<ckks_ct> outs(per_pass), kr(dim);
-    for (uint32_t g0 = 1; g0 < p.G; g0 += per_pass) {
-        const uint32_t ng = std::min(per_pass, p.G - g0);
-        for (uint32_t x = 0; x < ng; x++) pk[x] = *find_key(c, keys, nkeys, p.tok[g0 - 1 + x]);
-        // every key operand is extended once and rotated to the pass's groups off the shared digits
-        for (uint32_t dd = 0; dd < dim; dd++) {
-            for (uint32_t x = 0; x < ng; x++) outs[x] = ckks_ct{(uint64_t *)(rk + ((size_t)x * dim + dd) * ctb), level, 2, 0.0};
-            if ((rc = ckks_rotate_hoisted(c, &k[dd], pk.data(), ng, outs.data(), sw, sw_bytes, stream))) return rc;
+    u64 *rk = (u64 *)ws;                                                 // [per_pass][dim] ciphertexts
+    void *sw = rk + (size_t)per_pass * dim * ctw;
+    cudaStream_t s = (cudaStream_t)stream;
+    std::vector<CtView> vq, vk;
+    for (uint32_t dd = 0; dd < dim; dd++) { vq.push_back(view(c, q[dd])); vk.push_back(view(c, k[dd])); }
+    DeviceGuard guard(c->device);
+    // group 0 takes the key operands as they are; every key operand is extended once per pass and rotated to the pass's groups
+    // off the shared digits
+    for (uint32_t g0 = 0; g0 < p.G;) {
+        const uint32_t first = g0 ? g0 : 1, ng = std::min(per_pass, p.G - first), last = p.G > 1 ? first + ng : 1;
+        std::vector<ckks_evk> pk;
+        for (uint32_t g = first; g < last; g++) pk.push_back(*find_key(c, keys, nkeys, p.tok[g - 1]));
+        rotate_grid(c, vk.data(), dim, pk.data(), (uint32_t)pk.size(), rk, dim * ctw, ctw, level, sw, s);
+        std::vector<std::vector<CtView>> a, b;
+        std::vector<u64 *> out;
+        for (uint32_t g = g0; g < last; g++) {
+            std::vector<CtView> kr = vk;
+            for (uint32_t dd = 0; dd < dim && g; dd++) kr[dd] = CtView{rk + ((size_t)(g - first) * dim + dd) * ctw, (size_t)level * N};
+            a.push_back(vq); b.push_back(kr); out.push_back((u64 *)scores[g].data);
         }
-        for (uint32_t x = 0; x < ng; x++) {
-            for (uint32_t dd = 0; dd < dim; dd++) kr[dd] = ckks_ct{(uint64_t *)(rk + ((size_t)x * dim + dd) * ctb), level, 2, k[dd].scale};
-            if ((rc = ckks_mul_relin_sum(c, q, kr.data(), dim, rlk, &prod, sw, sw_bytes, stream))) return rc;
-            if ((rc = ckks_rescale(c, &prod, &scores[g0 + x], sw, sw_bytes, stream))) return rc;
-        }
+        sum_rescale(c, a, b, out.data(), (uint32_t)out.size(), (const u64 *)rlk->data, level, sw, s);
+        g0 = last;
     }
-    return CKKS_OK;
+    rc = finish(c);
+    for (uint32_t g = 0; g < p.G && rc == CKKS_OK; g++) {
+        scores[g].level = level - 1; scores[g].ncomp = 2; scores[g].scale = q[0].scale * k[0].scale / (double)c->mod[level - 1];
+    }
+    return rc;
 }
 
 // ---- Softmax over rows spread across the groups ---------------------------------------------------------------------
 static bool rows_desc_ok(const ckks_softmax_desc *s) {
     return s && s->exp_coeffs && s->exp_degree >= 2 && (s->rounds == 0 || (s->rsqrt_coeffs && s->rsqrt_degree >= 2));
 }
-static size_t rows_scratch(const ckks_ctx *c, const ckks_softmax_desc *s, uint32_t level) {
-    return align256(std::max({ckks_workspace_bytes(c, CKKS_OP_POLY_EVAL_TREE, level, std::max(s->exp_degree, s->rsqrt_degree)),
-                              ckks_workspace_bytes(c, CKKS_OP_MUL_RELIN, level, 0), ckks_workspace_bytes(c, CKKS_OP_RESCALE, level, 0),
-                              ckks_workspace_bytes(c, CKKS_OP_ROTATE, level, 0)}));
+// The groups go through every step up to KS_MULTI at a time.
+static size_t rows_scratch(const ckks_ctx *c, const AttnPlan &p, const ckks_softmax_desc *s, uint32_t level) {
+    const uint32_t n = std::min(p.G, KS_MULTI);
+    return align256(std::max({poly_tree_bytes(c, level, s->exp_degree, n), s->rounds ? poly_tree_bytes(c, level, s->rsqrt_degree, 1) : 0,
+                              (size_t)n * product_bytes(c, level)}));
 }
 
-// workspace: the groups' running ciphertexts u_g, four temporaries, the scratch of the calls
+// workspace: the groups' running ciphertexts u_g and their other copy, the row sums (twice) and lambda, the scratch of the steps
 extern "C" size_t ckks_softmax_rows_workspace_bytes(const ckks_ctx *c, const ckks_attn_desc *d, const ckks_softmax_desc *s, uint32_t level) {
     AttnPlan p;
     if (!c || level < 1 || level > c->L || !rows_desc_ok(s) || make_attn_plan(c, d, p)) return 0;
-    // the groups' running ciphertexts u_g, the row sums and lambda, then per lane two temporaries and the scratch of the calls
-    return (size_t)(p.G + 2) * ct_bytes(c, level) + lane_count(c) * (2 * ct_bytes(c, level) + rows_scratch(c, s, level));
+    return (size_t)(2 * p.G + 3) * ct_bytes(c, level) + rows_scratch(c, p, s, level);
 }
 
 extern "C" int32_t ckks_softmax_rows(ckks_ctx *c, const ckks_attn_desc *d, const ckks_softmax_desc *s, const ckks_ct *in, const ckks_evk *rlk,
@@ -246,86 +237,88 @@ extern "C" int32_t ckks_softmax_rows(ckks_ctx *c, const ckks_attn_desc *d, const
     for (uint32_t g = 0; g < p.G; g++)
         if (!out[g].data) return CKKS_ERR_ARG;
     if (!ws || ws_bytes < ckks_softmax_rows_workspace_bytes(c, d, s, level)) return CKKS_ERR_WORKSPACE;
-    const size_t ctb = ct_bytes(c, level), N = c->N;
-    char *base = (char *)ws;
-    std::vector<ckks_ct> u(p.G);
-    for (uint32_t g = 0; g < p.G; g++) u[g] = ckks_ct{(uint64_t *)(base + (size_t)g * ctb), level, 2, 0.0};
-    ckks_ct B{(uint64_t *)(base + (size_t)p.G * ctb), level, 2, 0.0}, T{(uint64_t *)(base + (size_t)(p.G + 1) * ctb), level, 2, 0.0};
-    const Lanes lanes(c, stream);
-    const size_t sw_bytes = rows_scratch(c, s, level), lane_bytes = 2 * ctb + sw_bytes;
-    char *lane0 = base + (size_t)(p.G + 2) * ctb;
-    // lane l: temporaries A and X, then the scratch
-    auto lane_A = [&](uint32_t l) { return ckks_ct{(uint64_t *)(lane0 + l * lane_bytes), level, 2, 0.0}; };
-    auto lane_X = [&](uint32_t l) { return ckks_ct{(uint64_t *)(lane0 + l * lane_bytes + ctb), level, 2, 0.0}; };
-    auto lane_sw = [&](uint32_t l) { return (void *)(lane0 + l * lane_bytes + 2 * ctb); };
-    cudaStream_t st = (cudaStream_t)stream;
-    // the groups' exponentials are independent: spread over the lanes
-    lanes.fork();
-    for (uint32_t g = 0; g < p.G && !rc; g++) {
-        const uint32_t l = g % lanes.n;
-        ckks_ct A = lane_A(l);
-        if ((rc = ckks_add_const(c, &in[g], -s->shift, &A, lanes.at(g)))) break;
-        rc = ckks_poly_eval_tree(c, &A, s->exp_coeffs, s->exp_degree, rlk, &u[g], lane_sw(l), sw_bytes, lanes.at(g));
-    }
-    lanes.join();
-    if (rc) return rc;
+    // every plan (levels, scales, constants) before anything is launched
+    long long shift;
+    TreePlan pe;
+    if (!const_value(-s->shift, in[0].scale, &shift)) return CKKS_ERR_RANGE;
+    if ((rc = poly_tree_plan(c, level, in[0].scale, s->exp_coeffs, s->exp_degree, pe))) return rc;
+    struct Round { TreePlan poly; uint32_t lu, lt, lx; };                 // levels of u, of its row sums and of lambda u
+    std::vector<Round> rounds(s->rounds);
+    uint32_t lu = pe.Lt - 1;
+    double su = pe.out_scale;
     for (uint32_t j = 0; j < s->rounds; j++) {
-        ckks_ct A = lane_A(0);
-        void *sw = lane_sw(0);
-        // t = row sums of u^2: one relinearisation for the sum over the groups, then the ladder over the blocks
-        if ((rc = ckks_mul_relin_sum(c, u.data(), u.data(), p.G, rlk, &A, sw, sw_bytes, stream))) return rc;
-        if ((rc = ckks_rescale(c, &A, &T, sw, sw_bytes, stream))) return rc;
-        if ((rc = block_ladder(c, p, keys, nkeys, &T, &A, sw, sw_bytes, stream))) return rc;
-        // lambda = p_rsqrt_j(t), once for all groups
-        if ((rc = ckks_poly_eval_tree(c, &T, s->rsqrt_coeffs + (size_t)j * (s->rsqrt_degree + 1), s->rsqrt_degree, rlk, &B, sw, sw_bytes, stream)))
-            return rc;
-        // u_g = rescale(rescale(lambda u_g)^2): independent over the groups
-        lanes.fork();
-        for (uint32_t g = 0; g < p.G && !rc; g++) {
-            const uint32_t l = g % lanes.n;
-            ckks_ct Al = lane_A(l), X = lane_X(l);
-            void *ls = lanes.at(g), *lw = lane_sw(l);
-            // u_g truncated to lambda's level
-            int prev = 0;
-            cudaGetDevice(&prev);
-            cudaSetDevice(c->device);
-            for (uint32_t comp = 0; comp < 2; comp++)
-                cudaMemcpyAsync(X.data + (size_t)comp * B.level * N, u[g].data + (size_t)comp * u[g].level * N, (size_t)B.level * N * sizeof(uint64_t),
-                                cudaMemcpyDeviceToDevice, (cudaStream_t)ls);
-            cudaSetDevice(prev);
-            X.level = B.level; X.ncomp = 2; X.scale = u[g].scale;
-            if ((rc = ckks_mul_relin(c, &B, &X, rlk, &Al, lw, sw_bytes, ls))) break;
-            if ((rc = ckks_rescale(c, &Al, &X, lw, sw_bytes, ls))) break;
-            if ((rc = ckks_mul_relin(c, &X, &X, rlk, &Al, lw, sw_bytes, ls))) break;
-            rc = ckks_rescale(c, &Al, &u[g], lw, sw_bytes, ls);
-        }
-        lanes.join();
-        if (rc) return rc;
+        Round &r = rounds[j];
+        r.lu = lu; r.lt = lu - 1;
+        const double st = su * su / (double)c->mod[lu - 1];
+        if ((rc = poly_tree_plan(c, r.lt, st, s->rsqrt_coeffs + (size_t)j * (s->rsqrt_degree + 1), s->rsqrt_degree, r.poly))) return rc;
+        r.lx = r.poly.Lt - 2;
+        const double sx = r.poly.out_scale * su / (double)c->mod[r.poly.Lt - 2];
+        su = sx * sx / (double)c->mod[r.lx - 1];
+        lu = r.lx - 1;
     }
-    int prev = 0;
-    cudaGetDevice(&prev);
-    cudaSetDevice(c->device);
-    for (uint32_t g = 0; g < p.G; g++)
-        cudaMemcpyAsync(out[g].data, u[g].data, (size_t)2 * u[g].level * N * sizeof(uint64_t), cudaMemcpyDeviceToDevice, st);
-    cudaError_t e = cudaGetLastError();
-    cudaSetDevice(prev);
-    if (e != cudaSuccess) { c->cuda_error = cudaGetErrorString(e); return CKKS_ERR_CUDA; }
-    for (uint32_t g = 0; g < p.G; g++) { out[g].level = u[g].level; out[g].ncomp = 2; out[g].scale = u[g].scale; }
-    return CKKS_OK;
+    const size_t ctw = ct_bytes(c, level) / sizeof(u64), N = c->N;
+    u64 *U = (u64 *)ws, *X = U + p.G * ctw, *T = X + p.G * ctw, *T2 = T + ctw, *B = T2 + ctw;
+    void *sw = B + ctw;
+    const u64 *rd = (const u64 *)rlk->data;
+    cudaStream_t st = (cudaStream_t)stream;
+    DeviceGuard guard(c->device);
+    auto run = [&](uint32_t g0) { return std::min(KS_MULTI, p.G - g0); };
+    auto outs = [&](uint32_t g0, uint32_t n, bool final) {               // where step results of groups g0.. go
+        Ptrs o;
+        o.n = n;
+        for (uint32_t g = 0; g < n; g++) o.p[g] = final ? (const u64 *)out[g0 + g].data : U + (size_t)(g0 + g) * ctw;
+        return o;
+    };
+    // u = p_exp(x - shift)
+    for (uint32_t g0 = 0; g0 < p.G; g0 += KS_MULTI) {
+        Ptrs pi;
+        pi.n = run(g0);
+        for (uint32_t g = 0; g < pi.n; g++) pi.p[g] = (const u64 *)in[g0 + g].data;
+        const Ptrs z(X + g0 * ctw, ctw);
+        launch_const(c, pi, shift, false, z, 2, level, st, pi.n);
+        poly_tree_run(c, pe, z, outs(g0, pi.n, s->rounds == 0), pi.n, rd, sw, st);
+    }
+    for (uint32_t j = 0; j < s->rounds; j++) {
+        const Round &r = rounds[j];
+        // t = row sums of u^2: one relinearisation for the sum over the groups, then the ladder over the blocks, back and forth
+        std::vector<CtView> u;
+        for (uint32_t g = 0; g < p.G; g++) u.push_back(CtView{U + g * ctw, (size_t)r.lu * N});
+        sum_rescale(c, {u}, {u}, &T, 1, rd, r.lu, sw, st);
+        for (int64_t rot : p.lad) {
+            KsWorkspace w = ks_carve(c, r.lt, sw);
+            const Ptrs from(T, 0);
+            rotate_ks(c, find_key(c, keys, nkeys, rot), from, Ptrs(T2, 0), r.lt, w, st, 1, &from);
+            std::swap(T, T2);
+        }
+        // lambda = p_rsqrt_j(t), once for all groups; u_g = rescale(rescale(lambda u_g)^2)
+        poly_tree_run(c, r.poly, Ptrs(T, 0), Ptrs(B, 0), 1, rd, sw, st);
+        const uint32_t lb = r.poly.Lt - 1;
+        std::vector<CtView> lam(p.G, CtView{B, (size_t)lb * N}), x;
+        std::vector<u64 *> xo, uo;
+        for (uint32_t g = 0; g < p.G; g++) {
+            xo.push_back(X + g * ctw);
+            x.push_back(CtView{X + g * ctw, (size_t)r.lx * N});
+            uo.push_back(j + 1 == s->rounds ? (u64 *)out[g].data : U + g * ctw);
+        }
+        mul_rescale(c, lam.data(), u.data(), xo.data(), p.G, rd, lb, sw, KS_MULTI, st);
+        mul_rescale(c, x.data(), x.data(), uo.data(), p.G, rd, r.lx, sw, KS_MULTI, st);
+    }
+    rc = finish(c);
+    for (uint32_t g = 0; g < p.G && rc == CKKS_OK; g++) { out[g].level = lu; out[g].ncomp = 2; out[g].scale = su; }
+    return rc;
 }
 
 // ---- probability x value ------------------------------------------------------------------------------------------
-// The ladder over the blocks runs for VAL_CHUNK output channels at a time (ckks_rotate_batch: their key switches side by side).
+// VAL_CHUNK output channels at a time: their rotations, sums and the ladder over the blocks side by side.
 constexpr uint32_t VAL_CHUNK = 16;
 static size_t values_scratch(const ckks_ctx *c, uint32_t level, uint32_t nrot) {
-    return std::max(scratch_bytes(c, level, nrot), align256(ckks_workspace_bytes(c, CKKS_OP_ROTATE_BATCH, level - 1, VAL_CHUNK)));
+    return std::max(scratch_bytes(c, level, VAL_CHUNK, nrot, VAL_CHUNK), align256(VAL_CHUNK * ks_workspace_limbs(c, level - 1) * c->N * sizeof(u64)));
 }
-// workspace: the truncated value operand and its rotated copies, a product, the rotated outputs of a chunk, the scratch of the calls
+// workspace: a chunk's rotated value operands, its outputs' other copy for the ladder, the scratch of the steps
 extern "C" size_t ckks_attention_values_workspace_bytes(const ckks_ctx *c, const ckks_attn_desc *d, uint32_t level) {
     AttnPlan p;
     if (!c || level < 2 || level > c->L || make_attn_plan(c, d, p)) return 0;
-    // per lane: the truncated value operand with its rotated copies, a product, the scratch of the calls; then a ladder chunk
-    return lane_count(c) * ((size_t)(p.G + 1) * ct_bytes(c, level) + values_scratch(c, level, p.G - 1)) + (size_t)VAL_CHUNK * ct_bytes(c, level - 1);
+    return VAL_CHUNK * ((size_t)(p.G - 1) * ct_bytes(c, level) + ct_bytes(c, level - 1)) + values_scratch(c, level, p.G - 1);
 }
 
 extern "C" int32_t ckks_attention_values(ckks_ctx *c, const ckks_attn_desc *d, const ckks_ct *probs, const ckks_ct *v, uint32_t dim_v,
@@ -346,49 +339,46 @@ extern "C" int32_t ckks_attention_values(ckks_ctx *c, const ckks_attn_desc *d, c
     for (uint32_t dd = 0; dd < dim_v; dd++)
         if (!out[dd].data) return CKKS_ERR_ARG;
     if (!ws || ws_bytes < ckks_attention_values_workspace_bytes(c, d, lp)) return CKKS_ERR_WORKSPACE;
-    const size_t ctb = ct_bytes(c, lp), ctb1 = ct_bytes(c, lp - 1), N = c->N;
-    char *base = (char *)ws;
-    const Lanes lanes(c, stream);
-    const size_t sw_bytes = values_scratch(c, lp, p.G - 1), lane_bytes = (size_t)(p.G + 1) * ctb + sw_bytes;
-    char *rot = base + lanes.n * lane_bytes;                           // [VAL_CHUNK] rotated outputs of the ladder
+    const size_t ctw = ct_bytes(c, lp) / sizeof(u64), ctw1 = ct_bytes(c, lp - 1) / sizeof(u64), N = c->N;
+    u64 *vr = (u64 *)ws, *tmp = vr + VAL_CHUNK * (p.G - 1) * ctw;         // [G - 1][VAL_CHUNK] at lp, [VAL_CHUNK] at lp - 1
+    void *sw = tmp + VAL_CHUNK * ctw1;
+    cudaStream_t s = (cudaStream_t)stream;
     std::vector<ckks_evk> pk;
     for (int64_t r : p.tok) pk.push_back(*find_key(c, keys, nkeys, r));
-    // the channels are independent up to the ladder: spread over the lanes, each with its own buffers
-    lanes.fork();
-    std::vector<ckks_ct> vr(p.G);
-    for (uint32_t dd = 0; dd < dim_v; dd++) {
-        char *lb = base + (dd % lanes.n) * lane_bytes;
-        void *ls = lanes.at(dd);
-        for (uint32_t g = 0; g < p.G; g++) vr[g] = ckks_ct{(uint64_t *)(lb + (size_t)g * ctb), lp, 2, v[dd].scale};
-        ckks_ct prod{(uint64_t *)(lb + (size_t)p.G * ctb), lp, 2, 0.0};
-        void *sw = lb + (size_t)(p.G + 1) * ctb;
-        int prev = 0;
-        cudaGetDevice(&prev);
-        cudaSetDevice(c->device);
-        for (uint32_t comp = 0; comp < 2; comp++)
-            cudaMemcpyAsync(vr[0].data + (size_t)comp * lp * N, v[dd].data + (size_t)comp * lv * N, (size_t)lp * N * sizeof(uint64_t),
-                            cudaMemcpyDeviceToDevice, (cudaStream_t)ls);
-        cudaSetDevice(prev);
-        if (p.G > 1 && (rc = ckks_rotate_hoisted(c, &vr[0], pk.data(), p.G - 1, vr.data() + 1, sw, sw_bytes, ls))) break;
-        for (uint32_t g = 0; g < p.G; g++) vr[g].scale = v[dd].scale;
-        if ((rc = ckks_mul_relin_sum(c, probs, vr.data(), p.G, rlk, &prod, sw, sw_bytes, ls))) break;
-        if ((rc = ckks_rescale(c, &prod, &out[dd], sw, sw_bytes, ls))) break;
-    }
-    lanes.join();
-    if (rc) return rc;
-    // the ladder over the blocks, a rotation of a whole chunk of channels at a time: out += rotate(out, r), r ascending
-    void *sw = base;                                                   // lane 0's buffers are free again
-    std::vector<ckks_ct> tmp(VAL_CHUNK);
+    std::vector<CtView> vp, vv;
+    for (uint32_t g = 0; g < p.G; g++) vp.push_back(view(c, probs[g]));
+    for (uint32_t dd = 0; dd < dim_v; dd++) vv.push_back(view(c, v[dd]));         // read at level lp in place
+    DeviceGuard guard(c->device);
     for (uint32_t d0 = 0; d0 < dim_v; d0 += VAL_CHUNK) {
         const uint32_t nd = std::min(VAL_CHUNK, dim_v - d0);
+        rotate_grid(c, vv.data() + d0, nd, pk.data(), p.G - 1, vr, VAL_CHUNK * ctw, ctw, lp, sw, s);
+        Ptrs po;
+        po.n = nd;
+        for (uint32_t x = 0; x < nd; x++) po.p[x] = (const u64 *)out[d0 + x].data;
+        const Ptrs pt(tmp, ctw1);
+        // the ladder doubles back and forth between the outputs and their copy and has to end in the outputs
+        bool in_out = p.lad.size() % 2 == 0;
+        std::vector<std::vector<CtView>> a(nd, vp), b(nd);
+        std::vector<u64 *> so;
+        for (uint32_t x = 0; x < nd; x++) {
+            b[x].push_back(vv[d0 + x]);
+            for (uint32_t g = 1; g < p.G; g++) b[x].push_back(CtView{vr + ((size_t)(g - 1) * VAL_CHUNK + x) * ctw, (size_t)lp * N});
+            so.push_back(const_cast<u64 *>(in_out ? po.p[x] : tmp + x * ctw1));
+        }
+        sum_rescale(c, a, b, so.data(), nd, (const u64 *)rlk->data, lp, sw, s);
+        // out += rotate(out, r), r ascending
         for (int64_t r : p.lad) {
-            for (uint32_t x = 0; x < nd; x++) tmp[x] = ckks_ct{(uint64_t *)(rot + (size_t)x * ctb1), lp - 1, 2, 0.0};
-            if ((rc = ckks_rotate_batch(c, &out[d0], nd, find_key(c, keys, nkeys, r), tmp.data(), sw, lane_bytes, stream))) return rc;
-            for (uint32_t x = 0; x < nd; x++)
-                if ((rc = ckks_add(c, &out[d0 + x], &tmp[x], &out[d0 + x], stream))) return rc;
+            KsWorkspace w = ks_carve(c, lp - 1, sw, nd);
+            const Ptrs &from = in_out ? po : pt, &to = in_out ? pt : po;
+            rotate_ks(c, find_key(c, keys, nkeys, r), from, to, lp - 1, w, s, nd, &from);
+            in_out = !in_out;
         }
     }
-    return CKKS_OK;
+    rc = finish(c);
+    for (uint32_t dd = 0; dd < dim_v && rc == CKKS_OK; dd++) {
+        out[dd].level = lp - 1; out[dd].ncomp = 2; out[dd].scale = probs[0].scale * v[0].scale / (double)c->mod[lp - 1];
+    }
+    return rc;
 }
 
 // ---- the three steps in a row -------------------------------------------------------------------------------------

@@ -1,0 +1,114 @@
+// Sequences of launches that several entry points share, all over many ciphertexts side by side: one ciphertext's launches
+// are one or two waves of CTAs each, sixteen ciphertexts' fill the GPU, and a switching key is read once for all of them.
+#include "common.cuh"
+
+// o[i] (2 x level limbs) += key switch of e2[i], nb side by side
+void relinearise(const ckks_ctx *c, const u64 *rlk, const Ptrs &e2, const Ptrs &o, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb) {
+    ks_modup(c, e2, level, w, s, nb);
+    ks_inner(c, rlk, level, 1, w, s, nb);
+    KsOut ko;
+    ko.add = ko.out = o;
+    ko.add_comps = 3;
+    ks_moddown(c, level, w, ko, s, nb);
+}
+// One product's share of a batch: the tensor product's two parts and a key-switch workspace (whose bytes the rescale reuses)
+size_t product_bytes(const ckks_ctx *c, uint32_t level) { return ((size_t)3 * level + ks_workspace_limbs(c, level)) * c->N * sizeof(u64); }
+
+// out[i] = rescale(relin(a[i] b[i])), up to `chunk` products side by side; ws: min(n, chunk) * product_bytes
+void mul_rescale(const ckks_ctx *c, const CtView *a, const CtView *b, u64 *const *out, uint32_t n, const u64 *rlk, uint32_t level, void *ws, uint32_t chunk,
+                 cudaStream_t s) {
+    const size_t N = c->N, ctl = (size_t)2 * level * N, ptl = (size_t)level * N;
+    for (uint32_t i0 = 0; i0 < n; i0 += chunk) {
+        const uint32_t m = std::min(chunk, n - i0);
+        u64 *e01 = (u64 *)ws, *e2 = e01 + m * ctl, *ksw = e2 + m * ptl;
+        TensorArgs ta;
+        Ptrs po;
+        po.n = m;
+        for (uint32_t i = 0; i < m; i++) {
+            ta.a[i] = a[i0 + i]; ta.b[i] = b[i0 + i];
+            ta.e01[i] = e01 + i * ctl; ta.e2[i] = e2 + i * ptl;
+            po.p[i] = out[i0 + i];
+        }
+        launch_tensor(c, ta, m, level, s);
+        KsWorkspace w = ks_carve(c, level, ksw, m);
+        relinearise(c, rlk, Ptrs(e2, ptl), Ptrs(e01, ctl), level, w, s, m);
+        launch_rescale(c, Ptrs(e01, ctl), po, 2, level, ksw, s, m);
+    }
+}
+
+// out = rotation of nb ciphertexts by one key (+ acc, both components, where acc is given; acc may be out, out must not be in)
+void rotate_ks(const ckks_ctx *c, const ckks_evk *key, const Ptrs &in, const Ptrs &out, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb,
+               const Ptrs *acc) {
+    Ptrs c1 = in;
+    const size_t ptl = (size_t)level * c->N;
+    if (in.n) for (uint32_t b = 0; b < in.n; b++) c1.p[b] += ptl;
+    else c1.base += ptl;
+    ks_modup(c, c1, level, w, s, nb);
+    ks_inner(c, (const u64 *)key->data, level, key->galois, w, s, nb);
+    KsOut ko;
+    ko.add = in; ko.out = out;
+    ko.add_comps = 1; ko.galois = key->galois;
+    if (acc) ko.acc = *acc;
+    ks_moddown(c, level, w, ko, s, nb);
+}
+
+// out[i] = rescale(relin(sum_t a[i][t] b[i][t])) for n sums of nterm products; ws: min(n, KS_MULTI) * product_bytes
+void sum_rescale(const ckks_ctx *c, const std::vector<std::vector<CtView>> &a, const std::vector<std::vector<CtView>> &b, u64 *const *out, uint32_t n,
+                 const u64 *rlk, uint32_t level, void *ws, cudaStream_t s) {
+    const size_t N = c->N, ctl = (size_t)2 * level * N, ptl = (size_t)level * N;
+    for (uint32_t i0 = 0; i0 < n; i0 += KS_MULTI) {
+        const uint32_t m = std::min(KS_MULTI, n - i0);
+        u64 *e01 = (u64 *)ws, *e2 = e01 + m * ctl, *ksw = e2 + m * ptl;
+        Ptrs po;
+        po.n = m;
+        for (uint32_t i = 0; i < m; i++) {
+            launch_tensor_sum(c, a[i0 + i].data(), b[i0 + i].data(), (uint32_t)a[i0 + i].size(), e01 + i * ctl, e2 + i * ptl, level, s);
+            po.p[i] = out[i0 + i];
+        }
+        KsWorkspace w = ks_carve(c, level, ksw, m);
+        relinearise(c, rlk, Ptrs(e2, ptl), Ptrs(e01, ctl), level, w, s, m);
+        launch_rescale(c, Ptrs(e01, ctl), po, 2, level, ksw, s, m);
+    }
+}
+
+// ---- many ciphertexts times many rotations -------------------------------------------------------------------------
+// Up to GRID_CTS ciphertexts share a pass: each is extended once, every key is applied to all of them (and read once for
+// them), GRID_ENTRIES key switches side by side.
+constexpr uint32_t GRID_CTS = 8, GRID_ENTRIES = 32;
+static uint32_t grid_keys(uint32_t members, uint32_t nrot) { return std::min(nrot, std::min(KS_MULTI, std::max(1u, GRID_ENTRIES / members))); }
+size_t rotate_grid_bytes(const ckks_ctx *c, uint32_t level, uint32_t n, uint32_t nrot) {
+    const size_t beta = (level + c->alpha - 1) / c->alpha, nt = level + c->K;
+    const uint32_t m = std::min(n, GRID_CTS);
+    return (m * (level + beta * nt) + (size_t)m * grid_keys(m, nrot) * (2 * nt + 2 * level)) * c->N * sizeof(u64);
+}
+// rotation r of ciphertext i (components comp words apart, taken at `level`) -> out + r * rot_stride + i * ct_stride
+void rotate_grid(const ckks_ctx *c, const CtView *in, uint32_t n, const ckks_evk *keys, uint32_t nrot, u64 *out, size_t rot_stride, size_t ct_stride,
+                 uint32_t level, void *ws, cudaStream_t s) {
+    if (!n || !nrot) return;
+    const size_t beta = (level + c->alpha - 1) / c->alpha, nt = level + c->K, N = c->N;
+    const uint32_t mmax = std::min(n, GRID_CTS), kmax = grid_keys(mmax, nrot);
+    KsWorkspace w;
+    w.dcoef = (u64 *)ws;
+    w.ext = w.dcoef + (size_t)mmax * level * N;
+    w.u = w.ext + mmax * beta * nt * N;
+    w.conv = w.u + (size_t)mmax * kmax * 2 * nt * N;
+    for (uint32_t i0 = 0; i0 < n; i0 += mmax) {
+        const uint32_t m = std::min(mmax, n - i0);
+        KsOut ko;
+        ko.add.n = m; ko.add_comps = 1;
+        ko.out = Ptrs(out + i0 * ct_stride, ct_stride);
+        Ptrs c1;
+        c1.n = m;
+        for (uint32_t i = 0; i < m; i++) { ko.add.p[i] = in[i0 + i].p; c1.p[i] = in[i0 + i].p + in[i0 + i].comp; }
+        ks_modup(c, c1, level, w, s, m);
+        for (uint32_t r0 = 0; r0 < nrot; r0 += kmax) {
+            const uint32_t nr = std::min(kmax, nrot - r0);
+            KsMulti k{};
+            k.group = m; k.rot_stride = rot_stride;
+            for (uint32_t r = 0; r < nr; r++) { k.galois[r] = keys[r0 + r].galois; k.evk[r] = (const u64 *)keys[r0 + r].data; }
+            ko.out.base = out + r0 * rot_stride + i0 * ct_stride;
+            ks_inner(c, nullptr, level, 1, w, s, nr * m, false, &k);
+            ks_moddown(c, level, w, ko, s, nr * m, &k);
+        }
+    }
+}

@@ -75,9 +75,9 @@ struct ckks_ctx {
     int conv_kernel = 0;                     // basis conversions: 0 = FP64 pipe, 1 = tensor cores (conv_mma.cu)
     int mac_kernel = 82;                     // projection multiply-accumulate kernel (see launch_mac_mma)
     long long wait_cycles = 2000000000ll;    // clock bound of every device-side wait (about a second)
-    // Streams of the context.  Composite calls whose work is many independent single-ciphertext chains (the attention
-    // entry points) spread those chains over `lanes` streams, lane 0 being the caller's: a single ciphertext's kernels fill
-    // the GPU for at most one wave, so independent chains overlap.  Forked from and joined to the caller's stream by events.
+    // Streams of the context.  ckks_attention_pack, whose work is many independent single-ciphertext chains, spreads them over
+    // `lanes` streams, lane 0 being the caller's: a single ciphertext's kernels fill the GPU for at most one wave, so
+    // independent chains overlap.  Forked from and joined to the caller's stream by events.
     int lanes = 4;
     cudaStream_t lane_stream[3] = {nullptr, nullptr, nullptr};
     cudaEvent_t lane_event[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -307,21 +307,41 @@ struct Ptrs {
     __host__ __device__ const u64 *at(uint32_t b) const { return n ? p[b] : base + b * stride; }
 };
 
+// Two adjacent words with one 16-byte access (WIDE) or two 8-byte ones: kernels come in both forms, chosen by aligned16 on the
+// host, because callers' buffers need only be 8-byte aligned.
+template <bool WIDE>
+__device__ __forceinline__ ulonglong2 ld_pair(const u64 *p) {
+    return WIDE ? *reinterpret_cast<const ulonglong2 *>(p) : make_ulonglong2(p[0], p[1]);
+}
+template <bool WIDE>
+__device__ __forceinline__ void st_pair(u64 *p, ulonglong2 v) {
+    if (WIDE) *reinterpret_cast<ulonglong2 *>(p) = v;
+    else { p[0] = v.x; p[1] = v.y; }
+}
+inline bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
+inline bool aligned16(const Ptrs &p) {
+    if (!p.n) return aligned16(p.base) && (p.stride & 1) == 0;
+    for (uint32_t i = 0; i < p.n; i++)
+        if (!aligned16(p.p[i])) return false;
+    return true;
+}
+
 // Epilogue of the forward transform, for a buffer of limbs laid out [b][ncomp][level].
 //   mode 1: instead of storing NTT(conv) the last pass finishes a ModDown or a rescale:
-//           out[b][comp][i][p] (+)= (u[b][comp][i][p] - NTT(conv)[p]) pinv[i] + sigma_g(add[b][comp][i])[p]
+//           out[b][comp][i][p] = (u[b][comp][i][p] - NTT(conv)[p]) pinv[i] + sigma_g(add[b][comp][i])[p] + acc[b][comp][i][p]
 //           u: [ncomp][nt][N] words per entry; add: [..][level][N] words, taken for the components in the mask add_comps;
+//           acc (if given): [ncomp][level][N] words per entry;
 //           out: plain ([ncomp][level][N] per entry) or tiled (tl.R != 0, component comp of entry b in row
 //           tl.row0 + b * tl.row_stride + comp)
 //   mode 2: the transform's own result is stored, but into a tiled buffer (out.base): limb y = b * level + i becomes row
 //           tl.row0 + b * tl.row_stride, limb i
 struct NttEpilogue {
     int mode;
-    Ptrs u, add, out;
+    Ptrs u, add, out, acc;
     const double2 *pinv;   // [level] {constant, constant / q_i}
     uint32_t add_comps, ncomp, level, nt;
     u64 galois;
-    int accumulate;
+    int accumulate;        // acc is given
     TiledOut tl;
     int multi;             // batch entry b adds through mgalois[b]
     u64 mgalois[KS_MULTI];
@@ -353,16 +373,30 @@ void launch_ntt_int(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, 
 void launch_mul_plain_acc(const ckks_ctx *c, const u64 *const *cts, u64 *const *accs, uint32_t ncts, const u64 *pt,
                           uint32_t level, bool init, cudaStream_t s);
 void launch_add(const ckks_ctx *c, const u64 *a, const u64 *b, u64 *out, uint32_t ncomp, uint32_t level, cudaStream_t s);
-void launch_tensor(const ckks_ctx *c, const u64 *a, const u64 *b, u64 *e01, u64 *e2, uint32_t level, cudaStream_t s);
+// A two-component ciphertext at some level inside a buffer of a higher one: component 1 lies comp words behind component 0
+struct CtView { const u64 *p; size_t comp; };
+inline bool aligned16(const CtView &v) { return aligned16(v.p) && (v.comp & 1) == 0; }
+// e01[z], e2[z] = tensor(a[z], b[z]) for z < n
+struct TensorArgs { CtView a[KS_MULTI], b[KS_MULTI]; u64 *e01[KS_MULTI], *e2[KS_MULTI]; };
+void launch_tensor(const ckks_ctx *c, const TensorArgs &args, uint32_t n, uint32_t level, cudaStream_t s);
 // slot values 1.0 on the slots x with lo <= x / B < hi and t0 <= x % Ti < t1, else 0.0 (n doubles on the device)
 void launch_slot_mask(const ckks_ctx *c, double *out, uint32_t B, uint32_t lo, uint32_t hi, uint32_t Ti, uint32_t t0, uint32_t t1, cudaStream_t s);
 // out = in * v or in + v (component 0 only) for the constant polynomial v
-void launch_const(const ckks_ctx *c, const u64 *in, long long v, bool mul, u64 *out, uint32_t ncomp, uint32_t level, cudaStream_t s);
-// e01, e2 = sum_i tensor(a_i, b_i) (host arrays of n device pointers, [2][level][N] each)
+void launch_const(const ckks_ctx *c, const Ptrs &in, long long v, bool mul, const Ptrs &out, uint32_t ncomp, uint32_t level, cudaStream_t s, uint32_t n = 1);
+// e01, e2 (+)= sum_i tensor(a_i, b_i) (host arrays of n views)
 constexpr uint32_t TS_MAX = 16;
-struct TensorSumArgs { const u64 *a[TS_MAX]; const u64 *b[TS_MAX]; };
-void launch_tensor_sum(const ckks_ctx *c, const u64 *const *a, const u64 *const *b, uint32_t n, u64 *e01, u64 *e2, uint32_t level,
-                       cudaStream_t s);
+struct TensorSumArgs { CtView a[TS_MAX], b[TS_MAX]; };
+void launch_tensor_sum(const ckks_ctx *c, const CtView *a, const CtView *b, uint32_t n, u64 *e01, u64 *e2, uint32_t level, cudaStream_t s, bool init = true);
+// out[o] (+)= sum_{j < nx} v[o][j] x[j] + cst[o] q_{level-1} (first component), o < no, for n ciphertexts each (see lincomb_kernel)
+constexpr uint32_t LIN_MAX = 8;
+struct LinArgs {
+    Ptrs x[LIN_MAX], out[LIN_MAX];        // inputs: component 1 lies xc words behind component 0; outputs: [2][level][N]
+    size_t xc[LIN_MAX];
+    long long v[LIN_MAX][LIN_MAX], cst[LIN_MAX];
+    uint32_t nx, no;
+    int accumulate;
+};
+void launch_lincomb(const ckks_ctx *c, const LinArgs &args, uint32_t n, uint32_t level, cudaStream_t s);
 
 // Key switch pieces.  Sizes in limbs: d [level], ext [beta][level+K], u [2][level+K], conv [2][level].
 // d: the evaluation-domain input of the last ks_modup.  A digit's own limbs are not copied into ext; the inner product reads
@@ -382,12 +416,12 @@ void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, 
 // (w.u, nb entries); with acc_u it adds to what w.u holds, so that a sum of key-switched terms can share one ks_moddown.
 void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w, cudaStream_t s, uint32_t nb = 1,
               bool acc_u = false, const KsMulti *multi = nullptr);
-// ModDown and the final combination out_c (+)= sigma_galois(add_c) + k_c (add taken for the components in add_comps)
+// ModDown and the final combination out_c = sigma_galois(add_c) + k_c + acc_c (add taken for the components in add_comps, acc if
+// given: [2][level][N] words per entry, possibly out itself)
 struct KsOut {
-    Ptrs add, out;
+    Ptrs add, out, acc;
     uint32_t add_comps = 0;
     u64 galois = 1;
-    bool accumulate = false;
     TiledOut tiled;
 };
 void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb = 1, const KsMulti *multi = nullptr);
@@ -444,3 +478,42 @@ void launch_encode(const ckks_ctx *c, const double *re, const double *im, uint32
 void launch_extract_diagonals(const ckks_ctx *c, const double *W, uint32_t d_out_total, uint32_t in0, uint32_t m_in,
                               uint32_t out0, uint32_t m_out, uint32_t F, uint32_t T, uint32_t k0, uint32_t count,
                               uint32_t pre_rot, double *slots, cudaStream_t s);
+
+// ---- sequences shared by the entry points (api.cu, poly.cu, attention.cu) -------------------------------------------
+void relinearise(const ckks_ctx *c, const u64 *rlk, const Ptrs &e2, const Ptrs &o, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb = 1);
+void rotate_ks(const ckks_ctx *c, const ckks_evk *key, const Ptrs &in, const Ptrs &out, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb = 1,
+               const Ptrs *acc = nullptr);
+size_t product_bytes(const ckks_ctx *c, uint32_t level);
+void mul_rescale(const ckks_ctx *c, const CtView *a, const CtView *b, u64 *const *out, uint32_t n, const u64 *rlk, uint32_t level, void *ws, uint32_t chunk,
+                 cudaStream_t s);
+void sum_rescale(const ckks_ctx *c, const std::vector<std::vector<CtView>> &a, const std::vector<std::vector<CtView>> &b, u64 *const *out, uint32_t n,
+                 const u64 *rlk, uint32_t level, void *ws, cudaStream_t s);
+size_t rotate_grid_bytes(const ckks_ctx *c, uint32_t level, uint32_t n, uint32_t nrot);
+void rotate_grid(const ckks_ctx *c, const CtView *in, uint32_t n, const ckks_evk *keys, uint32_t nrot, u64 *out, size_t rot_stride, size_t ct_stride,
+                 uint32_t level, void *ws, cudaStream_t s);
+// The polynomial of ckks_poly_eval_tree for n ciphertexts side by side (at most KS_MULTI; all at one level and scale).  plan
+// first: it fixes levels, scales and constants and reports their errors before anything is launched.
+struct TreePlan {
+    uint32_t degree, level, Lt;
+    double out_scale;
+    std::vector<uint32_t> lvl;          // of x^k
+    std::vector<long long> v;           // constants of x^k, v[0] for the constant term
+};
+int poly_tree_plan(const ckks_ctx *c, uint32_t level, double scale, const double *coeffs, uint32_t degree, TreePlan &p);
+size_t poly_tree_bytes(const ckks_ctx *c, uint32_t level, uint32_t degree, uint32_t n);
+void poly_tree_run(const ckks_ctx *c, const TreePlan &p, const Ptrs &x, const Ptrs &out, uint32_t n, const u64 *rlk, void *ws, cudaStream_t s);
+bool const_value(double c, double scale, long long *v);
+inline bool poly_bsgs_shape_ok(uint32_t degree, uint32_t m) { return m >= 2 && !(m & (m - 1)) && m <= degree; }
+struct DeviceGuard {
+    int prev = 0;
+    explicit DeviceGuard(int dev) { cudaGetDevice(&prev); if (prev != dev) cudaSetDevice(dev); else prev = -1; }
+    ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
+};
+inline int finish(ckks_ctx *c) {
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) { c->cuda_error = cudaGetErrorString(e); return CKKS_ERR_CUDA; }
+    return CKKS_OK;
+}
+inline bool ct_ok(const ckks_ct *ct) { return ct && ct->data; }
+inline bool level_ok(const ckks_ctx *c, uint32_t level) { return level >= 1 && level <= c->L; }
+inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }

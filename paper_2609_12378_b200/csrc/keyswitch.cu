@@ -457,14 +457,6 @@ void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, 
     launch_ntt(c, w.ext, nb * beta * nt, ext_map(level, c->K, c->L, c->alpha, beta), false, s);
 }
 
-static bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
-static bool aligned16(const Ptrs &p) {
-    if (!p.n) return aligned16(p.base) && (p.stride & 1) == 0;
-    for (uint32_t i = 0; i < p.n; i++)
-        if (!aligned16(p.p[i])) return false;
-    return true;
-}
-
 void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w, cudaStream_t s, uint32_t nb,
               bool acc_u, const KsMulti *multi) {
     const uint32_t N = c->N, nt = level + c->K;
@@ -513,7 +505,7 @@ void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const K
     ep.add = o.add; ep.out = o.out; ep.add_comps = o.add_comps;
     ep.pinv = c->dev.dn_p_inv_d;
     ep.ncomp = 2; ep.level = level; ep.nt = nt;
-    ep.galois = o.galois; ep.accumulate = o.accumulate ? 1 : 0; ep.tl = o.tiled;
+    ep.galois = o.galois; ep.acc = o.acc; ep.accumulate = o.acc.n || o.acc.base ? 1 : 0; ep.tl = o.tiled;
     if (multi) {
         ep.multi = 1; ep.group = multi->group; ep.rot_rows = multi->rot_rows; ep.rot_stride = multi->rot_stride;
         for (uint32_t b = 0; b < KS_MULTI; b++) { ep.mgalois[b] = multi->galois[b]; ep.out.p[b] = multi->out[b]; }

@@ -344,19 +344,9 @@ __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 768 / ColShape<LOGR>:
 // 8-byte accesses of consecutive lanes and 16-byte accesses to the own block are both conflict free.  Words enter and leave
 // through the row too, as pairs: lane t of a half warp moves words 2 t + 32 k and 2 t + 32 k + 1, so that every global access
 // is 16 bytes per lane and 256 consecutive bytes per half warp (32 bytes per lane cost the load/store pipe one pass per lane,
-// and 128-byte bulk copies per thread keep issuing while they are waited for: 163 -> 141 us for the pass at 768 limbs).
+// and 128-byte bulk copies per thread keep issuing while they are waited for: forward 162 -> 155, inverse 159 -> 146 us at 768 limbs).
 __device__ __forceinline__ uint32_t padded(uint32_t i) { return i + 2 * (i >> 4); }
 constexpr uint32_t ROW_PAD = 256 + 32, ROW_CTA = 16;
-
-template <bool WIDE>
-__device__ __forceinline__ ulonglong2 ld_pair(const u64 *p) {
-    return WIDE ? *reinterpret_cast<const ulonglong2 *>(p) : make_ulonglong2(p[0], p[1]);
-}
-template <bool WIDE>
-__device__ __forceinline__ void st_pair(u64 *p, ulonglong2 v) {
-    if (WIDE) *reinterpret_cast<ulonglong2 *>(p) = v;
-    else { p[0] = v.x; p[1] = v.y; }
-}
 
 // forward, EP 0: in place; 1: the tail of a ModDown or rescale, (u - NTT(conv)) c + sigma_g(add), written to its final
 // place; 2: into a tiled buffer
@@ -399,6 +389,7 @@ __global__ void __launch_bounds__(16 * ROW_CTA, 4) ntt_fwd_rows(DevTables c, u64
         const uint32_t gal = (uint32_t)(ep.multi ? ep.mgalois[rot] : ep.galois);
         const u64 *up = ep.u.at(bz) + (((size_t)comp * ep.nt + i) << c.log_n) + p0;
         const u64 *add = (ep.add_comps >> comp & 1) ? ep.add.at(mem) + (((size_t)comp * ep.level + i) << c.log_n) : nullptr;
+        const u64 *acc = ep.accumulate ? ep.acc.at(bz) + (((size_t)comp * ep.level + i) << c.log_n) + p0 : nullptr;
         const uint32_t bstep = ep.tl.R ? ep.tl.R * 64 : 64;    // words from one 64-word block of the destination to the next
         u64 *dst = ep.tl.R ? const_cast<u64 *>(ep.out.base) + tiled_index(ep.tl.R, c.N, ep.tl.row0 + rot * ep.rot_rows + (ep.group ? mem : bz) * ep.tl.row_stride + comp, i, row * 256) + 2 * t
                            : const_cast<u64 *>(ep.group ? ep.out.base + rot * ep.rot_stride + mem * ep.out.stride : ep.out.at(bz)) +
@@ -432,7 +423,7 @@ __global__ void __launch_bounds__(16 * ROW_CTA, 4) ntt_fwd_rows(DevTables c, u64
                 r1 = __dadd_rn(r1, u64_to_d(odd ? a.x : a.y));
             }
             if (ep.accumulate) {
-                const ulonglong2 o = ld_pair<WIDE>(d);
+                const ulonglong2 o = ld_pair<WIDE>(acc + 32 * k);
                 r0 = __dadd_rn(r0, u64_to_d(o.x));
                 r1 = __dadd_rn(r1, u64_to_d(o.y));
             }
@@ -499,14 +490,6 @@ uint32_t rows_per_cta(uint32_t R, uint32_t ny) {
     while (rows > 4 && (uint64_t)ny * (R / rows) < 148) rows /= 2;
     return rows;
 }
-bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
-bool aligned16(const Ptrs &p) {
-    if (!p.n) return aligned16(p.base) && (p.stride & 1) == 0;
-    for (uint32_t i = 0; i < p.n; i++)
-        if (!aligned16(p.p[i])) return false;
-    return true;
-}
-
 template <uint32_t LOGR>
 void launch_cols(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, bool inverse, uint32_t share, const NttPrologue *pro, const double2 *scale, cudaStream_t s) {
     const dim3 grid(256 / ColShape<LOGR>::COLS, ny);
@@ -550,7 +533,7 @@ void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbM
         if (share > 0 && !inverse) {
             cols();
             bool wide = aligned16(ep ? (const void *)nullptr : (const void *)b);
-            if (ep) wide = aligned16(ep->u) && aligned16(ep->add) && aligned16(ep->out) && (ep->rot_stride & 1) == 0;
+            if (ep) wide = aligned16(ep->u) && aligned16(ep->add) && aligned16(ep->acc) && aligned16(ep->out) && (ep->rot_stride & 1) == 0;
             NttEpilogue e = ep ? *ep : NttEpilogue{};
             e.y0 = y0;
             const int mode = ep ? ep->mode : 0;

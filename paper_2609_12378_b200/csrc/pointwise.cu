@@ -51,28 +51,44 @@ __global__ void __launch_bounds__(THREADS) add_kernel(DevTables c, const u64 *a,
     reinterpret_cast<ulonglong2 *>(out)[off] = make_ulonglong2(add_mod(u.x, v.x, q), add_mod(u.y, v.y, q));
 }
 
-// (a0 b0, a0 b1 + a1 b0) -> e01 [2][level][N];  a1 b1 -> e2 [level][N]
-__global__ void __launch_bounds__(THREADS) tensor_kernel(DevTables c, const u64 *a, const u64 *b, u64 *e01, u64 *e2, uint32_t level) {
+// Operands enter the product kernels as 50-bit residues in doubles: a product is six FP64 instructions (mulmod_dd, |r| <= 0.75 q),
+// where the integer pipe's 128-bit product and Barrett step cost about four times as much issue time.
+template <bool WIDE>
+__device__ __forceinline__ void pair_d(const u64 *p, double (&v)[2]) {
+    const ulonglong2 w = ld_pair<WIDE>(p);
+    v[0] = u64_to_d(w.x); v[1] = u64_to_d(w.y);
+}
+template <bool WIDE>
+__device__ __forceinline__ void store_pair(u64 *p, const double (&v)[2], double q, double qinv) {
+    st_pair<WIDE>(p, make_ulonglong2(canonical_d(reduce_d(v[0], q, qinv), q), canonical_d(reduce_d(v[1], q, qinv), q)));
+}
+
+// (a0 b0, a0 b1 + a1 b0) -> e01 [2][level][N];  a1 b1 -> e2 [level][N], for the products blockIdx.z; two coefficients per thread
+template <bool WIDE>
+__global__ void __launch_bounds__(THREADS) tensor_kernel(DevTables c, const __grid_constant__ TensorArgs t, uint32_t level) {
+    const uint32_t k = (blockIdx.x * THREADS + threadIdx.x) * 2, limb = blockIdx.y, z = blockIdx.z;
+    const double q = c.modd[limb].x, qinv = c.modd[limb].y;
+    const size_t o = (size_t)limb * c.N + k;
+    const CtView va = t.a[z], vb = t.b[z];
     grid_dep_sync();
-    const uint32_t k = blockIdx.x * THREADS + threadIdx.x;
-    if (k >= c.N) return;
-    const uint32_t limb = blockIdx.y;
-    const u64 q = c.mod[limb], mu = c.mu[limb];
-    const size_t o0 = (size_t)limb * c.N + k, o1 = o0 + (size_t)level * c.N;
-    const u64 a0 = a[o0], a1 = a[o1], b0 = b[o0], b1 = b[o1];
-    u64 hi = 0, lo = 0;
-    mac128(hi, lo, a0, b1);
-    mac128(hi, lo, a1, b0);
-    const u64 r0 = mul_mod(a0, b0, q, mu), r1 = barrett112(hi, lo, q, mu), r2 = mul_mod(a1, b1, q, mu);
-    e01[o0] = r0;
-    e01[o1] = r1;
-    e2[o0] = r2;
+    double a0[2], a1[2], b0[2], b1[2], r0[2], r1[2], r2[2];
+    pair_d<WIDE>(va.p + o, a0); pair_d<WIDE>(va.p + va.comp + o, a1);
+    pair_d<WIDE>(vb.p + o, b0); pair_d<WIDE>(vb.p + vb.comp + o, b1);
+#pragma unroll
+    for (uint32_t i = 0; i < 2; i++) {
+        r0[i] = mulmod_dd(a0[i], b0[i], q, qinv);
+        r1[i] = __dadd_rn(mulmod_dd(a0[i], b1[i], q, qinv), mulmod_dd(a1[i], b0[i], q, qinv));
+        r2[i] = mulmod_dd(a1[i], b1[i], q, qinv);
+    }
+    store_pair<WIDE>(t.e01[z] + o, r0, q, qinv);
+    store_pair<WIDE>(t.e01[z] + (size_t)level * c.N + o, r1, q, qinv);
+    store_pair<WIDE>(t.e2[z] + o, r2, q, qinv);
 }
 
 // out = in * v (MUL) or in + v on component 0 (the constant polynomial v, a signed integer, has the value v mod q in
 // every position of the evaluation domain); blockIdx.y = component * level + limb
 template <bool MUL>
-__global__ void __launch_bounds__(THREADS) const_kernel(DevTables c, const u64 *in, long long v, u64 *out, uint32_t level) {
+__global__ void __launch_bounds__(THREADS) const_kernel(DevTables c, const __grid_constant__ Ptrs inp, long long v, const __grid_constant__ Ptrs outp, uint32_t level) {
     grid_dep_sync();
     const uint32_t half = c.N / 2;
     const uint32_t x = blockIdx.x * THREADS + threadIdx.x;
@@ -83,34 +99,82 @@ __global__ void __launch_bounds__(THREADS) const_kernel(DevTables c, const u64 *
     u64 r = (v < 0 && m) ? q - m : m;
     if (!MUL && blockIdx.y >= level) r = 0;
     const size_t off = (size_t)blockIdx.y * half + x;
-    const ulonglong2 u = reinterpret_cast<const ulonglong2 *>(in)[off];
-    reinterpret_cast<ulonglong2 *>(out)[off] =
+    const ulonglong2 u = reinterpret_cast<const ulonglong2 *>(inp.at(blockIdx.z))[off];
+    reinterpret_cast<ulonglong2 *>(const_cast<u64 *>(outp.at(blockIdx.z)))[off] =
         MUL ? make_ulonglong2(mul_mod(u.x, r, q, mu), mul_mod(u.y, r, q, mu)) : make_ulonglong2(add_mod(u.x, r, q), add_mod(u.y, r, q));
 }
 
-// e (+)= sum_{i < n} tensor(a_i, b_i): lazy 128-bit sums (n <= TS_MAX pairs per launch: 2 n products stay below
-// 2^112), one Barrett step per component, then the previous partial sum is added unless INIT
-template <bool INIT>
-__global__ void __launch_bounds__(THREADS) tensor_sum_kernel(DevTables c, TensorSumArgs args, uint32_t n, u64 *e01, u64 *e2, uint32_t level) {
-    grid_dep_sync();
-    const uint32_t k = blockIdx.x * THREADS + threadIdx.x;
-    if (k >= c.N) return;
-    const uint32_t limb = blockIdx.y;
-    const u64 q = c.mod[limb], mu = c.mu[limb];
+// e (+)= sum_{i < n} tensor(a_i, b_i), n <= TS_MAX pairs per launch.  Sums of products of size 0.75 q (1.5 q for the middle
+// component) are reduced every four pairs; one canonical step per component at the end, with the previous partial sum added
+// unless INIT.  Bound by the operands' HBM traffic.
+template <bool INIT, bool WIDE>
+__global__ void __launch_bounds__(THREADS) tensor_sum_kernel(DevTables c, const __grid_constant__ TensorSumArgs t, uint32_t n, u64 *e01, u64 *e2, uint32_t level) {
+    const uint32_t k = (blockIdx.x * THREADS + threadIdx.x) * 2, limb = blockIdx.y;
+    const double q = c.modd[limb].x, qinv = c.modd[limb].y;
     const size_t o0 = (size_t)limb * c.N + k, o1 = o0 + (size_t)level * c.N;
-    u64 h0 = 0, l0 = 0, h1 = 0, l1 = 0, h2 = 0, l2 = 0;
+    grid_dep_sync();
+    double s0[2] = {0.0, 0.0}, s1[2] = {0.0, 0.0}, s2[2] = {0.0, 0.0};
+    if (!INIT) { pair_d<WIDE>(e01 + o0, s0); pair_d<WIDE>(e01 + o1, s1); pair_d<WIDE>(e2 + o0, s2); }
     for (uint32_t i = 0; i < n; i++) {
-        const u64 a0 = args.a[i][o0], a1 = args.a[i][o1], b0 = args.b[i][o0], b1 = args.b[i][o1];
-        mac128(h0, l0, a0, b0);
-        mac128(h1, l1, a0, b1);
-        mac128(h1, l1, a1, b0);
-        mac128(h2, l2, a1, b1);
+        double a0[2], a1[2], b0[2], b1[2];
+        pair_d<WIDE>(t.a[i].p + o0, a0); pair_d<WIDE>(t.a[i].p + t.a[i].comp + o0, a1);
+        pair_d<WIDE>(t.b[i].p + o0, b0); pair_d<WIDE>(t.b[i].p + t.b[i].comp + o0, b1);
+#pragma unroll
+        for (uint32_t j = 0; j < 2; j++) {
+            s0[j] = __dadd_rn(s0[j], mulmod_dd(a0[j], b0[j], q, qinv));
+            s1[j] = __dadd_rn(s1[j], __dadd_rn(mulmod_dd(a0[j], b1[j], q, qinv), mulmod_dd(a1[j], b0[j], q, qinv)));
+            s2[j] = __dadd_rn(s2[j], mulmod_dd(a1[j], b1[j], q, qinv));
+            if ((i & 3) == 3) { s0[j] = reduce_d(s0[j], q, qinv); s1[j] = reduce_d(s1[j], q, qinv); s2[j] = reduce_d(s2[j], q, qinv); }
+        }
     }
-    u64 r0 = barrett112(h0, l0, q, mu), r1 = barrett112(h1, l1, q, mu), r2 = barrett112(h2, l2, q, mu);
-    if (!INIT) { r0 = add_mod(r0, e01[o0], q); r1 = add_mod(r1, e01[o1], q); r2 = add_mod(r2, e2[o0], q); }
-    e01[o0] = r0;
-    e01[o1] = r1;
-    e2[o0] = r2;
+    store_pair<WIDE>(e01 + o0, s0, q, qinv);
+    store_pair<WIDE>(e01 + o1, s1, q, qinv);
+    store_pair<WIDE>(e2 + o0, s2, q, qinv);
+}
+
+// out[o] (+)= sum_j v[o][j] x[j] for up to LIN_MAX inputs and outputs of the ciphertexts blockIdx.z / 2 (component blockIdx.z & 1),
+// constants as signed integers; cst[o] q_{level-1} is added to the first component (so that a rescale turns it into the
+// constant cst[o]).  The inputs are read once for all outputs; the constants' residues modulo this limb's prime are formed
+// once per CTA.
+template <bool WIDE>
+__global__ void __launch_bounds__(THREADS) lincomb_kernel(DevTables c, const __grid_constant__ LinArgs t, uint32_t level) {
+    __shared__ double s_v[LIN_MAX][LIN_MAX + 1];
+    const uint32_t k = (blockIdx.x * THREADS + threadIdx.x) * 2, limb = blockIdx.y, comp = blockIdx.z & 1, z = blockIdx.z >> 1;
+    const double q = c.modd[limb].x, qinv = c.modd[limb].y;
+    for (uint32_t e = threadIdx.x; e < t.no * (LIN_MAX + 1); e += THREADS) {
+        const uint32_t o = e / (LIN_MAX + 1), j = e % (LIN_MAX + 1);
+        const long long v = j < LIN_MAX ? t.v[o][j] : t.cst[o];
+        const u64 m = c.mod[limb], r = (u64)(v < 0 ? -v : v) % m;
+        double d = v < 0 ? -(double)r : (double)r;
+        if (j == LIN_MAX) d = comp || limb + 1 == level ? 0.0 : mulmod_dd(d, (double)(c.mod[level - 1] % m), q, qinv);
+        s_v[o][j] = d;
+    }
+    grid_dep_sync();
+    const size_t off = (size_t)limb * c.N + k, oo = (size_t)comp * level * c.N + off;
+    ulonglong2 x[LIN_MAX];
+#pragma unroll
+    for (uint32_t j = 0; j < LIN_MAX; j++)
+        if (j < t.nx) x[j] = ld_pair<WIDE>(t.x[j].at(z) + comp * t.xc[j] + off);
+    __syncthreads();
+    for (uint32_t o = 0; o < t.no; o++) {
+        u64 *dst = const_cast<u64 *>(t.out[o].at(z)) + oo;
+        double r[2] = {s_v[o][LIN_MAX], s_v[o][LIN_MAX]};
+        if (t.accumulate) {
+            double old[2];
+            pair_d<WIDE>(dst, old);
+            r[0] = __dadd_rn(r[0], old[0]); r[1] = __dadd_rn(r[1], old[1]);
+        }
+        // |sum| <= (0.75 + 1) q + LIN_MAX / 2 * 0.75 q, twice with a reduction between: below 8 q
+#pragma unroll
+        for (uint32_t j = 0; j < LIN_MAX; j++) {
+            if (j < t.nx) {
+                r[0] = __dadd_rn(r[0], mulmod_dd(u64_to_d(x[j].x), s_v[o][j], q, qinv));
+                r[1] = __dadd_rn(r[1], mulmod_dd(u64_to_d(x[j].y), s_v[o][j], q, qinv));
+            }
+            if (j == LIN_MAX / 2 - 1) { r[0] = reduce_d(r[0], q, qinv); r[1] = reduce_d(r[1], q, qinv); }
+        }
+        store_pair<WIDE>(dst, r, q, qinv);
+    }
 }
 
 }  // namespace
@@ -129,22 +193,32 @@ void launch_slot_mask(const ckks_ctx *c, double *out, uint32_t B, uint32_t lo, u
     launch(slot_mask_kernel, (c->n + THREADS - 1) / THREADS, THREADS, 0, s, out, c->n, B, lo, hi, Ti, t0, t1);
 }
 
-void launch_const(const ckks_ctx *c, const u64 *in, long long v, bool mul, u64 *out, uint32_t ncomp, uint32_t level, cudaStream_t s) {
-    dim3 grid((c->N / 2 + THREADS - 1) / THREADS, ncomp * level);
+void launch_const(const ckks_ctx *c, const Ptrs &in, long long v, bool mul, const Ptrs &out, uint32_t ncomp, uint32_t level, cudaStream_t s, uint32_t n) {
+    dim3 grid((c->N / 2 + THREADS - 1) / THREADS, ncomp * level, n);
     if (mul) launch(const_kernel<true>, grid, THREADS, 0, s, c->dev, in, v, out, level);
     else launch(const_kernel<false>, grid, THREADS, 0, s, c->dev, in, v, out, level);
 }
 
-void launch_tensor_sum(const ckks_ctx *c, const u64 *const *a, const u64 *const *b, uint32_t n, u64 *e01, u64 *e2, uint32_t level,
-                       cudaStream_t s) {
-    dim3 grid((c->N + THREADS - 1) / THREADS, level);
+void launch_tensor_sum(const ckks_ctx *c, const CtView *a, const CtView *b, uint32_t n, u64 *e01, u64 *e2, uint32_t level, cudaStream_t s, bool init) {
+    const dim3 grid(c->N / (2 * THREADS), level);
     for (uint32_t i0 = 0; i0 < n; i0 += TS_MAX) {
         TensorSumArgs args;
-        const uint32_t m = n - i0 < TS_MAX ? n - i0 : TS_MAX;
-        for (uint32_t i = 0; i < m; i++) { args.a[i] = a[i0 + i]; args.b[i] = b[i0 + i]; }
-        if (i0 == 0) launch(tensor_sum_kernel<true>, grid, THREADS, 0, s, c->dev, args, m, e01, e2, level);
-        else launch(tensor_sum_kernel<false>, grid, THREADS, 0, s, c->dev, args, m, e01, e2, level);
+        const uint32_t m = std::min(TS_MAX, n - i0);
+        std::copy(a + i0, a + i0 + m, args.a);
+        std::copy(b + i0, b + i0 + m, args.b);
+        bool wide = aligned16(e01) && aligned16(e2);
+        for (uint32_t i = 0; i < m; i++) wide = wide && aligned16(args.a[i]) && aligned16(args.b[i]);
+        auto *k = init && i0 == 0 ? (wide ? tensor_sum_kernel<true, true> : tensor_sum_kernel<true, false>)
+                                  : (wide ? tensor_sum_kernel<false, true> : tensor_sum_kernel<false, false>);
+        launch(k, grid, THREADS, 0, s, c->dev, args, m, e01, e2, level);
     }
+}
+
+void launch_lincomb(const ckks_ctx *c, const LinArgs &args, uint32_t n, uint32_t level, cudaStream_t s) {
+    bool wide = true;
+    for (uint32_t j = 0; j < args.nx; j++) wide = wide && aligned16(args.x[j]) && (args.xc[j] & 1) == 0;
+    for (uint32_t o = 0; o < args.no; o++) wide = wide && aligned16(args.out[o]);
+    launch(wide ? lincomb_kernel<true> : lincomb_kernel<false>, dim3(c->N / (2 * THREADS), level, 2 * n), THREADS, 0, s, c->dev, args, level);
 }
 
 void launch_mul_plain_acc(const ckks_ctx *c, const u64 *const *cts, u64 *const *accs, uint32_t ncts, const u64 *pt,
@@ -163,7 +237,8 @@ void launch_add(const ckks_ctx *c, const u64 *a, const u64 *b, u64 *out, uint32_
     launch(add_kernel, grid, THREADS, 0, s, c->dev, a, b, out, level);
 }
 
-void launch_tensor(const ckks_ctx *c, const u64 *a, const u64 *b, u64 *e01, u64 *e2, uint32_t level, cudaStream_t s) {
-    dim3 grid((c->N + THREADS - 1) / THREADS, level);
-    launch(tensor_kernel, grid, THREADS, 0, s, c->dev, a, b, e01, e2, level);
+void launch_tensor(const ckks_ctx *c, const TensorArgs &args, uint32_t n, uint32_t level, cudaStream_t s) {
+    bool wide = true;
+    for (uint32_t i = 0; i < n; i++) wide = wide && aligned16(args.a[i]) && aligned16(args.b[i]) && aligned16(args.e01[i]) && aligned16(args.e2[i]);
+    launch(wide ? tensor_kernel<true> : tensor_kernel<false>, dim3(c->N / (2 * THREADS), level, n), THREADS, 0, s, c->dev, args, level);
 }

@@ -107,3 +107,69 @@ def test_encode_coefficients_of_every_size(log_n):
         got = host(ctx.encode(dev(zz), None, scale, 3))
         for b in range(4):
             assert np.array_equal(got[b], P.oracle.encode(zz[b], scale, 3)), (scale, b)
+
+
+@pytest.mark.parametrize("degree,m,count", [(40, 16, 5), (23, 2, 1), (16, 16, 2)])
+def test_polynomial_batches_and_combinations(degree, m, count):
+    """More inputs (15) and more blocks (11) than one combination launch takes, a block that is only a constant, zero
+    coefficients, ciphertexts of two scales in one batch, and the power tree of the same degree."""
+    from tests.gpu_util import context, ct_dev, host, key_dev
+    P, ctx = params(10, 10, 4, 3), context(10, 10, 4, 3)
+    o, g = P.oracle, inputs.rng(740, degree)
+    rlk = inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, 6).reshape(3, 2, 14, P.N)
+    coeffs = g.uniform(-1, 1, degree + 1)
+    coeffs[m + 1:2 * m] = 0.0
+    coeffs[3] = 0.0
+    cts = [inputs.uniform_residues(g, P.q[:9], P.N, 2) for _ in range(count)]
+    scales = [2.0 ** 50 * (1.0 if i != 2 else 1.0 - 2.0 ** -6) for i in range(count)]
+    got = ctx.poly_eval_bsgs_batch([ct_dev(c, s) for c, s in zip(cts, scales)], coeffs, m, key_dev(rlk, 0))
+    for x, c, s in zip(got, cts, scales):
+        want, so = o.poly_eval_bsgs(c, s, coeffs, rlk, m)
+        assert x.level == want.shape[1] and x.scale == so and np.array_equal(host(x.data), want)
+    want, so = o.poly_eval_tree(cts[0], scales[0], coeffs, rlk)
+    x = ctx.poly_eval_tree(ct_dev(cts[0], scales[0]), coeffs, key_dev(rlk, 0))
+    assert x.level == want.shape[1] and x.scale == so and np.array_equal(host(x.data), want)
+
+
+@pytest.mark.parametrize("level", [1, 4, 6])
+def test_products_and_rotations_in_place_and_unaligned(level):
+    """Batches of 17 (a full chunk and one) whose results lie on their own operands or on another product's, rotations onto
+    their own and each other's inputs, and operands that are only 8-byte aligned."""
+    import torch
+    from paper_2609_12378_b200 import binding
+    from tests.gpu_util import context, ct_dev, host, key_dev
+    P, ctx = params(10, 6, 2, 3), context(10, 6, 2, 3)
+    o, g = P.oracle, inputs.rng(750, level)
+    allp = list(P.q) + list(P.p)
+    key = inputs.uniform_residues(g, allp, P.N, 6).reshape(3, 2, 8, P.N)
+    gal = o.galois_element(5)
+    x = [inputs.uniform_residues(g, P.q[:level], P.N, 2) for _ in range(17)]
+    y = [inputs.uniform_residues(g, P.q[:level], P.N, 2) for _ in range(17)]
+    prod, rot = [o.mul_relin(a, b, key) for a, b in zip(x, y)], [o.rotate(a, key, gal) for a in x]
+
+    def unaligned(a):
+        buf = torch.zeros(a.size + 1, dtype=torch.int64, device="cuda").view(torch.uint64)
+        t = buf[1:].view(*a.shape)
+        t.copy_(torch.from_numpy(a))
+        return binding.Ciphertext(t, 1.0)
+
+    for put in (lambda a: ct_dev(a, 1.0), unaligned):
+        for shift in (0, 1):        # results onto the same product's operand, or onto the next one's
+            dx, dy = [put(a) for a in x], [put(b) for b in y]
+            outs = dx[shift:] + dx[:shift]
+            if shift == 0:
+                ctx.mul_relin_batch(dx, dy, key_dev(key, 0), outs=outs)
+            else:                   # the last result goes to an operand of the chunk before it, already used
+                ctx.mul_relin_batch(dx[:16], dy[:16], key_dev(key, 0), outs=dx[1:16] + dx[:1])
+                outs, want = dx[1:16] + dx[:1], prod[:16]
+            for i, w in enumerate(prod if shift == 0 else want):
+                assert np.array_equal(host(outs[i].data), w), (shift, i)
+            dx = [put(a) for a in x[:16]]
+            outs = dx[shift:] + dx[:shift]
+            ctx.rotate_batch(dx, key_dev(key, gal), outs=outs)
+            for i in range(16):
+                assert np.array_equal(host(outs[i].data), rot[i]), (shift, i)
+        assert np.array_equal(host(ctx.mul_relin(put(x[0]), put(y[0]), key_dev(key, 0)).data), prod[0])
+        assert np.array_equal(host(ctx.rotate(put(x[0]), key_dev(key, gal)).data), rot[0])
+        s = ctx.mul_relin_sum([put(a) for a in x], [put(b) for b in y], key_dev(key, 0))
+        assert np.array_equal(host(s.data), o.mul_relin_sum(np.stack(x), np.stack(y), key))
