@@ -187,10 +187,16 @@ class SwitchKey:
     galois: int             # 0 for a relinearisation key
 
 
+# The raw handle of the current stream without building a torch.cuda.Stream object
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _dev_u64(t: torch.Tensor) -> torch.Tensor:
@@ -200,8 +206,9 @@ def _dev_u64(t: torch.Tensor) -> torch.Tensor:
 
 
 def _cct(ct: Ciphertext) -> CCt:
-    _dev_u64(ct.data)
-    return CCt(ct.data.data_ptr(), ct.level, ct.ncomp, ct.scale)
+    t = _dev_u64(ct.data)
+    shape = t.shape
+    return CCt(t.data_ptr(), shape[1], shape[0], ct.scale)
 
 
 class Context:
@@ -223,6 +230,7 @@ class Context:
             raise CkksError(rc)
         self._h = h
         self._ws = None
+        self._ws_bytes = {}         # (operation, level, count) -> bytes: fixed for a context
 
     def close(self):
         if getattr(self, "_h", None):
@@ -241,7 +249,7 @@ class Context:
             raise CkksError(rc, load().ckks_last_cuda_error(self._h).decode() if rc == ERR_CUDA else "")
 
     def set_option(self, option: int, value: int):
-        self._check(load().ckks_context_set_option(self._h, option, int(value)))
+        self._check(_lib.ckks_context_set_option(self._h, option, int(value)))
 
     def get_option(self, option: int) -> int:
         return int(load().ckks_context_get_option(self._h, option))
@@ -254,7 +262,11 @@ class Context:
         return self._ws
 
     def workspace_bytes(self, op: int, level: int, count: int = 0) -> int:
-        return int(load().ckks_workspace_bytes(self._h, op, level, count))
+        key = (op, level, count)
+        n = self._ws_bytes.get(key)
+        if n is None:
+            n = self._ws_bytes[key] = int(load().ckks_workspace_bytes(self._h, op, level, count))
+        return n
 
     def galois_element(self, r: int) -> int:
         return int(load().ckks_galois_element(self._h, r))
@@ -268,21 +280,21 @@ class Context:
         _dev_u64(polys)
         nl = polys.shape[-2]
         batch = polys.numel() // (nl * self.N)
-        self._check(load().ckks_ntt(self._h, polys.data_ptr(), batch, first_prime, nl, _stream_ptr(stream)))
+        self._check(_lib.ckks_ntt(self._h, polys.data_ptr(), batch, first_prime, nl, _stream_ptr(stream)))
         return polys
 
     def intt(self, polys: torch.Tensor, first_prime: int = 0, stream=None):
         _dev_u64(polys)
         nl = polys.shape[-2]
         batch = polys.numel() // (nl * self.N)
-        self._check(load().ckks_intt(self._h, polys.data_ptr(), batch, first_prime, nl, _stream_ptr(stream)))
+        self._check(_lib.ckks_intt(self._h, polys.data_ptr(), batch, first_prime, nl, _stream_ptr(stream)))
         return polys
 
     def ntt_butterfly_probe(self, iters: int, scratch: torch.Tensor, stream=None) -> int:
         """Launches the register-resident butterfly kernel; returns the number of butterflies it performs."""
         _dev_u64(scratch)
         n = C.c_uint64(0)
-        self._check(load().ckks_ntt_butterfly_probe(self._h, iters, scratch.data_ptr(), scratch.numel(), C.byref(n), _stream_ptr(stream)))
+        self._check(_lib.ckks_ntt_butterfly_probe(self._h, iters, scratch.data_ptr(), scratch.numel(), C.byref(n), _stream_ptr(stream)))
         return int(n.value)
 
     def encode(self, re: torch.Tensor, im, scale: float, level: int, out: torch.Tensor = None, stream=None):
@@ -294,7 +306,7 @@ class Context:
             out = torch.empty((batch, level, self.N), dtype=torch.uint64, device=self.device)
         nb = self.workspace_bytes(OP_ENCODE, level, batch)
         ws = self.workspace(nb)
-        self._check(load().ckks_encode(self._h, re.data_ptr(), im.data_ptr() if im is not None else None, batch,
+        self._check(_lib.ckks_encode(self._h, re.data_ptr(), im.data_ptr() if im is not None else None, batch,
                                        float(scale), level, _dev_u64(out).data_ptr(), ws.data_ptr(), ws.numel(),
                                        _stream_ptr(stream)))
         return out
@@ -314,7 +326,7 @@ class Context:
         ca = (CCt * n)(*[_cct(c) for c in cts])
         aa = (CCt * n)(*[_cct(a) for a in accs])
         cp = CPt(_dev_u64(pt.data).data_ptr(), pt.level, pt.scale)
-        self._check(load().ckks_mul_plain_acc(self._h, ca, n, C.byref(cp), aa, int(init), _stream_ptr(stream)))
+        self._check(_lib.ckks_mul_plain_acc(self._h, ca, n, C.byref(cp), aa, int(init), _stream_ptr(stream)))
         for a, c in zip(accs, aa):
             a.scale = c.scale
         return accs
@@ -322,7 +334,7 @@ class Context:
     def add(self, a: Ciphertext, b: Ciphertext, out: Ciphertext = None, stream=None):
         out = out or self.empty_ct(a.level, a.ncomp)
         co = _cct(out)
-        self._check(load().ckks_add(self._h, C.byref(_cct(a)), C.byref(_cct(b)), C.byref(co), _stream_ptr(stream)))
+        self._check(_lib.ckks_add(self._h, C.byref(_cct(a)), C.byref(_cct(b)), C.byref(co), _stream_ptr(stream)))
         out.scale = co.scale
         return out
 
@@ -330,7 +342,7 @@ class Context:
         out = out or self.empty_ct(a.level)
         ws = self.workspace(self.workspace_bytes(OP_MUL_RELIN, a.level))
         co, ck = _cct(out), CEvk(_dev_u64(rlk.data).data_ptr(), rlk.galois)
-        self._check(load().ckks_mul_relin(self._h, C.byref(_cct(a)), C.byref(_cct(b)), C.byref(ck), C.byref(co),
+        self._check(_lib.ckks_mul_relin(self._h, C.byref(_cct(a)), C.byref(_cct(b)), C.byref(ck), C.byref(co),
                                           ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
         out.scale = co.scale
         return out
@@ -339,14 +351,14 @@ class Context:
         """ct times the constant c encoded at cscale (0: the last prime of ct's level)."""
         out = out or Ciphertext(torch.empty_like(ct.data), ct.scale)
         co = _cct(out)
-        self._check(load().ckks_mul_const(self._h, C.byref(_cct(ct)), c, cscale, C.byref(co), _stream_ptr(stream)))
+        self._check(_lib.ckks_mul_const(self._h, C.byref(_cct(ct)), c, cscale, C.byref(co), _stream_ptr(stream)))
         out.scale = co.scale
         return out
 
     def add_const(self, ct: Ciphertext, c: float, out: Ciphertext = None, stream=None):
         out = out or Ciphertext(torch.empty_like(ct.data), ct.scale)
         co = _cct(out)
-        self._check(load().ckks_add_const(self._h, C.byref(_cct(ct)), c, C.byref(co), _stream_ptr(stream)))
+        self._check(_lib.ckks_add_const(self._h, C.byref(_cct(ct)), c, C.byref(co), _stream_ptr(stream)))
         out.scale = co.scale
         return out
 
@@ -358,7 +370,7 @@ class Context:
         ca = (C.c_double * (d + 1))(*[float(v) for v in coeffs])
         co = _cct(out)
         ck = CEvk(_dev_u64(rlk.data).data_ptr() if rlk is not None else None, rlk.galois if rlk is not None else 0)
-        self._check(load().ckks_poly_eval(self._h, C.byref(_cct(x)), ca, d, C.byref(ck), C.byref(co), ws.data_ptr(), ws.numel(),
+        self._check(_lib.ckks_poly_eval(self._h, C.byref(_cct(x)), ca, d, C.byref(ck), C.byref(co), ws.data_ptr(), ws.numel(),
                                           _stream_ptr(stream)))
         out.scale = co.scale
         return out
@@ -372,7 +384,7 @@ class Context:
         ca = (C.c_double * (d + 1))(*[float(v) for v in coeffs])
         co = _cct(out)
         ck = CEvk(_dev_u64(rlk.data).data_ptr(), rlk.galois)
-        self._check(load().ckks_poly_eval_tree(self._h, C.byref(_cct(x)), ca, d, C.byref(ck), C.byref(co), ws.data_ptr(), ws.numel(),
+        self._check(_lib.ckks_poly_eval_tree(self._h, C.byref(_cct(x)), ca, d, C.byref(ck), C.byref(co), ws.data_ptr(), ws.numel(),
                                                _stream_ptr(stream)))
         out.scale = co.scale
         return out
@@ -388,12 +400,12 @@ class Context:
         ca = (C.c_double * (d + 1))(*[float(v) for v in coeffs])
         co = _cct(out)
         ck = CEvk(_dev_u64(rlk.data).data_ptr(), rlk.galois)
-        self._check(load().ckks_poly_eval_bsgs(self._h, C.byref(_cct(x)), ca, d, m, C.byref(ck), C.byref(co), ws.data_ptr(), ws.numel(),
+        self._check(_lib.ckks_poly_eval_bsgs(self._h, C.byref(_cct(x)), ca, d, m, C.byref(ck), C.byref(co), ws.data_ptr(), ws.numel(),
                                                _stream_ptr(stream)))
         return Ciphertext(out.data.view(-1)[: 2 * co.level * self.N].view(2, co.level, self.N), co.scale)
 
     def poly_eval_bsgs_batch(self, xs, coeffs, m: int, rlk: SwitchKey, stream=None):
-        """[poly_eval_bsgs(x, coeffs, m) for x in xs], the independent evaluations spread over the context's lanes."""
+        """[poly_eval_bsgs(x, coeffs, m) for x in xs], up to four evaluations of one scale side by side."""
         d, n, level = len(coeffs) - 1, len(xs), xs[0].level
         need = int(load().ckks_poly_eval_bsgs_batch_workspace_bytes(self._h, level, d, m, n))
         if need == 0:
@@ -404,7 +416,7 @@ class Context:
         xa = (CCt * n)(*[_cct(x) for x in xs])
         oa = (CCt * n)(*[_cct(o) for o in outs])
         ck = CEvk(_dev_u64(rlk.data).data_ptr(), rlk.galois)
-        self._check(load().ckks_poly_eval_bsgs_batch(self._h, xa, n, ca, d, m, C.byref(ck), oa, ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
+        self._check(_lib.ckks_poly_eval_bsgs_batch(self._h, xa, n, ca, d, m, C.byref(ck), oa, ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
         return [self._cut(o, c) for o, c in zip(outs, oa)]
 
     def softmax(self, ct: Ciphertext, shift: float, rounds: int, row_len: int, exp_coeffs, rsqrt_coeffs, rlk: SwitchKey, keys,
@@ -426,7 +438,7 @@ class Context:
         ci, co = _cct(ct), _cct(out)
         crlk = CEvk(_dev_u64(rlk.data).data_ptr(), 0)
         ka = (CEvk * max(1, len(keys)))(*[CEvk(_dev_u64(k.data).data_ptr(), k.galois) for k in keys])
-        self._check(load().ckks_softmax(self._h, C.byref(d), C.byref(ci), C.byref(crlk), ka, len(keys), C.byref(co), ws.data_ptr(), ws.numel(),
+        self._check(_lib.ckks_softmax(self._h, C.byref(d), C.byref(ci), C.byref(crlk), ka, len(keys), C.byref(co), ws.data_ptr(), ws.numel(),
                                         _stream_ptr(stream)))
         res = Ciphertext(out.data.view(-1)[: 2 * co.level * self.N].view(2, co.level, self.N), co.scale)
         return res
@@ -479,7 +491,7 @@ class Context:
         ia = (CCt * len(cts))(*[_cct(x) for x in cts])
         oa = (CCt * nout)(*[_cct(x) for x in outs])
         ra = (CEvk * max(1, len(keys)))(*[CEvk(_dev_u64(x.data).data_ptr(), x.galois) for x in keys])
-        self._check(load().ckks_attention_pack(self._h, C.byref(d), kind, ia, dim, ra, len(keys), oa, ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
+        self._check(_lib.ckks_attention_pack(self._h, C.byref(d), kind, ia, dim, ra, len(keys), oa, ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
         return [self._cut(o, c) for o, c in zip(outs, oa)]
 
     def attention_scores(self, q, k, rlk: SwitchKey, keys, tokens, heads, diag_block, ws: torch.Tensor = None, stream=None,
@@ -496,7 +508,7 @@ class Context:
         oa = (CCt * G)(*[_cct(x) for x in outs])
         ck = CEvk(_dev_u64(rlk.data).data_ptr(), 0)
         ra = (CEvk * max(1, len(keys)))(*[CEvk(_dev_u64(x.data).data_ptr(), x.galois) for x in keys])
-        self._check(load().ckks_attention_scores(self._h, C.byref(d), qa, ka, len(q), C.byref(ck), ra, len(keys), oa, ws.data_ptr(), ws.numel(),
+        self._check(_lib.ckks_attention_scores(self._h, C.byref(d), qa, ka, len(q), C.byref(ck), ra, len(keys), oa, ws.data_ptr(), ws.numel(),
                                                  _stream_ptr(stream)))
         for o, c in zip(outs, oa):
             o.scale = c.scale
@@ -516,7 +528,7 @@ class Context:
         oa = (CCt * len(outs))(*[_cct(x) for x in outs])
         ck = CEvk(_dev_u64(rlk.data).data_ptr(), 0)
         ra = (CEvk * max(1, len(keys)))(*[CEvk(_dev_u64(x.data).data_ptr(), x.galois) for x in keys])
-        self._check(load().ckks_softmax_rows(self._h, C.byref(d), C.byref(sd), ia, C.byref(ck), ra, len(keys), oa, ws.data_ptr(), ws.numel(),
+        self._check(_lib.ckks_softmax_rows(self._h, C.byref(d), C.byref(sd), ia, C.byref(ck), ra, len(keys), oa, ws.data_ptr(), ws.numel(),
                                              _stream_ptr(stream)))
         return [self._cut(o, c) for o, c in zip(outs, oa)]
 
@@ -531,7 +543,7 @@ class Context:
         oa = (CCt * len(outs))(*[_cct(x) for x in outs])
         ck = CEvk(_dev_u64(rlk.data).data_ptr(), 0)
         ra = (CEvk * max(1, len(keys)))(*[CEvk(_dev_u64(x.data).data_ptr(), x.galois) for x in keys])
-        self._check(load().ckks_attention_values(self._h, C.byref(d), pa, va, len(v), C.byref(ck), ra, len(keys), oa, ws.data_ptr(), ws.numel(),
+        self._check(_lib.ckks_attention_values(self._h, C.byref(d), pa, va, len(v), C.byref(ck), ra, len(keys), oa, ws.data_ptr(), ws.numel(),
                                                  _stream_ptr(stream)))
         for o, c in zip(outs, oa):
             o.scale = c.scale
@@ -555,7 +567,7 @@ class Context:
         oa = (CCt * len(outs))(*[_cct(x) for x in outs])
         ck = CEvk(_dev_u64(rlk.data).data_ptr(), 0)
         ra = (CEvk * max(1, len(keys)))(*[CEvk(_dev_u64(x.data).data_ptr(), x.galois) for x in keys])
-        self._check(load().ckks_attention(self._h, C.byref(d), C.byref(sd), qa, ka, len(q), va, len(v), C.byref(ck), ra, len(keys), oa,
+        self._check(_lib.ckks_attention(self._h, C.byref(d), C.byref(sd), qa, ka, len(q), va, len(v), C.byref(ck), ra, len(keys), oa,
                                           ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
         return [self._cut(o, c) for o, c in zip(outs, oa)]
 
@@ -568,7 +580,7 @@ class Context:
         ia = (CCt * len(cts))(*[_cct(x) for x in cts])
         ka = (CEvk * len(keys))(*[CEvk(_dev_u64(k.data).data_ptr(), k.galois) for k in keys])
         co = _cct(out)
-        self._check(load().ckks_rotate_sum(self._h, ia, ka, len(cts), C.byref(co), ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
+        self._check(_lib.ckks_rotate_sum(self._h, ia, ka, len(cts), C.byref(co), ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
         out.scale = co.scale
         return out
 
@@ -581,7 +593,7 @@ class Context:
         ia = (CCt * len(cts))(*[_cct(x) for x in cts])
         oa = (CCt * len(outs))(*[_cct(x) for x in outs])
         ck = CEvk(_dev_u64(key.data).data_ptr(), key.galois)
-        self._check(load().ckks_rotate_batch(self._h, ia, len(cts), C.byref(ck), oa, ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
+        self._check(_lib.ckks_rotate_batch(self._h, ia, len(cts), C.byref(ck), oa, ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
         for o, c in zip(outs, oa):
             o.scale = c.scale
         return outs
@@ -598,7 +610,7 @@ class Context:
         ba = (CCt * len(b))(*[_cct(x) for x in b])
         oa = (CCt * len(outs))(*[_cct(x) for x in outs])
         ck = CEvk(_dev_u64(rlk.data).data_ptr(), rlk.galois)
-        self._check(load().ckks_mul_relin_batch(self._h, aa, ba, len(a), C.byref(ck), oa, ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
+        self._check(_lib.ckks_mul_relin_batch(self._h, aa, ba, len(a), C.byref(ck), oa, ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
         for o, c in zip(outs, oa):
             o.scale = c.scale
         return outs
@@ -613,7 +625,7 @@ class Context:
         aa = (CCt * len(a))(*[_cct(x) for x in a])
         ba = (CCt * len(b))(*[_cct(x) for x in b])
         co, ck = _cct(out), CEvk(_dev_u64(rlk.data).data_ptr(), rlk.galois)
-        self._check(load().ckks_mul_relin_sum(self._h, aa, ba, len(a), C.byref(ck), C.byref(co), ws.data_ptr(), ws.numel(),
+        self._check(_lib.ckks_mul_relin_sum(self._h, aa, ba, len(a), C.byref(ck), C.byref(co), ws.data_ptr(), ws.numel(),
                                               _stream_ptr(stream)))
         out.scale = co.scale
         return out
@@ -622,7 +634,7 @@ class Context:
         out = out or self.empty_ct(ct.level)
         ws = self.workspace(self.workspace_bytes(OP_ROTATE, ct.level))
         co, ck = _cct(out), CEvk(_dev_u64(key.data).data_ptr(), key.galois)
-        self._check(load().ckks_rotate(self._h, C.byref(_cct(ct)), C.byref(ck), C.byref(co), ws.data_ptr(), ws.numel(),
+        self._check(_lib.ckks_rotate(self._h, C.byref(_cct(ct)), C.byref(ck), C.byref(co), ws.data_ptr(), ws.numel(),
                                        _stream_ptr(stream)))
         out.scale = co.scale
         return out
@@ -633,7 +645,7 @@ class Context:
         ws = self.workspace(self.workspace_bytes(OP_ROTATE_HOISTED, ct.level, n))
         ka = (CEvk * n)(*[CEvk(_dev_u64(k.data).data_ptr(), k.galois) for k in keys])
         oa = (CCt * n)(*[_cct(o) for o in outs])
-        self._check(load().ckks_rotate_hoisted(self._h, C.byref(_cct(ct)), ka, n, oa, ws.data_ptr(), ws.numel(),
+        self._check(_lib.ckks_rotate_hoisted(self._h, C.byref(_cct(ct)), ka, n, oa, ws.data_ptr(), ws.numel(),
                                                _stream_ptr(stream)))
         for o, c in zip(outs, oa):
             o.scale = c.scale
@@ -659,7 +671,7 @@ class Context:
         oa = (CCt * len(flat))(*[_cct(o) for o in flat])
         wa = (C.c_void_p * nmat)(*[W.data_ptr() for W in Ws])
         ka = (CEvk * len(keys))(*[CEvk(_dev_u64(k.data).data_ptr(), k.galois) for k in keys])
-        self._check(load().ckks_linear_proj_multi(self._h, da, nmat, ia, wa, ka, len(keys), oa, ws.data_ptr(), ws.numel(),
+        self._check(_lib.ckks_linear_proj_multi(self._h, da, nmat, ia, wa, ka, len(keys), oa, ws.data_ptr(), ws.numel(),
                                                   _stream_ptr(stream)))
         for o, c in zip(flat, oa):
             o.scale = c.scale
@@ -670,7 +682,7 @@ class Context:
         ws = self.workspace(self.workspace_bytes(OP_RESCALE, ct.level))
         co = _cct(out)
         co.level = ct.level - 1
-        self._check(load().ckks_rescale(self._h, C.byref(_cct(ct)), C.byref(co), ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
+        self._check(_lib.ckks_rescale(self._h, C.byref(_cct(ct)), C.byref(co), ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
         out.scale = co.scale
         return out
 
@@ -710,7 +722,7 @@ class Context:
         for o in oa:
             o.level = level - 1
         ka = (CEvk * len(keys))(*[CEvk(_dev_u64(k.data).data_ptr(), k.galois) for k in keys])
-        self._check(load().ckks_linear_proj(self._h, C.byref(d), ia, W.data_ptr(), ka, len(keys), oa, ws.data_ptr(),
+        self._check(_lib.ckks_linear_proj(self._h, C.byref(d), ia, W.data_ptr(), ka, len(keys), oa, ws.data_ptr(),
                                             ws.numel(), _stream_ptr(stream)))
         for o, c in zip(outs, oa):
             o.scale = c.scale
