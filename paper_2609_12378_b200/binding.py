@@ -187,6 +187,7 @@ class SwitchKey:
     galois: int             # 0 for a relinearisation key
 
 
+_U64 = torch.uint64
 # The raw handle of the current stream without building a torch.cuda.Stream object
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
@@ -200,7 +201,7 @@ def _stream_ptr(stream):
 
 
 def _dev_u64(t: torch.Tensor) -> torch.Tensor:
-    if not (t.is_cuda and t.dtype == torch.uint64 and t.is_contiguous()):
+    if not (t.is_cuda and t.dtype is _U64 and t.is_contiguous()):
         raise TypeError("expected a contiguous CUDA uint64 tensor")
     return t
 
@@ -278,16 +279,22 @@ class Context:
     def ntt(self, polys: torch.Tensor, first_prime: int = 0, stream=None):
         """In-place forward NTT of [batch][nlimbs][N] (or [nlimbs][N])."""
         _dev_u64(polys)
-        nl = polys.shape[-2]
-        batch = polys.numel() // (nl * self.N)
-        self._check(_lib.ckks_ntt(self._h, polys.data_ptr(), batch, first_prime, nl, _stream_ptr(stream)))
+        shape = polys.shape
+        nl = shape[-2]
+        batch = shape[0] if len(shape) == 3 and shape[2] == self.N else polys.numel() // (nl * self.N)
+        rc = _lib.ckks_ntt(self._h, polys.data_ptr(), batch, first_prime, nl, _stream_ptr(stream))
+        if rc:
+            self._check(rc)
         return polys
 
     def intt(self, polys: torch.Tensor, first_prime: int = 0, stream=None):
         _dev_u64(polys)
-        nl = polys.shape[-2]
-        batch = polys.numel() // (nl * self.N)
-        self._check(_lib.ckks_intt(self._h, polys.data_ptr(), batch, first_prime, nl, _stream_ptr(stream)))
+        shape = polys.shape
+        nl = shape[-2]
+        batch = shape[0] if len(shape) == 3 and shape[2] == self.N else polys.numel() // (nl * self.N)
+        rc = _lib.ckks_intt(self._h, polys.data_ptr(), batch, first_prime, nl, _stream_ptr(stream))
+        if rc:
+            self._check(rc)
         return polys
 
     def ntt_butterfly_probe(self, iters: int, scratch: torch.Tensor, stream=None) -> int:

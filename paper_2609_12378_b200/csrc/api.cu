@@ -163,7 +163,9 @@ extern "C" int32_t ckks_ntt(ckks_ctx *c, uint64_t *polys, uint32_t batch, uint32
     if (!c || !polys || !batch || !nlimbs) return CKKS_ERR_ARG;
     if ((uint64_t)first + nlimbs > c->T) return CKKS_ERR_LEVEL;
     DeviceGuard g(c->device);
-    launch_ntt(c, (u64 *)polys, batch * nlimbs, plain_map(first, nlimbs), false, (cudaStream_t)stream);
+    const LimbMap map = plain_map(first, nlimbs);
+    if (!launch_ntt_small(c, (u64 *)polys, batch * nlimbs, map, false, (cudaStream_t)stream))
+        launch_ntt(c, (u64 *)polys, batch * nlimbs, map, false, (cudaStream_t)stream);
     return finish(c);
 }
 
@@ -171,7 +173,9 @@ extern "C" int32_t ckks_intt(ckks_ctx *c, uint64_t *polys, uint32_t batch, uint3
     if (!c || !polys || !batch || !nlimbs) return CKKS_ERR_ARG;
     if ((uint64_t)first + nlimbs > c->T) return CKKS_ERR_LEVEL;
     DeviceGuard g(c->device);
-    launch_ntt(c, (u64 *)polys, batch * nlimbs, plain_map(first, nlimbs), true, (cudaStream_t)stream);
+    const LimbMap map = plain_map(first, nlimbs);
+    if (!launch_ntt_small(c, (u64 *)polys, batch * nlimbs, map, true, (cudaStream_t)stream))
+        launch_ntt(c, (u64 *)polys, batch * nlimbs, map, true, (cudaStream_t)stream);
     return finish(c);
 }
 

@@ -484,6 +484,167 @@ __global__ void __launch_bounds__(16 * ROW_CTA, 3) ntt_inv_rows(DevTables c, u64
     for (uint32_t k = 0; k < 16; k++) reinterpret_cast<double *>(g)[t + 16 * k] = x[k];
 }
 
+// ---- both passes in one kernel: a cluster of CTAs per limb --------------------------------------------------------------
+// CL CTAs hold a limb in shared memory: CTA c does the column stages of 256 / CL columns, the values cross to the CTAs that
+// own their rows through distributed shared memory, and CTA d does the row stages of R / CL rows (inverse: the other way
+// round).  Two cluster barriers: one, split around the second group's arithmetic, keeps values from landing in an exchange buffer
+// that is still being read; the other follows the crossing.
+template <uint32_t LOGR>
+struct ClShape {
+    static constexpr uint32_t LOG = LOGR, R = 1u << LOGR, CL = LOGR == 6 ? 8 : 4;
+    static constexpr uint32_t A = 4, B = LOGR - 4;                             // column stages: 4, then 0 .. 2
+    static constexpr uint32_t COLS = 256 / CL, ROWS = R / CL, THREADS = ROWS * 16;
+    static constexpr uint32_t SMEM = (ROWS * ROW_PAD > R * COLS ? ROWS * ROW_PAD : R * COLS) * 8;
+};
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_addr(const double *p, uint32_t rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, double v) { asm volatile("st.shared::cluster.f64 [%0], %1;\n" ::"r"(a), "d"(v) : "memory"); }
+
+template <uint32_t LOGR>
+__global__ void __launch_bounds__(ClShape<LOGR>::THREADS, 1024 / ClShape<LOGR>::THREADS) ntt_fwd_cluster(DevTables c, u64 *base, LimbMap map) {
+    using S = ClShape<LOGR>;
+    extern __shared__ __align__(16) double dsm[];
+    const int prime = limb_prime(map, blockIdx.y);
+    if (prime < 0) return;                  // the whole cluster
+    const double q = c.modd[prime].x, qinv = c.modd[prime].y;
+    const double *tw = c.twd_fwd + ((size_t)prime << c.log_n);
+    const uint32_t rank = blockIdx.x;
+    u64 *limb = base + (limb_index(map, blockIdx.y) << c.log_n);
+    double x[16];
+    {
+        const uint32_t cc = threadIdx.x % S::COLS, r = threadIdx.x / S::COLS;
+        constexpr uint32_t RS = S::R / 16;
+        const u64 *gs = limb + rank * S::COLS + cc;
+        grid_dep_sync();
+#pragma unroll
+        for (uint32_t k = 0; k < 16; k++) x[k] = u64_to_d(gs[(size_t)(r + RS * k) * 256]);
+        __syncwarp();
+        fwd_col_group<LOGR, 0, 4>(x, 0, tw, 1, q, qinv);
+        if constexpr (S::B > 0) {
+#pragma unroll
+            for (uint32_t k = 0; k < 16; k++) dsm[(r + RS * k) * S::COLS + cc] = x[k];
+            __syncthreads();
+#pragma unroll
+            for (uint32_t k = 0; k < 16; k++) x[k] = dsm[(16 * r + k) * S::COLS + cc];
+            cluster_arrive();
+#pragma unroll
+            for (uint32_t j = 0; j < (16u >> S::B); j++) fwd_col_group<LOGR, 4, S::B>(x, j << S::B, tw, 16 + r * (16 >> S::B) + j, q, qinv);
+        } else {
+            cluster_arrive();
+        }
+        cluster_wait();                     // (without a second group: the peers have started)
+        // 16 consecutive rows (S::B = 0: all of them) of one column to the CTAs that own them
+        const uint32_t col = padded(rank * S::COLS + cc);
+#pragma unroll
+        for (uint32_t k0 = 0; k0 < 16; k0 += S::ROWS) {
+            const uint32_t row = (S::B ? 16 * r : 0) + k0;
+            const uint32_t a = cluster_addr(dsm + col, row / S::ROWS);
+#pragma unroll
+            for (uint32_t k = 0; k < S::ROWS; k++) cluster_store(a + k * ROW_PAD * 8, x[k0 + k]);
+        }
+        cluster_arrive();
+        cluster_wait();
+    }
+    const uint32_t t = threadIdx.x & 15, rl = threadIdx.x >> 4, row = rank * S::ROWS + rl;
+    double *s = dsm + rl * ROW_PAD, *blk = s + 18 * t;
+#pragma unroll
+    for (uint32_t k = 0; k < 16; k++) x[k] = s[padded(t + 16 * k)];
+    fwd_row_open(x, tw, S::R + row, q, qinv);
+#pragma unroll
+    for (uint32_t k = 0; k < 16; k++) s[padded(t + 16 * k)] = x[k];
+    __syncwarp();
+#pragma unroll
+    for (uint32_t k = 0; k < 16; k += 2) {
+        const double2 v = *reinterpret_cast<const double2 *>(blk + k);
+        x[k] = v.x; x[k + 1] = v.y;
+    }
+    fwd_row_close(x, tw, 16 * (S::R + row) + t, q, qinv);
+#pragma unroll
+    for (uint32_t k = 0; k < 16; k += 2) *reinterpret_cast<double2 *>(blk + k) = make_double2(x[k], x[k + 1]);
+    __syncwarp();
+    const double *sp = s + 2 * t + 2 * (t >> 3);
+    u64 *dst = limb + (size_t)row * 256 + 2 * t;
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) {
+        const double2 v = *reinterpret_cast<const double2 *>(sp + 36 * k);
+        st_pair<true>(dst + 32 * k, make_ulonglong2(canonical_d(reduce_d(v.x, q, qinv), q), canonical_d(reduce_d(v.y, q, qinv), q)));
+    }
+}
+
+template <uint32_t LOGR>
+__global__ void __launch_bounds__(ClShape<LOGR>::THREADS, 1024 / ClShape<LOGR>::THREADS) ntt_inv_cluster(DevTables c, u64 *base, LimbMap map) {
+    using S = ClShape<LOGR>;
+    extern __shared__ __align__(16) double dsm[];
+    const int prime = limb_prime(map, blockIdx.y);
+    if (prime < 0) return;
+    const double q = c.modd[prime].x, qinv = c.modd[prime].y;
+    const double *tw = c.twd_inv + ((size_t)prime << c.log_n);
+    const uint32_t rank = blockIdx.x;
+    u64 *limb = base + (limb_index(map, blockIdx.y) << c.log_n);
+    double x[16];
+    {
+        const uint32_t t = threadIdx.x & 15, rl = threadIdx.x >> 4, row = rank * S::ROWS + rl;
+        const u64 *gs = limb + (size_t)row * 256;
+        double *s = dsm + rl * ROW_PAD, *blk = s + 18 * t, *sp = s + 2 * t + 2 * (t >> 3);
+        grid_dep_sync();
+#pragma unroll
+        for (uint32_t k = 0; k < 8; k++) {
+            const ulonglong2 v = ld_pair<true>(gs + 2 * t + 32 * k);
+            x[2 * k] = u64_to_d(v.x); x[2 * k + 1] = u64_to_d(v.y);
+        }
+#pragma unroll
+        for (uint32_t k = 0; k < 8; k++) *reinterpret_cast<double2 *>(sp + 36 * k) = make_double2(x[2 * k], x[2 * k + 1]);
+        __syncwarp();
+#pragma unroll
+        for (uint32_t k = 0; k < 16; k += 2) {
+            const double2 v = *reinterpret_cast<const double2 *>(blk + k);
+            x[k] = v.x; x[k + 1] = v.y;
+        }
+        inv_row_group<1>(x, tw, 16 * (S::R + row) + t, q, qinv);
+#pragma unroll
+        for (uint32_t k = 0; k < 16; k += 2) *reinterpret_cast<double2 *>(blk + k) = make_double2(x[k], x[k + 1]);
+        __syncwarp();
+#pragma unroll
+        for (uint32_t k = 0; k < 16; k++) x[k] = s[padded(t + 16 * k)];
+        cluster_arrive();
+        inv_row_group<2>(x, tw, S::R + row, q, qinv);
+        cluster_wait();
+        // columns t + 16 k of this row to the CTAs that own them
+        constexpr uint32_t KC = S::COLS / 16;
+#pragma unroll
+        for (uint32_t k0 = 0; k0 < 16; k0 += KC) {
+            const uint32_t a = cluster_addr(dsm + row * S::COLS + t, k0 / KC);
+#pragma unroll
+            for (uint32_t k = 0; k < KC; k++) cluster_store(a + k * 128, x[k0 + k]);
+        }
+        cluster_arrive();
+        cluster_wait();
+    }
+    const uint32_t cc = threadIdx.x % S::COLS, r = threadIdx.x / S::COLS;
+    constexpr uint32_t RS = S::R / 16;
+    const double2 c0 = c.n_inv_d[2 * prime], c1 = c.n_inv_d[2 * prime + 1];
+    if constexpr (S::B > 0) {
+#pragma unroll
+        for (uint32_t k = 0; k < 16; k++) x[k] = dsm[(16 * r + k) * S::COLS + cc];
+#pragma unroll
+        for (uint32_t j = 0; j < (16u >> S::B); j++) inv_col_open<S::B>(x, j << S::B, tw, 16 + r * (16 >> S::B) + j, q, qinv);
+#pragma unroll
+        for (uint32_t k = 0; k < 16; k++) dsm[(16 * r + k) * S::COLS + cc] = x[k];
+        __syncthreads();
+    }
+#pragma unroll
+    for (uint32_t k = 0; k < 16; k++) x[k] = dsm[(r + RS * k) * S::COLS + cc];
+    inv_col_last<4, S::B>(x, tw, q, qinv, c0, c1);
+    u64 *g = limb + rank * S::COLS + cc;
+#pragma unroll
+    for (uint32_t k = 0; k < 16; k++) g[(size_t)(r + RS * k) * 256] = canonical_d(x[k], q);
+}
+
 // rows per CTA: 16, or fewer while that would leave SMs without a CTA
 uint32_t rows_per_cta(uint32_t R, uint32_t ny) {
     uint32_t rows = R < ROW_CTA ? R : ROW_CTA;
@@ -549,6 +710,22 @@ void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbM
         }
         if (share < 8) launch_ntt_int(c, b, ny, map, inverse, src ? sr.ptr.base : nullptr, src ? (uint32_t)(sr.ptr.stride >> c->log_n) : 0, s);
     }
+}
+
+// In-place transforms of a few limbs of a small ring, both passes in one launch: a call of its own is bound by the host, whom a
+// launch costs 2 us (both directions of 12 limbs at N = 2^13: 20.4 -> 17.7 us).  Returns false outside its range, N = 2^12 .. 2^14
+// and at most two CTAs per SM.  Inside chains of launches the two-pass form stays the better one: the device then is the bound,
+// and the passes' 2.2 to 2.9 us each, back to back, beat this kernel's 5.8 (product and rescale at N = 2^14: 42 against 53 us).
+// At N = 2^16 the same form with 8 and 16 CTAs per cluster took 431 and 417 us against 305 for 768 limbs.
+bool launch_ntt_small(const ckks_ctx *c, u64 *base, uint32_t nlimbs, const LimbMap &map, bool inverse, cudaStream_t s) {
+    if (c->log_n < 12 || c->log_n > 14 || !aligned16(base)) return false;
+    auto run = [&](auto shape) {
+        using S = decltype(shape);
+        if (nlimbs * S::CL > 2 * (uint32_t)c->sms) return false;
+        launch_clusters(inverse ? ntt_inv_cluster<S::LOG> : ntt_fwd_cluster<S::LOG>, S::CL, dim3(S::CL, nlimbs), S::THREADS, S::SMEM, s, c->dev, base, map);
+        return true;
+    };
+    return c->log_n == 14 ? run(ClShape<6>()) : c->log_n == 13 ? run(ClShape<5>()) : run(ClShape<4>());
 }
 
 // grid: three CTAs per SM, the residency of the transform kernels.  Returns the butterflies one launch performs.

@@ -173,3 +173,13 @@ def test_products_and_rotations_in_place_and_unaligned(level):
         assert np.array_equal(host(ctx.rotate(put(x[0]), key_dev(key, gal)).data), rot[0])
         s = ctx.mul_relin_sum([put(a) for a in x], [put(b) for b in y], key_dev(key, 0))
         assert np.array_equal(host(s.data), o.mul_relin_sum(np.stack(x), np.stack(y), key))
+
+
+@pytest.mark.parametrize("log_n,batch,limbs", [(12, 1, 3), (12, 24, 3), (12, 25, 3), (13, 24, 3), (13, 25, 3), (14, 12, 3), (14, 13, 3)])
+def test_transforms_at_the_cluster_limit(log_n, batch, limbs):
+    """The last batch that one cluster per limb transforms and the first that goes in two passes: both directions."""
+    from tests.gpu_util import context, dev, host
+    P, ctx = params(log_n, 3, 1, 3), context(log_n, 3, 1, 3)
+    x = inputs.uniform_residues(inputs.rng(770, log_n), P.q[:limbs], P.N, batch)
+    assert np.array_equal(host(ctx.ntt(dev(x))), P.oracle.ntt(x))
+    assert np.array_equal(host(ctx.intt(dev(x))), P.oracle.intt(x))
