@@ -22,15 +22,17 @@
 
 namespace {
 
-constexpr uint32_t MG = 16, MS = 16, MK = 32, STAGES = 3;
+constexpr uint32_t MG = 16, MK = 32;
 
-template <uint32_t COEF>
+// COEF coefficients per CTA, tiles of NC column halves (8 columns each), STAGES steps in the ring
+template <uint32_t COEF, uint32_t NC, uint32_t NSTAGES>
 struct Geo {
+    static constexpr uint32_t MS = 8 * NC, STAGES = NSTAGES;
     static constexpr uint32_t CH = COEF / 2;                        // 16-byte chunks per row
     static constexpr uint32_t ROW = COEF * 8;                       // bytes per row
     static constexpr uint32_t GPITCH = MK * ROW + (CH == 4 ? 64 : 16);   // bytes per g (or s') block of 32 rows
-    static constexpr uint32_t BOX_BYTES = MG * GPITCH;              // one operand of one stage
-    static constexpr uint32_t STAGE_BYTES = 2 * BOX_BYTES;
+    static constexpr uint32_t BOX_BYTES = MG * GPITCH;              // the plaintext operand of one stage; the ciphertexts follow
+    static constexpr uint32_t STAGE_BYTES = BOX_BYTES + MS * GPITCH;
     static constexpr uint32_t OBUF_BYTES = MG * MS * COEF * 8;      // one tile of results, staged for whole-row stores
     static constexpr size_t SMEM_BYTES = (size_t)STAGES * STAGE_BYTES + OBUF_BYTES + 64 /* mbarriers */ + 128 /* alignment slack */;
     // byte offset of (block a, row j, 16-byte chunk ch) inside an operand tile
@@ -90,22 +92,23 @@ struct TileIt {
     }
 };
 
-template <uint32_t COEF, uint32_t NW>
-__global__ void __launch_bounds__(COEF * 64 / NW, 8 / COEF) mac_mma_kernel(DevTables c, const u64 *__restrict__ baby,
+// NW column halves per warp of the tile's NC
+template <uint32_t COEF, uint32_t NW, uint32_t NC, uint32_t NSTAGES, uint32_t CTAS>
+__global__ void __launch_bounds__(COEF * 32 * NC / NW, CTAS) mac_mma_kernel(DevTables c, const u64 *__restrict__ baby,
                                                                            const u64 *__restrict__ pts, u64 *__restrict__ acc, uint32_t J,
                                                                            uint32_t S, uint32_t G, uint32_t level, uint32_t ntiles,
                                                                            uint32_t Jx, uint32_t j0, uint32_t accumulate) {
     grid_dep_sync();
-    using T = Geo<COEF>;
-    constexpr uint32_t THREADS = COEF * 64 / NW, CH = T::CH;
+    using T = Geo<COEF, NC, NSTAGES>;
+    constexpr uint32_t THREADS = COEF * 32 * NC / NW, CH = T::CH, MS = T::MS, STAGES = T::STAGES;
     constexpr uint32_t AH = THREADS / (CH * MK);      // blocks a loaded side by side; a thread walks a = arow + AH it
-    constexpr uint32_t NIT = MG / AH;                 // cp.async per operand per thread and step
+    constexpr uint32_t NIT = MG / AH, NIX = MS / AH;  // cp.async per thread and step for the plaintexts and the ciphertexts
     constexpr uint32_t XB64 = 64 / COEF;              // tiles per 64-coefficient block
     extern __shared__ uint8_t smem_raw[];
     uint8_t *ring = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
     u64 *obuf = reinterpret_cast<u64 *>(ring + STAGES * T::STAGE_BYTES);
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
-    const uint32_t coef = NW == 2 ? warp : warp >> 1, n0 = NW == 2 ? 0 : (warp & 1);
+    const uint32_t coef = warp / (NC / NW), n0 = warp % (NC / NW);
     const uint32_t ncol = 2 * S, coltiles = (ncol + MS - 1) / MS, gtiles = (G + MG - 1) / MG;
     const uint32_t xblocks = c.N / COEF;
     const uint32_t nk = J / MK;
@@ -158,7 +161,7 @@ __global__ void __launch_bounds__(COEF * 64 / NW, 8 / COEF) mac_mma_kernel(DevTa
     for (uint32_t s = 0; s < STAGES - 1; s++) {
         load_begin();
 #pragma unroll
-        for (uint32_t k = 0; k < NIT; k++) { load_w(k); load_x(k); }
+        for (uint32_t k = 0; k < NIT; k++) { load_w(k); if (k < NIX) load_x(k); }
         load_end();
     }
 
@@ -176,7 +179,7 @@ __global__ void __launch_bounds__(COEF * 64 / NW, 8 / COEF) mac_mma_kernel(DevTa
     auto flush = [&]() {
 #pragma unroll
         for (uint32_t k = 0; k < MG * MS * COEF / THREADS; k++) {
-            const uint32_t row = k * (THREADS / COEF) + tid / COEF, sl = tid % COEF, gl = row >> 4, cl = row & 15;
+            const uint32_t row = k * (THREADS / COEF) + tid / COEF, sl = tid % COEF, gl = row / MS, cl = row % MS;
             const uint32_t g = pend_g0 + gl, col = pend_col0 + cl;
             if (g < G && col < ncol) {
                 u64 *dst = pend + ((size_t)g * ncol + col) * lN + (sl ^ (gl % COEF));
@@ -232,7 +235,7 @@ __global__ void __launch_bounds__(COEF * 64 / NW, 8 / COEF) mac_mma_kernel(DevTa
 #pragma unroll
                 for (uint32_t b = 0; b < 7; b++) mma_u8(dsum[n][a + b], A[a], Bf[b]);
                 // the next-but-one step's loads go out a few at a time between the products
-                constexpr uint32_t SLOTS = 7 * NW, NCP = 2 * NIT;
+                constexpr uint32_t SLOTS = 7 * NW, NCP = NIT + NIX;
                 const uint32_t sl = n * 7 + a;
 #pragma unroll
                 for (uint32_t k = 0; k < NCP; k++)
@@ -260,7 +263,7 @@ __global__ void __launch_bounds__(COEF * 64 / NW, 8 / COEF) mac_mma_kernel(DevTa
                     }
                     const u64 lo = e[0] + (e[1] << 32);
                     const u64 hi = (e[1] >> 32) + e[2] + ((u64)(uint32_t)dsum[n][12][r] << 32) + (lo < e[0]);
-                    obuf[(gl * 16 + cl) * COEF + (coef ^ (gl % COEF))] = barrett112(hi, lo, q, mu);
+                    obuf[(gl * MS + cl) * COEF + (coef ^ (gl % COEF))] = barrett112(hi, lo, q, mu);
                 }
             pend_g0 = ct.zg * MG;
             pend_col0 = ct.zc * MS;
@@ -313,7 +316,8 @@ __global__ void __launch_bounds__(COEF * 64 / NW, 8 / COEF) mac_mma_async_kernel
                                                                                  uint32_t ntiles, uint32_t Jx, uint32_t j0, uint32_t accumulate,
                                                                                  long long wait_limit) {
     grid_dep_sync();
-    using T = Geo<COEF>;
+    using T = Geo<COEF, 2, 3>;
+    constexpr uint32_t MS = T::MS, STAGES = T::STAGES;
     constexpr uint32_t THREADS = COEF * 64 / NW, CH = T::CH, NWARPS = THREADS / 32;
     constexpr uint32_t AH = THREADS / (CH * MK), NIT = MG / AH, XB64 = 64 / COEF;
     extern __shared__ uint8_t smem_raw[];
@@ -506,21 +510,16 @@ __global__ void __launch_bounds__(COEF * 64 / NW, 8 / COEF) mac_mma_async_kernel
     if (!alive) atomicExch(c.range_flag + 1, 1);
 }
 
-template <uint32_t COEF, uint32_t NW, bool ASYNC = false>
-bool launch_as(const ckks_ctx *c, const u64 *baby, const u64 *pts, u64 *acc, uint32_t J, uint32_t S, uint32_t G, uint32_t level, cudaStream_t s,
-               uint32_t Jx, uint32_t j0, bool accumulate) {
+struct MacArgsMma { const u64 *baby, *pts; u64 *acc; uint32_t J, S, G, level, Jx, j0, accumulate; };
+
+template <uint32_t COEF, uint32_t NC, uint32_t NSTAGES, class K, class... A>
+bool launch_as(K *kernel, uint32_t threads, uint32_t ctas_per_sm, const ckks_ctx *c, const MacArgsMma &m, cudaStream_t s, A... more) {
+    using T = Geo<COEF, NC, NSTAGES>;
     // per device, so set on every launch (a host-side table update)
-    const void *kernel = ASYNC ? (const void *)mac_mma_async_kernel<COEF, NW> : (const void *)mac_mma_kernel<COEF, NW>;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<COEF>::SMEM_BYTES) != cudaSuccess) return false;
-    const uint32_t coltiles = (2 * S + MS - 1) / MS, gt = (G + MG - 1) / MG;
-    const uint32_t ntiles = (c->N / COEF) * level * coltiles * gt;
-    const uint32_t ctas = (uint32_t)c->sms * (8 / COEF), grid = ntiles < ctas ? ntiles : ctas;
-    if (ASYNC)
-        launch(mac_mma_async_kernel<COEF, NW>, grid, COEF * 64 / NW, Geo<COEF>::SMEM_BYTES, s, c->dev, baby, pts, acc, J, S, G, level, ntiles, Jx, j0,
-               accumulate ? 1u : 0u, c->wait_cycles);
-    else
-        launch(mac_mma_kernel<COEF, NW>, grid, COEF * 64 / NW, Geo<COEF>::SMEM_BYTES, s, c->dev, baby, pts, acc, J, S, G, level, ntiles, Jx, j0,
-               accumulate ? 1u : 0u);
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::SMEM_BYTES) != cudaSuccess) return false;
+    const uint32_t coltiles = (2 * m.S + T::MS - 1) / T::MS, gt = (m.G + MG - 1) / MG;
+    const uint32_t ntiles = (c->N / COEF) * m.level * coltiles * gt, ctas = (uint32_t)c->sms * ctas_per_sm;
+    launch(kernel, std::min(ntiles, ctas), threads, T::SMEM_BYTES, s, c->dev, m.baby, m.pts, m.acc, m.J, m.S, m.G, m.level, ntiles, m.Jx, m.j0, m.accumulate, more...);
     return true;
 }
 
@@ -536,14 +535,22 @@ bool launch_mac_mma(const ckks_ctx *c, const u64 *baby, const u64 *pts, u64 *acc
     if (!mac_mma_supported(c, J)) return false;
     if (!Jx) Jx = J;
     // context option CKKS_OPT_MAC_KERNEL: CKKS_MAC_TCGEN05 (the tcgen05 / TMEM kernel of mac_umma.cu, J <= 64), CKKS_MAC_MMA
-    // (mma.sync, 8 coefficients per CTA, a warp per coefficient: the default), CKKS_MAC_MMA_ASYNC (the same without
-    // CTA-wide barriers: 7 % faster, bounded mbarrier waits), CKKS_MAC_MMA_SPLIT (two warps per coefficient, 10 % slower)
-    // or CKKS_MAC_MMA_HALF (4 coefficients per CTA, two CTAs per SM: the products overlap better, but operand rows
-    // fetched 32 bytes at a time make the loads twice as slow as the whole kernel otherwise is)
-    const int shape = c->mac_kernel;
-    if (shape == 100 && launch_mac_umma(c, baby, pts, acc, J, S, G, level, s, Jx, j0, accumulate)) return true;
-    if (shape == 83) return launch_as<8, 2, true>(c, baby, pts, acc, J, S, G, level, s, Jx, j0, accumulate);
-    if (shape == 42) return launch_as<4, 2>(c, baby, pts, acc, J, S, G, level, s, Jx, j0, accumulate);
-    if (shape == 81) return launch_as<8, 1>(c, baby, pts, acc, J, S, G, level, s, Jx, j0, accumulate);
-    return launch_as<8, 2>(c, baby, pts, acc, J, S, G, level, s, Jx, j0, accumulate);
+    // (mma.sync: the default), CKKS_MAC_MMA_ASYNC (16-column tiles without CTA-wide barriers: bounded mbarrier waits),
+    // CKKS_MAC_MMA_SPLIT (16-column tiles, two warps per coefficient) or CKKS_MAC_MMA_HALF (4 coefficients per CTA)
+    const MacArgsMma m{baby, pts, acc, J, S, G, level, Jx, j0, accumulate ? 1u : 0u};
+    switch (c->mac_kernel) {
+        case CKKS_MAC_TCGEN05:
+            if (launch_mac_umma(c, baby, pts, acc, J, S, G, level, s, Jx, j0, accumulate)) return true;
+            break;
+        case CKKS_MAC_MMA_ASYNC: return launch_as<8, 2, 3>(mac_mma_async_kernel<8, 2>, 256, 1, c, m, s, c->wait_cycles);
+        case CKKS_MAC_MMA_HALF: return launch_as<4, 2, 3>(mac_mma_kernel<4, 2, 2, 3, 2>, 128, 2, c, m, s);
+        case CKKS_MAC_MMA_SPLIT: return launch_as<8, 2, 3>(mac_mma_kernel<8, 1, 2, 3, 1>, 512, 1, c, m, s);
+    }
+    // Default: tiles of 16 columns, one CTA per SM with the whole register file, or (where that takes less) of 8 columns, two
+    // CTAs per SM.  An 8-column tile costs about 0.57 of a 16-column one (16 giants, J = 64, N = 2^16, level 24: 6 columns take
+    // 7.0 ms in a tile of 16 and 4.1 in one of 8; 32 columns 15.2 ms in two tiles of 16 and 17.2 in four of 8), so the narrow
+    // form takes the batches whose last 16-column tile would be at most half full, up to a few tiles.
+    const uint32_t narrow = (2 * S + 7) / 8, full = (2 * S + 15) / 16;
+    if (narrow * 4 < full * 7) return launch_as<8, 1, 2>(mac_mma_kernel<8, 1, 1, 2, 2>, 256, 2, c, m, s);
+    return launch_as<8, 2, 3>(mac_mma_kernel<8, 2, 2, 3, 1>, 256, 1, c, m, s);
 }

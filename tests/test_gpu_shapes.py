@@ -183,3 +183,10 @@ def test_transforms_at_the_cluster_limit(log_n, batch, limbs):
     x = inputs.uniform_residues(inputs.rng(770, log_n), P.q[:limbs], P.N, batch)
     assert np.array_equal(host(ctx.ntt(dev(x))), P.oracle.ntt(x))
     assert np.array_equal(host(ctx.intt(dev(x))), P.oracle.intt(x))
+
+
+@pytest.mark.parametrize("d,S", [(64, 4), (64, 5), (64, 9), (64, 12), (64, 17)])
+def test_multiply_accumulate_tile_widths(d, S):
+    """Shard counts at which the multiply-accumulate changes between 8- and 16-column tiles, with partly filled tiles."""
+    from tests.test_gpu_linear import _run
+    _run(10, 3, 1, 3, 2, d, d, 8, S, 32, seed=780 + S, check_slots=False)
