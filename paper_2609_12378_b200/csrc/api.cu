@@ -64,9 +64,14 @@ int make_plan(const ckks_ctx *c, const ckks_proj_desc *d, ProjPlan &p) {
     return CKKS_OK;
 }
 
-struct ProjWs { size_t baby, xin, pts, ptt, slots, enc, acc, total, tmp, ks, ksx, rs, bytes; uint32_t gg, gacc, eg; bool per_block, ib_outer; };
+struct ProjWs { size_t baby, xin, pts, ptt, slots, enc, acc, total, rot, ks, ksx, rs, bytes; uint32_t gg, gacc, eg; bool per_block, ib_outer; };
 
-constexpr uint32_t BABY_ROTS = 4;            // baby-step rotations per key-switch pass
+// Key switches side by side.  Sixteen fill the GPU at N = 2^16, level 24 (768 limbs per transform); with fewer ciphertexts the
+// passes take more rotations each.  Four rotations per baby-step pass at least: a limb's digits are fetched once for them.
+constexpr uint32_t SIDE = 16;
+inline uint32_t baby_rots(uint32_t nx, uint32_t B) { return std::max(1u, std::min(std::min(B - 1, KS_MULTI), std::max(4u, SIDE / nx))); }
+inline uint32_t eager_giants(uint32_t S) { return std::max(1u, SIDE / S); }
+inline uint32_t lazy_giants(uint32_t S) { return std::max(IP_TERMS, SIDE / S / IP_TERMS * IP_TERMS); }
 constexpr uint32_t MAC_GT = 4;               // giants per register tile of the fallback multiply-accumulate kernel
 constexpr uint32_t ENC_PTS = 128;            // plaintexts per encode call of the tensor-core path (its scratch is 13.25 MiB each)
 
@@ -94,17 +99,19 @@ ProjWs proj_layout(const ckks_ctx *c, const ProjPlan &p, uint32_t level, bool la
     w.eg = w.per_block ? std::max<uint32_t>(1, std::min<uint32_t>(w.gg, ENC_PTS / p.B)) : w.gg;
     const size_t nenc = w.per_block ? (size_t)w.eg * p.B : npt;
     const size_t knt = level + c->K, kbeta = (level + c->alpha - 1) / c->alpha;
-    // all shards' key switches run side by side; the baby steps take BABY_ROTS rotations per pass, which needs that
-    // many inner-product and conversion buffers per input ciphertext
-    const size_t ks_sz = align256(ks_bytes(c, level) * p.S * nbb + (size_t)(BABY_ROTS - 1) * p.S * nbb * (2 * knt + 2 * level) * c->N * sizeof(u64));
-    // lazy giant steps: coefficient copies and extended digits of IP_TERMS giant steps of every shard
-    const size_t ksx_sz = lazy ? align256((size_t)IP_TERMS * p.S * (level + kbeta * (level + c->K)) * c->N * sizeof(u64)) : 0;
+    // all shards' key switches run side by side; the baby steps take several rotations per pass, the eager giant steps several
+    // giants (both schedules get the eager one's share: a call of several matrices may mix them)
+    const uint32_t nx = p.S * (uint32_t)nbb, gb = eager_giants(p.S);
+    const size_t up = level + kbeta * knt, down = 2 * knt + 2 * level;
+    const size_t ks_sz = align256(std::max(nx * (up + baby_rots(nx, p.B) * down), (size_t)gb * p.S * (up + down)) * c->N * sizeof(u64));
+    // lazy giant steps: coefficient copies and extended digits of several giant steps of every shard
+    const size_t ksx_sz = lazy ? align256((size_t)lazy_giants(p.S) * p.S * up * c->N * sizeof(u64)) : 0;
     size_t off = 0;
     w.baby = off;  off += align256(ct * p.S * nbb * p.B);   // tiled: rows (shard * J + j) * 2 + component
     w.xin = off;   off += align256(ct * p.S * nbb);         // the inputs of the resident blocks side by side, plain layout
     w.acc = off;   off += align256(ct * p.S * w.gacc);
     w.total = off; off += align256(ct * p.S);
-    w.tmp = off;   off += align256(ct);
+    w.rot = off;   off += gb > 1 ? align256(ct * p.S * gb) : 0;        // rotated accumulators of a pass of eager giant steps
     w.rs = off;    off += align256(rescale_bytes(c, level, 2) * std::min(p.S, KS_MULTI));
     const size_t shared = off;
     w.ptt = off;   off += align256(pt * npt);               // encoded plaintexts of a group, tiled: rows g * J + j
@@ -763,12 +770,12 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
     if (!L.ib_outer)
         for (uint32_t x = 0; x < S * nib; x++)
             cudaMemcpyAsync(xin + (size_t)x * ctl, in[x].data, ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
-    KsWorkspace kw = ks_carve(c, level, base + L.ks, S * nbb);
-    // lazy giant steps: digits of IP_TERMS x S accumulators side by side; the running sum and the ModDown use kw's buffers
+    KsWorkspace kw = ks_carve(c, level, base + L.ks, S);
+    // lazy giant steps: digits of lazy_giants(S) x S accumulators side by side; the running sum and the ModDown use kw's buffers
     const uint32_t kbeta = (level + c->alpha - 1) / c->alpha, knt = level + c->K;
     KsWorkspace kx = kw;
     kx.dcoef = (u64 *)(base + L.ksx);
-    kx.ext = kx.dcoef + (size_t)IP_TERMS * S * level * N;
+    kx.ext = kx.dcoef + (size_t)lazy_giants(S) * S * level * N;
     auto baby_steps = [&](uint32_t ib0) {
         const u64 *xb = xin;                                           // first ciphertext of the set
         const size_t xs = ctl;                                         // from one ciphertext of the set to the next
@@ -776,17 +783,16 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
         if (L.ib_outer)
             for (uint32_t sh = 0; sh < S; sh++)
                 cudaMemcpyAsync(xin + (size_t)sh * ctl, in[sh * nib + ib0].data, ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
-        for (uint32_t comp = 0; comp < 2; comp++)
-            launch_to_tiled(c, xb + comp * ptl, xs, nx, baby, Rx, comp, 2 * B, level, s);
+        launch_to_tiled(c, xb, xs, nx, baby, Rx, 0, 2 * B, level, s);
         if (B <= 1) return;
-        ks_modup(c, Ptrs(xb + ptl, xs), level, kw, s, nx);
-        // BABY_ROTS rotations of all inputs per pass (the digits of a limb are fetched once for all of them and the launches
-        // are four times larger); the inner-product and conversion buffers follow the digits
-        KsWorkspace kb = kw;
-        kb.u = kw.ext + (size_t)nx * kbeta * knt * N;
-        kb.conv = kb.u + (size_t)BABY_ROTS * nx * 2 * knt * N;
-        for (uint32_t b = 1; b < B; b += BABY_ROTS) {
-            const uint32_t nr = std::min(BABY_ROTS, B - b);
+        // several rotations of all inputs per pass (the digits of a limb are fetched once for all of them and the launches are as
+        // many times larger); the inner-product and conversion buffers follow the digits
+        const uint32_t rots = baby_rots(nx, B);
+        KsWorkspace kb = ks_carve(c, level, base + L.ks, nx);
+        kb.conv = kb.u + (size_t)rots * nx * 2 * knt * N;
+        ks_modup(c, Ptrs(xb + ptl, xs), level, kb, s, nx);
+        for (uint32_t b = 1; b < B; b += rots) {
+            const uint32_t nr = std::min(rots, B - b);
             KsOut ko;
             ko.add = Ptrs(xb, xs); ko.out = Ptrs(baby, 0);
             ko.add_comps = 1;
@@ -821,48 +827,69 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
             }
             // the giant steps of a group of accumulators accg (giants g0 .. g0 + ng - 1, all shards)
             auto giant_steps = [&](u64 *acc, uint32_t g0, uint32_t ng) {
-                for (uint32_t gl = 0; gl < ng && !lazy; gl++) {
-                    const uint32_t gi = g0 + gl;
-                    u64 *ag = acc + (size_t)gl * S * ctl;
-                    if (gi == 0) {
-                        cudaMemcpyAsync(total, ag, (size_t)S * ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
-                        continue;
+                // eager: total = acc_0 + sum_g rotate(acc_g), several giants of all shards in one batch
+                const uint32_t gb = eager_giants(S);
+                for (uint32_t gl = 0; gl < ng && !lazy;) {
+                    const u64 *first = total;
+                    if (g0 + gl == 0) { first = acc; gl++; }
+                    const uint32_t nr = std::min(gb, ng - gl);
+                    if (first != total && (!nr || gb == 1)) cudaMemcpyAsync(total, first, (size_t)S * ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
+                    if (!nr) break;
+                    const u64 *ag = acc + (size_t)gl * S * ctl;
+                    auto key = [&](uint32_t r) { return find_key(keys, nkeys, ckks_galois_element(c, (int64_t)(g0 + gl + r) * B * T)); };
+                    if (gb == 1) {
+                        const Ptrs tot(total, ctl);
+                        rotate_ks(c, key(0), Ptrs(ag, ctl), tot, level, kw, s, S, &tot);
+                    } else {
+                        u64 *rot = (u64 *)(base + L.rot);
+                        KsWorkspace kg = ks_carve(c, level, base + L.ks, nr * S);
+                        KsMulti m{};
+                        m.group = S; m.own = 1; m.rot_stride = (size_t)S * ctl;
+                        for (uint32_t r = 0; r < nr; r++) { m.galois[r] = key(r)->galois; m.evk[r] = (const u64 *)key(r)->data; }
+                        KsOut ko;
+                        ko.add = Ptrs(ag, ctl); ko.out = Ptrs(rot, ctl);
+                        ko.add_comps = 1;
+                        ks_modup(c, Ptrs(ag + ptl, ctl), level, kg, s, nr * S);
+                        ks_inner(c, nullptr, level, 1, kg, s, nr * S, false, &m);
+                        ks_moddown(c, level, kg, ko, s, nr * S, &m);
+                        launch_sum(c, total, first, rot, nr, S, level, s);
                     }
-                    const u64 ge = ckks_galois_element(c, (int64_t)gi * B * T);
-                    // total[sh] += rotate(acc_g[sh]) for all shards in one batch
-                    const Ptrs tot(total, ctl);
-                    rotate_ks(c, find_key(keys, nkeys, ge), Ptrs(ag, ctl), tot, level, kw, s, S, &tot);
+                    gl += nr;
                 }
-                // lazy: the key-switched parts of up to IP_TERMS giant steps (all shards) are extended in one batch and
-                // added to the running sum in the key-switching basis in one pass, their first components with them
+                // lazy: the key-switched parts of several giant steps (all shards) are extended in one batch and added to the
+                // running sum in the key-switching basis, IP_TERMS of them in one pass, their first components with them
                 for (uint32_t gl = 0; gl < ng && lazy;) {
                     if (g0 + gl == 0) {
                         cudaMemcpyAsync(total, acc, (size_t)S * ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
                         gl++;
                         continue;
                     }
-                    const uint32_t nterm = std::min(IP_TERMS, ng - gl);
+                    const uint32_t nup = std::min(lazy_giants(S), ng - gl);
                     u64 *ag = acc + (size_t)gl * S * ctl;
-                    ks_modup(c, Ptrs(ag + ptl, ctl), level, kx, s, nterm * S);
-                    IpTerms tm{};
-                    for (uint32_t t = 0; t < nterm; t++) {
-                        const u64 ge = ckks_galois_element(c, (int64_t)(g0 + gl + t) * B * T);
-                        tm.evk[t] = (const u64 *)find_key(keys, nkeys, ge)->data;
-                        tm.galois[t] = ge;
-                        tm.c0[t] = ag + (size_t)t * S * ctl;
+                    ks_modup(c, Ptrs(ag + ptl, ctl), level, kx, s, nup * S);
+                    for (uint32_t t0 = 0; t0 < nup; t0 += IP_TERMS) {
+                        const uint32_t nterm = std::min(IP_TERMS, nup - t0);
+                        IpTerms tm{};
+                        for (uint32_t t = 0; t < nterm; t++) {
+                            const u64 ge = ckks_galois_element(c, (int64_t)(g0 + gl + t0 + t) * B * T);
+                            tm.evk[t] = (const u64 *)find_key(keys, nkeys, ge)->data;
+                            tm.galois[t] = ge;
+                            tm.c0[t] = ag + (size_t)(t0 + t) * S * ctl;
+                        }
+                        KsWorkspace kt = kx;
+                        kt.ext = kx.ext + (size_t)t0 * S * kbeta * knt * N;
+                        kt.d.base += (size_t)t0 * S * ctl;
+                        ks_inner_terms(c, level, kt, (size_t)S * kbeta * knt * N, tm, nterm, ctl, s, S, u_live);
+                        u_live = true;
                     }
-                    ks_inner_terms(c, level, kx, (size_t)S * kbeta * knt * N, tm, nterm, ctl, s, S, u_live);
-                    u_live = true;
-                    gl += nterm;
+                    gl += nup;
                 }
             };
             // the diagonals of giants g0 .. g0 + ngi - 1 of a block pair, encoded into rows 0 .. ngi B - 1 of the tiled buffer
             auto encode_group = [&](const Block &i, uint32_t g0, uint32_t ngi) {
                 for (uint32_t e0 = 0; e0 < ngi; e0 += L.eg) {
                     const uint32_t ne = std::min(L.eg, ngi - e0);
-                    for (uint32_t gl = 0; gl < ne; gl++)
-                        launch_extract_diagonals(c, W, d->d_out, i.start, i.size, o.start, o.size, p.F, T, (g0 + e0 + gl) * B, B,
-                                                 (g0 + e0 + gl) * B, slots + (size_t)gl * B * c->n, s);
+                    launch_extract_diagonals(c, W, d->d_out, i.start, i.size, o.start, o.size, p.F, T, (g0 + e0) * B, ne * B, B, slots, s);
                     TiledOut to;
                     to.R = ngi * B; to.row0 = e0 * B; to.row_stride = 1;
                     launch_encode(c, slots, nullptr, ne * B, pt_scale, level, pts, encw, s, to, ptt);
@@ -911,14 +938,17 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
                     for (uint32_t ib = 0; ib < nib; ib++)
                         if (g0 + gl >= std::min(p.ins[ib].size, o.size) / B) ragged = true;
                 if (ragged) cudaMemsetAsync(ptt, 0, (size_t)ng * J * ptl * sizeof(u64), s);
+                if (nib == 1 && !ragged) {
+                    const Block &i = p.ins[0];
+                    launch_extract_diagonals(c, W, d->d_out, i.start, i.size, o.start, o.size, p.F, T, g0 * B, ng * B, B, slots, s);
+                } else
                 for (uint32_t gl = 0; gl < ng; gl++)
                     for (uint32_t ib = 0; ib < nib; ib++) {
                         const Block &i = p.ins[ib];
                         const uint32_t gi = g0 + gl;
                         if (gi >= std::min(i.size, o.size) / B) continue;
                         const size_t idx = ((size_t)gl * nib + ib) * B;
-                        launch_extract_diagonals(c, W, d->d_out, i.start, i.size, o.start, o.size, p.F, T, gi * B, B, gi * B,
-                                                 slots + idx * c->n, s);
+                        launch_extract_diagonals(c, W, d->d_out, i.start, i.size, o.start, o.size, p.F, T, gi * B, B, B, slots + idx * c->n, s);
                         if (ragged) {
                             TiledOut to;
                             to.R = ng * J; to.row0 = (uint32_t)idx; to.row_stride = 1;

@@ -306,8 +306,8 @@ struct KsMulti {
     // group > 0: `group` ciphertexts with their own digits take every one of the keys; batch entry b = r * group + m is key r
     // applied to member m's digits, added to member m's addend, and written to the tiled row
     // row0 + r * rot_rows + m * row_stride + component, or (plain layout) to out + r * rot_stride + m * out_stride words
-    // (out[] is not used)
-    uint32_t group, rot_rows;
+    // (out[] is not used); own != 0: entry b has digits and an addend of its own instead of member m's
+    uint32_t group, own, rot_rows;
     size_t rot_stride;
 };
 
@@ -362,7 +362,7 @@ struct NttEpilogue {
     u64 mgalois[KS_MULTI];
     // KsMulti's grouped form: entry b = r * group + m takes mgalois[r] and add.at(m) and goes to row
     // tl.row0 + r * rot_rows + m * tl.row_stride + comp, or to out.base + r * rot_stride + m * out.stride
-    uint32_t group, rot_rows;
+    uint32_t group, own, rot_rows;
     size_t rot_stride;
     uint32_t y0;           // (filled in) first limb of the launch
 };
@@ -458,9 +458,11 @@ void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, siz
 // The basis conversions on the tensor cores (contexts with byte matrices: at most 8 sources)
 void launch_modup_mma(const ckks_ctx *c, const u64 *dcoef, u64 *ext, uint32_t level, uint32_t nb, cudaStream_t s);
 void launch_moddown_conv_mma(const ckks_ctx *c, const u64 *u, u64 *conv, uint32_t level, uint32_t nb, cudaStream_t s);
-// rows of [level][N] words, src_stride words apart, into rows row0, row0 + row_step, .. of a tiled buffer with R rows
-void launch_to_tiled(const ckks_ctx *c, const u64 *src, size_t src_stride, uint32_t nrows, u64 *dst, uint32_t R, uint32_t row0,
+// both components of n ciphertexts, src_stride words apart, into rows row0 + i * row_step + component of a tiled buffer with R rows
+void launch_to_tiled(const ckks_ctx *c, const u64 *src, size_t src_stride, uint32_t n, u64 *dst, uint32_t R, uint32_t row0,
                      uint32_t row_step, uint32_t level, cudaStream_t s);
+// dst = first + sum_{r < n} terms[r] for nct ciphertexts side by side (terms n * nct of them); first may be dst
+void launch_sum(const ckks_ctx *c, u64 *dst, const u64 *first, const u64 *terms, uint32_t n, uint32_t nct, uint32_t level, cudaStream_t s);
 
 // Tensor-core multiply-accumulate of a giant-step group (mac_mma.cu)
 bool mac_mma_supported(const ckks_ctx *c, uint32_t J);
@@ -490,10 +492,11 @@ size_t encode_workspace_bytes(const ckks_ctx *c, uint32_t batch);
 // `tiled_out`; `out` is then only the scratch between the two NTT passes.
 void launch_encode(const ckks_ctx *c, const double *re, const double *im, uint32_t batch, double scale, uint32_t level,
                    u64 *out, void *ws, cudaStream_t s, TiledOut tiled = TiledOut(), u64 *tiled_out = nullptr);
-// Slot vectors of pre-rotated generalised diagonals, [count][n] fp64, for k = k0 .. k0+count-1 of one block pair.
+// Slot vectors of generalised diagonals, [count][n] fp64, for k = k0 .. k0+count-1 of one block pair, diagonal k pre-rotated by its
+// giant step's share k - k % B.
 void launch_extract_diagonals(const ckks_ctx *c, const double *W, uint32_t d_out_total, uint32_t in0, uint32_t m_in,
                               uint32_t out0, uint32_t m_out, uint32_t F, uint32_t T, uint32_t k0, uint32_t count,
-                              uint32_t pre_rot, double *slots, cudaStream_t s);
+                              uint32_t B, double *slots, cudaStream_t s);
 
 // ---- sequences shared by the entry points (api.cu, poly.cu, attention.cu) -------------------------------------------
 void relinearise(const ckks_ctx *c, const u64 *rlk, const Ptrs &e2, const Ptrs &o, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb = 1);

@@ -113,16 +113,16 @@ __global__ void __launch_bounds__(THREADS) fft_strips_round(DevTables c, const d
     }
 }
 
-// slots[kk][r*T + t] = d'_k[r],  k = k0 + kk,  d'_k[r] = d_k[(r - pre_rot) mod F],
+// slots[kk][r*T + t] = d'_k[r],  k = k0 + kk,  d'_k[r] = d_k[(r - (k - k mod B)) mod F],
 // d_k[r'] = W^T[out0 + r' mod m_out, in0 + (r' + k) mod m_in]
 __global__ void __launch_bounds__(THREADS) extract_diagonals(const double *W, uint32_t d_out_total, uint32_t in0, uint32_t m_in,
                                                              uint32_t out0, uint32_t m_out, uint32_t F, uint32_t T, uint32_t k0,
-                                                             uint32_t pre_rot, double *slots, uint32_t n) {
+                                                             uint32_t B, double *slots, uint32_t n) {
     const uint32_t x = blockIdx.x * THREADS + threadIdx.x;
     grid_dep_sync();
     if (x >= n) return;
     const uint32_t r = x / T, k = k0 + blockIdx.y;
-    const uint32_t rp = (r + F - pre_rot % F) % F;
+    const uint32_t rp = (r + F - (k - k % B) % F) % F;
     const uint32_t ro = rp % m_out, ci = (rp + k) % m_in;
     slots[(size_t)blockIdx.y * n + x] = W[(size_t)(in0 + ci) * d_out_total + out0 + ro];
 }
@@ -153,6 +153,6 @@ void launch_encode(const ckks_ctx *c, const double *re, const double *im, uint32
 
 void launch_extract_diagonals(const ckks_ctx *c, const double *W, uint32_t d_out_total, uint32_t in0, uint32_t m_in,
                               uint32_t out0, uint32_t m_out, uint32_t F, uint32_t T, uint32_t k0, uint32_t count,
-                              uint32_t pre_rot, double *slots, cudaStream_t s) {
-    launch(extract_diagonals, dim3((c->n + THREADS - 1) / THREADS, count), THREADS, 0, s, W, d_out_total, in0, m_in, out0, m_out, F, T, k0, pre_rot, slots, c->n);
+                              uint32_t B, double *slots, cudaStream_t s) {
+    launch(extract_diagonals, dim3((c->n + THREADS - 1) / THREADS, count), THREADS, 0, s, W, d_out_total, in0, m_in, out0, m_out, F, T, k0, B, slots, c->n);
 }

@@ -173,11 +173,11 @@ __global__ void __launch_bounds__(THREADS) inner_product_generic_kernel(DevTable
     u[((size_t)1 * nt + x) * c.N + p] = r1;
 }
 
-// The same for BETA <= 4 digits, two adjacent coefficients per thread.  pi_g maps the pair (p, p + 1), p even, onto a
+// The same for BETA <= 8 digits, two adjacent coefficients per thread.  pi_g maps the pair (p, p + 1), p even, onto a
 // pair (s, s ^ 1), so digits and key words both move as 16-byte loads.  Without `multi` a thread walks `bch` batch
 // entries (blockIdx.y picks the chunk) with the key words of its pair held in registers; with it, an entry is one
 // of up to KS_MULTI keys applied to the same digits.
-constexpr uint32_t IP_MAX_BETA = 4;
+constexpr uint32_t IP_MAX_BETA = 8, IP_TERMS_MAX_BETA = 4;
 template <uint32_t BETA>
 __global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, const u64 *ext, const __grid_constant__ Ptrs d, const u64 *evk, u64 g, u64 *u,
                                                                 uint32_t level, uint32_t nb, uint32_t bch, int has_multi, const __grid_constant__ KsMulti multi,
@@ -193,6 +193,7 @@ __global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, con
         const uint32_t cpr = (multi.group + bch - 1) / bch, r = blockIdx.y / cpr, ch = blockIdx.y % cpr;
         e0 = ch * bch;
         b0 = r * multi.group + e0;
+        if (multi.own) e0 = b0;
         b1 = min(b0 + bch, (r + 1) * multi.group);
         evk = multi.evk[r]; g = multi.galois[r];
     } else if (has_multi) { evk = multi.evk[b0]; g = multi.galois[b0]; }
@@ -398,13 +399,27 @@ void launch_moddown_conv(const ckks_ctx *c, const u64 *u, u64 *conv, uint32_t le
         else { CALL(64); }                          \
     } while (0)
 
-// dst row (row0 + r * row_step) of a tiled buffer <- src + r * src_stride ([level][N] words)
+// dst row (row0 + i * row_step + comp) of a tiled buffer <- component comp of ciphertext i, blockIdx.z = 2 i + comp
 __global__ void __launch_bounds__(THREADS) to_tiled_kernel(DevTables c, const u64 *src, size_t src_stride, u64 *dst, uint32_t R,
                                                            uint32_t row0, uint32_t row_step) {
     grid_dep_sync();
-    const uint32_t p = (blockIdx.x * THREADS + threadIdx.x) * 2, i = blockIdx.y, r = blockIdx.z;
-    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(src + r * src_stride + (size_t)i * c.N + p);
-    *reinterpret_cast<ulonglong2 *>(dst + tiled_index(R, c.N, row0 + r * row_step, i, p)) = v;
+    const uint32_t p = (blockIdx.x * THREADS + threadIdx.x) * 2, i = blockIdx.y, r = blockIdx.z >> 1, comp = blockIdx.z & 1;
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(src + r * src_stride + ((size_t)comp * gridDim.y + i) * c.N + p);
+    *reinterpret_cast<ulonglong2 *>(dst + tiled_index(R, c.N, row0 + r * row_step + comp, i, p)) = v;
+}
+
+// dst[x] = first[x] + sum_r terms[r][x] over [nct][2][level][N] words (grid y: limbs of all ciphertexts)
+__global__ void __launch_bounds__(THREADS) sum_kernel(DevTables c, u64 *dst, const u64 *first, const u64 *terms, uint32_t n, size_t stride, uint32_t level) {
+    const size_t off = (size_t)blockIdx.y * c.N + (blockIdx.x * THREADS + threadIdx.x) * 2;
+    const u64 q = c.mod[blockIdx.y % level];
+    grid_dep_sync();
+    ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(first + off);
+    for (uint32_t r = 0; r < n; r++) {
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(terms + r * stride + off);
+        a.x = add_mod(a.x, b.x, q);
+        a.y = add_mod(a.y, b.y, q);
+    }
+    *reinterpret_cast<ulonglong2 *>(dst + off) = a;
 }
 
 // u[b][0][i][p] += P sigma_g(c0[b][i])[p]   (first component's q-limbs of the extended-basis sum)
@@ -470,6 +485,10 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
         for (uint32_t r = 0; r < nkeys; r++) {
             KsWorkspace wr = w;
             wr.u = w.u + (size_t)r * multi->group * 2 * nt * N;
+            if (multi->own) {
+                wr.ext = w.ext + (size_t)r * multi->group * beta * nt * N;
+                wr.d.base += r * multi->group * w.d.stride;
+            }
             ks_inner(c, multi->evk[r], level, multi->galois[r], wr, s, multi->group, acc_u, nullptr);
         }
         return;
@@ -480,7 +499,9 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
         const uint32_t grp = multi ? multi->group : 0, per = grp ? grp : nb;
         const uint32_t bch = (multi && !grp) ? 1 : (per >= 8 ? 4 : (per >= 4 ? 2 : 1));
         const dim3 grid(N / (2 * THREADS), grp ? (nb / grp) * ((grp + bch - 1) / bch) : (nb + bch - 1) / bch, nt);
-        auto *k = beta == 1 ? inner_product_kernel<1> : beta == 2 ? inner_product_kernel<2> : beta == 3 ? inner_product_kernel<3> : inner_product_kernel<4>;
+        static constexpr decltype(&inner_product_kernel<1>) kernels[IP_MAX_BETA] = {inner_product_kernel<1>, inner_product_kernel<2>, inner_product_kernel<3>, inner_product_kernel<4>,
+                                                                                   inner_product_kernel<5>, inner_product_kernel<6>, inner_product_kernel<7>, inner_product_kernel<8>};
+        auto *k = kernels[beta - 1];
         launch(k, grid, THREADS, 0, s, c->dev, w.ext, w.d, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au);
     } else {
         launch(inner_product_generic_kernel, dim3(N / THREADS, nb, nt), THREADS, 0, s, c->dev, w.ext, w.d, 0u, evk, ext_galois, w.u, level, multi ? 1 : 0, m, au);
@@ -507,7 +528,7 @@ void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const K
     ep.ncomp = 2; ep.level = level; ep.nt = nt;
     ep.galois = o.galois; ep.acc = o.acc; ep.accumulate = o.acc.n || o.acc.base ? 1 : 0; ep.tl = o.tiled;
     if (multi) {
-        ep.multi = 1; ep.group = multi->group; ep.rot_rows = multi->rot_rows; ep.rot_stride = multi->rot_stride;
+        ep.multi = 1; ep.group = multi->group; ep.own = multi->own; ep.rot_rows = multi->rot_rows; ep.rot_stride = multi->rot_stride;
         for (uint32_t b = 0; b < KS_MULTI; b++) { ep.mgalois[b] = multi->galois[b]; ep.out.p[b] = multi->out[b]; }
         if (!multi->group) ep.out.n = nb;
     }
@@ -519,7 +540,7 @@ void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, siz
     const uint32_t N = c->N, nt = level + c->K, beta = (level + c->alpha - 1) / c->alpha;
     bool aligned = aligned16(w.ext) && aligned16(w.u) && (term_stride & 1) == 0 && (c0_stride & 1) == 0 && aligned16(w.d);
     for (uint32_t t = 0; t < nterm; t++) aligned = aligned && aligned16(terms.evk[t]) && aligned16(terms.c0[t]);
-    if (beta <= IP_MAX_BETA && aligned) {
+    if (beta <= IP_TERMS_MAX_BETA && aligned) {
         const dim3 grid(N / (2 * THREADS), (nb + IP_BCH - 1) / IP_BCH, nt);
         auto *k = beta == 1 ? inner_product_terms_kernel<1> : beta == 2 ? inner_product_terms_kernel<2> : beta == 3 ? inner_product_terms_kernel<3> : inner_product_terms_kernel<4>;
         launch(k, grid, THREADS, 0, s, c->dev, w.ext, term_stride, w.d.base, w.d.stride, terms, nterm, c0_stride, w.u, level, nb, acc_u ? 1 : 0);
@@ -534,12 +555,20 @@ void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, siz
     }
 }
 
-void launch_to_tiled(const ckks_ctx *c, const u64 *src, size_t src_stride, uint32_t nrows, u64 *dst, uint32_t R, uint32_t row0,
+void launch_to_tiled(const ckks_ctx *c, const u64 *src, size_t src_stride, uint32_t n, u64 *dst, uint32_t R, uint32_t row0,
                      uint32_t row_step, uint32_t level, cudaStream_t s) {
-    for (uint32_t r0 = 0; r0 < nrows; r0 += 32768) {
-        const uint32_t nr = nrows - r0 < 32768 ? nrows - r0 : 32768;
-        launch(to_tiled_kernel, dim3(c->N / (2 * THREADS), level, nr), THREADS, 0, s, c->dev, src + r0 * src_stride, src_stride, dst, R,
+    for (uint32_t r0 = 0; r0 < n; r0 += 16384) {
+        const uint32_t nr = std::min(16384u, n - r0);
+        launch(to_tiled_kernel, dim3(c->N / (2 * THREADS), level, 2 * nr), THREADS, 0, s, c->dev, src + r0 * src_stride, src_stride, dst, R,
                row0 + r0 * row_step, row_step);
+    }
+}
+
+void launch_sum(const ckks_ctx *c, u64 *dst, const u64 *first, const u64 *terms, uint32_t n, uint32_t nct, uint32_t level, cudaStream_t s) {
+    const size_t ct = (size_t)2 * level * c->N;
+    for (uint32_t i0 = 0; i0 < nct; i0 += 256) {        // grid y holds 2 level (at most 128) limbs per ciphertext
+        const uint32_t m = std::min(256u, nct - i0);
+        launch(sum_kernel, dim3(c->N / (2 * THREADS), m * 2 * level), THREADS, 0, s, c->dev, dst + i0 * ct, first + i0 * ct, terms + i0 * ct, n, nct * ct, level);
     }
 }
 

@@ -384,11 +384,11 @@ __global__ void __launch_bounds__(16 * ROW_CTA, 4) ntt_fwd_rows(DevTables c, u64
         const uint32_t y = blockIdx.y + ep.y0, i = y % ep.level, comp = (y / ep.level) % ep.ncomp, bz = y / (ep.ncomp * ep.level);
         const double2 pinv = ep.pinv[i];
         const uint32_t p0 = row * 256 + 2 * t;
-        // grouped: entry bz is key bz / group applied to member bz % group
+        // grouped: entry bz is key bz / group applied to member bz % group (own: to the entry itself)
         const uint32_t rot = ep.group ? bz / ep.group : bz, mem = ep.group ? bz % ep.group : bz;
         const uint32_t gal = (uint32_t)(ep.multi ? ep.mgalois[rot] : ep.galois);
         const u64 *up = ep.u.at(bz) + (((size_t)comp * ep.nt + i) << c.log_n) + p0;
-        const u64 *add = (ep.add_comps >> comp & 1) ? ep.add.at(mem) + (((size_t)comp * ep.level + i) << c.log_n) : nullptr;
+        const u64 *add = (ep.add_comps >> comp & 1) ? ep.add.at(ep.own ? bz : mem) + (((size_t)comp * ep.level + i) << c.log_n) : nullptr;
         const u64 *acc = ep.accumulate ? ep.acc.at(bz) + (((size_t)comp * ep.level + i) << c.log_n) + p0 : nullptr;
         const uint32_t bstep = ep.tl.R ? ep.tl.R * 64 : 64;    // words from one 64-word block of the destination to the next
         u64 *dst = ep.tl.R ? const_cast<u64 *>(ep.out.base) + tiled_index(ep.tl.R, c.N, ep.tl.row0 + rot * ep.rot_rows + (ep.group ? mem : bz) * ep.tl.row_stride + comp, i, row * 256) + 2 * t

@@ -190,3 +190,18 @@ def test_multiply_accumulate_tile_widths(d, S):
     """Shard counts at which the multiply-accumulate changes between 8- and 16-column tiles, with partly filled tiles."""
     from tests.test_gpu_linear import _run
     _run(10, 3, 1, 3, 2, d, d, 8, S, 32, seed=780 + S, check_slots=False)
+
+
+@pytest.mark.parametrize("lazy", [False, True])
+@pytest.mark.parametrize("dnum,d_in,d_out,S,B", [
+    (6, 128, 128, 1, 8),      # sixteen eager giants (fifteen rotations) in one pass, seven baby rotations in one
+    (6, 64, 32, 3, 4),        # five giants per pass: a partial last pass; folded
+    (3, 128, 128, 5, 4),      # lazy: two passes of the sum over four giants each
+    (6, 64, 64, 17, 8),       # one giant per pass
+    (8, 24, 16, 2, 4),        # eight digits; two input blocks
+    (9, 16, 16, 2, 4),        # nine digits: one key at a time
+])
+def test_projection_passes_by_shard_count(dnum, d_in, d_out, S, B, lazy):
+    """How many rotations share a pass depends on the number of shards and digits."""
+    from tests.test_gpu_linear import _run
+    _run(10, 9, -(-9 // dnum), dnum, 9, d_in, d_out, 4 if d_in > 24 else 32, S, B, seed=760 + S, check_slots=False, lazy=lazy)
