@@ -20,8 +20,18 @@
 namespace {
 
 // ML consecutive twiddles w (ML = 1, 2, 4, 8; the index is a multiple of ML) with the widest loads that fit.
-template <uint32_t ML>
+// SH: from a copy in shared memory.
+template <uint32_t ML, bool SH = false>
 __device__ __forceinline__ void load_tw(const double *p, double (&v)[ML]) {
+    if (SH) {
+        if (ML == 1) v[0] = *p;
+#pragma unroll
+        for (uint32_t i = 0; i + 1 < ML; i += 2) {
+            const double2 w = *reinterpret_cast<const double2 *>(p + i);
+            v[i] = w.x; v[(i + 1) % ML] = w.y;
+        }
+        return;
+    }
     if (ML == 1) v[0] = __ldg(p);
     if (ML == 2) asm volatile("ld.global.nc.v2.f64 {%0,%1}, [%2];" : "=d"(v[0]), "=d"(v[ML > 1 ? 1 : 0]) : "l"(p));
     if (ML >= 4) {
@@ -49,11 +59,11 @@ __host__ __device__ constexpr bool col_coarse(uint32_t s) { return s >= 5 && s <
 __host__ __device__ constexpr bool col_reduce(uint32_t logr, uint32_t s) { return logr >= 4 && s == (logr < 7 ? logr : 7); }
 
 // one Cooley-Tukey stage on 2 ML tl registers starting at x: blocks of 2 tl, twiddles tw[ML * base + i]
-template <uint32_t ML, uint32_t RADIX, bool COARSE, bool REDUCE_U, uint32_t E>
+template <uint32_t ML, uint32_t RADIX, bool COARSE, bool REDUCE_U, bool SH = false, uint32_t E>
 __device__ __forceinline__ void fwd_stage(double (&x)[E], uint32_t x0, const double *__restrict__ tw, uint32_t base, double q, double qinv) {
     constexpr uint32_t tl = RADIX / 2 / ML;
     double w[ML];
-    load_tw<ML>(tw + ML * base, w);
+    load_tw<ML, SH>(tw + ML * base, w);
 #pragma unroll
     for (uint32_t i = 0; i < ML; i++)
 #pragma unroll
@@ -66,13 +76,13 @@ __device__ __forceinline__ void fwd_stage(double (&x)[E], uint32_t x0, const dou
         }
 }
 // stages S0 + 1 .. S0 + G of the column pass on one sub-transform of 2^G registers
-template <uint32_t LOGR, uint32_t S0, uint32_t G, uint32_t E>
+template <uint32_t LOGR, uint32_t S0, uint32_t G, bool SH = false, uint32_t E>
 __device__ __forceinline__ void fwd_col_group(double (&x)[E], uint32_t x0, const double *__restrict__ tw, uint32_t base, double q, double qinv) {
     constexpr uint32_t RX = 1u << G;
-    fwd_stage<1, RX, col_coarse(S0 + 1), col_reduce(LOGR, S0 + 1)>(x, x0, tw, base, q, qinv);
-    if constexpr (G >= 2) fwd_stage<2, RX, col_coarse(S0 + 2), col_reduce(LOGR, S0 + 2)>(x, x0, tw, base, q, qinv);
-    if constexpr (G >= 3) fwd_stage<4, RX, col_coarse(S0 + 3), col_reduce(LOGR, S0 + 3)>(x, x0, tw, base, q, qinv);
-    if constexpr (G >= 4) fwd_stage<8, RX, col_coarse(S0 + 4), col_reduce(LOGR, S0 + 4)>(x, x0, tw, base, q, qinv);
+    fwd_stage<1, RX, col_coarse(S0 + 1), col_reduce(LOGR, S0 + 1), SH>(x, x0, tw, base, q, qinv);
+    if constexpr (G >= 2) fwd_stage<2, RX, col_coarse(S0 + 2), col_reduce(LOGR, S0 + 2), SH>(x, x0, tw, base, q, qinv);
+    if constexpr (G >= 3) fwd_stage<4, RX, col_coarse(S0 + 3), col_reduce(LOGR, S0 + 3), SH>(x, x0, tw, base, q, qinv);
+    if constexpr (G >= 4) fwd_stage<8, RX, col_coarse(S0 + 4), col_reduce(LOGR, S0 + 4), SH>(x, x0, tw, base, q, qinv);
 }
 // row pass, first four stages: 3.20 q in, 4.10 5.61c 7.31c | u reduced 2.42c out
 __device__ __forceinline__ void fwd_row_open(double (&x)[16], const double *__restrict__ tw, uint32_t base, double q, double qinv) {
@@ -143,11 +153,11 @@ __device__ __forceinline__ void reduce_masked(double (&x)[E], uint32_t x0, doubl
         if (MASK >> k & 1) x[x0 + k] = reduce_d(x[x0 + k], q, qinv);
 }
 // stage s (distance 2^s) of a group of G stages
-template <uint32_t S, uint32_t G, uint32_t PRE, uint32_t COARSE, uint32_t E>
+template <uint32_t S, uint32_t G, uint32_t PRE, uint32_t COARSE, bool SH, uint32_t E>
 __device__ __forceinline__ void inv_stage(double (&x)[E], uint32_t x0, const double *__restrict__ tw, uint32_t base, double q, double qinv) {
     constexpr uint32_t tl = 1u << S, ML = (1u << G) / 2 / tl;
     double w[ML];
-    load_tw<ML>(tw + ML * base, w);
+    load_tw<ML, SH>(tw + ML * base, w);
     reduce_masked<PRE, (1u << G)>(x, x0, q, qinv);
 #pragma unroll
     for (uint32_t i = 0; i < ML; i++)
@@ -160,10 +170,11 @@ __device__ __forceinline__ void inv_stage(double (&x)[E], uint32_t x0, const dou
         }
 }
 // the first NST of a group of G stages, entry bound IN(group) of the plan (G, in, thr, LAST)
-#define INV_STAGE(S, G, IN, THR, LAST) inv_stage<S, G, gs_pre(G, IN, THR, LAST, S), gs_coarse(G, IN, THR, LAST, S)>(x, x0, tw, base, q, qinv)
+#define INV_STAGE(S, G, IN, THR, LAST) inv_stage<S, G, gs_pre(G, IN, THR, LAST, S), gs_coarse(G, IN, THR, LAST, S), SH>(x, x0, tw, base, q, qinv)
 template <int GROUP>        // 1, 2: the row pass
 __device__ __forceinline__ void inv_row_group(double (&x)[16], const double *__restrict__ tw, uint32_t base, double q, double qinv) {
     constexpr uint32_t x0 = 0;
+    constexpr bool SH = false;
     constexpr double in = inv_in(GROUP), thr = GROUP == 1 ? 1.75 : 2.01;
     INV_STAGE(0, 4, in, thr, false);
     INV_STAGE(1, 4, in, thr, false);
@@ -171,7 +182,7 @@ __device__ __forceinline__ void inv_row_group(double (&x)[16], const double *__r
     INV_STAGE(3, 4, in, thr, false);
     reduce_masked<gs_post(4, in, thr, false), 16>(x, 0, q, qinv);
 }
-template <uint32_t G, uint32_t E>       // the column pass's first group (of two)
+template <uint32_t G, bool SH = false, uint32_t E>       // the column pass's first group (of two)
 __device__ __forceinline__ void inv_col_open(double (&x)[E], uint32_t x0, const double *__restrict__ tw, uint32_t base, double q, double qinv) {
     constexpr double in = inv_in(3), thr = 1.01;
     INV_STAGE(0, G, in, thr, false);
@@ -183,7 +194,7 @@ __device__ __forceinline__ void inv_col_open(double (&x)[E], uint32_t x0, const 
 // The last group (twiddle base 1); the last stage has N^-1 (or the caller's constant) folded in: x1 = (u + v) c0,
 // x2 = (u - v) c1, both products of values below 4 q rounded to nearest, so the results are below q and one conditional
 // addition makes them canonical.  c0 = {N^-1, N^-1/q}, c1 = {w_1 N^-1, that / q}, centred.
-template <uint32_t G, uint32_t B, uint32_t E>     // B: stages of the open group before it (0: none)
+template <uint32_t G, uint32_t B, bool SH = false, uint32_t E>     // B: stages of the open group before it (0: none)
 __device__ __forceinline__ void inv_col_last(double (&x)[E], const double *__restrict__ tw, double q, double qinv, double2 c0, double2 c1) {
     constexpr uint32_t x0 = 0, base = 1;
     constexpr double in = B ? gs_out(B, inv_in(3), 1.01) : inv_in(3);
@@ -223,6 +234,17 @@ __global__ void __launch_bounds__(F_THREADS, 3) butterfly_probe_kernel(DevTables
     if (acc == 0.5) sink[blockIdx.x * F_THREADS + threadIdx.x] = 1;      // never true for integer-valued sums
 }
 
+// The column pass of a limb uses entries 1 .. R - 1 of its twiddle table (2 KiB at N = 2^16).  At that size a CTA fetches them
+// once into shared memory: stage by stage from global memory they cost every stage a trip to L2, because the streamed data
+// leaves them nothing of L1 (768 limbs: forward 150 -> 141 us, inverse 161 -> 156).  Smaller rings' few CTAs are bound by latency
+// and keep the direct loads (the barrier costs them 0.2 us), and so do the row passes, where a CTA's entries are its own
+// (forward 155 -> 157, inverse 147 -> 171 us with its first-group entries in shared memory).
+template <uint32_t LOGR> constexpr bool TW_SHARED = LOGR == 8;
+template <uint32_t R>
+__device__ __forceinline__ void stage_tw(double *dst, const double *tw) {
+    for (uint32_t e = threadIdx.x; e < R; e += blockDim.x) dst[e] = tw[e];
+}
+
 // ---- column passes -------------------------------------------------------------------------------------------------
 // Shape per LOGR: the R-point column transform is split into a first group of A stages (registers R/2^A rows apart) and a
 // second of B stages (2^B consecutive rows; a thread holds 2^(A-B) of these), E = 2^A registers per thread, COLS columns per
@@ -245,6 +267,8 @@ __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 1024 / ColShape<LOGR>
                                                                                                     const u64 *src, uint32_t src_prime) {
     using S = ColShape<LOGR>;
     __shared__ double sm[S::B ? S::R * S::COLS : 1];
+    constexpr bool SH = TW_SHARED<LOGR>;
+    __shared__ __align__(16) double stw[SH ? S::R : 2];
     const int prime = limb_prime(map, blockIdx.y);
     if (prime < 0 || (blockIdx.y & 7) >= fp_share) return;
     const double q = c.modd[prime].x, qinv = c.modd[prime].y;
@@ -254,6 +278,8 @@ __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 1024 / ColShape<LOGR>
     const u64 *gs = SRC == SRC_LIMBS ? g : src + ((size_t)(blockIdx.y / map.period) << c.log_n) + blockIdx.x * S::COLS + cc;
     constexpr uint32_t RS = S::R / S::E;          // rows between a thread's registers in the first group
     double x[S::E];
+    if (SH) stage_tw<S::R>(stw, tw);
+    const double *tws = SH ? stw : tw;
     grid_dep_sync();
     if (SRC == SRC_COEFS) {
         // coefficients below 2^49 (every weight of ordinary size at the scale of a prime) are residues as they are, signed;
@@ -285,8 +311,9 @@ __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 1024 / ColShape<LOGR>
 #pragma unroll
         for (uint32_t k = 0; k < S::E; k++) x[k] = u64_to_d(gs[(size_t)(r + RS * k) * 256]);
     }
-    __syncwarp();       // keeps all loads in front of the butterflies: interleaved with them they were 10 % slower
-    fwd_col_group<LOGR, 0, S::A>(x, 0, tw, 1, q, qinv);
+    if (SH) __syncthreads();
+    else __syncwarp();  // keeps all loads in front of the butterflies: interleaved with them they were 10 % slower
+    fwd_col_group<LOGR, 0, S::A, SH>(x, 0, tws, 1, q, qinv);
     if constexpr (S::B > 0) {
 #pragma unroll
         for (uint32_t k = 0; k < S::E; k++) sm[(r + RS * k) * S::COLS + cc] = x[k];
@@ -295,7 +322,7 @@ __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 1024 / ColShape<LOGR>
         for (uint32_t k = 0; k < S::E; k++) x[k] = sm[(S::E * r + k) * S::COLS + cc];
 #pragma unroll
         for (uint32_t j = 0; j < (S::E >> S::B); j++)
-            fwd_col_group<LOGR, S::A, S::B>(x, j << S::B, tw, (1u << S::A) + r * (S::E >> S::B) + j, q, qinv);
+            fwd_col_group<LOGR, S::A, S::B, SH>(x, j << S::B, tws, (1u << S::A) + r * (S::E >> S::B) + j, q, qinv);
     }
     constexpr uint32_t OS = S::B ? 1 : RS;        // without a second group the registers are still RS rows apart
 #pragma unroll
@@ -308,6 +335,8 @@ __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 768 / ColShape<LOGR>:
                                                                                                    const double2 *scale) {
     using S = ColShape<LOGR>;
     __shared__ double sm[S::B ? S::R * S::COLS : 1];
+    constexpr bool SH = TW_SHARED<LOGR>;
+    __shared__ __align__(16) double stw[SH ? S::R : 2];
     const int prime = limb_prime(map, blockIdx.y);
     if (prime < 0 || (blockIdx.y & 7) >= fp_share) return;
     const double q = c.modd[prime].x, qinv = c.modd[prime].y;
@@ -318,12 +347,15 @@ __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 768 / ColShape<LOGR>:
     const double2 c0 = sc[0], c1 = sc[1];
     constexpr uint32_t RS = S::R / S::E;
     double x[S::E];
+    if (SH) stage_tw<S::R>(stw, tw);
+    const double *tws = SH ? stw : tw;
     grid_dep_sync();
     if constexpr (S::B > 0) {
 #pragma unroll
         for (uint32_t k = 0; k < S::E; k++) x[k] = reinterpret_cast<const double *>(g)[(size_t)(S::E * r + k) * 256];
+        if (SH) __syncthreads();
 #pragma unroll
-        for (uint32_t j = 0; j < (S::E >> S::B); j++) inv_col_open<S::B>(x, j << S::B, tw, (1u << S::A) + r * (S::E >> S::B) + j, q, qinv);
+        for (uint32_t j = 0; j < (S::E >> S::B); j++) inv_col_open<S::B, SH>(x, j << S::B, tws, (1u << S::A) + r * (S::E >> S::B) + j, q, qinv);
 #pragma unroll
         for (uint32_t k = 0; k < S::E; k++) sm[(S::E * r + k) * S::COLS + cc] = x[k];
         __syncthreads();
@@ -332,8 +364,9 @@ __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 768 / ColShape<LOGR>:
     } else {
 #pragma unroll
         for (uint32_t k = 0; k < S::E; k++) x[k] = reinterpret_cast<const double *>(g)[(size_t)(r + RS * k) * 256];
+        if (SH) __syncthreads();
     }
-    inv_col_last<S::A, S::B>(x, tw, q, qinv, c0, c1);
+    inv_col_last<S::A, S::B, SH>(x, tws, q, qinv, c0, c1);
 #pragma unroll
     for (uint32_t k = 0; k < S::E; k++) g[(size_t)(r + RS * k) * 256] = canonical_d(x[k], q);
 }
