@@ -74,13 +74,14 @@ __device__ __forceinline__ void conv_store(u64 *p, const double (&v)[CPT], doubl
 // coefficients per thread: two while their sources fit the registers and the buffers take 16-byte accesses
 inline uint32_t conv_cpt(uint32_t ns, const void *a, const void *b) { return ns <= 8 && (((uintptr_t)a | (uintptr_t)b) & 15) == 0 ? 2 : 1; }
 
-// targets per CTA (grid y) for `items` conversions of `targets` targets over gx CTAs: as many as leave the machine three
-// waves of CTAs (4 per SM), so that large batches read their sources once and single ciphertexts still fill the GPU
+// targets per CTA (grid y) for `items` conversions of `targets` targets over gx CTAs: all of them, unless that leaves fewer than
+// two CTAs per SM.  Every chunk loads and centres its sources again, which costs more than a machine that is only partly
+// filled (one ciphertext at N = 2^16, level 24: ModUp with 24, 8, 5 targets per CTA 21.7, 22.7, 26.0 us).
 constexpr uint32_t CONV_CHUNK_MAX = 32;
 inline uint32_t conv_chunk(uint32_t gx, uint32_t items, uint32_t targets) {
-    const uint32_t want = 3 * 148 * 4;
+    const uint32_t want = 2 * 148;
     uint32_t chunks = (want + gx * items - 1) / (gx * items);
-    chunks = std::max(1u, std::min(chunks, (targets + 3) / 4));
+    chunks = std::max(1u, std::min(chunks, (targets + 1) / 2));
     return std::min(CONV_CHUNK_MAX, (targets + chunks - 1) / chunks);
 }
 
