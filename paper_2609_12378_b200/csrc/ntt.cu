@@ -372,25 +372,26 @@ __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 768 / ColShape<LOGR>:
 }
 
 // ---- row passes ----------------------------------------------------------------------------------------------------
-// 16 threads per row, a row in one half warp, 16 rows per CTA at most (blockDim / 16).  In the exchange row two spare words
+// 16 threads per row, a row in one half warp, so warps need no barrier between them; 4 rows per CTA (16 were
+// 2 % slower: finer CTAs keep the phases of an SM's warps apart).  In the exchange row two spare words
 // follow every 16, so that a thread's own 16 consecutive coefficients are a 16-byte aligned block at a pitch of 144 bytes:
 // 8-byte accesses of consecutive lanes and 16-byte accesses to the own block are both conflict free.  Words enter and leave
 // through the row too, as pairs: lane t of a half warp moves words 2 t + 32 k and 2 t + 32 k + 1, so that every global access
 // is 16 bytes per lane and 256 consecutive bytes per half warp (32 bytes per lane cost the load/store pipe one pass per lane,
 // and 128-byte bulk copies per thread keep issuing while they are waited for: forward 162 -> 155, inverse 159 -> 146 us at 768 limbs).
 __device__ __forceinline__ uint32_t padded(uint32_t i) { return i + 2 * (i >> 4); }
-constexpr uint32_t ROW_PAD = 256 + 32, ROW_CTA = 16;
+constexpr uint32_t ROW_PAD = 256 + 32, ROW_CTA = 4;
 
 // forward, EP 0: in place; 1: the tail of a ModDown or rescale, (u - NTT(conv)) c + sigma_g(add), written to its final
 // place; 2: into a tiled buffer
 template <int EP, bool WIDE>
-__global__ void __launch_bounds__(16 * ROW_CTA, 4) ntt_fwd_rows(DevTables c, u64 *base, LimbMap map, uint32_t fp_share, const __grid_constant__ NttEpilogue ep) {
+__global__ void __launch_bounds__(16 * ROW_CTA, 64 / ROW_CTA) ntt_fwd_rows(DevTables c, u64 *base, LimbMap map, uint32_t fp_share, const __grid_constant__ NttEpilogue ep) {
     __shared__ __align__(16) double sm[ROW_CTA * ROW_PAD];
     const int prime = limb_prime(map, blockIdx.y);
     if (prime < 0 || (blockIdx.y & 7) >= fp_share) return;
     const double q = c.modd[prime].x, qinv = c.modd[prime].y;
     const double *tw = c.twd_fwd + ((size_t)prime << c.log_n);
-    const uint32_t t = threadIdx.x & 15, rl = threadIdx.x >> 4, row = blockIdx.x * (blockDim.x >> 4) + rl, R = c.N >> 8;
+    const uint32_t t = threadIdx.x & 15, rl = threadIdx.x >> 4, row = blockIdx.x * ROW_CTA + rl, R = c.N >> 8;
     u64 *g = base + (limb_index(map, blockIdx.y) << c.log_n) + (size_t)row * 256;
     double *s = sm + rl * ROW_PAD;
     double x[16];
@@ -480,13 +481,13 @@ __global__ void __launch_bounds__(16 * ROW_CTA, 4) ntt_fwd_rows(DevTables c, u64
 
 // inverse (the first pass); src (if any): the input limbs lie elsewhere, entry y / period at src.ptr.at(), limbs src.lpitch apart
 template <bool WIDE>
-__global__ void __launch_bounds__(16 * ROW_CTA, 3) ntt_inv_rows(DevTables c, u64 *base, LimbMap map, uint32_t fp_share, const __grid_constant__ NttSource src) {
+__global__ void __launch_bounds__(16 * ROW_CTA, 48 / ROW_CTA) ntt_inv_rows(DevTables c, u64 *base, LimbMap map, uint32_t fp_share, const __grid_constant__ NttSource src) {
     __shared__ __align__(16) double sm[ROW_CTA * ROW_PAD];
     const int prime = limb_prime(map, blockIdx.y);
     if (prime < 0 || (blockIdx.y & 7) >= fp_share) return;
     const double q = c.modd[prime].x, qinv = c.modd[prime].y;
     const double *tw = c.twd_inv + ((size_t)prime << c.log_n);
-    const uint32_t t = threadIdx.x & 15, rl = threadIdx.x >> 4, row = blockIdx.x * (blockDim.x >> 4) + rl, R = c.N >> 8;
+    const uint32_t t = threadIdx.x & 15, rl = threadIdx.x >> 4, row = blockIdx.x * ROW_CTA + rl, R = c.N >> 8;
     u64 *g = base + (limb_index(map, blockIdx.y) << c.log_n) + (size_t)row * 256;
     const u64 *gs = src.lpitch ? src.ptr.at(blockIdx.y / map.period) + (((size_t)(blockIdx.y % map.period) * src.lpitch) << c.log_n) + (size_t)row * 256 : g;
     double *s = sm + rl * ROW_PAD, *blk = s + 18 * t;
@@ -678,12 +679,6 @@ __global__ void __launch_bounds__(ClShape<LOGR>::THREADS, 1024 / ClShape<LOGR>::
     for (uint32_t k = 0; k < 16; k++) g[(size_t)(r + RS * k) * 256] = canonical_d(x[k], q);
 }
 
-// rows per CTA: 16, or fewer while that would leave SMs without a CTA
-uint32_t rows_per_cta(uint32_t R, uint32_t ny) {
-    uint32_t rows = R < ROW_CTA ? R : ROW_CTA;
-    while (rows > 4 && (uint64_t)ny * (R / rows) < 148) rows /= 2;
-    return rows;
-}
 template <uint32_t LOGR>
 void launch_cols(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, bool inverse, uint32_t share, const NttPrologue *pro, const double2 *scale, cudaStream_t s) {
     const dim3 grid(256 / ColShape<LOGR>::COLS, ny);
@@ -722,8 +717,7 @@ void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbM
                 default: return launch_cols<2>(c, b, ny, map, inverse, share, pro ? &pr : nullptr, inv_scale, s);
             }
         };
-        const uint32_t rows = rows_per_cta(R, ny);
-        const dim3 grid(R / rows, ny);
+        const dim3 grid(R / ROW_CTA, ny);
         if (share > 0 && !inverse) {
             cols();
             bool wide = aligned16(ep ? (const void *)nullptr : (const void *)b);
@@ -734,11 +728,11 @@ void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbM
             auto *k = mode == 1 ? (wide ? ntt_fwd_rows<1, true> : ntt_fwd_rows<1, false>)
                     : mode == 2 ? (wide ? ntt_fwd_rows<2, true> : ntt_fwd_rows<2, false>)
                                 : (wide ? ntt_fwd_rows<0, true> : ntt_fwd_rows<0, false>);
-            launch(k, grid, rows * 16, 0, s, c->dev, b, map, share, e);
+            launch(k, grid, 16 * ROW_CTA, 0, s, c->dev, b, map, share, e);
         } else if (share > 0) {
             const NttSource none{};
             const bool wide = src ? aligned16(src->ptr) : aligned16(b);
-            launch(wide ? ntt_inv_rows<true> : ntt_inv_rows<false>, grid, rows * 16, 0, s, c->dev, b, map, share, src ? sr : none);
+            launch(wide ? ntt_inv_rows<true> : ntt_inv_rows<false>, grid, 16 * ROW_CTA, 0, s, c->dev, b, map, share, src ? sr : none);
             cols();
         }
         if (share < 8) launch_ntt_int(c, b, ny, map, inverse, src ? sr.ptr.base : nullptr, src ? (uint32_t)(sr.ptr.stride >> c->log_n) : 0, s);
