@@ -363,7 +363,8 @@ extern "C" int32_t ckks_mul_relin_sum(ckks_ctx *c, const ckks_ct *a, const ckks_
     u64 *o = (u64 *)out->data;
     std::vector<CtView> pa(n), pb(n);
     for (uint32_t i = 0; i < n; i++) { pa[i] = CtView{(const u64 *)a[i].data, (size_t)level * c->N}; pb[i] = CtView{(const u64 *)b[i].data, (size_t)level * c->N}; }
-    launch_tensor_sum(c, pa.data(), pb.data(), n, o, e2, level, s);
+    const CtView *vb = pb.data();
+    launch_tensor_sum(c, pa.data(), &vb, n, &o, &e2, 1, level, s);
     relinearise(c, (const u64 *)rlk->data, Ptrs(e2, 0), Ptrs(o, 0), level, w, s);
     int rc = finish(c);
     if (rc == CKKS_OK) { out->level = level; out->ncomp = 2; out->scale = a[0].scale * b[0].scale; }

@@ -52,6 +52,10 @@ void rotate_ks(const ckks_ctx *c, const ckks_evk *key, const Ptrs &in, const Ptr
     ks_moddown(c, level, w, ko, s, nb);
 }
 
+static bool same_views(const std::vector<CtView> &x, const std::vector<CtView> &y) {
+    return x.size() == y.size() && std::equal(x.begin(), x.end(), y.begin(), [](const CtView &u, const CtView &v) { return u.p == v.p && u.comp == v.comp; });
+}
+
 // out[i] = rescale(relin(sum_t a[i][t] b[i][t])) for n sums of nterm products; ws: min(n, KS_MULTI) * product_bytes
 void sum_rescale(const ckks_ctx *c, const std::vector<std::vector<CtView>> &a, const std::vector<std::vector<CtView>> &b, u64 *const *out, uint32_t n,
                  const u64 *rlk, uint32_t level, void *ws, cudaStream_t s) {
@@ -61,9 +65,18 @@ void sum_rescale(const ckks_ctx *c, const std::vector<std::vector<CtView>> &a, c
         u64 *e01 = (u64 *)ws, *e2 = e01 + m * ctl, *ksw = e2 + m * ptl;
         Ptrs po;
         po.n = m;
-        for (uint32_t i = 0; i < m; i++) {
-            launch_tensor_sum(c, a[i0 + i].data(), b[i0 + i].data(), (uint32_t)a[i0 + i].size(), e01 + i * ctl, e2 + i * ptl, level, s);
-            po.p[i] = out[i0 + i];
+        for (uint32_t i = 0; i < m;) {
+            // neighbours with the same first operands share a pass over them
+            const CtView *pb[KS_MULTI];
+            u64 *p01[KS_MULTI], *p2[KS_MULTI];
+            uint32_t r = 0;
+            for (; i + r < m && (r == 0 || same_views(a[i0 + i], a[i0 + i + r])); r++) {
+                pb[r] = b[i0 + i + r].data();
+                p01[r] = e01 + (i + r) * ctl; p2[r] = e2 + (i + r) * ptl;
+                po.p[i + r] = out[i0 + i + r];
+            }
+            launch_tensor_sum(c, a[i0 + i].data(), pb, (uint32_t)a[i0 + i].size(), p01, p2, r, level, s);
+            i += r;
         }
         KsWorkspace w = ks_carve(c, level, ksw, m);
         relinearise(c, rlk, Ptrs(e2, ptl), Ptrs(e01, ctl), level, w, s, m);

@@ -399,10 +399,11 @@ void launch_tensor(const ckks_ctx *c, const TensorArgs &args, uint32_t n, uint32
 void launch_slot_mask(const ckks_ctx *c, double *out, uint32_t B, uint32_t lo, uint32_t hi, uint32_t Ti, uint32_t t0, uint32_t t1, cudaStream_t s);
 // out = in * v or in + v (component 0 only) for the constant polynomial v
 void launch_const(const ckks_ctx *c, const Ptrs &in, long long v, bool mul, const Ptrs &out, uint32_t ncomp, uint32_t level, cudaStream_t s, uint32_t n = 1);
-// e01, e2 (+)= sum_i tensor(a_i, b_i) (host arrays of n views)
-constexpr uint32_t TS_MAX = 16;
-struct TensorSumArgs { CtView a[TS_MAX], b[TS_MAX]; };
-void launch_tensor_sum(const ckks_ctx *c, const CtView *a, const CtView *b, uint32_t n, u64 *e01, u64 *e2, uint32_t level, cudaStream_t s, bool init = true);
+// e01[o], e2[o] = sum_i tensor(a_i, b[o]_i) for `no` outputs that share the first operands (host arrays of n views each)
+constexpr uint32_t TS_MAX = 16, TS_OUT = 4;
+struct TensorSumArgs { CtView a[TS_MAX], b[TS_OUT][TS_MAX]; u64 *e01[TS_OUT], *e2[TS_OUT]; };
+void launch_tensor_sum(const ckks_ctx *c, const CtView *a, const CtView *const *b, uint32_t n, u64 *const *e01, u64 *const *e2, uint32_t no, uint32_t level,
+                       cudaStream_t s);
 // out[o] (+)= sum_{j < nx} v[o][j] x[j] + cst[o] q_{level-1} (first component), o < no, for n ciphertexts each (see lincomb_kernel)
 constexpr uint32_t LIN_MAX = 8;
 struct LinArgs {

@@ -104,32 +104,45 @@ __global__ void __launch_bounds__(THREADS) const_kernel(DevTables c, const __gri
         MUL ? make_ulonglong2(mul_mod(u.x, r, q, mu), mul_mod(u.y, r, q, mu)) : make_ulonglong2(add_mod(u.x, r, q), add_mod(u.y, r, q));
 }
 
-// e (+)= sum_{i < n} tensor(a_i, b_i), n <= TS_MAX pairs per launch.  Sums of products of size 0.75 q (1.5 q for the middle
-// component) are reduced every four pairs; one canonical step per component at the end, with the previous partial sum added
-// unless INIT.  Bound by the operands' HBM traffic.
-template <bool INIT, bool WIDE>
-__global__ void __launch_bounds__(THREADS) tensor_sum_kernel(DevTables c, const __grid_constant__ TensorSumArgs t, uint32_t n, u64 *e01, u64 *e2, uint32_t level) {
+// e[o] (+)= sum_{i < n} tensor(a_i, b[o]_i), n <= TS_MAX terms per launch, NO outputs that share the first operands.  Sums of
+// products of size 0.75 q (1.5 q for the middle component) are reduced every four terms; one canonical step per component at the
+// end, with the previous partial sum added unless INIT.  Bound by the operands' HBM traffic, which four outputs at a time cut to
+// 5/8 of one at a time (the attention products: one query set against several key sets, the probabilities against every value
+// channel).
+template <bool INIT, bool WIDE, uint32_t NO>
+__global__ void __launch_bounds__(THREADS) tensor_sum_kernel(DevTables c, const __grid_constant__ TensorSumArgs t, uint32_t n, uint32_t level) {
     const uint32_t k = (blockIdx.x * THREADS + threadIdx.x) * 2, limb = blockIdx.y;
     const double q = c.modd[limb].x, qinv = c.modd[limb].y;
     const size_t o0 = (size_t)limb * c.N + k, o1 = o0 + (size_t)level * c.N;
     grid_dep_sync();
-    double s0[2] = {0.0, 0.0}, s1[2] = {0.0, 0.0}, s2[2] = {0.0, 0.0};
-    if (!INIT) { pair_d<WIDE>(e01 + o0, s0); pair_d<WIDE>(e01 + o1, s1); pair_d<WIDE>(e2 + o0, s2); }
-    for (uint32_t i = 0; i < n; i++) {
-        double a0[2], a1[2], b0[2], b1[2];
-        pair_d<WIDE>(t.a[i].p + o0, a0); pair_d<WIDE>(t.a[i].p + t.a[i].comp + o0, a1);
-        pair_d<WIDE>(t.b[i].p + o0, b0); pair_d<WIDE>(t.b[i].p + t.b[i].comp + o0, b1);
+    double s[NO][3][2];
 #pragma unroll
-        for (uint32_t j = 0; j < 2; j++) {
-            s0[j] = __dadd_rn(s0[j], mulmod_dd(a0[j], b0[j], q, qinv));
-            s1[j] = __dadd_rn(s1[j], __dadd_rn(mulmod_dd(a0[j], b1[j], q, qinv), mulmod_dd(a1[j], b0[j], q, qinv)));
-            s2[j] = __dadd_rn(s2[j], mulmod_dd(a1[j], b1[j], q, qinv));
-            if ((i & 3) == 3) { s0[j] = reduce_d(s0[j], q, qinv); s1[j] = reduce_d(s1[j], q, qinv); s2[j] = reduce_d(s2[j], q, qinv); }
-        }
+    for (uint32_t o = 0; o < NO; o++)
+        if (INIT) s[o][0][0] = s[o][0][1] = s[o][1][0] = s[o][1][1] = s[o][2][0] = s[o][2][1] = 0.0;
+        else { pair_d<WIDE>(t.e01[o] + o0, s[o][0]); pair_d<WIDE>(t.e01[o] + o1, s[o][1]); pair_d<WIDE>(t.e2[o] + o0, s[o][2]); }
+    for (uint32_t i = 0; i < n; i++) {
+        double a0[2], a1[2], b0[NO][2], b1[NO][2];
+        pair_d<WIDE>(t.a[i].p + o0, a0); pair_d<WIDE>(t.a[i].p + t.a[i].comp + o0, a1);
+#pragma unroll
+        for (uint32_t o = 0; o < NO; o++) { pair_d<WIDE>(t.b[o][i].p + o0, b0[o]); pair_d<WIDE>(t.b[o][i].p + t.b[o][i].comp + o0, b1[o]); }
+#pragma unroll
+        for (uint32_t o = 0; o < NO; o++)
+#pragma unroll
+            for (uint32_t j = 0; j < 2; j++) {
+                s[o][0][j] = __dadd_rn(s[o][0][j], mulmod_dd(a0[j], b0[o][j], q, qinv));
+                s[o][1][j] = __dadd_rn(s[o][1][j], __dadd_rn(mulmod_dd(a0[j], b1[o][j], q, qinv), mulmod_dd(a1[j], b0[o][j], q, qinv)));
+                s[o][2][j] = __dadd_rn(s[o][2][j], mulmod_dd(a1[j], b1[o][j], q, qinv));
+                if ((i & 3) == 3)
+#pragma unroll
+                    for (uint32_t m = 0; m < 3; m++) s[o][m][j] = reduce_d(s[o][m][j], q, qinv);
+            }
     }
-    store_pair<WIDE>(e01 + o0, s0, q, qinv);
-    store_pair<WIDE>(e01 + o1, s1, q, qinv);
-    store_pair<WIDE>(e2 + o0, s2, q, qinv);
+#pragma unroll
+    for (uint32_t o = 0; o < NO; o++) {
+        store_pair<WIDE>(t.e01[o] + o0, s[o][0], q, qinv);
+        store_pair<WIDE>(t.e01[o] + o1, s[o][1], q, qinv);
+        store_pair<WIDE>(t.e2[o] + o0, s[o][2], q, qinv);
+    }
 }
 
 // out[o] (+)= sum_j v[o][j] x[j] for up to LIN_MAX inputs and outputs of the ciphertexts blockIdx.z / 2 (component blockIdx.z & 1),
@@ -199,19 +212,30 @@ void launch_const(const ckks_ctx *c, const Ptrs &in, long long v, bool mul, cons
     else launch(const_kernel<false>, grid, THREADS, 0, s, c->dev, in, v, out, level);
 }
 
-void launch_tensor_sum(const ckks_ctx *c, const CtView *a, const CtView *b, uint32_t n, u64 *e01, u64 *e2, uint32_t level, cudaStream_t s, bool init) {
+template <uint32_t NO>
+static void tensor_sum(const ckks_ctx *c, const CtView *a, const CtView *const *b, uint32_t n, u64 *const *e01, u64 *const *e2, uint32_t level, cudaStream_t s) {
     const dim3 grid(c->N / (2 * THREADS), level);
     for (uint32_t i0 = 0; i0 < n; i0 += TS_MAX) {
         TensorSumArgs args;
         const uint32_t m = std::min(TS_MAX, n - i0);
-        std::copy(a + i0, a + i0 + m, args.a);
-        std::copy(b + i0, b + i0 + m, args.b);
-        bool wide = aligned16(e01) && aligned16(e2);
-        for (uint32_t i = 0; i < m; i++) wide = wide && aligned16(args.a[i]) && aligned16(args.b[i]);
-        auto *k = init && i0 == 0 ? (wide ? tensor_sum_kernel<true, true> : tensor_sum_kernel<true, false>)
-                                  : (wide ? tensor_sum_kernel<false, true> : tensor_sum_kernel<false, false>);
-        launch(k, grid, THREADS, 0, s, c->dev, args, m, e01, e2, level);
+        bool wide = true;
+        for (uint32_t i = 0; i < m; i++) { args.a[i] = a[i0 + i]; wide = wide && aligned16(args.a[i]); }
+        for (uint32_t o = 0; o < NO; o++) {
+            args.e01[o] = e01[o]; args.e2[o] = e2[o];
+            wide = wide && aligned16(e01[o]) && aligned16(e2[o]);
+            for (uint32_t i = 0; i < m; i++) { args.b[o][i] = b[o][i0 + i]; wide = wide && aligned16(args.b[o][i]); }
+        }
+        auto *k = i0 == 0 ? (wide ? tensor_sum_kernel<true, true, NO> : tensor_sum_kernel<true, false, NO>)
+                          : (wide ? tensor_sum_kernel<false, true, NO> : tensor_sum_kernel<false, false, NO>);
+        launch(k, grid, THREADS, 0, s, c->dev, args, m, level);
     }
+}
+
+void launch_tensor_sum(const ckks_ctx *c, const CtView *a, const CtView *const *b, uint32_t n, u64 *const *e01, u64 *const *e2, uint32_t no, uint32_t level,
+                       cudaStream_t s) {
+    for (; no >= 4; no -= 4, b += 4, e01 += 4, e2 += 4) tensor_sum<4>(c, a, b, n, e01, e2, level, s);
+    if (no >= 2) { tensor_sum<2>(c, a, b, n, e01, e2, level, s); no -= 2; b += 2; e01 += 2; e2 += 2; }
+    if (no) tensor_sum<1>(c, a, b, n, e01, e2, level, s);
 }
 
 void launch_lincomb(const ckks_ctx *c, const LinArgs &args, uint32_t n, uint32_t level, cudaStream_t s) {

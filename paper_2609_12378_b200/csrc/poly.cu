@@ -255,7 +255,9 @@ void bsgs_run(const ckks_ctx *c, const BsgsPlan &p, const Ptrs &x, const Ptrs &o
             A.push_back(CtView{blk + ((size_t)b * n + i) * blkw, (size_t)(p.Lb - 1) * N});
             B.push_back(gat(i, p.blocks[b]));
         }
-        launch_tensor_sum(c, A.data(), B.data(), nblk, S + i * sw, e2 + i * ew, p.Lc, s);
+        const CtView *pb = B.data();
+        u64 *p01 = S + i * sw, *p2 = e2 + i * ew;
+        launch_tensor_sum(c, A.data(), &pb, nblk, &p01, &p2, 1, p.Lc, s);
     }
     Lin l;
     l.out = {Ptrs(S, sw)};
