@@ -443,14 +443,12 @@ extern "C" int32_t ckks_poly_eval(ckks_ctx *c, const ckks_ct *x, const double *c
     launch_const(c, Ptrs(rb, 0), vs[degree - 1], false, Ptrs(rb, 0), 2, lvl, s);
     u64 *cur = rb, *other = ra;
     for (uint32_t k = degree - 1; k-- > 0;) {
-        KsWorkspace w = ks_carve(c, lvl, ksw);
         TensorArgs ta;
         ta.a[0] = CtView{cur, (size_t)lvl * N};
         ta.b[0] = CtView{xd, (size_t)level * N};         // x truncated to lvl limbs per component
         ta.e01[0] = other; ta.e2[0] = e2;
         launch_tensor(c, ta, 1, lvl, s);
-        relinearise(c, (const u64 *)rlk->data, Ptrs(e2, 0), Ptrs(other, 0), lvl, w, s);
-        launch_rescale(c, Ptrs(other, 0), Ptrs(cur, 0), 2, lvl, rsw, s);
+        relin_rescale(c, (const u64 *)rlk->data, Ptrs(e2, 0), Ptrs(other, 0), Ptrs(cur, 0), lvl, ksw, s);
         lvl--;
         launch_const(c, Ptrs(cur, 0), vs[k], false, Ptrs(cur, 0), 2, lvl, s);
     }

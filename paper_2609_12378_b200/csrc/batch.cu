@@ -11,6 +11,18 @@ void relinearise(const ckks_ctx *c, const u64 *rlk, const Ptrs &e2, const Ptrs &
     ko.add_comps = 3;
     ks_moddown(c, level, w, ko, s, nb);
 }
+// out[i] = rescale(e01[i] + key switch of e2[i]); ksw: the workspace of nb key switches
+void relin_rescale(const ckks_ctx *c, const u64 *rlk, const Ptrs &e2, const Ptrs &e01, const Ptrs &out, uint32_t level, u64 *ksw, cudaStream_t s, uint32_t nb) {
+    KsWorkspace w = ks_carve(c, level, ksw, nb);
+    if (!ks_fused_rescale(c)) {
+        relinearise(c, rlk, e2, e01, level, w, s, nb);
+        launch_rescale(c, e01, out, 2, level, ksw, s, nb);
+        return;
+    }
+    ks_modup(c, e2, level, w, s, nb);
+    ks_inner(c, rlk, level, 1, w, s, nb, false, nullptr, &e01);
+    ks_moddown_rescale(c, level, w, out, s, nb);
+}
 // One product's share of a batch: the tensor product's two parts and a key-switch workspace (whose bytes the rescale reuses)
 size_t product_bytes(const ckks_ctx *c, uint32_t level) { return ((size_t)3 * level + ks_workspace_limbs(c, level)) * c->N * sizeof(u64); }
 
@@ -30,9 +42,7 @@ void mul_rescale(const ckks_ctx *c, const CtView *a, const CtView *b, u64 *const
             po.p[i] = out[i0 + i];
         }
         launch_tensor(c, ta, m, level, s);
-        KsWorkspace w = ks_carve(c, level, ksw, m);
-        relinearise(c, rlk, Ptrs(e2, ptl), Ptrs(e01, ctl), level, w, s, m);
-        launch_rescale(c, Ptrs(e01, ctl), po, 2, level, ksw, s, m);
+        relin_rescale(c, rlk, Ptrs(e2, ptl), Ptrs(e01, ctl), po, level, ksw, s, m);
     }
 }
 
@@ -78,9 +88,7 @@ void sum_rescale(const ckks_ctx *c, const std::vector<std::vector<CtView>> &a, c
             launch_tensor_sum(c, a[i0 + i].data(), pb, (uint32_t)a[i0 + i].size(), p01, p2, r, level, s);
             i += r;
         }
-        KsWorkspace w = ks_carve(c, level, ksw, m);
-        relinearise(c, rlk, Ptrs(e2, ptl), Ptrs(e01, ctl), level, w, s, m);
-        launch_rescale(c, Ptrs(e01, ctl), po, 2, level, ksw, s, m);
+        relin_rescale(c, rlk, Ptrs(e2, ptl), Ptrs(e01, ctl), po, level, ksw, s, m);
     }
 }
 

@@ -35,6 +35,7 @@ struct DevTables {
     // {N^-1 qhat^-1, last inverse twiddle times that}, each {v, v / prime} centred
     const double2 *inv_scale_up;   // [(L+1)][L][2]   ModUp: level, limb
     const double2 *inv_scale_dn;   // [K][2]          ModDown: special limb
+    const double2 *inv_scale_rs;   // [L][1 + K][2]   ModDown with rescale: dropped limb (N^-1 alone), then the special limbs
     // ModUp, per level l (1..L), digit j, source a < alpha:
     const ulonglong2 *up_hat_inv;  // [(L+1)][dnum][alpha]        {qhat^-1 mod q_src, Shoup}
     const double *up_hat_mod_d;    // [(L+1)][dnum][T][alpha]     centred qhat mod target
@@ -52,6 +53,7 @@ struct DevTables {
     uint32_t conv_groups;
     // Rescale:
     const double2 *rs_inv_d;       // [L(last)][L(i)] {q_last^-1 mod q_i, that / q_i} as doubles
+    const double2 *rs_p_inv_d;     // [L(last)][L(i)] {(q_last P)^-1 mod q_i, that / q_i}
     // Encode:
     const uint32_t *enc_src;       // [n] slot index feeding FFT input position pos (bit-reversed e_j)
     const double2 *enc_omega;      // [n] exp(2 pi i t / n)
@@ -149,6 +151,8 @@ inline LimbMap same_map(uint32_t prime, uint32_t period) { return LimbMap{2, pri
 inline LimbMap ext_map(uint32_t level, uint32_t K, uint32_t L, uint32_t alpha, uint32_t beta) {
     return LimbMap{1, 0, level + K, level + K, level, L, alpha, beta, 1};
 }
+// limbs first .. level + K - 1 of every polynomial of the extended basis, polynomials level + K limbs apart
+inline LimbMap tail_map(uint32_t first, uint32_t level, uint32_t K, uint32_t L) { return LimbMap{1, first, level + K - first, level + K, level, L, 0, 1, 0}; }
 
 __host__ __device__ inline int limb_prime(const LimbMap &m, uint32_t y) {
     uint32_t x = y % m.period;
@@ -158,6 +162,7 @@ __host__ __device__ inline int limb_prime(const LimbMap &m, uint32_t y) {
         uint32_t j = (y / m.period) % m.nbeta, lo = j * m.alpha, hi = lo + m.alpha < m.level ? lo + m.alpha : m.level;
         if (x >= lo && x < hi) return -1;
     }
+    x += m.first;
     return x < m.level ? (int)x : (int)(m.L + (x - m.level));
 }
 // index (in limbs) of limb y from the base pointer
@@ -430,9 +435,10 @@ KsWorkspace ks_carve(const ckks_ctx *c, uint32_t level, void *ws, uint32_t nb = 
 // sigma_g(d), and d is never copied.
 void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb = 1);
 // inner product with evk (digits read through sigma_{ext_galois}; 1 = identity): leaves u = <digits, evk> in the extended basis
-// (w.u, nb entries); with acc_u it adds to what w.u holds, so that a sum of key-switched terms can share one ks_moddown.
+// (w.u, nb entries); with acc_u it adds to what w.u holds, so that a sum of key-switched terms can share one ks_moddown; with
+// `add` ([2][level][N] words per entry, no multi) it adds P add to both components.
 void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w, cudaStream_t s, uint32_t nb = 1,
-              bool acc_u = false, const KsMulti *multi = nullptr);
+              bool acc_u = false, const KsMulti *multi = nullptr, const Ptrs *add = nullptr);
 // ModDown and the final combination out_c = sigma_galois(add_c) + k_c + acc_c (add taken for the components in add_comps, acc if
 // given: [2][level][N] words per entry, possibly out itself)
 struct KsOut {
@@ -442,6 +448,9 @@ struct KsOut {
     TiledOut tiled;
 };
 void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb = 1, const KsMulti *multi = nullptr);
+// out = rescale(ModDown(w.u)), level - 1 limbs per component, without the tensor-core conversions (see ks_fused_rescale)
+void ks_moddown_rescale(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const Ptrs &out, cudaStream_t s, uint32_t nb);
+bool ks_fused_rescale(const ckks_ctx *c);
 // A sum of up to IP_TERMS key-switched terms in one pass over the extended basis:
 //   u[b] (+)= sum_t ( <ext[t][b] read through sigma_{g_t}, evk_t>  +  P sigma_{g_t}(c0_t[b]) on component 0's q-limbs )
 // ext holds term t's digits of batch entry b at ext + t * term_stride + b * beta * (level + K) * N words, the own limbs of the
@@ -501,6 +510,8 @@ void launch_extract_diagonals(const ckks_ctx *c, const double *W, uint32_t d_out
 
 // ---- sequences shared by the entry points (api.cu, poly.cu, attention.cu) -------------------------------------------
 void relinearise(const ckks_ctx *c, const u64 *rlk, const Ptrs &e2, const Ptrs &o, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb = 1);
+void relin_rescale(const ckks_ctx *c, const u64 *rlk, const Ptrs &e2, const Ptrs &e01, const Ptrs &out, uint32_t level, u64 *ksw, cudaStream_t s,
+                   uint32_t nb = 1);
 void rotate_ks(const ckks_ctx *c, const ckks_evk *key, const Ptrs &in, const Ptrs &out, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb = 1,
                const Ptrs *acc = nullptr);
 size_t product_bytes(const ckks_ctx *c, uint32_t level);

@@ -383,6 +383,20 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
                 rs[(size_t)last * L + i] = make_double2(inv, inv / (double)mod[i]);
             }
 
+    // ModDown and rescale in one step: (q_last P)^-1 mod q_i, and the inverse transform's scalings of the limbs it takes back
+    // ({last q-limb: N^-1}, then the special limbs' as above), index [last][1 + K][2]
+    std::vector<double2> rsp((size_t)L * L, make_double2(0.0, 0.0)), isc_rs((size_t)L * (K + 1) * 2);
+    for (uint32_t last = 0; last < L; last++) {
+        for (uint32_t i = 0; i < L; i++)
+            if (i != last) {
+                const double inv = (double)h_mul((u64)rs[(size_t)last * L + i].x, (u64)dn_pinv_d[i].x, mod[i]);
+                rsp[(size_t)last * L + i] = make_double2(inv, inv / (double)mod[i]);
+            }
+        double2 *e = &isc_rs[(size_t)last * (K + 1) * 2];
+        e[0] = ninvd[2 * last]; e[1] = ninvd[2 * last + 1];
+        for (uint32_t a = 0; a < 2 * K; a++) e[2 + a] = isc_dn[a];
+    }
+
     // ---- Encode tables: input permutation and fp64 twiddles from the host libm
     std::vector<uint32_t> enc_src(n);
     std::vector<double2> om(n), ze(n);
@@ -418,7 +432,7 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
     if ((rc = upload(c, mod, &d.mod)) || (rc = upload(c, mu, &d.mu)) || (rc = upload(c, mu64, &d.mu64)) || (rc = upload(c, modd, &d.modd)) || (rc = upload(c, twf, &d.tw_fwd)) ||
         (rc = upload(c, twi, &d.tw_inv)) || (rc = upload(c, twdf, &d.twd_fwd)) || (rc = upload(c, twdi, &d.twd_inv)) || (rc = upload(c, ninvd, &d.n_inv_d)) || (rc = upload(c, isc_up, &d.inv_scale_up)) || (rc = upload(c, isc_dn, &d.inv_scale_dn)) || (rc = upload(c, ninv, &d.n_inv)) || (rc = upload(c, up_inv, &d.up_hat_inv)) ||
         (rc = upload(c, up_mod_d, &d.up_hat_mod_d)) || (rc = upload(c, dn_mod_d, &d.dn_hat_mod_d)) || (rc = upload(c, dn_inv, &d.dn_hat_inv)) ||
-        (rc = upload(c, dn_pinv_d, &d.dn_p_inv_d)) || (rc = upload(c, dn_pmod_d, &d.dn_p_mod_d)) || (rc = upload(c, up_bmat, &d.up_bmat)) || (rc = upload(c, dn_bmat, &d.dn_bmat)) || (rc = upload(c, two52, &d.two52_d)) || (rc = upload(c, rs, &d.rs_inv_d)) ||
+        (rc = upload(c, dn_pinv_d, &d.dn_p_inv_d)) || (rc = upload(c, dn_pmod_d, &d.dn_p_mod_d)) || (rc = upload(c, up_bmat, &d.up_bmat)) || (rc = upload(c, dn_bmat, &d.dn_bmat)) || (rc = upload(c, two52, &d.two52_d)) || (rc = upload(c, rs, &d.rs_inv_d)) || (rc = upload(c, rsp, &d.rs_p_inv_d)) || (rc = upload(c, isc_rs, &d.inv_scale_rs)) ||
         (rc = upload(c, enc_src, &d.enc_src)) || (rc = upload(c, om, &d.enc_omega)) || (rc = upload(c, om_st, &d.enc_omega_st)) || (rc = upload(c, om_st2, &d.enc_omega_st2)) || (rc = upload(c, ze, &d.enc_zeta)) ||
         (rc = upload(c, flag, &flag_dev))) {
         cudaSetDevice(prev);

@@ -272,11 +272,8 @@ void bsgs_run(const ckks_ctx *c, const BsgsPlan &p, const Ptrs &x, const Ptrs &o
         l.v[0].push_back(p.cv[k]);
     }
     lincomb(c, l, n, p.Lc, nblk > 0, s);
-    if (nblk) {
-        KsWorkspace w = ks_carve(c, p.Lc, ksw, n);
-        relinearise(c, rlk, Ptrs(e2, ew), Ptrs(S, sw), p.Lc, w, s, n);
-    }
-    launch_rescale(c, Ptrs(S, sw), out, 2, p.Lc, ksw, s, n);
+    if (nblk) relin_rescale(c, rlk, Ptrs(e2, ew), Ptrs(S, sw), out, p.Lc, ksw, s, n);
+    else launch_rescale(c, Ptrs(S, sw), out, 2, p.Lc, ksw, s, n);
 }
 
 constexpr uint32_t POLY_BATCH = 4;      // ciphertexts evaluated side by side by the batch entry point
