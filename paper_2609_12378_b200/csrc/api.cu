@@ -670,8 +670,7 @@ extern "C" int32_t ckks_rotate_hoisted(ckks_ctx *c, const ckks_ct *in, const ckk
         const uint32_t nb = std::min(nbh, nrot - r0);
         KsMulti m{};
         for (uint32_t b = 0; b < nb; b++) { m.evk[b] = (const u64 *)keys[r0 + b].data; m.galois[b] = keys[r0 + b].galois; m.out[b] = (u64 *)outs[r0 + b].data; }
-        ks_inner(c, nullptr, level, 1, w, s, nb, false, &m);
-        ks_moddown(c, level, w, ko, s, nb, &m);
+        ks_apply(c, nullptr, level, w, ko, s, nb, &m);
     }
     rc = finish(c);
     if (rc == CKKS_OK)
@@ -802,8 +801,7 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
                 m.galois[r] = ckks_galois_element(c, (int64_t)(b + r) * T);
                 m.evk[r] = (const u64 *)find_key(keys, nkeys, m.galois[r])->data;
             }
-            ks_inner(c, nullptr, level, 1, kb, s, nr * nx, false, &m);
-            ks_moddown(c, level, kb, ko, s, nr * nx, &m);
+            ks_apply(c, nullptr, level, kb, ko, s, nr * nx, &m);
         }
     };
     if (!L.ib_outer) baby_steps(0);
@@ -849,8 +847,7 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
                         ko.add = Ptrs(ag, ctl); ko.out = Ptrs(rot, ctl);
                         ko.add_comps = 1;
                         ks_modup(c, Ptrs(ag + ptl, ctl), level, kg, s, nr * S);
-                        ks_inner(c, nullptr, level, 1, kg, s, nr * S, false, &m);
-                        ks_moddown(c, level, kg, ko, s, nr * S, &m);
+                        ks_apply(c, nullptr, level, kg, ko, s, nr * S, &m);
                         launch_sum(c, total, first, rot, nr, S, level, s);
                     }
                     gl += nr;

@@ -5,11 +5,10 @@
 // o[i] (2 x level limbs) += key switch of e2[i], nb side by side
 void relinearise(const ckks_ctx *c, const u64 *rlk, const Ptrs &e2, const Ptrs &o, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb) {
     ks_modup(c, e2, level, w, s, nb);
-    ks_inner(c, rlk, level, 1, w, s, nb);
     KsOut ko;
     ko.add = ko.out = o;
     ko.add_comps = 3;
-    ks_moddown(c, level, w, ko, s, nb);
+    ks_apply(c, rlk, level, w, ko, s, nb);
 }
 // out[i] = rescale(e01[i] + key switch of e2[i]); ksw: the workspace of nb key switches
 void relin_rescale(const ckks_ctx *c, const u64 *rlk, const Ptrs &e2, const Ptrs &e01, const Ptrs &out, uint32_t level, u64 *ksw, cudaStream_t s, uint32_t nb) {
@@ -20,8 +19,7 @@ void relin_rescale(const ckks_ctx *c, const u64 *rlk, const Ptrs &e2, const Ptrs
         return;
     }
     ks_modup(c, e2, level, w, s, nb);
-    ks_inner(c, rlk, level, 1, w, s, nb, false, nullptr, &e01);
-    ks_moddown_rescale(c, level, w, out, s, nb);
+    ks_apply_rescale(c, rlk, level, w, e01, out, s, nb);
 }
 // One product's share of a batch: the tensor product's two parts and a key-switch workspace (whose bytes the rescale reuses)
 size_t product_bytes(const ckks_ctx *c, uint32_t level) { return ((size_t)3 * level + ks_workspace_limbs(c, level)) * c->N * sizeof(u64); }
@@ -54,12 +52,11 @@ void rotate_ks(const ckks_ctx *c, const ckks_evk *key, const Ptrs &in, const Ptr
     if (in.n) for (uint32_t b = 0; b < in.n; b++) c1.p[b] += ptl;
     else c1.base += ptl;
     ks_modup(c, c1, level, w, s, nb);
-    ks_inner(c, (const u64 *)key->data, level, key->galois, w, s, nb);
     KsOut ko;
     ko.add = in; ko.out = out;
     ko.add_comps = 1; ko.galois = key->galois;
     if (acc) ko.acc = *acc;
-    ks_moddown(c, level, w, ko, s, nb);
+    ks_apply(c, (const u64 *)key->data, level, w, ko, s, nb);
 }
 
 static bool same_views(const std::vector<CtView> &x, const std::vector<CtView> &y) {
@@ -128,8 +125,7 @@ void rotate_grid(const ckks_ctx *c, const CtView *in, uint32_t n, const ckks_evk
             k.group = m; k.rot_stride = rot_stride;
             for (uint32_t r = 0; r < nr; r++) { k.galois[r] = keys[r0 + r].galois; k.evk[r] = (const u64 *)keys[r0 + r].data; }
             ko.out.base = out + r0 * rot_stride + i0 * ct_stride;
-            ks_inner(c, nullptr, level, 1, w, s, nr * m, false, &k);
-            ks_moddown(c, level, w, ko, s, nr * m, &k);
+            ks_apply(c, nullptr, level, w, ko, s, nr * m, &k);
         }
     }
 }

@@ -353,8 +353,11 @@ inline bool aligned16(const Ptrs &p) {
 //           acc (if given): [ncomp][level][N] words per entry;
 //           out: plain ([ncomp][level][N] per entry) or tiled (tl.R != 0, component comp of entry b in row
 //           tl.row0 + b * tl.row_stride + comp)
+//   mode 3: as mode 1, but the sum u is not read: it is formed here, u = <digits, key> (add_p: + P add, and nothing is
+//           added afterwards).  Digits are read through sigma_galois as well; beta <= IP_FUSED_BETA of them
 //   mode 2: the transform's own result is stored, but into a tiled buffer (out.base): limb y = b * level + i becomes row
 //           tl.row0 + b * tl.row_stride, limb i
+constexpr uint32_t IP_FUSED_BETA = 4;
 struct NttEpilogue {
     int mode;
     Ptrs u, add, out, acc;
@@ -369,6 +372,11 @@ struct NttEpilogue {
     // tl.row0 + r * rot_rows + m * tl.row_stride + comp, or to out.base + r * rot_stride + m * out.stride
     uint32_t group, own, rot_rows;
     size_t rot_stride;
+    // mode 3: extended digits [entry][beta][nt][N] and the digits' own limbs (shared: entry 0 for all), the key (multi: one per
+    // rotation), the limbs per component of `add`, the batch
+    const u64 *ext, *evk, *mevk[KS_MULTI];
+    Ptrs d;
+    uint32_t beta, shared, add_level, add_p, nb;
     uint32_t y0;           // (filled in) first limb of the launch
 };
 // Prologue of the forward transform: the first pass reads one buffer [batch][N] (batch = limb index / map.period) instead of
@@ -437,8 +445,9 @@ void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, 
 // inner product with evk (digits read through sigma_{ext_galois}; 1 = identity): leaves u = <digits, evk> in the extended basis
 // (w.u, nb entries); with acc_u it adds to what w.u holds, so that a sum of key-switched terms can share one ks_moddown; with
 // `add` ([2][level][N] words per entry, no multi) it adds P add to both components.
+// Only limbs x0 .. level + K - 1 of the extended basis are formed.
 void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w, cudaStream_t s, uint32_t nb = 1,
-              bool acc_u = false, const KsMulti *multi = nullptr, const Ptrs *add = nullptr);
+              bool acc_u = false, const KsMulti *multi = nullptr, const Ptrs *add = nullptr, uint32_t x0 = 0);
 // ModDown and the final combination out_c = sigma_galois(add_c) + k_c + acc_c (add taken for the components in add_comps, acc if
 // given: [2][level][N] words per entry, possibly out itself)
 struct KsOut {
@@ -448,8 +457,10 @@ struct KsOut {
     TiledOut tiled;
 };
 void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb = 1, const KsMulti *multi = nullptr);
-// out = rescale(ModDown(w.u)), level - 1 limbs per component, without the tensor-core conversions (see ks_fused_rescale)
-void ks_moddown_rescale(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const Ptrs &out, cudaStream_t s, uint32_t nb);
+// Both together: out = ModDown(<digits, key>) and the final combination, digits read through the permutation of o.galois
+void ks_apply(const ckks_ctx *c, const u64 *evk, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb = 1, const KsMulti *multi = nullptr);
+// out = rescale(ModDown(<digits, key>) + add), level - 1 limbs per component, without the tensor-core conversions (see ks_fused_rescale)
+void ks_apply_rescale(const ckks_ctx *c, const u64 *evk, uint32_t level, const KsWorkspace &w, const Ptrs &add, const Ptrs &out, cudaStream_t s, uint32_t nb);
 bool ks_fused_rescale(const ckks_ctx *c);
 // A sum of up to IP_TERMS key-switched terms in one pass over the extended basis:
 //   u[b] (+)= sum_t ( <ext[t][b] read through sigma_{g_t}, evk_t>  +  P sigma_{g_t}(c0_t[b]) on component 0's q-limbs )

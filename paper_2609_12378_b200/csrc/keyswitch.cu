@@ -145,9 +145,9 @@ void launch_modup(const ckks_ctx *c, const u64 *dcoef, u64 *ext, uint32_t level,
 // u[comp][x][p] = sum_j ext[j][x][pi_g(p)] * evk[j][comp][kt(x)][p]          (any number of digits)
 __global__ void __launch_bounds__(THREADS) inner_product_generic_kernel(DevTables c, const u64 *ext, const __grid_constant__ Ptrs dp, uint32_t d0, const u64 *evk, u64 g,
                                                                         u64 *u, uint32_t level, int has_multi, const __grid_constant__ KsMulti multi, int acc_u, int has_add,
-                                                                        const __grid_constant__ Ptrs add) {
+                                                                        const __grid_constant__ Ptrs add, uint32_t x0) {
     const uint32_t p = blockIdx.x * THREADS + threadIdx.x;
-    const uint32_t x = blockIdx.z, bz = blockIdx.y;     // batch varies faster than the limb: a key limb is reused from L2
+    const uint32_t x = blockIdx.z + x0, bz = blockIdx.y;     // batch varies faster than the limb: a key limb is reused from L2
     const uint32_t nt = level + c.K, beta = (level + c.alpha - 1) / c.alpha;
     const uint32_t kt = x < level ? x : c.L + (x - level);
     if (has_multi) { evk = multi.evk[bz]; g = multi.galois[bz]; }     // shared digits, per-entry key and permutation
@@ -189,9 +189,9 @@ constexpr uint32_t IP_MAX_BETA = 8, IP_TERMS_MAX_BETA = 4;
 template <uint32_t BETA, bool ADD>
 __global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, const u64 *ext, const __grid_constant__ Ptrs d, const u64 *evk, u64 g, u64 *u,
                                                                 uint32_t level, uint32_t nb, uint32_t bch, int has_multi, const __grid_constant__ KsMulti multi,
-                                                                int acc_u, const __grid_constant__ Ptrs add) {
+                                                                int acc_u, const __grid_constant__ Ptrs add, uint32_t x0) {
     const uint32_t p = (blockIdx.x * THREADS + threadIdx.x) * 2;
-    const uint32_t x = blockIdx.z;     // chunks of a limb run together: its key words (and shared digits) come from L2
+    const uint32_t x = blockIdx.z + x0;     // chunks of a limb run together: its key words (and shared digits) come from L2
     uint32_t b0 = blockIdx.y * bch, b1 = min(b0 + bch, nb), e0 = has_multi ? 0 : b0;      // entries; first digits entry
     const uint32_t nt = level + c.K;
     const uint32_t kt = x < level ? x : c.L + (x - level);
@@ -511,7 +511,7 @@ void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, 
 }
 
 void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w, cudaStream_t s, uint32_t nb,
-              bool acc_u, const KsMulti *multi, const Ptrs *add) {
+              bool acc_u, const KsMulti *multi, const Ptrs *add, uint32_t x0) {
     const uint32_t N = c->N, nt = level + c->K;
     const uint32_t beta = (level + c->alpha - 1) / c->alpha;
     const int au = acc_u ? 1 : 0;
@@ -529,7 +529,7 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
                 wr.ext = w.ext + (size_t)r * multi->group * beta * nt * N;
                 wr.d.base += r * multi->group * w.d.stride;
             }
-            ks_inner(c, multi->evk[r], level, multi->galois[r], wr, s, multi->group, acc_u, nullptr);
+            ks_inner(c, multi->evk[r], level, multi->galois[r], wr, s, multi->group, acc_u, nullptr, nullptr, x0);
         }
         return;
     }
@@ -538,20 +538,59 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
         // batch entries per thread: enough chunks left to fill the machine, key words reused across a chunk
         const uint32_t grp = multi ? multi->group : 0, per = grp ? grp : nb;
         const uint32_t bch = (multi && !grp) ? 1 : (per >= 8 ? 4 : (per >= 4 ? 2 : 1));
-        const dim3 grid(N / (2 * THREADS), grp ? (nb / grp) * ((grp + bch - 1) / bch) : (nb + bch - 1) / bch, nt);
+        const dim3 grid(N / (2 * THREADS), grp ? (nb / grp) * ((grp + bch - 1) / bch) : (nb + bch - 1) / bch, nt - x0);
         using K = decltype(&inner_product_kernel<1, false>);
         static constexpr K plain[IP_MAX_BETA] = {inner_product_kernel<1, false>, inner_product_kernel<2, false>, inner_product_kernel<3, false>, inner_product_kernel<4, false>,
                                                  inner_product_kernel<5, false>, inner_product_kernel<6, false>, inner_product_kernel<7, false>, inner_product_kernel<8, false>};
         static constexpr K adding[IP_MAX_BETA] = {inner_product_kernel<1, true>, inner_product_kernel<2, true>, inner_product_kernel<3, true>, inner_product_kernel<4, true>,
                                                   inner_product_kernel<5, true>, inner_product_kernel<6, true>, inner_product_kernel<7, true>, inner_product_kernel<8, true>};
-        launch((add ? adding : plain)[beta - 1], grid, THREADS, 0, s, c->dev, w.ext, w.d, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au, pa);
+        launch((add ? adding : plain)[beta - 1], grid, THREADS, 0, s, c->dev, w.ext, w.d, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au, pa, x0);
     } else {
-        launch(inner_product_generic_kernel, dim3(N / THREADS, nb, nt), THREADS, 0, s, c->dev, w.ext, w.d, 0u, evk, ext_galois, w.u, level, multi ? 1 : 0, m, au,
-               add ? 1 : 0, pa);
+        launch(inner_product_generic_kernel, dim3(N / THREADS, nb, nt - x0), THREADS, 0, s, c->dev, w.ext, w.d, 0u, evk, ext_galois, w.u, level, multi ? 1 : 0, m, au,
+               add ? 1 : 0, pa, x0);
     }
 }
 
-void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb, const KsMulti *multi) {
+// Whether the row pass that ends a ModDown forms the inner product's q-limbs itself (mode 3 of the epilogue), so that the sum u
+// is written and read back for the special limbs only.  It does where a key word serves fewer than four entries (four or more share
+// it from registers in inner_product_kernel, where this form would read it from L2 for each) and the pass fills the GPU once:
+// below that its eight steps of dependent reads cost more than the traffic (64 hoisted rotations at N = 2^16, level 24:
+// 4550 -> 4110 us; the key/value projections of 24 tokens 35.9 -> 34.3 ms).  Operands have to take 16-byte accesses.
+static bool inner_fused(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const u64 *evk, uint32_t nb, const KsMulti *multi) {
+    const uint32_t beta = (level + c->alpha - 1) / c->alpha, nkeys = multi ? (multi->group ? nb / multi->group : nb) : 0, per = multi ? multi->group : nb;
+    bool ok = per < 4 && beta <= IP_FUSED_BETA && nb * 2 * level <= 32768 && (uint64_t)nb * 2 * level * (c->N >> 10) >= 16 * (uint64_t)c->sms &&
+              aligned16(w.ext) && aligned16(w.d) && (multi || aligned16(evk));
+    for (uint32_t b = 0; b < nkeys; b++) ok = ok && aligned16(multi->evk[b]);
+    return ok;
+}
+// the part of the epilogue that describes the inner product
+static void fuse_inner(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const u64 *evk, uint32_t nb, const KsMulti *multi, NttEpilogue &ep) {
+    ep.mode = 3;
+    ep.ext = w.ext; ep.d = w.d; ep.evk = evk; ep.nb = nb;
+    ep.beta = (level + c->alpha - 1) / c->alpha;
+    ep.shared = multi && !multi->group;
+    ep.add_level = level;
+    if (multi) for (uint32_t b = 0; b < KS_MULTI; b++) ep.mevk[b] = multi->evk[b];
+}
+static bool out_aligned(const NttEpilogue &ep) { return aligned16(ep.add) && aligned16(ep.acc) && aligned16(ep.out) && (ep.rot_stride & 1) == 0; }
+
+// the ModDown of w.u; fused: of a w.u whose special limbs alone exist
+static NttEpilogue moddown_epilogue(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const KsOut &o, uint32_t nb, const KsMulti *multi) {
+    NttEpilogue ep{};      // the last NTT pass finishes the ModDown itself
+    ep.mode = 1;
+    ep.u = Ptrs(w.u, (size_t)2 * (level + c->K) * c->N);
+    ep.add = o.add; ep.out = o.out; ep.add_comps = o.add_comps;
+    ep.pinv = c->dev.dn_p_inv_d;
+    ep.ncomp = 2; ep.level = level; ep.nt = level + c->K;
+    ep.galois = o.galois; ep.acc = o.acc; ep.accumulate = o.acc.n || o.acc.base ? 1 : 0; ep.tl = o.tiled;
+    if (multi) {
+        ep.multi = 1; ep.group = multi->group; ep.own = multi->own; ep.rot_rows = multi->rot_rows; ep.rot_stride = multi->rot_stride;
+        for (uint32_t b = 0; b < KS_MULTI; b++) { ep.mgalois[b] = multi->galois[b]; ep.out.p[b] = multi->out[b]; }
+        if (!multi->group) ep.out.n = nb;
+    }
+    return ep;
+}
+static void moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const NttEpilogue &ep, cudaStream_t s, uint32_t nb) {
     const uint32_t N = c->N, nt = level + c->K, K = c->K;
     // the K special limbs of every (batch, component): groups of K limbs, nt limbs apart
     launch_ntt(c, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, nullptr, nullptr, nullptr,
@@ -563,19 +602,17 @@ void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const K
         DISPATCH_POW2(K, CALL_DN);
 #undef CALL_DN
     }
-    NttEpilogue ep{};      // the last NTT pass finishes the ModDown itself
-    ep.mode = 1;
-    ep.u = Ptrs(w.u, (size_t)2 * nt * N);
-    ep.add = o.add; ep.out = o.out; ep.add_comps = o.add_comps;
-    ep.pinv = c->dev.dn_p_inv_d;
-    ep.ncomp = 2; ep.level = level; ep.nt = nt;
-    ep.galois = o.galois; ep.acc = o.acc; ep.accumulate = o.acc.n || o.acc.base ? 1 : 0; ep.tl = o.tiled;
-    if (multi) {
-        ep.multi = 1; ep.group = multi->group; ep.own = multi->own; ep.rot_rows = multi->rot_rows; ep.rot_stride = multi->rot_stride;
-        for (uint32_t b = 0; b < KS_MULTI; b++) { ep.mgalois[b] = multi->galois[b]; ep.out.p[b] = multi->out[b]; }
-        if (!multi->group) ep.out.n = nb;
-    }
     launch_ntt(c, w.conv, nb * 2 * level, plain_map(0, level), false, s, &ep);
+}
+void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb, const KsMulti *multi) {
+    moddown(c, level, w, moddown_epilogue(c, level, w, o, nb, multi), s, nb);
+}
+void ks_apply(const ckks_ctx *c, const u64 *evk, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb, const KsMulti *multi) {
+    NttEpilogue ep = moddown_epilogue(c, level, w, o, nb, multi);
+    const bool fused = inner_fused(c, level, w, evk, nb, multi) && out_aligned(ep);
+    ks_inner(c, evk, level, o.galois, w, s, nb, false, multi, nullptr, fused ? level : 0);
+    if (fused) fuse_inner(c, level, w, evk, nb, multi, ep);
+    moddown(c, level, w, ep, s, nb);
 }
 
 // The tensor-core conversions have no form that carries the dropped limb along
@@ -583,19 +620,25 @@ bool ks_fused_rescale(const ckks_ctx *c) { return !conv_tensor(c); }
 
 // ModDown and rescale at once, bit for bit what they give one after the other (see moddown_conv_kernel); the polynomial of
 // degree 63 at N = 2^16, level 24, whose products all end this way: 2615 -> 2295 us.
-void ks_moddown_rescale(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const Ptrs &out, cudaStream_t s, uint32_t nb) {
+void ks_apply_rescale(const ckks_ctx *c, const u64 *evk, uint32_t level, const KsWorkspace &w, const Ptrs &add, const Ptrs &out, cudaStream_t s, uint32_t nb) {
     const uint32_t N = c->N, K = c->K, nt = level + K, m = level - 1;
-    // the dropped limb and the K special limbs of every (batch, component), nt limbs apart
-    launch_ntt(c, w.u + (size_t)m * N, nb * 2 * (K + 1), tail_map(m, level, K, c->L), true, s, nullptr, nullptr, nullptr, c->dev.inv_scale_rs + (size_t)m * (K + 1) * 2);
-#define CALL_DN(A) launch_moddown_conv<A, true>(c, w.u, w.conv, level, nb, s)
-    DISPATCH_POW2(K, CALL_DN);
-#undef CALL_DN
     NttEpilogue ep{};
     ep.mode = 1;
     ep.u = Ptrs(w.u, (size_t)2 * nt * N);
     ep.out = out;
     ep.pinv = c->dev.rs_p_inv_d + (size_t)m * c->L;
     ep.ncomp = 2; ep.level = m; ep.nt = nt; ep.galois = 1;
+    const bool fused = inner_fused(c, level, w, evk, nb, nullptr) && out_aligned(ep) && aligned16(add);
+    ks_inner(c, evk, level, 1, w, s, nb, false, nullptr, &add, fused ? m : 0);
+    if (fused) {
+        fuse_inner(c, level, w, evk, nb, nullptr, ep);
+        ep.add = add; ep.add_comps = 3; ep.add_p = 1;
+    }
+    // the dropped limb and the K special limbs of every (batch, component), nt limbs apart
+    launch_ntt(c, w.u + (size_t)m * N, nb * 2 * (K + 1), tail_map(m, level, K, c->L), true, s, nullptr, nullptr, nullptr, c->dev.inv_scale_rs + (size_t)m * (K + 1) * 2);
+#define CALL_DN(A) launch_moddown_conv<A, true>(c, w.u, w.conv, level, nb, s)
+    DISPATCH_POW2(K, CALL_DN);
+#undef CALL_DN
     launch_ntt(c, w.conv, nb * 2 * m, plain_map(0, m), false, s, &ep);
 }
 
@@ -613,7 +656,7 @@ void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, siz
     // any number of digits, any alignment: one term at a time through the generic kernel, then its P c0
     for (uint32_t t = 0; t < nterm; t++) {
         launch(inner_product_generic_kernel, dim3(N / THREADS, nb, nt), THREADS, 0, s, c->dev, w.ext + t * term_stride, w.d, t * nb, terms.evk[t], terms.galois[t],
-               w.u, level, 0, KsMulti{}, (acc_u || t > 0) ? 1 : 0, 0, Ptrs());
+               w.u, level, 0, KsMulti{}, (acc_u || t > 0) ? 1 : 0, 0, Ptrs(), 0u);
         if (terms.c0[t])
             launch(p_c0_acc_kernel, dim3(N / THREADS, level, nb), THREADS, 0, s, c->dev, terms.c0[t], c0_stride, terms.galois[t], w.u, (size_t)2 * nt * N);
     }

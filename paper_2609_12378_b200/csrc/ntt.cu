@@ -383,16 +383,20 @@ __device__ __forceinline__ uint32_t padded(uint32_t i) { return i + 2 * (i >> 4)
 constexpr uint32_t ROW_PAD = 256 + 32, ROW_CTA = 4;
 
 // forward, EP 0: in place; 1: the tail of a ModDown or rescale, (u - NTT(conv)) c + sigma_g(add), written to its final
-// place; 2: into a tiled buffer
-template <int EP, bool WIDE>
+// place; 2: into a tiled buffer; 3: as 1 with u formed here from BETA digits and the key.  EP 3 is bound by HBM (the key words and the
+// results); one pair of words per step at 64 registers: two pairs at 96 registers and 20 warps per SM took 1750 us for 64
+// rotations, four pairs at 128 registers 1910, against 1550.
+template <int EP, bool WIDE, uint32_t BETA = 1, bool ADDP = false>
 __global__ void __launch_bounds__(16 * ROW_CTA, 64 / ROW_CTA) ntt_fwd_rows(DevTables c, u64 *base, LimbMap map, uint32_t fp_share, const __grid_constant__ NttEpilogue ep) {
     __shared__ __align__(16) double sm[ROW_CTA * ROW_PAD];
-    const int prime = limb_prime(map, blockIdx.y);
-    if (prime < 0 || (blockIdx.y & 7) >= fp_share) return;
+    // EP 3: the entries and components of a limb next to each other, for the sake of its digits and key words in L2
+    const uint32_t yl = EP == 3 ? ((blockIdx.y >> 1) % ep.nb * 2 + (blockIdx.y & 1)) * ep.level + (blockIdx.y >> 1) / ep.nb : blockIdx.y;
+    const int prime = limb_prime(map, yl);
+    if (prime < 0 || (yl & 7) >= fp_share) return;
     const double q = c.modd[prime].x, qinv = c.modd[prime].y;
     const double *tw = c.twd_fwd + ((size_t)prime << c.log_n);
     const uint32_t t = threadIdx.x & 15, rl = threadIdx.x >> 4, row = blockIdx.x * ROW_CTA + rl, R = c.N >> 8;
-    u64 *g = base + (limb_index(map, blockIdx.y) << c.log_n) + (size_t)row * 256;
+    u64 *g = base + (limb_index(map, yl) << c.log_n) + (size_t)row * 256;
     double *s = sm + rl * ROW_PAD;
     double x[16];
     grid_dep_sync();
@@ -414,20 +418,65 @@ __global__ void __launch_bounds__(16 * ROW_CTA, 64 / ROW_CTA) ntt_fwd_rows(DevTa
     for (uint32_t k = 0; k < 16; k += 2) *reinterpret_cast<double2 *>(blk + k) = make_double2(x[k], x[k + 1]);
     __syncwarp();
     const double *sp = s + 2 * t + 2 * (t >> 3);          // padded(2 t); word 2 t + 32 k is 36 k further
-    if (EP == 1) {
-        const uint32_t y = blockIdx.y + ep.y0, i = y % ep.level, comp = (y / ep.level) % ep.ncomp, bz = y / (ep.ncomp * ep.level);
+    if (EP == 1 || EP == 3) {
+        const uint32_t y = yl + ep.y0, i = y % ep.level, comp = (y / ep.level) % ep.ncomp, bz = y / (ep.ncomp * ep.level);
         const double2 pinv = ep.pinv[i];
         const uint32_t p0 = row * 256 + 2 * t;
         // grouped: entry bz is key bz / group applied to member bz % group (own: to the entry itself)
         const uint32_t rot = ep.group ? bz / ep.group : bz, mem = ep.group ? bz % ep.group : bz;
         const uint32_t gal = (uint32_t)(ep.multi ? ep.mgalois[rot] : ep.galois);
-        const u64 *up = ep.u.at(bz) + (((size_t)comp * ep.nt + i) << c.log_n) + p0;
-        const u64 *add = (ep.add_comps >> comp & 1) ? ep.add.at(ep.own ? bz : mem) + (((size_t)comp * ep.level + i) << c.log_n) : nullptr;
+        const u64 *add = (ep.add_comps >> comp & 1) ? ep.add.at(ep.own ? bz : mem) + (((size_t)comp * (EP == 3 ? ep.add_level : ep.level) + i) << c.log_n) : nullptr;
         const u64 *acc = ep.accumulate ? ep.acc.at(bz) + (((size_t)comp * ep.level + i) << c.log_n) + p0 : nullptr;
         const uint32_t bstep = ep.tl.R ? ep.tl.R * 64 : 64;    // words from one 64-word block of the destination to the next
         u64 *dst = ep.tl.R ? const_cast<u64 *>(ep.out.base) + tiled_index(ep.tl.R, c.N, ep.tl.row0 + rot * ep.rot_rows + (ep.group ? mem : bz) * ep.tl.row_stride + comp, i, row * 256) + 2 * t
                            : const_cast<u64 *>(ep.group ? ep.out.base + rot * ep.rot_stride + mem * ep.out.stride : ep.out.at(bz)) +
                                  (((size_t)comp * ep.level + i) << c.log_n) + p0;
+        if (EP == 3) {
+            // u = sum_j digit_j key_j; add joins it times P (rescale: the result is scaled by (P q_l)^-1) or the result as it is
+            const size_t ks = (size_t)2 * c.T << c.log_n;
+            const uint32_t de = ep.shared ? 0 : ep.group && !ep.own ? mem : bz, own = i / c.alpha;
+            const u64 *kp = (ep.multi ? ep.mevk[rot] : ep.evk) + (((size_t)comp * c.T + i) << c.log_n) + p0;
+            const u64 *eb = ep.ext + (((size_t)de * BETA * ep.nt + i) << c.log_n), *od = ep.d.at(de) + ((size_t)i << c.log_n);
+            const double pq = ADDP ? c.dn_p_mod_d[i] : 0.0;
+#pragma unroll
+            for (uint32_t k = 0; k < 8; k++) {
+                const uint32_t sr = galois_src(p0 + 32 * k, gal, c.log_n), so = sr & ~1u;
+                const bool odd = sr & 1;
+                ulonglong2 kv[BETA], ev[BETA], z;
+#pragma unroll
+                for (uint32_t j = 0; j < BETA; j++) {
+                    kv[j] = ld_pair<true>(kp + j * ks + 32 * k);
+                    ev[j] = ld_pair<true>((j == own ? od : eb + (((size_t)j * ep.nt) << c.log_n)) + so);
+                }
+                if (add) z = ld_pair<true>(add + so);
+                __syncwarp();
+                // the permutation maps the pair onto a pair, possibly swapped: summed in the digits' order, crossed with the key's
+                double s0 = 0.0, s1 = 0.0;
+                if (ADDP && add) { s0 = mulmod_dd(u64_to_d(z.x), pq, q, qinv); s1 = mulmod_dd(u64_to_d(z.y), pq, q, qinv); }
+#pragma unroll
+                for (uint32_t j = 0; j < BETA; j++) {
+                    s0 = __dadd_rn(s0, mulmod_dd(u64_to_d(ev[j].x), u64_to_d(odd ? kv[j].y : kv[j].x), q, qinv));
+                    s1 = __dadd_rn(s1, mulmod_dd(u64_to_d(ev[j].y), u64_to_d(odd ? kv[j].x : kv[j].y), q, qinv));
+                }
+                // |u - v| < (0.75 (BETA + 1) + 0.5) q <= 3.5 q, below 2^52: the product may round its quotient to even
+                if (BETA > 3) { s0 = reduce_d(s0, q, qinv); s1 = reduce_d(s1, q, qinv); }
+                const double2 v = *reinterpret_cast<const double2 *>(sp + 36 * k);
+                double r0 = mulmod_d<1>(__dsub_rn(odd ? s1 : s0, reduce_d(v.x, q, qinv)), pinv, q);
+                double r1 = mulmod_d<1>(__dsub_rn(odd ? s0 : s1, reduce_d(v.y, q, qinv)), pinv, q);
+                if (!ADDP && add) {
+                    r0 = __dadd_rn(r0, u64_to_d(odd ? z.y : z.x));
+                    r1 = __dadd_rn(r1, u64_to_d(odd ? z.x : z.y));
+                }
+                if (ep.accumulate) {
+                    const ulonglong2 o = ld_pair<true>(acc + 32 * k);
+                    r0 = __dadd_rn(r0, u64_to_d(o.x));
+                    r1 = __dadd_rn(r1, u64_to_d(o.y));
+                }
+                st_pair<true>(dst + (k >> 1) * bstep + (k & 1) * 32, make_ulonglong2(canonical_d(reduce_d(r0, q, qinv), q), canonical_d(reduce_d(r1, q, qinv), q)));
+            }
+            return;
+        }
+        const u64 *up = ep.u.at(bz) + (((size_t)comp * ep.nt + i) << c.log_n) + p0;
         // the other operands are fetched four pairs at a time, all in flight together (one pair per step, behind the step's
         // arithmetic, was latency bound: 332 us against 243 for 16 key switches at level 24)
         ulonglong2 ua[4], aa[4];
@@ -725,7 +774,11 @@ void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbM
             NttEpilogue e = ep ? *ep : NttEpilogue{};
             e.y0 = y0;
             const int mode = ep ? ep->mode : 0;
-            auto *k = mode == 1 ? (wide ? ntt_fwd_rows<1, true> : ntt_fwd_rows<1, false>)
+            static constexpr decltype(&ntt_fwd_rows<0, true>) inner[2][IP_FUSED_BETA] = {
+                {ntt_fwd_rows<3, true, 1>, ntt_fwd_rows<3, true, 2>, ntt_fwd_rows<3, true, 3>, ntt_fwd_rows<3, true, 4>},
+                {ntt_fwd_rows<3, true, 1, true>, ntt_fwd_rows<3, true, 2, true>, ntt_fwd_rows<3, true, 3, true>, ntt_fwd_rows<3, true, 4, true>}};
+            auto *k = mode == 3 ? inner[e.add_p][e.beta - 1]
+                    : mode == 1 ? (wide ? ntt_fwd_rows<1, true> : ntt_fwd_rows<1, false>)
                     : mode == 2 ? (wide ? ntt_fwd_rows<2, true> : ntt_fwd_rows<2, false>)
                                 : (wide ? ntt_fwd_rows<0, true> : ntt_fwd_rows<0, false>);
             launch(k, grid, 16 * ROW_CTA, 0, s, c->dev, b, map, share, e);
