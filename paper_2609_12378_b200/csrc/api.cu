@@ -171,8 +171,7 @@ extern "C" int32_t ckks_ntt(ckks_ctx *c, uint64_t *polys, uint32_t batch, uint32
     if ((uint64_t)first + nlimbs > c->T) return CKKS_ERR_LEVEL;
     DeviceGuard g(c->device);
     const LimbMap map = plain_map(first, nlimbs);
-    if (!launch_ntt_small(c, (u64 *)polys, batch * nlimbs, map, false, (cudaStream_t)stream))
-        launch_ntt(c, (u64 *)polys, batch * nlimbs, map, false, (cudaStream_t)stream);
+    launch_ntt(c, (u64 *)polys, batch * nlimbs, map, false, (cudaStream_t)stream, nullptr, nullptr, nullptr, nullptr, true);
     return finish(c);
 }
 
@@ -181,8 +180,7 @@ extern "C" int32_t ckks_intt(ckks_ctx *c, uint64_t *polys, uint32_t batch, uint3
     if ((uint64_t)first + nlimbs > c->T) return CKKS_ERR_LEVEL;
     DeviceGuard g(c->device);
     const LimbMap map = plain_map(first, nlimbs);
-    if (!launch_ntt_small(c, (u64 *)polys, batch * nlimbs, map, true, (cudaStream_t)stream))
-        launch_ntt(c, (u64 *)polys, batch * nlimbs, map, true, (cudaStream_t)stream);
+    launch_ntt(c, (u64 *)polys, batch * nlimbs, map, true, (cudaStream_t)stream, nullptr, nullptr, nullptr, nullptr, true);
     return finish(c);
 }
 
@@ -275,6 +273,7 @@ extern "C" int32_t ckks_mul_relin(ckks_ctx *c, const ckks_ct *a, const ckks_ct *
     cudaStream_t s = (cudaStream_t)stream;
     u64 *e2 = (u64 *)ws;
     KsWorkspace w = ks_carve(c, level, e2 + (size_t)level * c->N);
+    w.alone = true;
     u64 *o = (u64 *)out->data;
     auto view = [&](const ckks_ct *t) { return CtView{(const u64 *)t->data, (size_t)level * c->N}; };
     TensorArgs ta;
@@ -552,6 +551,7 @@ extern "C" int32_t ckks_rotate(ckks_ctx *c, const ckks_ct *in, const ckks_evk *k
     cudaStream_t s = (cudaStream_t)stream;
     const uint32_t level = in->level;
     KsWorkspace w = ks_carve(c, level, ws);
+    w.alone = true;
     rotate_ks(c, key, Ptrs((const u64 *)in->data, 0), Ptrs((const u64 *)out->data, 0), level, w, s);
     rc = finish(c);
     if (rc == CKKS_OK) { out->level = level; out->ncomp = 2; out->scale = in->scale; }
@@ -657,6 +657,7 @@ extern "C" int32_t ckks_rotate_hoisted(ckks_ctx *c, const ckks_ct *in, const ckk
     while (nbh > 1 && hoisted_bytes(c, level, nbh) > ws_bytes) nbh--;
     const size_t beta = (level + c->alpha - 1) / c->alpha, nt = level + c->K, N = c->N;
     KsWorkspace w;
+    w.alone = true;
     w.dcoef = (u64 *)ws;
     w.ext = w.dcoef + (size_t)level * N;
     w.u = w.ext + beta * nt * N;
@@ -684,7 +685,7 @@ extern "C" int32_t ckks_rescale(ckks_ctx *c, const ckks_ct *in, ckks_ct *out, vo
     if (!out->data || (in->ncomp > 1 && in->data == out->data)) return CKKS_ERR_ARG;
     if (!ws || ws_bytes < rescale_bytes(c, in->level, in->ncomp)) return CKKS_ERR_WORKSPACE;
     DeviceGuard g(c->device);
-    launch_rescale(c, Ptrs((const u64 *)in->data, 0), Ptrs((u64 *)out->data, 0), in->ncomp, in->level, (u64 *)ws, (cudaStream_t)stream);
+    launch_rescale(c, Ptrs((const u64 *)in->data, 0), Ptrs((u64 *)out->data, 0), in->ncomp, in->level, (u64 *)ws, (cudaStream_t)stream, 1, true);
     int rc = finish(c);
     if (rc == CKKS_OK) {
         const double ql = (double)c->mod[in->level - 1];

@@ -392,11 +392,11 @@ struct NttSource {
     Ptrs ptr;
     uint32_t lpitch = 0;
 };
+// alone: the chain of launches belongs to a short call of its own, which for a small ring the host bounds: fewest launches.
 // inv_scale (inverse): pairs [map.period][2] that replace {N^-1, last twiddle N^-1} for limb x of every period (device
 // pointer), so that the output is scaled by a per-limb constant.
 void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbMap &map, bool inverse, cudaStream_t s,
-                const NttEpilogue *ep = nullptr, const NttPrologue *pro = nullptr, const NttSource *src = nullptr, const double2 *inv_scale = nullptr);
-bool launch_ntt_small(const ckks_ctx *c, u64 *base, uint32_t nlimbs, const LimbMap &map, bool inverse, cudaStream_t s);
+                const NttEpilogue *ep = nullptr, const NttPrologue *pro = nullptr, const NttSource *src = nullptr, const double2 *inv_scale = nullptr, bool alone = false);
 void launch_ntt_int(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, bool inverse, const u64 *src, uint32_t src_pitch, cudaStream_t s);
 
 void launch_mul_plain_acc(const ckks_ctx *c, const u64 *const *cts, u64 *const *accs, uint32_t ncts, const u64 *pt,
@@ -434,6 +434,7 @@ void launch_lincomb(const ckks_ctx *c, const LinArgs &args, uint32_t n, uint32_t
 struct KsWorkspace {
     u64 *dcoef, *ext, *u, *conv;
     Ptrs d;
+    bool alone = false;     // the key switch is an entry point's only one: see launch_ntt
 };
 size_t ks_workspace_limbs(const ckks_ctx *c, uint32_t level);
 KsWorkspace ks_carve(const ckks_ctx *c, uint32_t level, void *ws, uint32_t nb = 1);
@@ -506,7 +507,8 @@ bool launch_mac_umma(const ckks_ctx *c, const u64 *baby, const u64 *pts, u64 *ac
                      cudaStream_t s, uint32_t Jx = 0, uint32_t j0 = 0, bool accumulate = false);
 
 // nb ciphertexts (at most KS_MULTI when the pointers are scattered) of ncomp components; ws: nb * ncomp * level limbs
-void launch_rescale(const ckks_ctx *c, const Ptrs &in, const Ptrs &out, uint32_t ncomp, uint32_t level, u64 *ws, cudaStream_t s, uint32_t nb = 1);
+void launch_rescale(const ckks_ctx *c, const Ptrs &in, const Ptrs &out, uint32_t ncomp, uint32_t level, u64 *ws, cudaStream_t s, uint32_t nb = 1,
+                    bool alone = false);
 
 size_t encode_workspace_bytes(const ckks_ctx *c, uint32_t batch);
 // tiled.R != 0: plaintext b is written as row tiled.row0 + b * tiled.row_stride of the tiled buffer

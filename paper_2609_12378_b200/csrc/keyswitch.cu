@@ -499,7 +499,7 @@ void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, 
     NttSource src;
     src.ptr = d; src.lpitch = 1;
     launch_ntt(c, w.dcoef, nb * level, plain_map(0, level), true, s, nullptr, nullptr, &src,
-               conv_tensor(c) ? nullptr : c->dev.inv_scale_up + (size_t)level * c->L * 2);
+               conv_tensor(c) ? nullptr : c->dev.inv_scale_up + (size_t)level * c->L * 2, w.alone);
     if (conv_tensor(c)) {
         launch_modup_mma(c, w.dcoef, w.ext, level, nb, s);
     } else {
@@ -507,7 +507,7 @@ void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, 
         DISPATCH_POW2(c->alpha, CALL_UP);
 #undef CALL_UP
     }
-    launch_ntt(c, w.ext, nb * beta * nt, ext_map(level, c->K, c->L, c->alpha, beta), false, s);
+    launch_ntt(c, w.ext, nb * beta * nt, ext_map(level, c->K, c->L, c->alpha, beta), false, s, nullptr, nullptr, nullptr, nullptr, w.alone);
 }
 
 void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w, cudaStream_t s, uint32_t nb,
@@ -594,7 +594,7 @@ static void moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, con
     const uint32_t N = c->N, nt = level + c->K, K = c->K;
     // the K special limbs of every (batch, component): groups of K limbs, nt limbs apart
     launch_ntt(c, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, nullptr, nullptr, nullptr,
-               conv_tensor(c) ? nullptr : c->dev.inv_scale_dn);
+               conv_tensor(c) ? nullptr : c->dev.inv_scale_dn, w.alone);
     if (conv_tensor(c)) {
         launch_moddown_conv_mma(c, w.u, w.conv, level, nb, s);
     } else {
@@ -684,14 +684,14 @@ void launch_sum(const ckks_ctx *c, u64 *dst, const u64 *first, const u64 *terms,
 // Four launches for the whole batch; copies of the last limbs, the lift and the final step were kernels of their own before
 // (10 operations, 63 -> 36 us for one ciphertext at N = 2^16, level 17).
 // ws: [nb][ncomp][N] last limbs + [nb][ncomp][level-1][N]
-void launch_rescale(const ckks_ctx *c, const Ptrs &in, const Ptrs &out, uint32_t ncomp, uint32_t level, u64 *ws, cudaStream_t s, uint32_t nb) {
+void launch_rescale(const ckks_ctx *c, const Ptrs &in, const Ptrs &out, uint32_t ncomp, uint32_t level, u64 *ws, cudaStream_t s, uint32_t nb, bool alone) {
     const size_t N = c->N;
     u64 *last = ws, *tmp = ws + (size_t)nb * ncomp * N;
     NttSource src;
     src.ptr = in; src.lpitch = level;
     if (in.n) for (uint32_t b = 0; b < in.n; b++) src.ptr.p[b] += (size_t)(level - 1) * N;
     else src.ptr.base += (size_t)(level - 1) * N;
-    launch_ntt(c, last, nb * ncomp, same_map(level - 1, ncomp), true, s, nullptr, nullptr, &src);
+    launch_ntt(c, last, nb * ncomp, same_map(level - 1, ncomp), true, s, nullptr, nullptr, &src, nullptr, alone);
     NttPrologue pro{last, true, level - 1};
     NttEpilogue ep{};
     ep.mode = 1;

@@ -660,7 +660,8 @@ __global__ void __launch_bounds__(ClShape<LOGR>::THREADS, 1024 / ClShape<LOGR>::
 }
 
 template <uint32_t LOGR>
-__global__ void __launch_bounds__(ClShape<LOGR>::THREADS, 1024 / ClShape<LOGR>::THREADS) ntt_inv_cluster(DevTables c, u64 *base, LimbMap map) {
+__global__ void __launch_bounds__(ClShape<LOGR>::THREADS, 1024 / ClShape<LOGR>::THREADS) ntt_inv_cluster(DevTables c, u64 *base, LimbMap map, const __grid_constant__ NttSource src,
+                                                                                                           const double2 *scale) {
     using S = ClShape<LOGR>;
     extern __shared__ __align__(16) double dsm[];
     const int prime = limb_prime(map, blockIdx.y);
@@ -672,7 +673,7 @@ __global__ void __launch_bounds__(ClShape<LOGR>::THREADS, 1024 / ClShape<LOGR>::
     double x[16];
     {
         const uint32_t t = threadIdx.x & 15, rl = threadIdx.x >> 4, row = rank * S::ROWS + rl;
-        const u64 *gs = limb + (size_t)row * 256;
+        const u64 *gs = (src.lpitch ? src.ptr.at(blockIdx.y / map.period) + (((size_t)(blockIdx.y % map.period) * src.lpitch) << c.log_n) : limb) + (size_t)row * 256;
         double *s = dsm + rl * ROW_PAD, *blk = s + 18 * t, *sp = s + 2 * t + 2 * (t >> 3);
         grid_dep_sync();
 #pragma unroll
@@ -710,7 +711,8 @@ __global__ void __launch_bounds__(ClShape<LOGR>::THREADS, 1024 / ClShape<LOGR>::
     }
     const uint32_t cc = threadIdx.x % S::COLS, r = threadIdx.x / S::COLS;
     constexpr uint32_t RS = S::R / 16;
-    const double2 c0 = c.n_inv_d[2 * prime], c1 = c.n_inv_d[2 * prime + 1];
+    const double2 *sc = scale ? scale + 2 * (blockIdx.y % map.period) : c.n_inv_d + 2 * prime;
+    const double2 c0 = sc[0], c1 = sc[1];
     if constexpr (S::B > 0) {
 #pragma unroll
         for (uint32_t k = 0; k < 16; k++) x[k] = dsm[(16 * r + k) * S::COLS + cc];
@@ -740,8 +742,27 @@ void launch_cols(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, boo
 
 }  // namespace
 
+// Transforms of a few limbs of a small ring without a fused prologue or epilogue, both passes in one launch.  Returns false outside
+// its range, N = 2^12 .. 2^14 and at most two CTAs per SM.  For short calls: these are bound by the host, whom a launch costs
+// 2 us (N = 2^14: product and rescale 53 -> 47 us; N = 2^13: rotation 33.5 -> 29.5 us), while on the device this kernel's 5.8 to
+// 7.8 us lose to the two passes' 2.3 to 3.7 us each, so that longer calls keep those (a 64 x 64 projection at N = 2^13: 177 against
+// 188 us).  At N = 2^16 the same form with 8 and 16 CTAs per cluster took 431 and 417 us against 305 for 768 limbs.
+static bool launch_ntt_small(const ckks_ctx *c, u64 *base, uint32_t nlimbs, const LimbMap &map, bool inverse, cudaStream_t s, const NttSource *src, const double2 *inv_scale) {
+    if (c->log_n < 12 || c->log_n > 14 || !aligned16(base) || (src && !aligned16(src->ptr))) return false;
+    auto run = [&](auto shape) {
+        using S = decltype(shape);
+        if (nlimbs * S::CL > 2 * (uint32_t)c->sms) return false;
+        const dim3 grid(S::CL, nlimbs);
+        if (inverse) launch_clusters(ntt_inv_cluster<S::LOG>, S::CL, grid, S::THREADS, S::SMEM, s, c->dev, base, map, src ? *src : NttSource{}, inv_scale);
+        else launch_clusters(ntt_fwd_cluster<S::LOG>, S::CL, grid, S::THREADS, S::SMEM, s, c->dev, base, map);
+        return true;
+    };
+    return c->log_n == 14 ? run(ClShape<6>()) : c->log_n == 13 ? run(ClShape<5>()) : run(ClShape<4>());
+}
+
 void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbMap &map, bool inverse, cudaStream_t s, const NttEpilogue *ep,
-                const NttPrologue *pro, const NttSource *src, const double2 *inv_scale) {
+                const NttPrologue *pro, const NttSource *src, const double2 *inv_scale, bool alone) {
+    if (alone && !ep && !pro && launch_ntt_small(c, base, nlimbs_total, map, inverse, s, src, inv_scale)) return;
     const uint32_t R = c->N >> 8;
     // the integer path (an option, N = 2^16) has no fused forms: those take all limbs on the FP64 pipe
     const uint32_t share = (ep || pro || inv_scale || (src && src->ptr.n) || c->log_n != 16) ? 8 : c->ntt_fp_share;
@@ -790,22 +811,6 @@ void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbM
         }
         if (share < 8) launch_ntt_int(c, b, ny, map, inverse, src ? sr.ptr.base : nullptr, src ? (uint32_t)(sr.ptr.stride >> c->log_n) : 0, s);
     }
-}
-
-// In-place transforms of a few limbs of a small ring, both passes in one launch: a call of its own is bound by the host, whom a
-// launch costs 2 us (both directions of 12 limbs at N = 2^13: 20.4 -> 17.7 us).  Returns false outside its range, N = 2^12 .. 2^14
-// and at most two CTAs per SM.  Inside chains of launches the two-pass form stays the better one: the device then is the bound,
-// and the passes' 2.2 to 2.9 us each, back to back, beat this kernel's 5.8 (product and rescale at N = 2^14: 42 against 53 us).
-// At N = 2^16 the same form with 8 and 16 CTAs per cluster took 431 and 417 us against 305 for 768 limbs.
-bool launch_ntt_small(const ckks_ctx *c, u64 *base, uint32_t nlimbs, const LimbMap &map, bool inverse, cudaStream_t s) {
-    if (c->log_n < 12 || c->log_n > 14 || !aligned16(base)) return false;
-    auto run = [&](auto shape) {
-        using S = decltype(shape);
-        if (nlimbs * S::CL > 2 * (uint32_t)c->sms) return false;
-        launch_clusters(inverse ? ntt_inv_cluster<S::LOG> : ntt_fwd_cluster<S::LOG>, S::CL, dim3(S::CL, nlimbs), S::THREADS, S::SMEM, s, c->dev, base, map);
-        return true;
-    };
-    return c->log_n == 14 ? run(ClShape<6>()) : c->log_n == 13 ? run(ClShape<5>()) : run(ClShape<4>());
 }
 
 // grid: three CTAs per SM, the residency of the transform kernels.  Returns the butterflies one launch performs.
