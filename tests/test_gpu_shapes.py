@@ -205,3 +205,51 @@ def test_projection_passes_by_shard_count(dnum, d_in, d_out, S, B, lazy):
     """How many rotations share a pass depends on the number of shards and digits."""
     from tests.test_gpu_linear import _run
     _run(10, 9, -(-9 // dnum), dnum, 9, d_in, d_out, 4 if d_in > 24 else 32, S, B, seed=760 + S, check_slots=False, lazy=lazy)
+
+
+@pytest.mark.parametrize("L,K,dnum,level", [(3, 1, 3, 3), (9, 9, 1, 9), (17, 17, 1, 16), (7, 4, 3, 5), (8, 1, 8, 8)])
+def test_products_that_drop_a_limb(L, K, dnum, level):
+    """ModDown and rescale in one step: one, two and three groups of eight special primes, full and partial digits, more digits
+    than the unrolled inner products take, the lowest level; inputs at the ends of the residues."""
+    from tests.gpu_util import context, ct_dev, host, key_dev
+    P, ctx = params(10, L, K, dnum), context(10, L, K, dnum)
+    o, g = P.oracle, inputs.rng(770, level + 100 * L)
+    x = inputs.uniform_residues(g, P.q[:level], P.N, 2)
+    for i in range(level):
+        x[:, i, ::7] = int(P.q[i]) - 1
+    rlk = inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, dnum * 2).reshape(dnum, 2, L + K, P.N)
+    coeffs = [0.25, -0.5, 0.75]
+    want, so = o.poly_eval(x, 2.0 ** 50, coeffs, rlk)
+    got = ctx.poly_eval(ct_dev(x, 2.0 ** 50), coeffs, key_dev(rlk, 0))
+    assert got.scale == so and np.array_equal(host(got.data), want)
+
+
+@pytest.mark.parametrize("dnum", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("level", [9, 10])
+def test_hoisted_rotations_with_and_without_a_stored_inner_product(dnum, level):
+    """Sixteen rotations at N = 2^13: at ten limbs and up to four digits they form the inner product in the last row pass, at nine
+    limbs or with five digits in a launch of its own."""
+    from tests.gpu_util import context, ct_dev, host, key_dev
+    K = -(-10 // dnum)
+    P, ctx = params(13, 10, K, dnum), context(13, 10, K, dnum)
+    o, g = P.oracle, inputs.rng(780, level + 100 * dnum)
+    ct = inputs.uniform_residues(g, P.q[:level], P.N, 2)
+    keys = [inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, dnum * 2).reshape(dnum, 2, 10 + K, P.N) for _ in range(16)]
+    gs = [o.galois_element(r) for r in range(1, 17)]
+    got = ctx.rotate_hoisted(ct_dev(ct, 1.0), [key_dev(k, e) for k, e in zip(keys, gs)])
+    for x, want in zip(got, o.rotate_hoisted(ct, keys, gs)):
+        assert np.array_equal(host(x.data), want)
+
+
+@pytest.mark.parametrize("dnum,level", [(1, 21), (3, 22), (4, 22), (3, 19)])
+def test_large_product_with_and_without_a_stored_inner_product(dnum, level):
+    """x^2 at N = 2^16 on either side of the size from which the last row pass forms the inner product."""
+    from tests.gpu_util import context, ct_dev, host, key_dev
+    K = -(-22 // dnum)
+    P, ctx = params(16, 22, K, dnum), context(16, 22, K, dnum)
+    o, g = P.oracle, inputs.rng(790, level + 100 * dnum)
+    x = inputs.uniform_residues(g, P.q[:level], P.N, 2)
+    rlk = inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, dnum * 2).reshape(dnum, 2, 22 + K, P.N)
+    want, so = o.poly_eval(x, 2.0 ** 50, [0.0, 0.5, 1.0], rlk)
+    got = ctx.poly_eval(ct_dev(x, 2.0 ** 50), [0.0, 0.5, 1.0], key_dev(rlk, 0))
+    assert got.scale == so and np.array_equal(host(got.data), want)
