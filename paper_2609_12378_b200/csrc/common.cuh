@@ -355,6 +355,8 @@ inline bool aligned16(const Ptrs &p) {
 //           tl.row0 + b * tl.row_stride + comp)
 //   mode 3: as mode 1, but the sum u is not read: it is formed here, u = <digits, key> (add_p: + P add, and nothing is
 //           added afterwards).  Digits are read through sigma_galois as well; beta <= IP_FUSED_BETA of them
+//           (inverse: the input is not read but formed as u, for the limbs x0 .. of the extended basis; the map's periods are the
+//           entries' components)
 //   mode 2: the transform's own result is stored, but into a tiled buffer (out.base): limb y = b * level + i becomes row
 //           tl.row0 + b * tl.row_stride, limb i
 constexpr uint32_t IP_FUSED_BETA = 4;
@@ -376,7 +378,7 @@ struct NttEpilogue {
     // rotation), the limbs per component of `add`, the batch
     const u64 *ext, *evk, *mevk[KS_MULTI];
     Ptrs d;
-    uint32_t beta, shared, add_level, add_p, nb;
+    uint32_t beta, shared, add_level, add_p, nb, x0;    // x0: (inverse) extended-basis limb of the map's first
     uint32_t y0;           // (filled in) first limb of the launch
 };
 // Prologue of the forward transform: the first pass reads one buffer [batch][N] (batch = limb index / map.period) instead of
@@ -446,9 +448,8 @@ void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, 
 // inner product with evk (digits read through sigma_{ext_galois}; 1 = identity): leaves u = <digits, evk> in the extended basis
 // (w.u, nb entries); with acc_u it adds to what w.u holds, so that a sum of key-switched terms can share one ks_moddown; with
 // `add` ([2][level][N] words per entry, no multi) it adds P add to both components.
-// Only limbs x0 .. level + K - 1 of the extended basis are formed.
 void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w, cudaStream_t s, uint32_t nb = 1,
-              bool acc_u = false, const KsMulti *multi = nullptr, const Ptrs *add = nullptr, uint32_t x0 = 0);
+              bool acc_u = false, const KsMulti *multi = nullptr, const Ptrs *add = nullptr);
 // ModDown and the final combination out_c = sigma_galois(add_c) + k_c + acc_c (add taken for the components in add_comps, acc if
 // given: [2][level][N] words per entry, possibly out itself)
 struct KsOut {

@@ -145,9 +145,9 @@ void launch_modup(const ckks_ctx *c, const u64 *dcoef, u64 *ext, uint32_t level,
 // u[comp][x][p] = sum_j ext[j][x][pi_g(p)] * evk[j][comp][kt(x)][p]          (any number of digits)
 __global__ void __launch_bounds__(THREADS) inner_product_generic_kernel(DevTables c, const u64 *ext, const __grid_constant__ Ptrs dp, uint32_t d0, const u64 *evk, u64 g,
                                                                         u64 *u, uint32_t level, int has_multi, const __grid_constant__ KsMulti multi, int acc_u, int has_add,
-                                                                        const __grid_constant__ Ptrs add, uint32_t x0) {
+                                                                        const __grid_constant__ Ptrs add) {
     const uint32_t p = blockIdx.x * THREADS + threadIdx.x;
-    const uint32_t x = blockIdx.z + x0, bz = blockIdx.y;     // batch varies faster than the limb: a key limb is reused from L2
+    const uint32_t x = blockIdx.z, bz = blockIdx.y;     // batch varies faster than the limb: a key limb is reused from L2
     const uint32_t nt = level + c.K, beta = (level + c.alpha - 1) / c.alpha;
     const uint32_t kt = x < level ? x : c.L + (x - level);
     if (has_multi) { evk = multi.evk[bz]; g = multi.galois[bz]; }     // shared digits, per-entry key and permutation
@@ -189,9 +189,9 @@ constexpr uint32_t IP_MAX_BETA = 8, IP_TERMS_MAX_BETA = 4;
 template <uint32_t BETA, bool ADD>
 __global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, const u64 *ext, const __grid_constant__ Ptrs d, const u64 *evk, u64 g, u64 *u,
                                                                 uint32_t level, uint32_t nb, uint32_t bch, int has_multi, const __grid_constant__ KsMulti multi,
-                                                                int acc_u, const __grid_constant__ Ptrs add, uint32_t x0) {
+                                                                int acc_u, const __grid_constant__ Ptrs add) {
     const uint32_t p = (blockIdx.x * THREADS + threadIdx.x) * 2;
-    const uint32_t x = blockIdx.z + x0;     // chunks of a limb run together: its key words (and shared digits) come from L2
+    const uint32_t x = blockIdx.z;     // chunks of a limb run together: its key words (and shared digits) come from L2
     uint32_t b0 = blockIdx.y * bch, b1 = min(b0 + bch, nb), e0 = has_multi ? 0 : b0;      // entries; first digits entry
     const uint32_t nt = level + c.K;
     const uint32_t kt = x < level ? x : c.L + (x - level);
@@ -511,7 +511,7 @@ void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, 
 }
 
 void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w, cudaStream_t s, uint32_t nb,
-              bool acc_u, const KsMulti *multi, const Ptrs *add, uint32_t x0) {
+              bool acc_u, const KsMulti *multi, const Ptrs *add) {
     const uint32_t N = c->N, nt = level + c->K;
     const uint32_t beta = (level + c->alpha - 1) / c->alpha;
     const int au = acc_u ? 1 : 0;
@@ -529,7 +529,7 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
                 wr.ext = w.ext + (size_t)r * multi->group * beta * nt * N;
                 wr.d.base += r * multi->group * w.d.stride;
             }
-            ks_inner(c, multi->evk[r], level, multi->galois[r], wr, s, multi->group, acc_u, nullptr, nullptr, x0);
+            ks_inner(c, multi->evk[r], level, multi->galois[r], wr, s, multi->group, acc_u, nullptr);
         }
         return;
     }
@@ -538,16 +538,16 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
         // batch entries per thread: enough chunks left to fill the machine, key words reused across a chunk
         const uint32_t grp = multi ? multi->group : 0, per = grp ? grp : nb;
         const uint32_t bch = (multi && !grp) ? 1 : (per >= 8 ? 4 : (per >= 4 ? 2 : 1));
-        const dim3 grid(N / (2 * THREADS), grp ? (nb / grp) * ((grp + bch - 1) / bch) : (nb + bch - 1) / bch, nt - x0);
+        const dim3 grid(N / (2 * THREADS), grp ? (nb / grp) * ((grp + bch - 1) / bch) : (nb + bch - 1) / bch, nt);
         using K = decltype(&inner_product_kernel<1, false>);
         static constexpr K plain[IP_MAX_BETA] = {inner_product_kernel<1, false>, inner_product_kernel<2, false>, inner_product_kernel<3, false>, inner_product_kernel<4, false>,
                                                  inner_product_kernel<5, false>, inner_product_kernel<6, false>, inner_product_kernel<7, false>, inner_product_kernel<8, false>};
         static constexpr K adding[IP_MAX_BETA] = {inner_product_kernel<1, true>, inner_product_kernel<2, true>, inner_product_kernel<3, true>, inner_product_kernel<4, true>,
                                                   inner_product_kernel<5, true>, inner_product_kernel<6, true>, inner_product_kernel<7, true>, inner_product_kernel<8, true>};
-        launch((add ? adding : plain)[beta - 1], grid, THREADS, 0, s, c->dev, w.ext, w.d, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au, pa, x0);
+        launch((add ? adding : plain)[beta - 1], grid, THREADS, 0, s, c->dev, w.ext, w.d, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au, pa);
     } else {
-        launch(inner_product_generic_kernel, dim3(N / THREADS, nb, nt - x0), THREADS, 0, s, c->dev, w.ext, w.d, 0u, evk, ext_galois, w.u, level, multi ? 1 : 0, m, au,
-               add ? 1 : 0, pa, x0);
+        launch(inner_product_generic_kernel, dim3(N / THREADS, nb, nt), THREADS, 0, s, c->dev, w.ext, w.d, 0u, evk, ext_galois, w.u, level, multi ? 1 : 0, m, au,
+               add ? 1 : 0, pa);
     }
 }
 
@@ -590,10 +590,11 @@ static NttEpilogue moddown_epilogue(const ckks_ctx *c, uint32_t level, const KsW
     }
     return ep;
 }
-static void moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const NttEpilogue &ep, cudaStream_t s, uint32_t nb) {
+static void moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, NttEpilogue ep, cudaStream_t s, uint32_t nb) {
     const uint32_t N = c->N, nt = level + c->K, K = c->K;
     // the K special limbs of every (batch, component): groups of K limbs, nt limbs apart
-    launch_ntt(c, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, nullptr, nullptr, nullptr,
+    ep.x0 = level;
+    launch_ntt(c, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, ep.mode == 3 ? &ep : nullptr, nullptr, nullptr,
                conv_tensor(c) ? nullptr : c->dev.inv_scale_dn, w.alone);
     if (conv_tensor(c)) {
         launch_moddown_conv_mma(c, w.u, w.conv, level, nb, s);
@@ -610,8 +611,8 @@ void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const K
 void ks_apply(const ckks_ctx *c, const u64 *evk, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb, const KsMulti *multi) {
     NttEpilogue ep = moddown_epilogue(c, level, w, o, nb, multi);
     const bool fused = inner_fused(c, level, w, evk, nb, multi) && out_aligned(ep);
-    ks_inner(c, evk, level, o.galois, w, s, nb, false, multi, nullptr, fused ? level : 0);
     if (fused) fuse_inner(c, level, w, evk, nb, multi, ep);
+    else ks_inner(c, evk, level, o.galois, w, s, nb, false, multi);
     moddown(c, level, w, ep, s, nb);
 }
 
@@ -629,13 +630,14 @@ void ks_apply_rescale(const ckks_ctx *c, const u64 *evk, uint32_t level, const K
     ep.pinv = c->dev.rs_p_inv_d + (size_t)m * c->L;
     ep.ncomp = 2; ep.level = m; ep.nt = nt; ep.galois = 1;
     const bool fused = inner_fused(c, level, w, evk, nb, nullptr) && out_aligned(ep) && aligned16(add);
-    ks_inner(c, evk, level, 1, w, s, nb, false, nullptr, &add, fused ? m : 0);
     if (fused) {
         fuse_inner(c, level, w, evk, nb, nullptr, ep);
-        ep.add = add; ep.add_comps = 3; ep.add_p = 1;
+        ep.add = add; ep.add_comps = 3; ep.add_p = 1; ep.x0 = m;
+    } else {
+        ks_inner(c, evk, level, 1, w, s, nb, false, nullptr, &add);
     }
     // the dropped limb and the K special limbs of every (batch, component), nt limbs apart
-    launch_ntt(c, w.u + (size_t)m * N, nb * 2 * (K + 1), tail_map(m, level, K, c->L), true, s, nullptr, nullptr, nullptr, c->dev.inv_scale_rs + (size_t)m * (K + 1) * 2);
+    launch_ntt(c, w.u + (size_t)m * N, nb * 2 * (K + 1), tail_map(m, level, K, c->L), true, s, fused ? &ep : nullptr, nullptr, nullptr, c->dev.inv_scale_rs + (size_t)m * (K + 1) * 2);
 #define CALL_DN(A) launch_moddown_conv<A, true>(c, w.u, w.conv, level, nb, s)
     DISPATCH_POW2(K, CALL_DN);
 #undef CALL_DN
@@ -656,7 +658,7 @@ void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, siz
     // any number of digits, any alignment: one term at a time through the generic kernel, then its P c0
     for (uint32_t t = 0; t < nterm; t++) {
         launch(inner_product_generic_kernel, dim3(N / THREADS, nb, nt), THREADS, 0, s, c->dev, w.ext + t * term_stride, w.d, t * nb, terms.evk[t], terms.galois[t],
-               w.u, level, 0, KsMulti{}, (acc_u || t > 0) ? 1 : 0, 0, Ptrs(), 0u);
+               w.u, level, 0, KsMulti{}, (acc_u || t > 0) ? 1 : 0, 0, Ptrs());
         if (terms.c0[t])
             launch(p_c0_acc_kernel, dim3(N / THREADS, level, nb), THREADS, 0, s, c->dev, terms.c0[t], c0_stride, terms.galois[t], w.u, (size_t)2 * nt * N);
     }
