@@ -383,10 +383,12 @@ struct NttEpilogue {
 };
 // Prologue of the forward transform: the first pass reads one buffer [batch][N] (batch = limb index / map.period) instead of
 // `base`: signed 64-bit coefficients, or (lift) residues modulo prime src_prime whose centred representatives are meant.
+// doubles: the buffer itself, which holds signed doubles of at most half a prime (the conversions' output).
 struct NttPrologue {
-    const u64 *src;
-    bool lift;
-    uint32_t src_prime;
+    const u64 *src = nullptr;
+    bool lift = false;
+    uint32_t src_prime = 0;
+    bool doubles = false;
 };
 // Source of the inverse transform: the first pass reads limb x of entry b at ptr.at(b) + x * lpitch limbs, so the transform
 // runs out of place and the input stays as it is (b = limb index / map.period, x = limb index % map.period).

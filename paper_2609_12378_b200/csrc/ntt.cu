@@ -258,10 +258,11 @@ struct ColShape {
     static constexpr uint32_t THREADS = R * COLS / E;
 };
 
-enum { SRC_LIMBS = 0, SRC_COEFS = 1, SRC_LIFT = 2 };
+enum { SRC_LIMBS = 0, SRC_COEFS = 1, SRC_LIFT = 2, SRC_DOUBLES = 3 };
 
 // forward: SRC_LIMBS in place; SRC_COEFS: signed 64-bit coefficients [batch][N], reduced modulo the limb's prime on load;
-// SRC_LIFT: one residue limb per period modulo prime src_prime, lifted to its centred representative (rescale)
+// SRC_LIFT: one residue limb per period modulo prime src_prime, lifted to its centred representative (rescale);
+// SRC_DOUBLES in place, signed doubles of at most q / 2 instead of residues (the conversions)
 template <uint32_t LOGR, int SRC>
 __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 1024 / ColShape<LOGR>::THREADS) ntt_fwd_cols(DevTables c, u64 *base, LimbMap map, uint32_t fp_share,
                                                                                                     const u64 *src, uint32_t src_prime) {
@@ -275,7 +276,7 @@ __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 1024 / ColShape<LOGR>
     const double *tw = c.twd_fwd + ((size_t)prime << c.log_n);
     const uint32_t cc = threadIdx.x % S::COLS, r = threadIdx.x / S::COLS;
     u64 *g = base + (limb_index(map, blockIdx.y) << c.log_n) + blockIdx.x * S::COLS + cc;
-    const u64 *gs = SRC == SRC_LIMBS ? g : src + ((size_t)(blockIdx.y / map.period) << c.log_n) + blockIdx.x * S::COLS + cc;
+    const u64 *gs = SRC == SRC_LIMBS || SRC == SRC_DOUBLES ? g : src + ((size_t)(blockIdx.y / map.period) << c.log_n) + blockIdx.x * S::COLS + cc;
     constexpr uint32_t RS = S::R / S::E;          // rows between a thread's registers in the first group
     double x[S::E];
     if (SH) stage_tw<S::R>(stw, tw);
@@ -303,6 +304,9 @@ __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 1024 / ColShape<LOGR>
 #pragma unroll
             for (uint32_t k = 0; k < S::E; k++) x[k] = __dsub_rn(__longlong_as_double(v[k] + 0x4338000000000000ll), MAGIC0);
         }
+    } else if (SRC == SRC_DOUBLES) {
+#pragma unroll
+        for (uint32_t k = 0; k < S::E; k++) x[k] = reinterpret_cast<const double *>(gs)[(size_t)(r + RS * k) * 256];
     } else if (SRC == SRC_LIFT) {
         const u64 ql = c.mod[src_prime];
 #pragma unroll
@@ -629,7 +633,7 @@ __device__ __forceinline__ uint32_t cluster_addr(const double *p, uint32_t rank)
 __device__ __forceinline__ void cluster_store(uint32_t a, double v) { asm volatile("st.shared::cluster.f64 [%0], %1;\n" ::"r"(a), "d"(v) : "memory"); }
 
 template <uint32_t LOGR>
-__global__ void __launch_bounds__(ClShape<LOGR>::THREADS, 1024 / ClShape<LOGR>::THREADS) ntt_fwd_cluster(DevTables c, u64 *base, LimbMap map) {
+__global__ void __launch_bounds__(ClShape<LOGR>::THREADS, 1024 / ClShape<LOGR>::THREADS) ntt_fwd_cluster(DevTables c, u64 *base, LimbMap map, bool doubles) {
     using S = ClShape<LOGR>;
     extern __shared__ __align__(16) double dsm[];
     const int prime = limb_prime(map, blockIdx.y);
@@ -645,7 +649,10 @@ __global__ void __launch_bounds__(ClShape<LOGR>::THREADS, 1024 / ClShape<LOGR>::
         const u64 *gs = limb + rank * S::COLS + cc;
         grid_dep_sync();
 #pragma unroll
-        for (uint32_t k = 0; k < 16; k++) x[k] = u64_to_d(gs[(size_t)(r + RS * k) * 256]);
+        for (uint32_t k = 0; k < 16; k++) {
+            const u64 v = gs[(size_t)(r + RS * k) * 256];
+            x[k] = doubles ? __longlong_as_double((long long)v) : u64_to_d(v);
+        }
         __syncwarp();
         fwd_col_group<LOGR, 0, 4>(x, 0, tw, 1, q, qinv);
         if constexpr (S::B > 0) {
@@ -776,6 +783,7 @@ void launch_cols(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, boo
     const uint32_t th = ColShape<LOGR>::THREADS;
     if (inverse) launch(ntt_inv_cols<LOGR>, grid, th, 0, s, c->dev, b, map, share, scale);
     else if (!pro) launch(ntt_fwd_cols<LOGR, SRC_LIMBS>, grid, th, 0, s, c->dev, b, map, share, (const u64 *)nullptr, 0u);
+    else if (pro->doubles) launch(ntt_fwd_cols<LOGR, SRC_DOUBLES>, grid, th, 0, s, c->dev, b, map, share, (const u64 *)nullptr, 0u);
     else if (pro->lift) launch(ntt_fwd_cols<LOGR, SRC_LIFT>, grid, th, 0, s, c->dev, b, map, share, pro->src, pro->src_prime);
     else launch(ntt_fwd_cols<LOGR, SRC_COEFS>, grid, th, 0, s, c->dev, b, map, share, pro->src, 0u);
 }
@@ -787,14 +795,14 @@ void launch_cols(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, boo
 // 2 us (N = 2^14: product and rescale 53 -> 47 us; N = 2^13: rotation 33.5 -> 29.5 us), while on the device this kernel's 5.8 to
 // 7.8 us lose to the two passes' 2.3 to 3.7 us each, so that longer calls keep those (a 64 x 64 projection at N = 2^13: 177 against
 // 188 us).  At N = 2^16 the same form with 8 and 16 CTAs per cluster took 431 and 417 us against 305 for 768 limbs.
-static bool launch_ntt_small(const ckks_ctx *c, u64 *base, uint32_t nlimbs, const LimbMap &map, bool inverse, cudaStream_t s, const NttSource *src, const double2 *inv_scale) {
+static bool launch_ntt_small(const ckks_ctx *c, u64 *base, uint32_t nlimbs, const LimbMap &map, bool inverse, cudaStream_t s, const NttSource *src, const double2 *inv_scale, bool doubles) {
     if (c->log_n < 12 || c->log_n > 14 || !aligned16(base) || (src && !aligned16(src->ptr))) return false;
     auto run = [&](auto shape) {
         using S = decltype(shape);
         if (nlimbs * S::CL > 2 * (uint32_t)c->sms) return false;
         const dim3 grid(S::CL, nlimbs);
         if (inverse) launch_clusters(ntt_inv_cluster<S::LOG>, S::CL, grid, S::THREADS, S::SMEM, s, c->dev, base, map, src ? *src : NttSource{}, inv_scale);
-        else launch_clusters(ntt_fwd_cluster<S::LOG>, S::CL, grid, S::THREADS, S::SMEM, s, c->dev, base, map);
+        else launch_clusters(ntt_fwd_cluster<S::LOG>, S::CL, grid, S::THREADS, S::SMEM, s, c->dev, base, map, doubles);
         return true;
     };
     return c->log_n == 14 ? run(ClShape<6>()) : c->log_n == 13 ? run(ClShape<5>()) : run(ClShape<4>());
@@ -802,7 +810,7 @@ static bool launch_ntt_small(const ckks_ctx *c, u64 *base, uint32_t nlimbs, cons
 
 void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbMap &map, bool inverse, cudaStream_t s, const NttEpilogue *ep,
                 const NttPrologue *pro, const NttSource *src, const double2 *inv_scale, bool alone) {
-    if (alone && !ep && !pro && launch_ntt_small(c, base, nlimbs_total, map, inverse, s, src, inv_scale)) return;
+    if (alone && !ep && (!pro || pro->doubles) && launch_ntt_small(c, base, nlimbs_total, map, inverse, s, src, inv_scale, pro != nullptr)) return;
     const uint32_t R = c->N >> 8;
     // the integer path (an option, N = 2^16) has no fused forms: those take all limbs on the FP64 pipe
     const uint32_t share = (ep || pro || inv_scale || (src && src->ptr.n) || c->log_n != 16) ? 8 : c->ntt_fp_share;
@@ -813,7 +821,8 @@ void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbM
         const uint32_t ny = nlimbs_total - y0 < chunk ? nlimbs_total - y0 : chunk;
         u64 *b = base + (limb_index(map, y0) << c->log_n);
         NttPrologue pr;
-        if (pro) { pr = *pro; pr.src += (size_t)(y0 / map.period) << c->log_n; }
+        if (pro) pr = *pro;
+        if (pr.src) { pr.src += (size_t)(y0 / map.period) << c->log_n; }
         NttSource sr;
         if (src) { sr = *src; if (!sr.ptr.n) sr.ptr.base += (size_t)(y0 / map.period) * sr.ptr.stride; }
         auto cols = [&]() {
