@@ -14,7 +14,10 @@
 
 namespace {
 
-constexpr uint32_t THREADS = 256;
+constexpr uint32_t THREADS = 256, TERM_THREADS = 128;
+// of the conversions: 128 threads even out what an SM gets (ModDown of products 184 -> 172 us in the degree-63 polynomial, the
+// hoisted rotations' 615 -> 601; 64 threads fetch their constants too often, 618)
+constexpr uint32_t CONV_THREADS = 128;
 
 // ---------------------------------------------------------------------------
 // Basis conversions: out[x] = sum_a y_a C[a][x] mod t_x with centred sources |y_a| <= q_a / 2 and centred constants
@@ -82,7 +85,7 @@ inline uint32_t conv_cpt(uint32_t ns, const void *a, const void *b) { return ns 
 // filled (one ciphertext at N = 2^16, level 24: ModUp with 24, 8, 5 targets per CTA 21.7, 22.7, 26.0 us).
 constexpr uint32_t CONV_CHUNK_MAX = 32;
 inline uint32_t conv_chunk(uint32_t gx, uint32_t items, uint32_t targets) {
-    const uint32_t want = 2 * 148;
+    const uint32_t want = 2 * 148 * 256 / CONV_THREADS;
     uint32_t chunks = (want + gx * items - 1) / (gx * items);
     chunks = std::max(1u, std::min(chunks, (targets + 1) / 2));
     return std::min(CONV_CHUNK_MAX, (targets + chunks - 1) / chunks);
@@ -93,17 +96,17 @@ inline uint32_t conv_chunk(uint32_t gx, uint32_t items, uint32_t targets) {
 // limbs (blockIdx.y), so the source limbs are read once per chunk.
 // dcoef already holds [d_a qhat_a^-1] (the inverse transform multiplied it in), so only the centring is left.
 template <uint32_t ALPHA, uint32_t CPT>
-__global__ void __launch_bounds__(THREADS) modup_kernel(DevTables c, const u64 *dcoef, u64 *ext, uint32_t level, uint32_t CHUNK) {
+__global__ void __launch_bounds__(CONV_THREADS) modup_kernel(DevTables c, const u64 *dcoef, u64 *ext, uint32_t level, uint32_t CHUNK) {
     // the CTA's conversion constants (qhat_a mod t; t and 1/t), fetched once
     __shared__ __align__(16) double s_w[CONV_CHUNK_MAX][ALPHA];
     __shared__ double2 s_m[CONV_CHUNK_MAX];
-    const uint32_t k = (blockIdx.x * THREADS + threadIdx.x) * CPT;
+    const uint32_t k = (blockIdx.x * CONV_THREADS + threadIdx.x) * CPT;
     const uint32_t beta = (level + c.alpha - 1) / c.alpha, j = blockIdx.z % beta, bz = blockIdx.z / beta;
     const uint32_t nt = level + c.K, lo = j * c.alpha, hi = min(lo + c.alpha, level), nd = hi - lo;
     const uint32_t x0 = blockIdx.y * CHUNK, x1 = min(x0 + CHUNK, nt - nd);       // targets, counted without the digit's own limbs
     if (x0 >= x1) return;
     const size_t cb = (size_t)level * c.dnum + j;
-    for (uint32_t e = threadIdx.x; e < (x1 - x0) * ALPHA; e += THREADS) {
+    for (uint32_t e = threadIdx.x; e < (x1 - x0) * ALPHA; e += CONV_THREADS) {
         const uint32_t xi = e / ALPHA, a = e % ALPHA, xt = x0 + xi, x = xt < lo ? xt : xt + nd, t = x < level ? x : c.L + (x - level);
         s_w[xi][a] = a < nd ? c.up_hat_mod_d[(cb * c.T + t) * c.alpha + a] : 0.0;
         if (a == 0) s_m[xi] = c.modd[t];
@@ -137,11 +140,11 @@ __global__ void __launch_bounds__(THREADS) modup_kernel(DevTables c, const u64 *
 template <uint32_t ALPHA>
 void launch_modup(const ckks_ctx *c, const u64 *dcoef, u64 *ext, uint32_t level, uint32_t nb, cudaStream_t s) {
     const uint32_t nt = level + c->K, beta = (level + c->alpha - 1) / c->alpha;
-    const uint32_t cpt = conv_cpt(ALPHA, dcoef, ext), gx = c->N / (THREADS * cpt), targets = nt - (level - (beta - 1) * c->alpha);   // the last digit has the most targets
+    const uint32_t cpt = conv_cpt(ALPHA, dcoef, ext), gx = c->N / (CONV_THREADS * cpt), targets = nt - (level - (beta - 1) * c->alpha);   // the last digit has the most targets
     const uint32_t CHUNK = conv_chunk(gx, beta * nb, targets);
     const dim3 grid(gx, (targets + CHUNK - 1) / CHUNK, beta * nb);
     constexpr uint32_t WIDE = ALPHA <= 8 ? 2 : 1;
-    launch(cpt == WIDE ? modup_kernel<ALPHA, WIDE> : modup_kernel<ALPHA, 1>, grid, THREADS, 0, s, c->dev, dcoef, ext, level, CHUNK);
+    launch(cpt == WIDE ? modup_kernel<ALPHA, WIDE> : modup_kernel<ALPHA, 1>, grid, CONV_THREADS, 0, s, c->dev, dcoef, ext, level, CHUNK);
 }
 
 // u[comp][x][p] = sum_j ext[j][x][pi_g(p)] * evk[j][comp][kt(x)][p]          (any number of digits)
@@ -276,12 +279,14 @@ __global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, con
 // The inner product of several terms at once (see ks_inner_terms): like inner_product_kernel, but every term has its
 // own digits, key, permutation and first component, and the running sums of a chunk of IP_BCH batch entries stay in
 // registers over the terms.
-constexpr uint32_t IP_BCH = 4;
+// Two entries per thread at 64 registers and 32 warps per SM: four entries at 85 registers kept too few loads in flight (the
+// 4096 x 4096 projection's share: 20.2 -> 17.4 ms; one entry 19.9, two at 48 registers 21.3).
+constexpr uint32_t IP_BCH = 2;
 template <uint32_t BETA>
-__global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTables c, const u64 *ext, size_t term_stride, const u64 *d, size_t d_stride,
+__global__ void __launch_bounds__(TERM_THREADS, 8) inner_product_terms_kernel(DevTables c, const u64 *ext, size_t term_stride, const u64 *d, size_t d_stride,
                                                                          const __grid_constant__ IpTerms tm, uint32_t nterm, size_t c0_stride,
                                                                          u64 *u, uint32_t level, uint32_t nb, int acc_u) {
-    const uint32_t p = (blockIdx.x * THREADS + threadIdx.x) * 2;
+    const uint32_t p = (blockIdx.x * TERM_THREADS + threadIdx.x) * 2;
     const uint32_t x = blockIdx.z, b0 = blockIdx.y * IP_BCH;
     const uint32_t nt = level + c.K;
     const uint32_t kt = x < level ? x : c.L + (x - level);
@@ -366,15 +371,15 @@ __global__ void __launch_bounds__(THREADS, 3) inner_product_terms_kernel(DevTabl
 // gets P r on top, so that (u_i - NTT(conv_i + P r)) (P q_l)^-1 is the rescaled ModDown: one transform of each remaining
 // limb, where ModDown and rescale after each other take two (and four more launches).
 template <uint32_t KK, uint32_t CPT, bool RS>
-__global__ void __launch_bounds__(THREADS) moddown_conv_kernel(DevTables c, const u64 *u, u64 *conv, uint32_t level, uint32_t targets, uint32_t CHUNK) {
+__global__ void __launch_bounds__(CONV_THREADS) moddown_conv_kernel(DevTables c, const u64 *u, u64 *conv, uint32_t level, uint32_t targets, uint32_t CHUNK) {
     __shared__ __align__(16) double s_w[CONV_CHUNK_MAX + RS][KK];     // Phat_a mod q_i (the last row: of the dropped limb)
     __shared__ double2 s_m[CONV_CHUNK_MAX];                           // q_i, 1 / q_i
     __shared__ double s_p[RS ? CONV_CHUNK_MAX : 1];                   // P mod q_i
-    const uint32_t k = (blockIdx.x * THREADS + threadIdx.x) * CPT;
+    const uint32_t k = (blockIdx.x * CONV_THREADS + threadIdx.x) * CPT;
     const uint32_t comp = blockIdx.z & 1, bz = blockIdx.z >> 1;
     const uint32_t nt = level + c.K;
     const uint32_t i0 = blockIdx.y * CHUNK, i1 = min(i0 + CHUNK, targets);
-    for (uint32_t e = threadIdx.x; e < (i1 - i0) * KK; e += THREADS) {
+    for (uint32_t e = threadIdx.x; e < (i1 - i0) * KK; e += CONV_THREADS) {
         const uint32_t ii = e / KK, a = e % KK;
         s_w[ii][a] = a < c.K ? c.dn_hat_mod_d[(size_t)(i0 + ii) * c.K + a] : 0.0;
         if (a == 0) s_m[ii] = c.modd[i0 + ii];
@@ -421,10 +426,10 @@ __global__ void __launch_bounds__(THREADS) moddown_conv_kernel(DevTables c, cons
 
 template <uint32_t KK, bool RS>
 void launch_moddown_conv(const ckks_ctx *c, const u64 *u, u64 *conv, uint32_t level, uint32_t nb, cudaStream_t s) {
-    const uint32_t targets = level - RS, cpt = conv_cpt(KK, u, conv), gx = c->N / (THREADS * cpt), CHUNK = conv_chunk(gx, 2 * nb, targets);
+    const uint32_t targets = level - RS, cpt = conv_cpt(KK, u, conv), gx = c->N / (CONV_THREADS * cpt), CHUNK = conv_chunk(gx, 2 * nb, targets);
     const dim3 grid(gx, (targets + CHUNK - 1) / CHUNK, 2 * nb);
     constexpr uint32_t WIDE = KK <= 8 ? 2 : 1;
-    launch(cpt == WIDE ? moddown_conv_kernel<KK, WIDE, RS> : moddown_conv_kernel<KK, 1, RS>, grid, THREADS, 0, s, c->dev, u, conv, level, targets, CHUNK);
+    launch(cpt == WIDE ? moddown_conv_kernel<KK, WIDE, RS> : moddown_conv_kernel<KK, 1, RS>, grid, CONV_THREADS, 0, s, c->dev, u, conv, level, targets, CHUNK);
 }
 
 // register-array size for a digit / special-prime count: next of 1, 2, 4, 8, 16, 32, 64
@@ -654,9 +659,9 @@ void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, siz
     bool aligned = aligned16(w.ext) && aligned16(w.u) && (term_stride & 1) == 0 && (c0_stride & 1) == 0 && aligned16(w.d);
     for (uint32_t t = 0; t < nterm; t++) aligned = aligned && aligned16(terms.evk[t]) && aligned16(terms.c0[t]);
     if (beta <= IP_TERMS_MAX_BETA && aligned) {
-        const dim3 grid(N / (2 * THREADS), (nb + IP_BCH - 1) / IP_BCH, nt);
+        const dim3 grid(N / (2 * TERM_THREADS), (nb + IP_BCH - 1) / IP_BCH, nt);
         auto *k = beta == 1 ? inner_product_terms_kernel<1> : beta == 2 ? inner_product_terms_kernel<2> : beta == 3 ? inner_product_terms_kernel<3> : inner_product_terms_kernel<4>;
-        launch(k, grid, THREADS, 0, s, c->dev, w.ext, term_stride, w.d.base, w.d.stride, terms, nterm, c0_stride, w.u, level, nb, acc_u ? 1 : 0);
+        launch(k, grid, TERM_THREADS, 0, s, c->dev, w.ext, term_stride, w.d.base, w.d.stride, terms, nterm, c0_stride, w.u, level, nb, acc_u ? 1 : 0);
         return;
     }
     // any number of digits, any alignment: one term at a time through the generic kernel, then its P c0
