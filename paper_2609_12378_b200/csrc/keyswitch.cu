@@ -14,7 +14,7 @@
 
 namespace {
 
-constexpr uint32_t THREADS = 256, TERM_THREADS = 128;
+constexpr uint32_t THREADS = 256, IP_THREADS = 128;
 // of the conversions: 128 threads even out what an SM gets (ModDown of products 184 -> 172 us in the degree-63 polynomial, the
 // hoisted rotations' 615 -> 601; 64 threads fetch their constants too often, 618)
 constexpr uint32_t CONV_THREADS = 128;
@@ -192,10 +192,10 @@ __global__ void __launch_bounds__(THREADS) inner_product_generic_kernel(DevTable
 // of up to KS_MULTI keys applied to the same digits.
 constexpr uint32_t IP_MAX_BETA = 8, IP_TERMS_MAX_BETA = 4;
 template <uint32_t BETA, bool ADD>
-__global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, const u64 *ext, const __grid_constant__ Ptrs d, const u64 *evk, u64 g, u64 *u,
+__global__ void __launch_bounds__(IP_THREADS) inner_product_kernel(DevTables c, const u64 *ext, const __grid_constant__ Ptrs d, const u64 *evk, u64 g, u64 *u,
                                                                 uint32_t level, uint32_t nb, uint32_t bch, int has_multi, const __grid_constant__ KsMulti multi,
                                                                 int acc_u, const __grid_constant__ Ptrs add) {
-    const uint32_t p = (blockIdx.x * THREADS + threadIdx.x) * 2;
+    const uint32_t p = (blockIdx.x * IP_THREADS + threadIdx.x) * 2;
     const uint32_t x = blockIdx.z;     // chunks of a limb run together: its key words (and shared digits) come from L2
     uint32_t b0 = blockIdx.y * bch, b1 = min(b0 + bch, nb), e0 = has_multi ? 0 : b0;      // entries; first digits entry
     const uint32_t nt = level + c.K;
@@ -283,10 +283,10 @@ __global__ void __launch_bounds__(THREADS) inner_product_kernel(DevTables c, con
 // 4096 x 4096 projection's share: 20.2 -> 17.4 ms; one entry 19.9, two at 48 registers 21.3).
 constexpr uint32_t IP_BCH = 2;
 template <uint32_t BETA>
-__global__ void __launch_bounds__(TERM_THREADS, 8) inner_product_terms_kernel(DevTables c, const u64 *ext, size_t term_stride, const u64 *d, size_t d_stride,
+__global__ void __launch_bounds__(IP_THREADS, 8) inner_product_terms_kernel(DevTables c, const u64 *ext, size_t term_stride, const u64 *d, size_t d_stride,
                                                                          const __grid_constant__ IpTerms tm, uint32_t nterm, size_t c0_stride,
                                                                          u64 *u, uint32_t level, uint32_t nb, int acc_u) {
-    const uint32_t p = (blockIdx.x * TERM_THREADS + threadIdx.x) * 2;
+    const uint32_t p = (blockIdx.x * IP_THREADS + threadIdx.x) * 2;
     const uint32_t x = blockIdx.z, b0 = blockIdx.y * IP_BCH;
     const uint32_t nt = level + c.K;
     const uint32_t kt = x < level ? x : c.L + (x - level);
@@ -544,16 +544,17 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
     }
     const KsMulti m = multi ? *multi : KsMulti{};
     if (fast) {
-        // batch entries per thread: enough chunks left to fill the machine, key words reused across a chunk
+        // batch entries per thread: enough chunks left to fill the machine, key words reused across a chunk (sixteen entries, 4 ->
+        // 8 per thread: 13.9 -> 12.7 ms of the 4096 x 4096 projection; half of these shares: 15.9 ms)
         const uint32_t grp = multi ? multi->group : 0, per = grp ? grp : nb;
-        const uint32_t bch = (multi && !grp) ? 1 : (per >= 8 ? 4 : (per >= 4 ? 2 : 1));
-        const dim3 grid(N / (2 * THREADS), grp ? (nb / grp) * ((grp + bch - 1) / bch) : (nb + bch - 1) / bch, nt);
+        const uint32_t bch = (multi && !grp) ? 1 : (per >= 16 ? 8 : per >= 8 ? 4 : per >= 4 ? 2 : 1);
+        const dim3 grid(N / (2 * IP_THREADS), grp ? (nb / grp) * ((grp + bch - 1) / bch) : (nb + bch - 1) / bch, nt);
         using K = decltype(&inner_product_kernel<1, false>);
         static constexpr K plain[IP_MAX_BETA] = {inner_product_kernel<1, false>, inner_product_kernel<2, false>, inner_product_kernel<3, false>, inner_product_kernel<4, false>,
                                                  inner_product_kernel<5, false>, inner_product_kernel<6, false>, inner_product_kernel<7, false>, inner_product_kernel<8, false>};
         static constexpr K adding[IP_MAX_BETA] = {inner_product_kernel<1, true>, inner_product_kernel<2, true>, inner_product_kernel<3, true>, inner_product_kernel<4, true>,
                                                   inner_product_kernel<5, true>, inner_product_kernel<6, true>, inner_product_kernel<7, true>, inner_product_kernel<8, true>};
-        launch((add ? adding : plain)[beta - 1], grid, THREADS, 0, s, c->dev, w.ext, w.d, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au, pa);
+        launch((add ? adding : plain)[beta - 1], grid, IP_THREADS, 0, s, c->dev, w.ext, w.d, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au, pa);
     } else {
         launch(inner_product_generic_kernel, dim3(N / THREADS, nb, nt), THREADS, 0, s, c->dev, w.ext, w.d, 0u, evk, ext_galois, w.u, level, multi ? 1 : 0, m, au,
                add ? 1 : 0, pa);
@@ -659,9 +660,9 @@ void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, siz
     bool aligned = aligned16(w.ext) && aligned16(w.u) && (term_stride & 1) == 0 && (c0_stride & 1) == 0 && aligned16(w.d);
     for (uint32_t t = 0; t < nterm; t++) aligned = aligned && aligned16(terms.evk[t]) && aligned16(terms.c0[t]);
     if (beta <= IP_TERMS_MAX_BETA && aligned) {
-        const dim3 grid(N / (2 * TERM_THREADS), (nb + IP_BCH - 1) / IP_BCH, nt);
+        const dim3 grid(N / (2 * IP_THREADS), (nb + IP_BCH - 1) / IP_BCH, nt);
         auto *k = beta == 1 ? inner_product_terms_kernel<1> : beta == 2 ? inner_product_terms_kernel<2> : beta == 3 ? inner_product_terms_kernel<3> : inner_product_terms_kernel<4>;
-        launch(k, grid, TERM_THREADS, 0, s, c->dev, w.ext, term_stride, w.d.base, w.d.stride, terms, nterm, c0_stride, w.u, level, nb, acc_u ? 1 : 0);
+        launch(k, grid, IP_THREADS, 0, s, c->dev, w.ext, term_stride, w.d.base, w.d.stride, terms, nterm, c0_stride, w.u, level, nb, acc_u ? 1 : 0);
         return;
     }
     // any number of digits, any alignment: one term at a time through the generic kernel, then its P c0
