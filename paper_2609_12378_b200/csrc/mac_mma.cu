@@ -124,32 +124,34 @@ __global__ void __launch_bounds__(COEF * 32 * NC / NW, CTAS) mac_mma_kernel(DevT
     TileIt lt;                                    // tile of the step the loader issues next
     lt.init(t_begin, coltiles, gtiles, xblocks);
     uint32_t lks = 0, lstep = 0;
-    const u64 *wrow = nullptr, *xrow = nullptr;   // row j of the step, giant 0 / shard 0, this thread's chunk
-    uint32_t lg0 = 0, lsh0 = 0, lsm = 0;
+    // this thread's chunk of row j of the step at its first giant / shard, the bytes from one to the next, and how many follow it
+    const u64 *wrow = nullptr, *xrow = nullptr;
+    const uint32_t wstep = J * 512, xstep = Jx * 1024;
+    uint32_t wleft = 0, xleft = 0, lsm = 0;
     auto load_begin = [&]() {
         if (lstep < nsteps) {
             // tiled_index(R, N, r, i, p) = blk * R * 64 + r * 64 + p % 64, blk = i * N/64 + p/64
             const size_t blk = (size_t)lt.i * (c.N >> 6) + lt.xb / XB64;
             const uint32_t in_blk = (lt.xb % XB64) * COEF + 2 * ch, j = lks * MK + jj;
-            wrow = pts + blk * Rw * 64 + in_blk + (size_t)j * 64;
-            xrow = baby + blk * Rx * 64 + in_blk + (size_t)(2 * (j0 + j) + (arow & 1)) * 64;
-            lg0 = lt.zg * MG + arow;
-            lsh0 = lt.zc * (MS / 2) + (arow >> 1);
+            const uint32_t g = min(lt.zg * MG + arow, G - 1), sh = min(lt.zc * (MS / 2) + (arow >> 1), S - 1);
+            wrow = pts + blk * Rw * 64 + in_blk + ((size_t)g * J + j) * 64;
+            xrow = baby + blk * Rx * 64 + in_blk + ((size_t)sh * 2 * Jx + 2 * (j0 + j) + (arow & 1)) * 64;
+            wleft = G - 1 - g;
+            xleft = S - 1 - sh;
             lsm = sm_thread + (lstep % STAGES) * T::STAGE_BYTES;
         }
     };
     // rows beyond the last giant or shard re-read the last valid one; their results are never stored
     auto load_w = [&](uint32_t k) {
         if (lstep < nsteps) {
-            const uint32_t g = min(lg0 + AH * k, G - 1);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(lsm + k * AH * T::GPITCH), "l"(wrow + (size_t)g * J * 64) : "memory");
+            const u64 src = mad_wide(min(AH * k, wleft), wstep, (u64)(uintptr_t)wrow);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(lsm + k * AH * T::GPITCH), "l"(src) : "memory");
         }
     };
     auto load_x = [&](uint32_t k) {
         if (lstep < nsteps) {
-            const uint32_t sh = min(lsh0 + (AH / 2) * k, S - 1);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(lsm + T::BOX_BYTES + k * AH * T::GPITCH), "l"(xrow + (size_t)sh * Jx * 128)
-                         : "memory");
+            const u64 src = mad_wide(min((AH / 2) * k, xleft), xstep, (u64)(uintptr_t)xrow);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(lsm + T::BOX_BYTES + k * AH * T::GPITCH), "l"(src) : "memory");
         }
     };
     auto load_end = [&]() {
@@ -176,15 +178,23 @@ __global__ void __launch_bounds__(COEF * 32 * NC / NW, CTAS) mac_mma_kernel(DevT
     uint32_t pend_g0 = 0, pend_col0 = 0;
     u64 pend_q = 0;
     const size_t lN = (size_t)level * c.N;
+    // a thread writes one column: rows of giants fg, fg + FG, ..
+    constexpr uint32_t FG = THREADS / COEF / MS;
+    static_assert(FG * MS * COEF == THREADS, "a pass over the staged rows covers whole giants");
+    const uint32_t fsl = tid % COEF, fcol = (tid / COEF) % MS, fg = tid / COEF / MS;
+    const size_t fstep = FG * ncol * lN;
     auto flush = [&]() {
+        if (pend_col0 + fcol < ncol) {
+            u64 *dst = pend + ((size_t)(pend_g0 + fg) * ncol + pend_col0 + fcol) * lN;
+            const uint32_t gleft = G - pend_g0;
 #pragma unroll
-        for (uint32_t k = 0; k < MG * MS * COEF / THREADS; k++) {
-            const uint32_t row = k * (THREADS / COEF) + tid / COEF, sl = tid % COEF, gl = row / MS, cl = row % MS;
-            const uint32_t g = pend_g0 + gl, col = pend_col0 + cl;
-            if (g < G && col < ncol) {
-                u64 *dst = pend + ((size_t)g * ncol + col) * lN + (sl ^ (gl % COEF));
-                const u64 v = obuf[row * COEF + sl];
-                *dst = accumulate ? add_mod(v, *dst, pend_q) : v;
+            for (uint32_t k = 0; k < MG / FG; k++, dst += fstep) {
+                const uint32_t gl = fg + k * FG;
+                if (gl < gleft) {
+                    u64 *o = dst + (fsl ^ (gl % COEF));
+                    const u64 v = obuf[(gl * MS + fcol) * COEF + fsl];
+                    *o = accumulate ? add_mod(v, *o, pend_q) : v;
+                }
             }
         }
         pend = nullptr;
