@@ -583,7 +583,7 @@ def run_cuda(args):
     hbm_achieved = ntt_bytes / (ntt_fwd_ms * 1e-3) / 1e9
     roofline = alu(ops, ntt_fwd_ms)
     roofline.update({
-        "kernel": "ntt16_fwd_cols + ntt16_fwd_rows (forward NTT of 768 limbs, one launch each)",
+        "kernel": "ntt_fwd_cols + ntt_fwd_rows (forward NTT of 768 limbs, one launch each)",
         # ncu, dram read + write bytes of the two launches; None when no capture of the current kernels is recorded
         "traffic": profile_figure("ntt16_384limbs.md", "dram_bytes_per_launch_pair"),
         "ms_per_launch_pair": ntt_fwd_ms,
