@@ -401,7 +401,7 @@ struct NttSource {
 // pointer), so that the output is scaled by a per-limb constant.
 void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbMap &map, bool inverse, cudaStream_t s,
                 const NttEpilogue *ep = nullptr, const NttPrologue *pro = nullptr, const NttSource *src = nullptr, const double2 *inv_scale = nullptr, bool alone = false);
-void launch_ntt_int(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, bool inverse, const u64 *src, uint32_t src_pitch, cudaStream_t s);
+void launch_ntt_int(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, bool inverse, const NttSource &src, cudaStream_t s);
 
 void launch_mul_plain_acc(const ckks_ctx *c, const u64 *const *cts, u64 *const *accs, uint32_t ncts, const u64 *pt,
                           uint32_t level, bool init, cudaStream_t s);

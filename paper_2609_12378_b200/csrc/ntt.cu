@@ -861,7 +861,7 @@ void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbM
             else launch(wide ? ntt_inv_rows<true> : ntt_inv_rows<false>, grid, 16 * ROW_CTA, 0, s, c->dev, b, map, share, src ? sr : none);
             cols();
         }
-        if (share < 8) launch_ntt_int(c, b, ny, map, inverse, src ? sr.ptr.base : nullptr, src ? (uint32_t)(sr.ptr.stride >> c->log_n) : 0, s);
+        if (share < 8) launch_ntt_int(c, b, ny, map, inverse, sr, s);
     }
 }
 

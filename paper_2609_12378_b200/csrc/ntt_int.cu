@@ -125,7 +125,8 @@ __global__ void __launch_bounds__(THREADS) int_fwd_rows(DevTables c, u64 *base, 
     for (uint32_t k = 0; k < 16; k++) g[t + 16 * k] = s[padded(t + 16 * k)];
 }
 
-__global__ void __launch_bounds__(THREADS) int_inv_rows(DevTables c, u64 *base, LimbMap map, uint32_t fp_share, const u64 *src, uint32_t src_pitch) {
+// src (if any): limb x of entry y / period lies at src + entry * src_stride words + x * src_lpitch limbs
+__global__ void __launch_bounds__(THREADS) int_inv_rows(DevTables c, u64 *base, LimbMap map, uint32_t fp_share, const u64 *src, size_t src_stride, uint32_t src_lpitch) {
     grid_dep_sync();
     __shared__ u64 sm[16 * ROW_PAD];
     const int prime = limb_prime(map, blockIdx.y);
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(THREADS) int_inv_rows(DevTables c, u64 *base, 
     const ulonglong2 *tw = c.tw_inv + ((size_t)prime << 16);
     const uint32_t t = threadIdx.x & 15, rl = threadIdx.x >> 4, row = blockIdx.x * 16 + rl;
     u64 *g = base + (limb_index(map, blockIdx.y) << 16) + (size_t)row * 256;
-    const u64 *gs = src ? src + ((((size_t)(blockIdx.y / map.period) * src_pitch) + blockIdx.y % map.period) << 16) + (size_t)row * 256 : g;
+    const u64 *gs = src ? src + (blockIdx.y / map.period) * src_stride + (((size_t)(blockIdx.y % map.period) * src_lpitch) << 16) + (size_t)row * 256 : g;
     u64 *s = sm + rl * ROW_PAD;
     u64 x[16];
 #pragma unroll
@@ -182,14 +183,15 @@ __global__ void __launch_bounds__(THREADS) int_inv_cols(DevTables c, u64 *base, 
 }  // namespace
 
 // the limbs of a grid of ny limbs that the FP64 kernels leave out (whole periods of the map per call)
-void launch_ntt_int(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, bool inverse, const u64 *src, uint32_t src_pitch, cudaStream_t s) {
+// src: as launch_ntt's, in the unscattered form
+void launch_ntt_int(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, bool inverse, const NttSource &src, cudaStream_t s) {
     const dim3 grid(16, ny);
     const uint32_t share = c->ntt_fp_share;
     if (!inverse) {
         launch(int_fwd_cols, grid, THREADS, 0, s, c->dev, b, map, share);
         launch(int_fwd_rows, grid, THREADS, 0, s, c->dev, b, map, share);
     } else {
-        launch(int_inv_rows, grid, THREADS, 0, s, c->dev, b, map, share, src, src_pitch);
+        launch(int_inv_rows, grid, THREADS, 0, s, c->dev, b, map, share, src.lpitch ? src.ptr.base : nullptr, src.ptr.stride, src.lpitch);
         launch(int_inv_cols, grid, THREADS, 0, s, c->dev, b, map, share);
     }
 }

@@ -253,3 +253,35 @@ def test_large_product_with_and_without_a_stored_inner_product(dnum, level):
     want, so = o.poly_eval(x, 2.0 ** 50, [0.0, 0.5, 1.0], rlk)
     got = ctx.poly_eval(ct_dev(x, 2.0 ** 50), [0.0, 0.5, 1.0], key_dev(rlk, 0))
     assert got.scale == so and np.array_equal(host(got.data), want)
+
+
+@pytest.mark.parametrize("share", [0, 1, 4, 7])
+def test_integer_transforms_give_the_same_limbs(share):
+    """N = 2^16 with some or all limbs on the integer transform: nine limbs both ways, rescales of one to three components (their
+    dropped limbs lie a whole component apart) with a workspace and without, of four ciphertexts at once behind a projection,
+    and a rotation whose ModUp takes the transform's plain output."""
+    from paper_2609_12378_b200 import binding
+    from tests.gpu_util import context, ct_dev, dev, host, key_dev
+    from tests.test_gpu_linear import _run
+    from tests.test_zz_no_alloc import _call_static
+    P, ctx = params(16, 9, 3, 3), context(16, 9, 3, 3)
+    o, g = P.oracle, inputs.rng(800, share)
+    x = inputs.uniform_residues(g, P.q[:9], P.N, 3)
+    key = inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, 6).reshape(3, 2, 12, P.N)
+    gal = o.galois_element(5)
+    ctx.set_option(binding.OPT_NTT_FP_SHARE, share)
+    try:
+        assert np.array_equal(host(ctx.ntt(dev(x))), o.ntt(x))
+        assert np.array_equal(host(ctx.intt(dev(x))), o.intt(x))
+        for ncomp in (1, 2):
+            assert np.array_equal(host(ctx.rescale(ct_dev(x[:ncomp], 1.0)).data), o.rescale(x[:ncomp])), ncomp
+        short = np.ascontiguousarray(x[:, :2])
+        out = dev(np.zeros((3, 1, P.N), dtype=np.uint64))
+        assert _call_static(ctx, dev(short), 2, 3, 1.0, out)[0] == binding.OK
+        assert np.array_equal(host(out), o.rescale(short))
+        _run(16, 9, 3, 3, 2, 4, 4, 8192, 4, 2, seed=801, check_slots=False)
+        ctx.set_option(binding.OPT_CONV_KERNEL, binding.CONV_TENSOR)
+        assert np.array_equal(host(ctx.rotate(ct_dev(x[:2], 1.0), key_dev(key, gal)).data), o.rotate(x[:2], key, gal))
+    finally:
+        ctx.set_option(binding.OPT_CONV_KERNEL, binding.CONV_FP64)
+        ctx.set_option(binding.OPT_NTT_FP_SHARE, 8)
