@@ -295,19 +295,21 @@ static int32_t bsgs_entry(ckks_ctx *c, const ckks_ct *x, uint32_t n, const doubl
     if (!level_ok(c, x[0].level)) return CKKS_ERR_LEVEL;
     if (!rlk_ok(rlk)) return CKKS_ERR_NO_KEY;
     std::vector<BsgsPlan> plans(n);
+    std::vector<double> scale(n);           // x and out may be one array: its scales change on the way
+    for (uint32_t i = 0; i < n; i++) scale[i] = x[i].scale;
     for (uint32_t i = 0; i < n; i++)
-        if (i == 0 || x[i].scale != x[0].scale) {
-            const int rc = bsgs_plan(c, x[i].level, x[i].scale, coeffs, degree, m, plans[i]);
+        if (i == 0 || scale[i] != scale[0]) {
+            const int rc = bsgs_plan(c, x[i].level, scale[i], coeffs, degree, m, plans[i]);
             if (rc) return rc;
         }
     if (!ws || ws_bytes < need) return CKKS_ERR_WORKSPACE;
     DeviceGuard guard(c->device);
     for (uint32_t i = 0; i < n;) {
         // a run of ciphertexts of one scale: the constants depend on it
-        const bool own = i == 0 || x[i].scale != x[0].scale;
+        const bool own = i == 0 || scale[i] != scale[0];
         const BsgsPlan &p = own ? plans[i] : plans[0];
         uint32_t k = 1;
-        while (k < POLY_BATCH && i + k < n && x[i + k].scale == x[i].scale) k++;
+        while (k < POLY_BATCH && i + k < n && scale[i + k] == scale[i]) k++;
         Ptrs px, po;
         px.n = po.n = k;
         for (uint32_t j = 0; j < k; j++) { px.p[j] = (const u64 *)x[i + j].data; po.p[j] = (const u64 *)out[i + j].data; }

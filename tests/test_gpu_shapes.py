@@ -131,6 +131,39 @@ def test_polynomial_batches_and_combinations(degree, m, count):
     assert x.level == want.shape[1] and x.scale == so and np.array_equal(host(x.data), want)
 
 
+def test_polynomial_batch_in_place():
+    """Five ciphertexts (a run of four and one) in one array of descriptors for input and output, at a scale that multiplying and
+    dividing by the dropped prime does not give back."""
+    import ctypes as C
+    import torch
+    from paper_2609_12378_b200 import binding
+    from oracle.ckks_oracle import Oracle
+    from tests.gpu_util import GuardedContext, dev, host, key_dev
+    N, r, primes = 1024, 1 + int(1.37 * 2.0 ** 49) // 2048 * 2048, []
+    while len(primes) < 14:         # in the middle of the range: just below 2^50 every scale comes back
+        if inputs.is_prime(r):
+            primes.append(r)
+        r += 2048
+    qs, ps = (np.array(x, dtype=np.uint64) for x in (primes[:10], primes[10:]))
+    o, ctx, g = Oracle(10, qs, ps, 3), GuardedContext(10, qs, ps, 3), inputs.rng(745, 0)
+    rlk = inputs.uniform_residues(g, primes, N, 6).reshape(3, 2, 14, N)
+    coeffs, m, level = g.uniform(-1, 1, 16), 4, 9
+    cts = [inputs.uniform_residues(g, qs[:level], N, 2) for _ in range(5)]
+    lc = o.poly_eval_bsgs(cts[0], 2.0 ** 50, coeffs, rlk, m)[0].shape[1]
+    q = float(qs[lc])
+    scale = next(s for s in 2.0 ** 50 * g.uniform(0.9, 1.1, 1000) if s * q / q != s)
+    data, key = [dev(c) for c in cts], key_dev(rlk, 0)
+    arr = (binding.CCt * 5)(*[binding.CCt(d.data_ptr(), level, 2, scale) for d in data])
+    lib = binding.load()
+    ws = torch.empty(lib.ckks_poly_eval_bsgs_batch_workspace_bytes(ctx._h, level, 15, m, 5), dtype=torch.uint8, device="cuda")
+    ck = binding.CEvk(key.data.data_ptr(), 0)
+    assert lib.ckks_poly_eval_bsgs_batch(ctx._h, arr, 5, (C.c_double * 16)(*coeffs), 15, m, C.byref(ck), arr, ws.data_ptr(), ws.numel(), None) == binding.OK
+    for d, x, c in zip(data, arr, cts):
+        want, so = o.poly_eval_bsgs(c, scale, coeffs, rlk, m)
+        assert x.level == want.shape[1] and x.scale == so and so != scale
+        assert np.array_equal(host(d).reshape(-1)[:want.size].reshape(want.shape), want)
+
+
 @pytest.mark.parametrize("level", [1, 4, 6])
 def test_products_and_rotations_in_place_and_unaligned(level):
     """Batches of 17 (a full chunk and one) whose results lie on their own operands or on another product's, rotations onto
