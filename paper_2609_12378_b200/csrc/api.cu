@@ -8,8 +8,6 @@
 
 namespace {
 
-bool scales_agree(double a, double b) { return fabs(a - b) <= ldexp(fmax(fabs(a), fabs(b)), -30); }
-
 size_t ks_bytes(const ckks_ctx *c, uint32_t level) { return ks_workspace_limbs(c, level) * c->N * sizeof(u64); }
 // hoisted rotations: one set of digits, nbh rotations' worth of inner-product and ModDown buffers side by side
 size_t hoisted_bytes(const ckks_ctx *c, uint32_t level, uint32_t nbh) {

@@ -237,23 +237,35 @@ extern "C" int32_t ckks_softmax_rows(ckks_ctx *c, const ckks_attn_desc *d, const
     for (uint32_t g = 0; g < p.G; g++)
         if (!out[g].data) return CKKS_ERR_ARG;
     if (!ws || ws_bytes < ckks_softmax_rows_workspace_bytes(c, d, s, level)) return CKKS_ERR_WORKSPACE;
-    // every plan (levels, scales, constants) before anything is launched
-    long long shift;
-    TreePlan pe;
-    if (!const_value(-s->shift, in[0].scale, &shift)) return CKKS_ERR_RANGE;
-    if ((rc = poly_tree_plan(c, level, in[0].scale, s->exp_coeffs, s->exp_degree, pe))) return rc;
+    // every plan (levels, scales, constants) before anything is launched.  The groups' scales agree within 2^-30 and need not be
+    // equal: every u_g has a scale of its own, and the exponential's constants depend on it.
+    struct Run { uint32_t g0, n; long long shift; TreePlan poly; };       // neighbours of one scale
+    std::vector<Run> runs;
+    std::vector<double> su(p.G);
+    for (uint32_t g0 = 0; g0 < p.G;) {
+        Run r{g0, 1, 0, TreePlan()};
+        while (r.n < KS_MULTI && g0 + r.n < p.G && in[g0 + r.n].scale == in[g0].scale) r.n++;
+        if (!const_value(-s->shift, in[g0].scale, &r.shift)) return CKKS_ERR_RANGE;
+        if ((rc = poly_tree_plan(c, level, in[g0].scale, s->exp_coeffs, s->exp_degree, r.poly))) return rc;
+        for (uint32_t g = 0; g < r.n; g++) su[g0 + g] = r.poly.out_scale;
+        g0 += r.n;
+        runs.push_back(std::move(r));
+    }
     struct Round { TreePlan poly; uint32_t lu, lt, lx; };                 // levels of u, of its row sums and of lambda u
     std::vector<Round> rounds(s->rounds);
-    uint32_t lu = pe.Lt - 1;
-    double su = pe.out_scale;
+    uint32_t lu = runs[0].poly.Lt - 1;
     for (uint32_t j = 0; j < s->rounds; j++) {
         Round &r = rounds[j];
         r.lu = lu; r.lt = lu - 1;
-        const double st = su * su / (double)c->mod[lu - 1];
+        for (uint32_t g = 0; g < p.G; g++)
+            if (!scales_agree(su[g], su[0])) return CKKS_ERR_SCALE;
+        const double st = su[0] * su[0] / (double)c->mod[lu - 1];
         if ((rc = poly_tree_plan(c, r.lt, st, s->rsqrt_coeffs + (size_t)j * (s->rsqrt_degree + 1), s->rsqrt_degree, r.poly))) return rc;
         r.lx = r.poly.Lt - 2;
-        const double sx = r.poly.out_scale * su / (double)c->mod[r.poly.Lt - 2];
-        su = sx * sx / (double)c->mod[r.lx - 1];
+        for (uint32_t g = 0; g < p.G; g++) {
+            const double sx = r.poly.out_scale * su[g] / (double)c->mod[r.poly.Lt - 2];
+            su[g] = sx * sx / (double)c->mod[r.lx - 1];
+        }
         lu = r.lx - 1;
     }
     const size_t ctw = ct_bytes(c, level) / sizeof(u64), N = c->N;
@@ -262,21 +274,17 @@ extern "C" int32_t ckks_softmax_rows(ckks_ctx *c, const ckks_attn_desc *d, const
     const u64 *rd = (const u64 *)rlk->data;
     cudaStream_t st = (cudaStream_t)stream;
     DeviceGuard guard(c->device);
-    auto run = [&](uint32_t g0) { return std::min(KS_MULTI, p.G - g0); };
-    auto outs = [&](uint32_t g0, uint32_t n, bool final) {               // where step results of groups g0.. go
-        Ptrs o;
-        o.n = n;
-        for (uint32_t g = 0; g < n; g++) o.p[g] = final ? (const u64 *)out[g0 + g].data : U + (size_t)(g0 + g) * ctw;
-        return o;
-    };
     // u = p_exp(x - shift)
-    for (uint32_t g0 = 0; g0 < p.G; g0 += KS_MULTI) {
-        Ptrs pi;
-        pi.n = run(g0);
-        for (uint32_t g = 0; g < pi.n; g++) pi.p[g] = (const u64 *)in[g0 + g].data;
-        const Ptrs z(X + g0 * ctw, ctw);
-        launch_const(c, pi, shift, false, z, 2, level, st, pi.n);
-        poly_tree_run(c, pe, z, outs(g0, pi.n, s->rounds == 0), pi.n, rd, sw, st);
+    for (const Run &r : runs) {
+        Ptrs pi, po;
+        pi.n = po.n = r.n;
+        for (uint32_t g = 0; g < r.n; g++) {
+            pi.p[g] = (const u64 *)in[r.g0 + g].data;
+            po.p[g] = s->rounds ? U + (size_t)(r.g0 + g) * ctw : (const u64 *)out[r.g0 + g].data;
+        }
+        const Ptrs z(X + r.g0 * ctw, ctw);
+        launch_const(c, pi, r.shift, false, z, 2, level, st, r.n);
+        poly_tree_run(c, r.poly, z, po, r.n, rd, sw, st);
     }
     for (uint32_t j = 0; j < s->rounds; j++) {
         const Round &r = rounds[j];
@@ -304,7 +312,7 @@ extern "C" int32_t ckks_softmax_rows(ckks_ctx *c, const ckks_attn_desc *d, const
         mul_rescale(c, x.data(), x.data(), uo.data(), p.G, rd, r.lx, sw, KS_MULTI, st);
     }
     rc = finish(c);
-    for (uint32_t g = 0; g < p.G && rc == CKKS_OK; g++) { out[g].level = lu; out[g].ncomp = 2; out[g].scale = su; }
+    for (uint32_t g = 0; g < p.G && rc == CKKS_OK; g++) { out[g].level = lu; out[g].ncomp = 2; out[g].scale = su[g]; }
     return rc;
 }
 

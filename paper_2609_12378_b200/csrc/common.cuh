@@ -4,6 +4,7 @@
 #include <algorithm>
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <string>
@@ -561,6 +562,7 @@ inline int finish(ckks_ctx *c) {
     if (e != cudaSuccess) { c->cuda_error = cudaGetErrorString(e); return CKKS_ERR_CUDA; }
     return CKKS_OK;
 }
+inline bool scales_agree(double a, double b) { return fabs(a - b) <= ldexp(fmax(fabs(a), fabs(b)), -30); }
 inline bool ct_ok(const ckks_ct *ct) { return ct && ct->data; }
 inline bool level_ok(const ckks_ctx *c, uint32_t level) { return level >= 1 && level <= c->L; }
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }

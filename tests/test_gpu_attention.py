@@ -150,6 +150,42 @@ def test_attention_scores_in_passes_and_errors():
     assert binding.kernel_launches() == launches
 
 
+@pytest.mark.parametrize("rounds", [0, 1])
+def test_softmax_rows_of_groups_with_their_own_scales(rounds):
+    """Scales that agree within 2^-30 without being equal: every group's exponential takes the constants of its own scale and
+    every result carries its own, step by step as the checker's functions give them."""
+    from tests.gpu_util import context, ct_dev, host, key_dev
+    P, ctx = params(10, 13, 4, 4), context(10, 13, 4, 4)
+    o, g = P.oracle, inputs.rng(650, rounds)
+    a, level, shift = (16, 2, 4), 13, 2.0
+    desc = AttnDesc(*a)
+    G = desc.groups()
+    _, lad = o.attention_rotations(desc)
+    def key():
+        return inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, 8).reshape(4, 2, 17, P.N)
+    rlk, keys = key(), {o.galois_element(r): key() for r in lad}
+    ec, rc = g.uniform(-1, 1, 5), g.uniform(-1, 1, (rounds, 5))
+    scales = [2.0 ** 50, 2.0 ** 50 * (1.0 + 2.0 ** -31), 2.0 ** 50 * (1.0 + 2.0 ** -31), 2.0 ** 50]
+    S = [inputs.uniform_residues(g, P.q[:level], P.N, 2) for _ in range(G)]
+    u, su = map(list, zip(*[o.poly_eval_tree(o.add_const(x, int(np.rint(-shift * s))), s, ec, rlk) for x, s in zip(S, scales)]))
+    for j in range(rounds):
+        lv = u[0].shape[1]
+        t = o._block_ladder(desc, o.rescale(o.mul_relin_sum(np.stack(u), np.stack(u), rlk)), keys)
+        lam, sl = o.poly_eval_tree(t, su[0] * su[0] / float(P.q[lv - 1]), rc[j], rlk)
+        ll = lam.shape[1]
+        for x in range(G):
+            v = o.rescale(o.mul_relin(lam, u[x][:, :ll], rlk))
+            u[x] = o.rescale(o.mul_relin(v, v, rlk))
+            sv = sl * su[x] / float(P.q[ll - 1])
+            su[x] = sv * sv / float(P.q[ll - 2])
+    assert su[0] != su[1]
+    got = ctx.softmax_rows([ct_dev(x, s) for x, s in zip(S, scales)], shift, rounds, ec, rc, key_dev(rlk, 0),
+                           [key_dev(k, ge) for ge, k in keys.items()], *a)
+    for x in range(G):
+        assert got[x].scale == su[x] and got[x].level == u[x].shape[1], x
+        assert np.array_equal(host(got[x].data), u[x]), x
+
+
 @pytest.mark.slow
 def test_attention_full_ring():
     """N = 2^16 with the decoder layer's attention shape in the slots (128 tokens, 32 heads, 8 diagonals per ciphertext:
