@@ -383,8 +383,9 @@ extern "C" int32_t ckks_attention_values(ckks_ctx *c, const ckks_attn_desc *d, c
         }
     }
     rc = finish(c);
-    for (uint32_t dd = 0; dd < dim_v && rc == CKKS_OK; dd++) {
-        out[dd].level = lp - 1; out[dd].ncomp = 2; out[dd].scale = probs[0].scale * v[0].scale / (double)c->mod[lp - 1];
+    for (uint32_t dd = 0; dd < dim_v && rc == CKKS_OK; dd++) {        // out may be v: each entry is read before it is written
+        out[dd].scale = probs[0].scale * v[dd].scale / (double)c->mod[lp - 1];
+        out[dd].level = lp - 1; out[dd].ncomp = 2;
     }
     return rc;
 }

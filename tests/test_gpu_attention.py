@@ -186,6 +186,36 @@ def test_softmax_rows_of_groups_with_their_own_scales(rounds):
         assert np.array_equal(host(got[x].data), u[x]), x
 
 
+def test_attention_values_onto_their_operands():
+    """Results in the value operands' own descriptors and buffers (more channels than one pass takes), whose scales agree within
+    2^-30 without being equal: each result carries its own operand's."""
+    import ctypes as C
+
+    from tests.gpu_util import context, dev, host, key_dev
+    P, ctx = params(10, 6, 2, 3), context(10, 6, 2, 3)
+    o, g = P.oracle, inputs.rng(655, 0)
+    a, lp, lv, dim_v = (8, 2, 4), 4, 5, 18
+    desc = AttnDesc(*a)
+    tok, lad = o.attention_rotations(desc)
+    def key():
+        return inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, 6).reshape(3, 2, 8, P.N)
+    rlk, keys = key(), {o.galois_element(r): key() for r in tok + lad}
+    probs = [inputs.uniform_residues(g, P.q[:lp], P.N, 2) for _ in range(desc.groups())]
+    v = [inputs.uniform_residues(g, P.q[:lv], P.N, 2) for _ in range(dim_v)]
+    ps, vs = 2.0 ** 50, [2.0 ** 50 * (1.0 + d * 2.0 ** -40) for d in range(dim_v)]
+    want = o.attention_values(desc, np.stack(probs), np.stack(v), rlk, keys)
+    dp, dv, drlk, dkeys = [dev(x) for x in probs], [dev(x) for x in v], key_dev(rlk, 0), [key_dev(k, ge) for ge, k in keys.items()]
+    pa = (binding.CCt * len(dp))(*[binding.CCt(x.data_ptr(), lp, 2, ps) for x in dp])
+    va = (binding.CCt * dim_v)(*[binding.CCt(x.data_ptr(), lv, 2, s) for x, s in zip(dv, vs)])
+    ka = (binding.CEvk * len(dkeys))(*[binding.CEvk(k.data.data_ptr(), k.galois) for k in dkeys])
+    ck, d, lib = binding.CEvk(drlk.data.data_ptr(), 0), binding.CAttnDesc(*a), binding.load()
+    ws = ctx.workspace(int(lib.ckks_attention_values_workspace_bytes(ctx._h, C.byref(d), lp)))
+    assert lib.ckks_attention_values(ctx._h, C.byref(d), pa, va, dim_v, C.byref(ck), ka, len(dkeys), va, ws.data_ptr(), ws.numel(), None) == binding.OK
+    for x in range(dim_v):
+        assert va[x].level == lp - 1 and va[x].scale == ps * vs[x] / float(P.q[lp - 1]), x
+        assert np.array_equal(host(dv[x]).reshape(-1)[:want[x].size].reshape(want[x].shape), want[x]), x
+
+
 @pytest.mark.slow
 def test_attention_full_ring():
     """N = 2^16 with the decoder layer's attention shape in the slots (128 tokens, 32 heads, 8 diagonals per ciphertext:
