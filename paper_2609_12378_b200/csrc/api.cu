@@ -730,6 +730,7 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
     const ProjPlan &p0 = plans[0];
     const uint32_t nib = (uint32_t)p0.ins.size(), S = p0.S, B = p0.B, T = p0.T, N = c->N;
     const uint32_t level = in[0].level;
+    const double in_scale = in[0].scale;            // out may be in
     if (!level_ok(c, level) || level < 2) return CKKS_ERR_LEVEL;
     for (uint32_t x = 0; x < S * nib; x++) {
         if (!in[x].data || in[x].ncomp != 2) return CKKS_ERR_ARG;
@@ -990,7 +991,7 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
             const double pt_scale = descs[m].pt_scale > 0.0 ? descs[m].pt_scale : (double)c->mod[level - 1];
             for (uint32_t x = 0; x < S * nob; x++) {
                 out_m[x].level = level - 1; out_m[x].ncomp = 2;
-                out_m[x].scale = in[0].scale * pt_scale / (double)c->mod[level - 1];
+                out_m[x].scale = in_scale * pt_scale / (double)c->mod[level - 1];
             }
             out_m += S * nob;
         }

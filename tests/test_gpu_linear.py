@@ -101,6 +101,28 @@ def test_projection_lazy_moddown_many_groups():
     _run(11, 4, 2, 2, 3, 128, 128, 8, 2, 4, seed=490, lazy=True)
 
 
+def test_projection_onto_its_inputs():
+    """Results in the inputs' own descriptors and buffers, weights at a scale that changes the ciphertexts': three shards with
+    the limbs of a projection into other buffers and one scale for all."""
+    import ctypes as C
+
+    from tests.gpu_util import ct_dev, dev, host, key_dev
+    P = params(10, 4, 2, 2)
+    ctx, cts, keys = _run(10, 4, 2, 2, 4, 16, 16, 32, 3, 4, seed=470, pt_scale=2.0 ** 38, check_slots=False)
+    W = dev(inputs.weights_normal(inputs.rng(470, 2), 16, 16, 0.02))
+    dkeys = [key_dev(k, g_) for g_, k in keys.items()]
+    want = ctx.linear_proj([ct_dev(c, 2.0 ** 40) for c in cts], W, dkeys, 16, 16, 32, 3, 4, 2.0 ** 38)
+    data = [dev(c) for c in cts]
+    arr = (binding.CCt * 3)(*[binding.CCt(x.data_ptr(), 4, 2, 2.0 ** 40) for x in data])
+    ka = (binding.CEvk * len(dkeys))(*[binding.CEvk(k.data.data_ptr(), k.galois) for k in dkeys])
+    d, lib = binding.CProjDesc(16, 16, 32, 3, 4, 0, 2.0 ** 38), binding.load()
+    ws = ctx.workspace(int(lib.ckks_linear_proj_workspace_bytes(ctx._h, C.byref(d), 4)))
+    assert lib.ckks_linear_proj(ctx._h, C.byref(d), arr, W.data_ptr(), ka, len(dkeys), arr, ws.data_ptr(), ws.numel(), None) == binding.OK
+    for x, c, w in zip(data, arr, want):
+        assert c.level == 3 and c.scale == w.scale == 2.0 ** 40 * 2.0 ** 38 / float(P.q[3])
+        assert np.array_equal(host(x).reshape(-1)[:w.data.numel()].reshape(2, 3, P.N), host(w.data))
+
+
 @pytest.mark.parametrize("kernel", [binding.MAC_MMA_SPLIT, binding.MAC_MMA_ASYNC, binding.MAC_MMA_HALF, binding.MAC_TCGEN05])
 def test_projection_tensor_core_mac_other_shapes(kernel):
     """The kernel's other forms (two warps per coefficient; the barrier-free pipeline; four coefficients per CTA; tcgen05
