@@ -131,6 +131,12 @@ ProjWs proj_layout(const ckks_ctx *c, const ProjPlan &p, uint32_t level, bool la
     return w;
 }
 
+// whether the buffers of `words` words at a and b share any of them
+bool overlap(const void *a, const void *b, size_t words) {
+    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+    return (x > y ? x - y : y - x) < words * sizeof(u64);
+}
+
 const ckks_evk *find_key(const ckks_evk *keys, uint32_t nkeys, u64 g) {
     for (uint32_t i = 0; i < nkeys; i++)
         if (keys[i].galois == g && keys[i].data) return &keys[i];
@@ -312,11 +318,15 @@ extern "C" int32_t ckks_mul_relin_batch(ckks_ctx *c, const ckks_ct *a, const ckk
     for (uint32_t i0 = 0; i0 < n; i0 += MRB_CHUNK) {
         const uint32_t m = std::min(MRB_CHUNK, n - i0);
         u64 *stage = (u64 *)ws, *e2 = stage + (size_t)m * ctl;
-        // results go straight to their place unless another product of the chunk still has to read what lies there
+        // results go straight to their place unless a product of the chunk still has to read or write what lies there (a product
+        // exactly on its own operand is read word by word before it is written)
         bool staged = false;
         for (uint32_t i = 0; i < m; i++)
-            for (uint32_t j = 0; j < m; j++)
-                staged = staged || (i != j && (out[i0 + i].data == a[i0 + j].data || out[i0 + i].data == b[i0 + j].data || out[i0 + i].data == out[i0 + j].data));
+            for (uint32_t j = 0; j < m; j++) {
+                const u64 *o = (const u64 *)out[i0 + i].data, *x = (const u64 *)a[i0 + j].data, *y = (const u64 *)b[i0 + j].data;
+                staged = staged || (overlap(o, x, ctl) && (i != j || o != x)) || (overlap(o, y, ctl) && (i != j || o != y)) ||
+                         (i != j && overlap(o, out[i0 + j].data, ctl));
+            }
         TensorArgs ta;
         Ptrs o(stage, ctl);
         for (uint32_t i = 0; i < m; i++) {
@@ -572,7 +582,8 @@ extern "C" int32_t ckks_rotate_batch(ckks_ctx *c, const ckks_ct *in, uint32_t n,
     const size_t N = c->N, ctl = (size_t)2 * level * N, ptl = (size_t)level * N;
     for (uint32_t i0 = 0; i0 < n; i0 += MRB_CHUNK) {
         const uint32_t m = std::min(MRB_CHUNK, n - i0);
-        // a result may lie where an input of the chunk does: such inputs are copied first
+        // a result may lie where an input of the chunk does: such inputs are copied first.  Results that share words are written
+        // one run after the other, so that the last one stays.
         u64 *xin = (u64 *)ws;
         KsWorkspace w = ks_carve(c, level, xin + (size_t)m * ctl, m);
         Ptrs src, dst;
@@ -581,12 +592,20 @@ extern "C" int32_t ckks_rotate_batch(ckks_ctx *c, const ckks_ct *in, uint32_t n,
             src.p[i] = (const u64 *)in[i0 + i].data;
             dst.p[i] = (const u64 *)out[i0 + i].data;
             bool alias = false;
-            for (uint32_t j = 0; j < m; j++) alias = alias || out[i0 + j].data == in[i0 + i].data;
+            for (uint32_t j = 0; j < m; j++) alias = alias || overlap(out[i0 + j].data, in[i0 + i].data, ctl);
             if (!alias) continue;
             cudaMemcpyAsync(xin + (size_t)i * ctl, src.p[i], ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
             src.p[i] = xin + (size_t)i * ctl;
         }
-        rotate_ks(c, key, src, dst, level, w, s, m);
+        for (uint32_t r0 = 0, r1; r0 < m; r0 = r1) {
+            for (r1 = r0 + 1; r1 < m; r1++)
+                if (std::any_of(dst.p + r0, dst.p + r1, [&](const u64 *d) { return overlap(d, dst.p[r1], ctl); })) break;
+            Ptrs rs, rd;
+            rs.n = rd.n = r1 - r0;
+            std::copy(src.p + r0, src.p + r1, rs.p);
+            std::copy(dst.p + r0, dst.p + r1, rd.p);
+            rotate_ks(c, key, rs, rd, level, w, s, r1 - r0);
+        }
     }
     int rc = finish(c);
     if (rc == CKKS_OK)

@@ -208,6 +208,39 @@ def test_products_and_rotations_in_place_and_unaligned(level):
         assert np.array_equal(host(s.data), o.mul_relin_sum(np.stack(x), np.stack(y), key))
 
 
+@pytest.mark.parametrize("shift", [0, 1, 5])
+def test_batches_whose_results_share_words(shift):
+    """Sixteen products and rotations in one buffer whose results start `shift` limbs behind another product's operand (the last
+    one's for the first result), and two results in one place: as if every operand had been read first and the results then
+    written in order."""
+    from paper_2609_12378_b200 import binding
+    from tests.gpu_util import context, ct_dev, dev, host, key_dev
+    P, ctx = params(13, 6, 1, 6), context(13, 6, 1, 6)
+    o, g = P.oracle, inputs.rng(755, shift)
+    n, level, N = 16, 6, P.N
+    words = 2 * level * N
+    key = inputs.uniform_residues(g, list(P.q) + list(P.p), N, 12).reshape(6, 2, 7, N)
+    gal = o.galois_element(5)
+    x = [inputs.uniform_residues(g, P.q, N, 2) for _ in range(n)]
+    y = inputs.uniform_residues(g, P.q, N, 2)
+    for place in ([n - 1] + list(range(n - 1)), [0, 1] + [3] * 2 + list(range(4, n))):
+        for products in (True, False):
+            flat = np.concatenate([a.reshape(-1) for a in x] + [np.zeros(words, dtype=np.uint64)])
+            want = flat.copy()
+            for a, p in zip(x, place):
+                r = o.mul_relin(a, y, key) if products else o.rotate(a, key, gal)
+                want[p * words + shift * N:(p + 1) * words + shift * N] = r.reshape(-1)
+            buf = dev(flat)
+            def cts(starts):
+                return [binding.Ciphertext(buf[s:s + words].view(2, level, N), 1.0) for s in starts]
+            ins, outs = cts(i * words for i in range(n)), cts(p * words + shift * N for p in place)
+            if products:
+                ctx.mul_relin_batch(ins, [ct_dev(y, 1.0)] * n, key_dev(key, 0), outs=outs)
+            else:
+                ctx.rotate_batch(ins, key_dev(key, gal), outs=outs)
+            assert np.array_equal(host(buf), want), (place[0], products)
+
+
 @pytest.mark.parametrize("log_n,batch,limbs", [(12, 1, 3), (12, 24, 3), (12, 25, 3), (13, 24, 3), (13, 25, 3), (14, 12, 3), (14, 13, 3)])
 def test_transforms_at_the_cluster_limit(log_n, batch, limbs):
     """The last batch that one cluster per limb transforms and the first that goes in two passes: both directions."""
