@@ -814,9 +814,9 @@ void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbM
     const uint32_t R = c->N >> 8;
     // the integer path (an option, N = 2^16) has no fused forms: those take all limbs on the FP64 pipe
     const uint32_t share = (ep || pro || inv_scale || (src && src->ptr.n) || c->log_n != 16) ? 8 : c->ntt_fp_share;
-    // grid.y is limited to 65535: go in chunks that are whole periods of the limb map (a multiple of 8 limbs apart only
-    // matters to the integer share, which is a choice of limbs and not part of the result)
-    const uint32_t chunk = map.period >= 32768 ? map.period : (32768 / map.period) * map.period;
+    // grid.y is limited to 65535: go in chunks that are whole repeats of the limb map, a period of every digit where they differ (a
+    // multiple of 8 limbs apart only matters to the integer share, which is a choice of limbs and not part of the result)
+    const uint32_t repeat = map.period * map.nbeta, chunk = std::max(1u, 32768 / repeat) * repeat;
     for (uint32_t y0 = 0; y0 < nlimbs_total; y0 += chunk) {
         const uint32_t ny = nlimbs_total - y0 < chunk ? nlimbs_total - y0 : chunk;
         u64 *b = base + (limb_index(map, y0) << c->log_n);

@@ -123,6 +123,22 @@ def test_projection_onto_its_inputs():
         assert np.array_equal(host(x).reshape(-1)[:w.data.numel()].reshape(2, 3, P.N), host(w.data))
 
 
+def test_projection_of_more_digits_than_one_launch_takes():
+    """620 shards of seven digits: the extended digits' transforms take two launches, and the second one's first polynomial is not
+    a first digit.  Shards of one input give what a projection of five shards gives."""
+    from tests.gpu_util import ct_dev, dev, host, key_dev
+    ctx, cts, keys = _run(10, 7, 1, 7, 7, 4, 4, 128, 5, 2, seed=475, check_slots=False)
+    W = dev(inputs.weights_normal(inputs.rng(475, 2), 4, 4, 0.02))
+    dcts, dkeys = [ct_dev(c, 2.0 ** 40) for c in cts], [key_dev(k, g_) for g_, k in keys.items()]
+    want = [host(w.data) for w in ctx.linear_proj(dcts, W, dkeys, 4, 4, 128, 5, 2)]
+    for lazy in (False, True):
+        got = ctx.linear_proj([dcts[x % 5] for x in range(620)], W, dkeys, 4, 4, 128, 620, 2, lazy_moddown=lazy)
+        if lazy:
+            want = [host(w.data) for w in ctx.linear_proj(dcts, W, dkeys, 4, 4, 128, 5, 2, lazy_moddown=True)]
+        for x in range(620):
+            assert np.array_equal(host(got[x].data), want[x % 5]), (lazy, x)
+
+
 @pytest.mark.parametrize("kernel", [binding.MAC_MMA_SPLIT, binding.MAC_MMA_ASYNC, binding.MAC_MMA_HALF, binding.MAC_TCGEN05])
 def test_projection_tensor_core_mac_other_shapes(kernel):
     """The kernel's other forms (two warps per coefficient; the barrier-free pipeline; four coefficients per CTA; tcgen05
