@@ -169,10 +169,14 @@ extern "C" int32_t ckks_attention_scores(ckks_ctx *c, const ckks_attn_desc *d, c
         if (!ws || ws_bytes < ckks_attention_scores_workspace_bytes(c, d, level, dim)) return CKKS_ERR_WORKSPACE;
         return scores_split(c, p, q, k, dim, level, rlk, keys, nkeys, scores, ws, (cudaStream_t)stream);
     }
-    // as many groups per pass as the workspace holds (one at least)
-    const size_t ctb = ct_bytes(c, level), ctw = ctb / sizeof(u64), N = c->N, fixed = scratch_bytes(c, level, dim, p.G - 1, p.G);
-    uint32_t per_pass = p.G > 1 ? (uint32_t)std::min<size_t>(p.G - 1, ws_bytes > fixed ? (ws_bytes - fixed) / ((size_t)dim * ctb) : 0) : 0;
-    if (!ws || ws_bytes < fixed || (p.G > 1 && per_pass == 0)) return CKKS_ERR_WORKSPACE;
+    // As many groups per pass as the workspace holds.  A workspace too small for one next to the steps' full scratch takes one
+    // group per pass and fewer sums and rotations side by side, down to one product and one operand's rotations.
+    const size_t ctb = ct_bytes(c, level), ctw = ctb / sizeof(u64), N = c->N, set = p.G > 1 ? dim * ctb : 0, full = scratch_bytes(c, level, dim, p.G - 1, p.G);
+    const size_t least = ctb + align256(std::max(ckks_workspace_bytes(c, CKKS_OP_MUL_RELIN, level, 0),
+                                                 ckks_workspace_bytes(c, CKKS_OP_ROTATE_HOISTED, level, std::max(1u, p.G - 1))));
+    if (!ws || ws_bytes < least + set) return CKKS_ERR_WORKSPACE;
+    const uint32_t per_pass = p.G == 1 ? 0 : ws_bytes < full + set ? 1 : (uint32_t)std::min<size_t>(p.G - 1, (ws_bytes - full) / set);
+    const size_t sw_bytes = ws_bytes - per_pass * set;
     u64 *rk = (u64 *)ws;                                                 // [per_pass][dim] ciphertexts
     void *sw = rk + (size_t)per_pass * dim * ctw;
     cudaStream_t s = (cudaStream_t)stream;
@@ -185,7 +189,7 @@ extern "C" int32_t ckks_attention_scores(ckks_ctx *c, const ckks_attn_desc *d, c
         const uint32_t first = g0 ? g0 : 1, ng = std::min(per_pass, p.G - first), last = p.G > 1 ? first + ng : 1;
         std::vector<ckks_evk> pk;
         for (uint32_t g = first; g < last; g++) pk.push_back(*find_key(c, keys, nkeys, p.tok[g - 1]));
-        rotate_grid(c, vk.data(), dim, pk.data(), (uint32_t)pk.size(), rk, dim * ctw, ctw, level, sw, s);
+        rotate_grid(c, vk.data(), dim, pk.data(), (uint32_t)pk.size(), rk, dim * ctw, ctw, level, sw, s, sw_bytes);
         std::vector<std::vector<CtView>> a, b;
         std::vector<u64 *> out;
         for (uint32_t g = g0; g < last; g++) {
@@ -193,7 +197,7 @@ extern "C" int32_t ckks_attention_scores(ckks_ctx *c, const ckks_attn_desc *d, c
             for (uint32_t dd = 0; dd < dim && g; dd++) kr[dd] = CtView{rk + ((size_t)(g - first) * dim + dd) * ctw, (size_t)level * N};
             a.push_back(vq); b.push_back(kr); out.push_back((u64 *)scores[g].data);
         }
-        sum_rescale(c, a, b, out.data(), (uint32_t)out.size(), (const u64 *)rlk->data, level, sw, s);
+        sum_rescale(c, a, b, out.data(), (uint32_t)out.size(), (const u64 *)rlk->data, level, sw, s, sw_bytes);
         g0 = last;
     }
     rc = finish(c);

@@ -63,12 +63,14 @@ static bool same_views(const std::vector<CtView> &x, const std::vector<CtView> &
     return x.size() == y.size() && std::equal(x.begin(), x.end(), y.begin(), [](const CtView &u, const CtView &v) { return u.p == v.p && u.comp == v.comp; });
 }
 
-// out[i] = rescale(relin(sum_t a[i][t] b[i][t])) for n sums of nterm products; ws: min(n, KS_MULTI) * product_bytes
+// out[i] = rescale(relin(sum_t a[i][t] b[i][t])) for n sums of nterm products; ws: min(n, KS_MULTI) * product_bytes, or a ws_bytes
+// of at least one product_bytes, which takes as many sums side by side as it holds
 void sum_rescale(const ckks_ctx *c, const std::vector<std::vector<CtView>> &a, const std::vector<std::vector<CtView>> &b, u64 *const *out, uint32_t n,
-                 const u64 *rlk, uint32_t level, void *ws, cudaStream_t s) {
+                 const u64 *rlk, uint32_t level, void *ws, cudaStream_t s, size_t ws_bytes) {
     const size_t N = c->N, ctl = (size_t)2 * level * N, ptl = (size_t)level * N;
-    for (uint32_t i0 = 0; i0 < n; i0 += KS_MULTI) {
-        const uint32_t m = std::min(KS_MULTI, n - i0);
+    const uint32_t side = (uint32_t)std::min<size_t>(KS_MULTI, ws_bytes / product_bytes(c, level));
+    for (uint32_t i0 = 0; i0 < n; i0 += side) {
+        const uint32_t m = std::min(side, n - i0);
         u64 *e01 = (u64 *)ws, *e2 = e01 + m * ctl, *ksw = e2 + m * ptl;
         Ptrs po;
         po.n = m;
@@ -94,17 +96,23 @@ void sum_rescale(const ckks_ctx *c, const std::vector<std::vector<CtView>> &a, c
 // them), GRID_ENTRIES key switches side by side.
 constexpr uint32_t GRID_CTS = 8, GRID_ENTRIES = 32;
 static uint32_t grid_keys(uint32_t members, uint32_t nrot) { return std::min(nrot, std::min(KS_MULTI, std::max(1u, GRID_ENTRIES / members))); }
-size_t rotate_grid_bytes(const ckks_ctx *c, uint32_t level, uint32_t n, uint32_t nrot) {
+static size_t grid_bytes(const ckks_ctx *c, uint32_t level, uint32_t members, uint32_t keys) {
     const size_t beta = (level + c->alpha - 1) / c->alpha, nt = level + c->K;
+    return (members * (level + beta * nt) + (size_t)members * keys * (2 * nt + 2 * level)) * c->N * sizeof(u64);
+}
+size_t rotate_grid_bytes(const ckks_ctx *c, uint32_t level, uint32_t n, uint32_t nrot) {
     const uint32_t m = std::min(n, GRID_CTS);
-    return (m * (level + beta * nt) + (size_t)m * grid_keys(m, nrot) * (2 * nt + 2 * level)) * c->N * sizeof(u64);
+    return grid_bytes(c, level, m, grid_keys(m, nrot));
 }
 // rotation r of ciphertext i (components comp words apart, taken at `level`) -> out + r * rot_stride + i * ct_stride
+// ws: rotate_grid_bytes, or a ws_bytes of at least what one ciphertext and one key take, which lets as many share a pass as fit
 void rotate_grid(const ckks_ctx *c, const CtView *in, uint32_t n, const ckks_evk *keys, uint32_t nrot, u64 *out, size_t rot_stride, size_t ct_stride,
-                 uint32_t level, void *ws, cudaStream_t s) {
+                 uint32_t level, void *ws, cudaStream_t s, size_t ws_bytes) {
     if (!n || !nrot) return;
     const size_t beta = (level + c->alpha - 1) / c->alpha, nt = level + c->K, N = c->N;
-    const uint32_t mmax = std::min(n, GRID_CTS), kmax = grid_keys(mmax, nrot);
+    uint32_t mmax = std::min(n, GRID_CTS), kmax = grid_keys(mmax, nrot);
+    for (; mmax > 1 && grid_bytes(c, level, mmax, kmax) > ws_bytes; kmax = grid_keys(mmax, nrot)) mmax--;
+    while (kmax > 1 && grid_bytes(c, level, mmax, kmax) > ws_bytes) kmax--;
     KsWorkspace w;
     w.dcoef = (u64 *)ws;
     w.ext = w.dcoef + (size_t)mmax * level * N;

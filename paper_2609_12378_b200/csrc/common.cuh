@@ -535,10 +535,10 @@ size_t product_bytes(const ckks_ctx *c, uint32_t level);
 void mul_rescale(const ckks_ctx *c, const CtView *a, const CtView *b, u64 *const *out, uint32_t n, const u64 *rlk, uint32_t level, void *ws, uint32_t chunk,
                  cudaStream_t s);
 void sum_rescale(const ckks_ctx *c, const std::vector<std::vector<CtView>> &a, const std::vector<std::vector<CtView>> &b, u64 *const *out, uint32_t n,
-                 const u64 *rlk, uint32_t level, void *ws, cudaStream_t s);
+                 const u64 *rlk, uint32_t level, void *ws, cudaStream_t s, size_t ws_bytes = SIZE_MAX);
 size_t rotate_grid_bytes(const ckks_ctx *c, uint32_t level, uint32_t n, uint32_t nrot);
 void rotate_grid(const ckks_ctx *c, const CtView *in, uint32_t n, const ckks_evk *keys, uint32_t nrot, u64 *out, size_t rot_stride, size_t ct_stride,
-                 uint32_t level, void *ws, cudaStream_t s);
+                 uint32_t level, void *ws, cudaStream_t s, size_t ws_bytes = SIZE_MAX);
 // The polynomial of ckks_poly_eval_tree for n ciphertexts side by side (at most KS_MULTI; all at one level and scale).  plan
 // first: it fixes levels, scales and constants and reports their errors before anything is launched.
 struct TreePlan {

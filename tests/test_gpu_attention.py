@@ -150,6 +150,39 @@ def test_attention_scores_in_passes_and_errors():
     assert binding.kernel_launches() == launches
 
 
+@pytest.mark.parametrize("E,dim", [(1, 9), (4, 3), (16, 2)])
+def test_attention_scores_down_to_the_smallest_workspace(E, dim):
+    """Sixteen, four groups and one: every workspace from the one that holds one group's rotated operands, one product and one
+    operand's rotations gives the same scores, a smaller one is refused."""
+    import torch
+
+    from tests.gpu_util import GUARD_BYTES, GUARD_VALUE, context, ct_dev, host, key_dev
+    P, ctx = params(10, 5, 2, 3), context(10, 5, 2, 3)
+    o, g = P.oracle, inputs.rng(645, E)
+    a, level = (16, 2, E), 4
+    desc = AttnDesc(*a)
+    G = desc.groups()
+    tok, _ = o.attention_rotations(desc)
+    def key():
+        return inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, 6).reshape(3, 2, 7, P.N)
+    rlk, keys = key(), {o.galois_element(r): key() for r in tok}
+    q, k = ([inputs.uniform_residues(g, P.q[:level], P.N, 2) for _ in range(dim)] for _ in "qk")
+    want = o.attention_scores(desc, np.stack(q), np.stack(k), rlk, keys)
+    args = ([ct_dev(x, 1.0) for x in q], [ct_dev(x, 1.0) for x in k], key_dev(rlk, 0), [key_dev(x, ge) for ge, x in keys.items()])
+    ct = 2 * level * P.N * 8
+    least = ct + max(ctx.workspace_bytes(binding.OP_MUL_RELIN, level), ctx.workspace_bytes(binding.OP_ROTATE_HOISTED, level, max(1, G - 1)))
+    least += dim * ct if G > 1 else 0
+    for extra in (0, 3 * ct, 12 * ct, 40 * ct, 160 * ct):
+        buf = torch.full((least + extra + GUARD_BYTES,), GUARD_VALUE, dtype=torch.uint8, device="cuda")
+        got = ctx.attention_scores(*args, *a, ws=buf[:least + extra])
+        for x in range(G):
+            assert np.array_equal(host(got[x].data), want[x]), (extra, x)
+        assert bool((buf[least + extra:] == GUARD_VALUE).all())
+    with pytest.raises(binding.CkksError) as e:
+        ctx.attention_scores(*args, *a, ws=torch.empty(least - 256, dtype=torch.uint8, device="cuda"))
+    assert e.value.code == binding.ERR_WORKSPACE
+
+
 @pytest.mark.parametrize("rounds", [0, 1])
 def test_softmax_rows_of_groups_with_their_own_scales(rounds):
     """Scales that agree within 2^-30 without being equal: every group's exponential takes the constants of its own scale and
