@@ -278,17 +278,18 @@ extern "C" int32_t ckks_softmax_rows(ckks_ctx *c, const ckks_attn_desc *d, const
     const u64 *rd = (const u64 *)rlk->data;
     cudaStream_t st = (cudaStream_t)stream;
     DeviceGuard guard(c->device);
-    // u = p_exp(x - shift)
+    // u = p_exp(x - shift); all inputs are read before the first result, which may lie on any of them
     for (const Run &r : runs) {
-        Ptrs pi, po;
-        pi.n = po.n = r.n;
-        for (uint32_t g = 0; g < r.n; g++) {
-            pi.p[g] = (const u64 *)in[r.g0 + g].data;
-            po.p[g] = s->rounds ? U + (size_t)(r.g0 + g) * ctw : (const u64 *)out[r.g0 + g].data;
-        }
-        const Ptrs z(X + r.g0 * ctw, ctw);
-        launch_const(c, pi, r.shift, false, z, 2, level, st, r.n);
-        poly_tree_run(c, r.poly, z, po, r.n, rd, sw, st);
+        Ptrs pi;
+        pi.n = r.n;
+        for (uint32_t g = 0; g < r.n; g++) pi.p[g] = (const u64 *)in[r.g0 + g].data;
+        launch_const(c, pi, r.shift, false, Ptrs(X + r.g0 * ctw, ctw), 2, level, st, r.n);
+    }
+    for (const Run &r : runs) {
+        Ptrs po;
+        po.n = r.n;
+        for (uint32_t g = 0; g < r.n; g++) po.p[g] = s->rounds ? U + (size_t)(r.g0 + g) * ctw : (const u64 *)out[r.g0 + g].data;
+        poly_tree_run(c, r.poly, Ptrs(X + r.g0 * ctw, ctw), po, r.n, rd, sw, st);
     }
     for (uint32_t j = 0; j < s->rounds; j++) {
         const Round &r = rounds[j];

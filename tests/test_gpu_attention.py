@@ -219,6 +219,30 @@ def test_softmax_rows_of_groups_with_their_own_scales(rounds):
         assert np.array_equal(host(got[x].data), u[x]), x
 
 
+@pytest.mark.parametrize("rounds", [0, 1])
+def test_softmax_rows_onto_each_others_inputs(rounds):
+    """Thirty-two groups (two passes of the steps) whose results lie on one another's inputs, in reverse order."""
+    import ctypes as C
+
+    from tests.gpu_util import context, ct_dev, dev, host, key_dev
+    P, ctx = params(10, 11, 4, 3), context(10, 11, 4, 3)
+    o, g = P.oracle, inputs.rng(652, rounds)
+    a, level, shift, scale, G = (32, 1, 1), 4 + 6 * rounds, 2.0, 2.0 ** 50, 32
+    rlk = inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, 6).reshape(3, 2, 15, P.N)
+    ec, rc = g.uniform(-1, 1, 4), g.uniform(-1, 1, (rounds, 4))
+    S = np.stack([inputs.uniform_residues(g, P.q[:level], P.N, 2) for _ in range(G)])
+    want, so = o.softmax_rows(AttnDesc(*a), S, scale, shift, rounds, ec, rc, rlk, {})
+    data, drlk = [dev(x) for x in S], key_dev(rlk, 0)
+    ia = (binding.CCt * G)(*[binding.CCt(x.data_ptr(), level, 2, scale) for x in data])
+    oa = (binding.CCt * G)(*[binding.CCt(x.data_ptr(), level, 2, 0.0) for x in reversed(data)])
+    d, sd, ck, lib = binding.CAttnDesc(*a), ctx._softmax_desc(shift, rounds, ec, rc), binding.CEvk(drlk.data.data_ptr(), 0), binding.load()
+    ws = ctx.workspace(int(lib.ckks_softmax_rows_workspace_bytes(ctx._h, C.byref(d), C.byref(sd), level)))
+    assert lib.ckks_softmax_rows(ctx._h, C.byref(d), C.byref(sd), ia, C.byref(ck), None, 0, oa, ws.data_ptr(), ws.numel(), None) == binding.OK
+    for x in range(G):
+        assert oa[x].scale == so and oa[x].level == want.shape[2], x
+        assert np.array_equal(host(data[G - 1 - x]).reshape(-1)[:want[x].size].reshape(want[x].shape), want[x]), x
+
+
 def test_attention_values_onto_their_operands():
     """Results in the value operands' own descriptors and buffers (more channels than one pass takes), whose scales agree within
     2^-30 without being equal: each result carries its own operand's."""
