@@ -245,6 +245,12 @@ __device__ __forceinline__ void stage_tw(double *dst, const double *tw) {
     for (uint32_t e = threadIdx.x; e < R; e += blockDim.x) dst[e] = tw[e];
 }
 
+// The end of a CTA whose limb is left out.  With limbs on the integer path that may be every CTA of a grid (a digit's own limb and
+// seven integer ones), and a grid that has not waited for the one before it lets the one after it pass that too.
+__device__ __forceinline__ void leave_out(uint32_t fp_share) {
+    if (fp_share < 8) grid_dep_sync();
+}
+
 // ---- column passes -------------------------------------------------------------------------------------------------
 // Shape per LOGR: the R-point column transform is split into a first group of A stages (registers R/2^A rows apart) and a
 // second of B stages (2^B consecutive rows; a thread holds 2^(A-B) of these), E = 2^A registers per thread, COLS columns per
@@ -271,7 +277,7 @@ __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 1024 / ColShape<LOGR>
     constexpr bool SH = TW_SHARED<LOGR>;
     __shared__ __align__(16) double stw[SH ? S::R : 2];
     const int prime = limb_prime(map, blockIdx.y);
-    if (prime < 0 || (blockIdx.y & 7) >= fp_share) return;
+    if (prime < 0 || (blockIdx.y & 7) >= fp_share) return leave_out(fp_share);
     const double q = c.modd[prime].x, qinv = c.modd[prime].y;
     const double *tw = c.twd_fwd + ((size_t)prime << c.log_n);
     const uint32_t cc = threadIdx.x % S::COLS, r = threadIdx.x / S::COLS;
@@ -342,7 +348,7 @@ __global__ void __launch_bounds__(ColShape<LOGR>::THREADS, 768 / ColShape<LOGR>:
     constexpr bool SH = TW_SHARED<LOGR>;
     __shared__ __align__(16) double stw[SH ? S::R : 2];
     const int prime = limb_prime(map, blockIdx.y);
-    if (prime < 0 || (blockIdx.y & 7) >= fp_share) return;
+    if (prime < 0 || (blockIdx.y & 7) >= fp_share) return leave_out(fp_share);
     const double q = c.modd[prime].x, qinv = c.modd[prime].y;
     const double *tw = c.twd_inv + ((size_t)prime << c.log_n);
     const uint32_t cc = threadIdx.x % S::COLS, r = threadIdx.x / S::COLS;
@@ -396,7 +402,7 @@ __global__ void __launch_bounds__(16 * ROW_CTA, 64 / ROW_CTA) ntt_fwd_rows(DevTa
     // EP 3: the entries and components of a limb next to each other, for the sake of its digits and key words in L2
     const uint32_t yl = EP == 3 ? ((blockIdx.y >> 1) % ep.nb * 2 + (blockIdx.y & 1)) * ep.level + (blockIdx.y >> 1) / ep.nb : blockIdx.y;
     const int prime = limb_prime(map, yl);
-    if (prime < 0 || (yl & 7) >= fp_share) return;
+    if (prime < 0 || (yl & 7) >= fp_share) return leave_out(fp_share);
     const double q = c.modd[prime].x, qinv = c.modd[prime].y;
     const double *tw = c.twd_fwd + ((size_t)prime << c.log_n);
     const uint32_t t = threadIdx.x & 15, rl = threadIdx.x >> 4, row = blockIdx.x * ROW_CTA + rl, R = c.N >> 8;
@@ -539,7 +545,7 @@ template <bool WIDE, uint32_t BETA = 0, class Src = NttSource>
 __global__ void __launch_bounds__(16 * ROW_CTA, 48 / ROW_CTA) ntt_inv_rows(DevTables c, u64 *base, LimbMap map, uint32_t fp_share, const __grid_constant__ Src src) {
     __shared__ __align__(16) double sm[ROW_CTA * ROW_PAD];
     const int prime = limb_prime(map, blockIdx.y);
-    if (prime < 0 || (blockIdx.y & 7) >= fp_share) return;
+    if (prime < 0 || (blockIdx.y & 7) >= fp_share) return leave_out(fp_share);
     const double q = c.modd[prime].x, qinv = c.modd[prime].y;
     const double *tw = c.twd_inv + ((size_t)prime << c.log_n);
     const uint32_t t = threadIdx.x & 15, rl = threadIdx.x >> 4, row = blockIdx.x * ROW_CTA + rl, R = c.N >> 8;

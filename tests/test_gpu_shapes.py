@@ -351,3 +351,29 @@ def test_integer_transforms_give_the_same_limbs(share):
     finally:
         ctx.set_option(binding.OPT_CONV_KERNEL, binding.CONV_FP64)
         ctx.set_option(binding.OPT_NTT_FP_SHARE, 8)
+
+
+@pytest.mark.parametrize("share", [1, 7])
+def test_transforms_that_leave_out_every_limb_of_one_path(share):
+    """One limb and one special prime with the tensor-core ModUp: at share 1 the FP64 transform of the extended digits has the
+    digit's own limb alone, which it skips, and the integer one all the rest; eight rotations in a row without a pause."""
+    from paper_2609_12378_b200 import binding
+    from tests.gpu_util import context, ct_dev, host, key_dev
+    P, ctx = params(16, 3, 1, 3), context(16, 3, 1, 3)
+    o, g = P.oracle, inputs.rng(810, share)
+    x = inputs.uniform_residues(g, P.q[:1], P.N, 2)
+    key = inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, 6).reshape(3, 2, 4, P.N)
+    gal = o.galois_element(5)
+    ctx.set_option(binding.OPT_NTT_FP_SHARE, share)
+    ctx.set_option(binding.OPT_CONV_KERNEL, binding.CONV_TENSOR)
+    try:
+        ct, k = ct_dev(x, 1.0), key_dev(key, gal)
+        for _ in range(8):
+            ct = ctx.rotate(ct, k)
+        want = x
+        for _ in range(8):
+            want = o.rotate(want, key, gal)
+        assert np.array_equal(host(ct.data), want)
+    finally:
+        ctx.set_option(binding.OPT_CONV_KERNEL, binding.CONV_FP64)
+        ctx.set_option(binding.OPT_NTT_FP_SHARE, 8)
