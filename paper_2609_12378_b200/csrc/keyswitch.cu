@@ -81,11 +81,12 @@ __device__ __forceinline__ void conv_store(u64 *p, const double (&v)[CPT]) {
 inline uint32_t conv_cpt(uint32_t ns, const void *a, const void *b) { return ns <= 8 && (((uintptr_t)a | (uintptr_t)b) & 15) == 0 ? 2 : 1; }
 
 // targets per CTA (grid y) for `items` conversions of `targets` targets over gx CTAs: all of them, unless that leaves fewer than
-// two CTAs per SM.  Every chunk loads and centres its sources again, which costs more than a machine that is only partly
-// filled (one ciphertext at N = 2^16, level 24: ModUp with 24, 8, 5 targets per CTA 21.7, 22.7, 26.0 us).
+// 512 threads (four CTAs) per SM.  Every chunk loads and centres its sources again, which costs more than a machine that is
+// only partly filled (one ciphertext at N = 2^16, level 24: ModUp with 24, 8, 5 targets per CTA 21.7, 22.7, 26.0 us, taken with
+// CTAs of 256 threads, two per SM).
 constexpr uint32_t CONV_CHUNK_MAX = 32;
-inline uint32_t conv_chunk(uint32_t gx, uint32_t items, uint32_t targets) {
-    const uint32_t want = 2 * 148 * 256 / CONV_THREADS;
+inline uint32_t conv_chunk(const ckks_ctx *c, uint32_t gx, uint32_t items, uint32_t targets) {
+    const uint32_t want = (uint32_t)c->sms * (512 / CONV_THREADS);
     uint32_t chunks = (want + gx * items - 1) / (gx * items);
     chunks = std::max(1u, std::min(chunks, (targets + 1) / 2));
     return std::min(CONV_CHUNK_MAX, (targets + chunks - 1) / chunks);
@@ -141,7 +142,7 @@ template <uint32_t ALPHA>
 void launch_modup(const ckks_ctx *c, const u64 *dcoef, u64 *ext, uint32_t level, uint32_t nb, cudaStream_t s) {
     const uint32_t nt = level + c->K, beta = (level + c->alpha - 1) / c->alpha;
     const uint32_t cpt = conv_cpt(ALPHA, dcoef, ext), gx = c->N / (CONV_THREADS * cpt), targets = nt - (level - (beta - 1) * c->alpha);   // the last digit has the most targets
-    const uint32_t CHUNK = conv_chunk(gx, beta * nb, targets);
+    const uint32_t CHUNK = conv_chunk(c, gx, beta * nb, targets);
     const dim3 grid(gx, (targets + CHUNK - 1) / CHUNK, beta * nb);
     constexpr uint32_t WIDE = ALPHA <= 8 ? 2 : 1;
     launch(cpt == WIDE ? modup_kernel<ALPHA, WIDE> : modup_kernel<ALPHA, 1>, grid, CONV_THREADS, 0, s, c->dev, dcoef, ext, level, CHUNK);
@@ -426,7 +427,7 @@ __global__ void __launch_bounds__(CONV_THREADS) moddown_conv_kernel(DevTables c,
 
 template <uint32_t KK, bool RS>
 void launch_moddown_conv(const ckks_ctx *c, const u64 *u, u64 *conv, uint32_t level, uint32_t nb, cudaStream_t s) {
-    const uint32_t targets = level - RS, cpt = conv_cpt(KK, u, conv), gx = c->N / (CONV_THREADS * cpt), CHUNK = conv_chunk(gx, 2 * nb, targets);
+    const uint32_t targets = level - RS, cpt = conv_cpt(KK, u, conv), gx = c->N / (CONV_THREADS * cpt), CHUNK = conv_chunk(c, gx, 2 * nb, targets);
     const dim3 grid(gx, (targets + CHUNK - 1) / CHUNK, 2 * nb);
     constexpr uint32_t WIDE = KK <= 8 ? 2 : 1;
     launch(cpt == WIDE ? moddown_conv_kernel<KK, WIDE, RS> : moddown_conv_kernel<KK, 1, RS>, grid, CONV_THREADS, 0, s, c->dev, u, conv, level, targets, CHUNK);
