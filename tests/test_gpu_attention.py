@@ -448,24 +448,28 @@ def test_attention_block_from_projections_to_projection_bit_exact():
 
 
 def test_lanes_do_not_change_results():
-    """The attention entry points spread independent chains over the context's streams (option CKKS_OPT_LANES); one lane
-    (the caller's stream only) and four give the same limbs, on the caller's stream in both cases."""
-    from tests.gpu_util import host
-    P, ctx, o, cl, desc, c, scale, q, k, v, rlk, keys, dev = _setup(10, 13, 4, 4, 13, 16, 2, 4, 4, 3, 641)
-    a = (16, 2, 4)
+    """The layout conversions spread their channels over the context's streams (option CKKS_OPT_LANES): one lane (the caller's
+    stream only) to four give the checker's limbs, on the caller's stream in every case."""
+    from tests.gpu_util import context, ct_dev, host, key_dev
+    P, ctx = params(10, 6, 2, 3), context(10, 6, 2, 3)
+    o, g = P.oracle, inputs.rng(642, 0)
+    a, dim, level = (16, 8, 4, 4), 7, 6
+    desc = AttnDesc(*a[:3], 1, a[3])
+    rots = set(ctx.attention_pack_rotations(binding.ATTN_KEY_VALUE, dim, *a))
+    keys = {o.galois_element(r): inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, 6).reshape(3, 2, 8, P.N) for r in rots}
+    dkeys = [key_dev(k, ge) for ge, k in keys.items()]
+    shards = np.stack([inputs.uniform_residues(g, P.q[:level], P.N, 2) for _ in range(4)])
+    want = o.attention_pack(desc, 1, shards, dim, keys)
+    dcts = [ct_dev(x, 2.0 ** 40) for x in shards]
     assert ctx.get_option(binding.OPT_LANES) == 4
-    res = {}
     try:
-        for lanes in (1, 4, 2):
+        for lanes in (1, 4, 2, 3):
             ctx.set_option(binding.OPT_LANES, lanes)
-            out = ctx.attention(dev["q"], dev["k"], dev["v"], c["shift"], 1, c["exp_coeffs"], c["rsqrt_coeffs"], dev["rlk"], dev["keys"], *a)
-            res[lanes] = [host(x.data) for x in out]
+            out = ctx.attention_pack(binding.ATTN_KEY_VALUE, dcts, dim, dkeys, *a)
+            for d in range(dim):
+                assert np.array_equal(host(out[d].data), want[d]), (lanes, d)
     finally:
         ctx.set_option(binding.OPT_LANES, 4)
-    want, _ = o.attention(desc, q, k, v, scale, scale, c["shift"], 1, c["exp_coeffs"], c["rsqrt_coeffs"], rlk, keys)
-    for lanes in (1, 2, 4):
-        for d in range(3):
-            assert np.array_equal(res[lanes][d], want[d]), (lanes, d)
     with pytest.raises(binding.CkksError):
         ctx.set_option(binding.OPT_LANES, 5)
     assert ctx.device_status() == binding.OK
