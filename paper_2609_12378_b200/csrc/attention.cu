@@ -1,5 +1,5 @@
-// Attention in the diagonal-block layout: compositions of the entry points of api.cu on buffers carved from the caller's
-// workspace.  No kernels of its own.
+// Attention in the diagonal-block layout on buffers carved from the caller's workspace: the products from the batched steps of
+// batch.cu and poly.cu, the layout conversions from the entry points of api.cu.  No kernels of its own.
 //
 // Layout.  Every operand and every score ciphertext uses the slot index
 //     slot = ((e * tokens + i) * heads + h) * R + r,      R = n / (diag_block * tokens * heads),

@@ -214,7 +214,8 @@ __device__ __forceinline__ void inv_col_last(double (&x)[E], const double *__res
 
 // ---- measurement aid: the forward butterflies on registers only ------------------
 // Every thread runs `iters` radix-16 groups (4 stages, 32 butterflies, with the transform's range reductions and twiddle
-// fetches, the latter from a 64 KiB window that stays in L1/L2) on 16 registers; nothing else touches memory.
+// fetches, the latter from a 17 KiB window that stays in L1) on 16 registers; nothing else touches memory.  Three CTAs of 256
+// threads per SM: 24 warps, the inverse transform's occupancy (the forward passes run at 32).
 constexpr uint32_t F_THREADS = 256;
 __global__ void __launch_bounds__(F_THREADS, 3) butterfly_probe_kernel(DevTables c, uint32_t iters, u64 *sink) {
     grid_dep_sync();
@@ -871,7 +872,7 @@ void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbM
     }
 }
 
-// grid: three CTAs per SM, the residency of the transform kernels.  Returns the butterflies one launch performs.
+// grid: three CTAs per SM, all resident at once.  Returns the butterflies one launch performs.
 uint64_t launch_butterfly_probe(const ckks_ctx *c, uint32_t iters, u64 *sink, cudaStream_t s) {
     const uint32_t ctas = (uint32_t)c->sms * 3;
     launch(butterfly_probe_kernel, ctas, F_THREADS, 0, s, c->dev, iters, sink);

@@ -59,8 +59,8 @@ extern "C" int32_t ckks_rescale_static(ckks_ctx *c, const ckks_ct *in, ckks_ct *
     u64 *scratch = nullptr;
     cudaError_t e = scratch_address(c->device, &scratch);
     if (e != cudaSuccess) { c->cuda_error = cudaGetErrorString(e); return CKKS_ERR_CUDA; }
-    // Nothing in the scratch has to start at zero: the last limbs are copied in and every lifted limb is written
-    // before it is read, so whatever the previous call left there is simply overwritten.
+    // Nothing in the scratch has to start at zero: the dropped limbs' inverse transforms and every lifted limb are written
+    // before they are read, so whatever the previous call left there is simply overwritten.
     launch_rescale(c, Ptrs((const u64 *)in->data, 0), Ptrs((const u64 *)out->data, 0), in->ncomp, in->level, scratch, (cudaStream_t)stream, 1, true);
     e = cudaGetLastError();
     if (e != cudaSuccess) { c->cuda_error = cudaGetErrorString(e); return CKKS_ERR_CUDA; }
