@@ -637,6 +637,11 @@ extern "C" int32_t ckks_rotate_sum(ckks_ctx *c, const ckks_ct *in, const ckks_ev
         const uint32_t m = std::min(MRB_CHUNK, n - i0);
         for (uint32_t i = 0; i < m; i++)
             cudaMemcpyAsync(xin + (size_t)i * ctl, in[i0 + i].data, ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
+        w.mid = true;
+        for (uint32_t i = 0; i < m; i++) {
+            const u64 *evk = (const u64 *)keys[i0 + i].data;
+            w.mid = w.mid && ks_mid(c, level, w, Ptrs(xin + ptl, ctl), &evk, 1);
+        }
         ks_modup(c, Ptrs(xin + ptl, ctl), level, w, s, m);
         // every term has its own digits, key and first component; all of them add into entry 0 of the inner-product
         // buffer, the first components multiplied by P so that the one ModDown returns them unchanged
@@ -865,6 +870,7 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
                         KsOut ko;
                         ko.add = Ptrs(ag, ctl); ko.out = Ptrs(rot, ctl);
                         ko.add_comps = 1;
+                        kg.mid = ks_mid(c, level, kg, Ptrs(ag + ptl, ctl), m.evk, nr);
                         ks_modup(c, Ptrs(ag + ptl, ctl), level, kg, s, nr * S);
                         ks_apply(c, nullptr, level, kg, ko, s, nr * S, &m);
                         launch_sum(c, total, first, rot, nr, S, level, s);
@@ -881,20 +887,23 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
                     }
                     const uint32_t nup = std::min(lazy_giants(S), ng - gl);
                     u64 *ag = acc + (size_t)gl * S * ctl;
+                    std::vector<IpTerms> tms((nup + IP_TERMS - 1) / IP_TERMS);
+                    kx.mid = true;
+                    for (uint32_t t = 0; t < nup; t++) {
+                        IpTerms &tm = tms[t / IP_TERMS];
+                        const u64 ge = ckks_galois_element(c, (int64_t)(g0 + gl + t) * B * T);
+                        tm.evk[t % IP_TERMS] = (const u64 *)find_key(keys, nkeys, ge)->data;
+                        tm.galois[t % IP_TERMS] = ge;
+                        tm.c0[t % IP_TERMS] = ag + (size_t)t * S * ctl;
+                        kx.mid = kx.mid && ks_mid(c, level, kx, Ptrs(ag + ptl, ctl), &tm.evk[t % IP_TERMS], 1);
+                    }
                     ks_modup(c, Ptrs(ag + ptl, ctl), level, kx, s, nup * S);
                     for (uint32_t t0 = 0; t0 < nup; t0 += IP_TERMS) {
                         const uint32_t nterm = std::min(IP_TERMS, nup - t0);
-                        IpTerms tm{};
-                        for (uint32_t t = 0; t < nterm; t++) {
-                            const u64 ge = ckks_galois_element(c, (int64_t)(g0 + gl + t0 + t) * B * T);
-                            tm.evk[t] = (const u64 *)find_key(keys, nkeys, ge)->data;
-                            tm.galois[t] = ge;
-                            tm.c0[t] = ag + (size_t)(t0 + t) * S * ctl;
-                        }
                         KsWorkspace kt = kx;
                         kt.ext = kx.ext + (size_t)t0 * S * kbeta * knt * N;
                         kt.d.base += (size_t)t0 * S * ctl;
-                        ks_inner_terms(c, level, kt, (size_t)S * kbeta * knt * N, tm, nterm, ctl, s, S, u_live);
+                        ks_inner_terms(c, level, kt, (size_t)S * kbeta * knt * N, tms[t0 / IP_TERMS], nterm, ctl, s, S, u_live);
                         u_live = true;
                     }
                     gl += nup;

@@ -4,6 +4,7 @@
 
 // o[i] (2 x level limbs) += key switch of e2[i], nb side by side
 void relinearise(const ckks_ctx *c, const u64 *rlk, const Ptrs &e2, const Ptrs &o, uint32_t level, KsWorkspace &w, cudaStream_t s, uint32_t nb) {
+    w.mid = ks_mid(c, level, w, e2, &rlk, 1);
     ks_modup(c, e2, level, w, s, nb);
     KsOut ko;
     ko.add = ko.out = o;
@@ -18,6 +19,7 @@ void relin_rescale(const ckks_ctx *c, const u64 *rlk, const Ptrs &e2, const Ptrs
         launch_rescale(c, e01, out, 2, level, ksw, s, nb);
         return;
     }
+    w.mid = ks_mid(c, level, w, e2, &rlk, 1) && aligned16(e01);
     ks_modup(c, e2, level, w, s, nb);
     ks_apply_rescale(c, rlk, level, w, e01, out, s, nb);
 }
@@ -51,12 +53,14 @@ void rotate_ks(const ckks_ctx *c, const ckks_evk *key, const Ptrs &in, const Ptr
     const size_t ptl = (size_t)level * c->N;
     if (in.n) for (uint32_t b = 0; b < in.n; b++) c1.p[b] += ptl;
     else c1.base += ptl;
+    const u64 *evk = (const u64 *)key->data;
+    w.mid = ks_mid(c, level, w, c1, &evk, 1);
     ks_modup(c, c1, level, w, s, nb);
     KsOut ko;
     ko.add = in; ko.out = out;
     ko.add_comps = 1; ko.galois = key->galois;
     if (acc) ko.acc = *acc;
-    ks_apply(c, (const u64 *)key->data, level, w, ko, s, nb);
+    ks_apply(c, evk, level, w, ko, s, nb);
 }
 
 static bool same_views(const std::vector<CtView> &x, const std::vector<CtView> &y) {

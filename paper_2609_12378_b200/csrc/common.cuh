@@ -354,10 +354,9 @@ inline bool aligned16(const Ptrs &p) {
 //           acc (if given): [ncomp][level][N] words per entry;
 //           out: plain ([ncomp][level][N] per entry) or tiled (tl.R != 0, component comp of entry b in row
 //           tl.row0 + b * tl.row_stride + comp)
-//   mode 3: as mode 1, but the sum u is not read: it is formed here, u = <digits, key> (add_p: + P add, and nothing is
-//           added afterwards).  Digits are read through sigma_galois as well; beta <= IP_FUSED_BETA of them
-//           (inverse: the input is not read but formed as u, for the limbs x0 .. of the extended basis; the map's periods are the
-//           entries' components)
+//   mode 3: as mode 1, but the sum u is not read: it is formed here, u = <digits, key>.  Digits are read through sigma_galois
+//           as well; beta <= IP_FUSED_BETA of them (inverse: the input is not read but formed as u, for the special limbs; the
+//           map's periods are the entries' components)
 //   mode 2: the transform's own result is stored, but into a tiled buffer (out.base): limb y = b * level + i becomes row
 //           tl.row0 + b * tl.row_stride, limb i
 constexpr uint32_t IP_FUSED_BETA = 4;
@@ -376,10 +375,10 @@ struct NttEpilogue {
     uint32_t group, own, rot_rows;
     size_t rot_stride;
     // mode 3: extended digits [entry][beta][nt][N] and the digits' own limbs (shared: entry 0 for all), the key (multi: one per
-    // rotation), the limbs per component of `add`, the batch
+    // rotation), the batch
     const u64 *ext, *evk, *mevk[KS_MULTI];
     Ptrs d;
-    uint32_t beta, shared, add_level, add_p, nb, x0;    // x0: (inverse) extended-basis limb of the map's first
+    uint32_t beta, shared, nb;
     uint32_t y0;           // (filled in) first limb of the launch
 };
 // Prologue of the forward transform: the first pass reads one buffer [batch][N] (batch = limb index / map.period) instead of
@@ -402,6 +401,10 @@ struct NttSource {
 // pointer), so that the output is scaled by a per-limb constant.
 void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbMap &map, bool inverse, cudaStream_t s,
                 const NttEpilogue *ep = nullptr, const NttPrologue *pro = nullptr, const NttSource *src = nullptr, const double2 *inv_scale = nullptr, bool alone = false);
+// One of the two passes alone, or both; limbs are signed doubles between the passes
+enum NttPart { NTT_ROWS = 1, NTT_COLS = 2, NTT_BOTH = 3 };
+void launch_ntt_part(const ckks_ctx *c, NttPart part, u64 *base, uint32_t nlimbs_total, const LimbMap &map, bool inverse, cudaStream_t s, const NttEpilogue *ep = nullptr,
+                     const NttPrologue *pro = nullptr, const NttSource *src = nullptr, const double2 *inv_scale = nullptr);
 void launch_ntt_int(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, bool inverse, const NttSource &src, cudaStream_t s);
 
 void launch_mul_plain_acc(const ckks_ctx *c, const u64 *const *cts, u64 *const *accs, uint32_t ncts, const u64 *pt,
@@ -440,6 +443,7 @@ struct KsWorkspace {
     u64 *dcoef, *ext, *u, *conv;
     Ptrs d;
     bool alone = false;     // the key switch is an entry point's only one: see launch_ntt
+    bool mid = false;       // ext is left after the column pass, for launch_mid_rows (set before ks_modup, see ks_mid)
 };
 size_t ks_workspace_limbs(const ckks_ctx *c, uint32_t level);
 KsWorkspace ks_carve(const ckks_ctx *c, uint32_t level, void *ws, uint32_t nb = 1);
@@ -462,6 +466,8 @@ struct KsOut {
     TiledOut tiled;
 };
 void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb = 1, const KsMulti *multi = nullptr);
+// Whether launch_mid_rows takes the digits d of key switches, which serve one key each (nkeys keys in all)
+bool ks_mid(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const Ptrs &d, const u64 *const *evk, uint32_t nkeys);
 // Both together: out = ModDown(<digits, key>) and the final combination, digits read through the permutation of o.galois
 void ks_apply(const ckks_ctx *c, const u64 *evk, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb = 1, const KsMulti *multi = nullptr);
 // out = rescale(ModDown(<digits, key>) + add), level - 1 limbs per component, without the tensor-core conversions (see ks_fused_rescale)
@@ -481,6 +487,21 @@ struct IpTerms {
 };
 void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, size_t term_stride, const IpTerms &terms, uint32_t nterm,
                     size_t c0_stride, cudaStream_t s, uint32_t nb, bool acc_u);
+// The middle of a key switch whose digits serve one key each (mid_rows.cu): forward row pass of the extended digits (ext, after the
+// column pass), inner product, inverse row pass of the limbs from inv_from on.
+//   u[b] (+)= sum_t ( <ext[t][b] read through sigma_{g_t}, evk_t>  +  P sigma_{g_t}(c0_t[b]) )  +  P add[b]
+// terms as in ks_inner_terms; with one term, entry b may have key b / group instead (group > 0)
+struct MidArgs {
+    const u64 *ext;
+    Ptrs d, add;
+    u64 *u;
+    const u64 *evk[KS_MULTI], *c0[IP_TERMS];
+    u64 galois[KS_MULTI];
+    size_t term_stride, c0_stride;
+    uint32_t nterm, nb, level, group, inv_from;
+    int has_add, acc_u;
+};
+void launch_mid_rows(const ckks_ctx *c, const MidArgs &a, uint32_t beta, cudaStream_t s);
 // The basis conversions on the tensor cores (contexts with byte matrices: at most 8 sources)
 void launch_modup_mma(const ckks_ctx *c, const u64 *dcoef, u64 *ext, uint32_t level, uint32_t nb, cudaStream_t s);
 void launch_moddown_conv_mma(const ckks_ctx *c, const u64 *u, u64 *conv, uint32_t level, uint32_t nb, cudaStream_t s);

@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(THREADS) inner_product_generic_kernel(DevTable
 // pair (s, s ^ 1), so digits and key words both move as 16-byte loads.  Without `multi` a thread walks `bch` batch
 // entries (blockIdx.y picks the chunk) with the key words of its pair held in registers; with it, an entry is one
 // of up to KS_MULTI keys applied to the same digits.
-constexpr uint32_t IP_MAX_BETA = 8, IP_TERMS_MAX_BETA = 4;
+constexpr uint32_t IP_MAX_BETA = 8;
 template <uint32_t BETA, bool ADD>
 __global__ void __launch_bounds__(IP_THREADS) inner_product_kernel(DevTables c, const u64 *ext, const __grid_constant__ Ptrs d, const u64 *evk, u64 g, u64 *u,
                                                                 uint32_t level, uint32_t nb, uint32_t bch, int has_multi, const __grid_constant__ KsMulti multi,
@@ -269,94 +269,6 @@ __global__ void __launch_bounds__(IP_THREADS) inner_product_kernel(DevTables c, 
             if (acc_u) {
                 const ulonglong2 old = *reinterpret_cast<const ulonglong2 *>(o + cm * js);
                 const u64 m = c.mod[kt];
-                r.x = add_mod(r.x, old.x, m);
-                r.y = add_mod(r.y, old.y, m);
-            }
-            *reinterpret_cast<ulonglong2 *>(o + cm * js) = r;
-        }
-    }
-}
-
-// The inner product of several terms at once (see ks_inner_terms): like inner_product_kernel, but every term has its
-// own digits, key, permutation and first component, and the running sums of a chunk of IP_BCH batch entries stay in
-// registers over the terms.
-// Two entries per thread at 64 registers and 32 warps per SM: four entries at 85 registers kept too few loads in flight (the
-// 4096 x 4096 projection's share: 20.2 -> 17.4 ms; one entry 19.9, two at 48 registers 21.3).
-constexpr uint32_t IP_BCH = 2;
-template <uint32_t BETA>
-__global__ void __launch_bounds__(IP_THREADS, 8) inner_product_terms_kernel(DevTables c, const u64 *ext, size_t term_stride, const u64 *d, size_t d_stride,
-                                                                         const __grid_constant__ IpTerms tm, uint32_t nterm, size_t c0_stride,
-                                                                         u64 *u, uint32_t level, uint32_t nb, int acc_u) {
-    const uint32_t p = (blockIdx.x * IP_THREADS + threadIdx.x) * 2;
-    const uint32_t x = blockIdx.z, b0 = blockIdx.y * IP_BCH;
-    const uint32_t nt = level + c.K;
-    const uint32_t kt = x < level ? x : c.L + (x - level);
-    const double2 md = c.modd[kt];
-    const size_t js = (size_t)nt * c.N, ks = (size_t)c.T * c.N;
-    const double pq = x < level ? c.dn_p_mod_d[x] : 0.0;
-    const uint32_t own = x < level ? x / c.alpha : BETA;       // the digit that has x among its own limbs: it lies in d
-    double acc[IP_BCH][2][2];
-#pragma unroll
-    for (uint32_t bi = 0; bi < IP_BCH; bi++) acc[bi][0][0] = acc[bi][0][1] = acc[bi][1][0] = acc[bi][1][1] = 0.0;
-    grid_dep_sync();
-    for (uint32_t t = 0; t < nterm; t++) {
-        const uint32_t src = galois_src(p, (uint32_t)tm.galois[t], c.log_n);
-        const bool odd = src & 1;
-        const u64 *evk = tm.evk[t];
-        double k[BETA][2][2];
-#pragma unroll
-        for (uint32_t j = 0; j < BETA; j++)
-#pragma unroll
-            for (uint32_t cm = 0; cm < 2; cm++) {
-                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(evk + ((size_t)j * 2 + cm) * ks + (size_t)kt * c.N + p);
-                k[j][cm][0] = u64_to_d(v.x);
-                k[j][cm][1] = u64_to_d(v.y);
-            }
-        const uint32_t so = src & ~1u;
-        const u64 *z = (x < level && tm.c0[t]) ? tm.c0[t] + b0 * c0_stride + (size_t)x * c.N : nullptr;
-        // no branch in here, so that the loads of all entries of the chunk are in flight together: an entry past the end
-        // of the batch repeats the last one and is not stored
-#pragma unroll
-        for (uint32_t bi = 0; bi < IP_BCH; bi++) {
-            const uint32_t bc = min(bi, nb - 1 - b0);
-            double sum[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-#pragma unroll
-            for (uint32_t j = 0; j < BETA; j++) {
-                const u64 *ej = (j == own ? d + (size_t)(t * nb + b0 + bc) * d_stride
-                                          : ext + t * term_stride + ((size_t)(b0 + bc) * BETA + j) * js) + (size_t)x * c.N;
-                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(ej + so);
-                const double d0 = u64_to_d(odd ? v.y : v.x), d1 = u64_to_d(odd ? v.x : v.y);
-#pragma unroll
-                for (uint32_t cm = 0; cm < 2; cm++) {
-                    sum[cm][0] = __dadd_rn(sum[cm][0], mulmod_dd(d0, k[j][cm][0], md.x, md.y));
-                    sum[cm][1] = __dadd_rn(sum[cm][1], mulmod_dd(d1, k[j][cm][1], md.x, md.y));
-                }
-            }
-            if (z) {
-                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(z + bc * c0_stride + so);
-                sum[0][0] = __dadd_rn(sum[0][0], mulmod_dd(u64_to_d(odd ? v.y : v.x), pq, md.x, md.y));
-                sum[0][1] = __dadd_rn(sum[0][1], mulmod_dd(u64_to_d(odd ? v.x : v.y), pq, md.x, md.y));
-            }
-            // at most BETA + 1 products of size 0.75 m on top of a reduced sum: far below 2^53
-#pragma unroll
-            for (uint32_t cm = 0; cm < 2; cm++) {
-                acc[bi][cm][0] = reduce_d(__dadd_rn(acc[bi][cm][0], sum[cm][0]), md.x, md.y);
-                acc[bi][cm][1] = reduce_d(__dadd_rn(acc[bi][cm][1], sum[cm][1]), md.x, md.y);
-            }
-        }
-    }
-    const u64 m = c.mod[kt];
-#pragma unroll
-    for (uint32_t bi = 0; bi < IP_BCH; bi++) {
-        if (b0 + bi >= nb) break;
-        u64 *o = u + (size_t)(b0 + bi) * 2 * js + (size_t)x * c.N + p;
-#pragma unroll
-        for (uint32_t cm = 0; cm < 2; cm++) {
-            ulonglong2 r;
-            r.x = canonical_d(acc[bi][cm][0], md.x);
-            r.y = canonical_d(acc[bi][cm][1], md.x);
-            if (acc_u) {
-                const ulonglong2 old = *reinterpret_cast<const ulonglong2 *>(o + cm * js);
                 r.x = add_mod(r.x, old.x, m);
                 r.y = add_mod(r.y, old.y, m);
             }
@@ -517,7 +429,8 @@ void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, 
         DISPATCH_POW2(c->alpha, CALL_UP);
 #undef CALL_UP
     }
-    launch_ntt(c, w.ext, nb * beta * nt, ext_map(level, c->K, c->L, c->alpha, beta), false, s, nullptr, conv_tensor(c) ? nullptr : &CONV_OUT, nullptr, nullptr, w.alone);
+    if (w.mid) launch_ntt_part(c, NTT_COLS, w.ext, nb * beta * nt, ext_map(level, c->K, c->L, c->alpha, beta), false, s, nullptr, conv_tensor(c) ? nullptr : &CONV_OUT);
+    else launch_ntt(c, w.ext, nb * beta * nt, ext_map(level, c->K, c->L, c->alpha, beta), false, s, nullptr, conv_tensor(c) ? nullptr : &CONV_OUT, nullptr, nullptr, w.alone);
 }
 
 void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois, const KsWorkspace &w, cudaStream_t s, uint32_t nb,
@@ -562,11 +475,32 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
     }
 }
 
+// mid_rows takes up to IP_FUSED_BETA digits and 16-byte accesses (one rotation at N = 2^16, level 24: 153 -> 149.4 us, at N = 2^14 32.8 ->
+// 29.4; the degree-63 polynomial 2139 -> 2091; projections of 24 tokens, which sum their giant steps, 32.1 -> 31.7 ms)
+bool ks_mid(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const Ptrs &d, const u64 *const *evk, uint32_t nkeys) {
+    bool ok = (level + c->alpha - 1) / c->alpha <= IP_FUSED_BETA && aligned16(w.ext) && aligned16(w.u) && aligned16(d);
+    for (uint32_t k = 0; k < nkeys; k++) ok = ok && aligned16(evk[k]);
+    return ok;
+}
+static void mid_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 galois, const KsWorkspace &w, uint32_t inv_from, cudaStream_t s, uint32_t nb, const KsMulti *multi,
+                      const Ptrs *add) {
+    MidArgs a{};
+    a.ext = w.ext; a.d = w.d; a.u = w.u;
+    a.nterm = 1; a.nb = nb; a.level = level; a.inv_from = inv_from;
+    a.evk[0] = evk; a.galois[0] = galois;
+    if (multi) {
+        a.group = multi->group;
+        for (uint32_t r = 0; r < nb / multi->group; r++) { a.evk[r] = multi->evk[r]; a.galois[r] = multi->galois[r]; }
+    }
+    if (add) { a.has_add = 1; a.add = *add; }
+    launch_mid_rows(c, a, (level + c->alpha - 1) / c->alpha, s);
+}
+
 // Whether the row pass that ends a ModDown forms the inner product's q-limbs itself (mode 3 of the epilogue), so that the sum u
 // is written and read back for the special limbs only.  It does where a key word serves fewer than four entries (four or more share
 // it from registers in inner_product_kernel, where this form would read it from L2 for each) and the pass fills the GPU once:
 // below that its eight steps of dependent reads cost more than the traffic (64 hoisted rotations at N = 2^16, level 24:
-// 4550 -> 4110 us; the key/value projections of 24 tokens 35.9 -> 34.3 ms).  Operands have to take 16-byte accesses.
+// 4550 -> 4110 us; the key/value projections of 24 tokens 35.9 -> 34.3 ms).  Digits that serve one key go through mid_rows instead.  Operands have to take 16-byte accesses.
 static bool inner_fused(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const u64 *evk, uint32_t nb, const KsMulti *multi) {
     const uint32_t beta = (level + c->alpha - 1) / c->alpha, nkeys = multi ? (multi->group ? nb / multi->group : nb) : 0, per = multi ? multi->group : nb;
     bool ok = per < 4 && beta <= IP_FUSED_BETA && nb * 2 * level <= 32768 && (uint64_t)nb * 2 * level * (c->N >> 10) >= 16 * (uint64_t)c->sms &&
@@ -580,7 +514,6 @@ static void fuse_inner(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, 
     ep.ext = w.ext; ep.d = w.d; ep.evk = evk; ep.nb = nb;
     ep.beta = (level + c->alpha - 1) / c->alpha;
     ep.shared = multi && !multi->group;
-    ep.add_level = level;
     if (multi) for (uint32_t b = 0; b < KS_MULTI; b++) ep.mevk[b] = multi->evk[b];
 }
 static bool out_aligned(const NttEpilogue &ep) { return aligned16(ep.add) && aligned16(ep.acc) && aligned16(ep.out) && (ep.rot_stride & 1) == 0; }
@@ -604,9 +537,9 @@ static NttEpilogue moddown_epilogue(const ckks_ctx *c, uint32_t level, const KsW
 static void moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, NttEpilogue ep, cudaStream_t s, uint32_t nb) {
     const uint32_t N = c->N, nt = level + c->K, K = c->K;
     // the K special limbs of every (batch, component): groups of K limbs, nt limbs apart
-    ep.x0 = level;
-    launch_ntt(c, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, ep.mode == 3 ? &ep : nullptr, nullptr, nullptr,
-               conv_tensor(c) ? nullptr : c->dev.inv_scale_dn, w.alone);
+    const double2 *scale = conv_tensor(c) ? nullptr : c->dev.inv_scale_dn;
+    if (w.mid) launch_ntt_part(c, NTT_COLS, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, nullptr, nullptr, nullptr, scale);
+    else launch_ntt(c, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, ep.mode == 3 ? &ep : nullptr, nullptr, nullptr, scale, w.alone);
     if (conv_tensor(c)) {
         launch_moddown_conv_mma(c, w.u, w.conv, level, nb, s);
     } else {
@@ -617,10 +550,17 @@ static void moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, Ntt
     launch_ntt(c, w.conv, nb * 2 * level, plain_map(0, level), false, s, &ep, conv_tensor(c) ? nullptr : &CONV_OUT);
 }
 void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb, const KsMulti *multi) {
-    moddown(c, level, w, moddown_epilogue(c, level, w, o, nb, multi), s, nb);
+    KsWorkspace wd = w;
+    wd.mid = false;         // all of u is in the evaluation domain
+    moddown(c, level, wd, moddown_epilogue(c, level, wd, o, nb, multi), s, nb);
 }
 void ks_apply(const ckks_ctx *c, const u64 *evk, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb, const KsMulti *multi) {
     NttEpilogue ep = moddown_epilogue(c, level, w, o, nb, multi);
+    if (w.mid) {
+        mid_inner(c, evk, level, o.galois, w, level, s, nb, multi, nullptr);
+        moddown(c, level, w, ep, s, nb);
+        return;
+    }
     const bool fused = inner_fused(c, level, w, evk, nb, multi) && out_aligned(ep);
     if (fused) fuse_inner(c, level, w, evk, nb, multi, ep);
     else ks_inner(c, evk, level, o.galois, w, s, nb, false, multi);
@@ -640,15 +580,11 @@ void ks_apply_rescale(const ckks_ctx *c, const u64 *evk, uint32_t level, const K
     ep.out = out;
     ep.pinv = c->dev.rs_p_inv_d + (size_t)m * c->L;
     ep.ncomp = 2; ep.level = m; ep.nt = nt; ep.galois = 1;
-    const bool fused = inner_fused(c, level, w, evk, nb, nullptr) && out_aligned(ep) && aligned16(add);
-    if (fused) {
-        fuse_inner(c, level, w, evk, nb, nullptr, ep);
-        ep.add = add; ep.add_comps = 3; ep.add_p = 1; ep.x0 = m;
-    } else {
-        ks_inner(c, evk, level, 1, w, s, nb, false, nullptr, &add);
-    }
+    if (w.mid) mid_inner(c, evk, level, 1, w, m, s, nb, nullptr, &add);
+    else ks_inner(c, evk, level, 1, w, s, nb, false, nullptr, &add);
     // the dropped limb and the K special limbs of every (batch, component), nt limbs apart
-    launch_ntt(c, w.u + (size_t)m * N, nb * 2 * (K + 1), tail_map(m, level, K, c->L), true, s, fused ? &ep : nullptr, nullptr, nullptr, c->dev.inv_scale_rs + (size_t)m * (K + 1) * 2);
+    launch_ntt_part(c, w.mid ? NTT_COLS : NTT_BOTH, w.u + (size_t)m * N, nb * 2 * (K + 1), tail_map(m, level, K, c->L), true, s, nullptr, nullptr, nullptr,
+                    c->dev.inv_scale_rs + (size_t)m * (K + 1) * 2);
 #define CALL_DN(A) launch_moddown_conv<A, true>(c, w.u, w.conv, level, nb, s)
     DISPATCH_POW2(K, CALL_DN);
 #undef CALL_DN
@@ -658,12 +594,13 @@ void ks_apply_rescale(const ckks_ctx *c, const u64 *evk, uint32_t level, const K
 void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, size_t term_stride, const IpTerms &terms, uint32_t nterm,
                     size_t c0_stride, cudaStream_t s, uint32_t nb, bool acc_u) {
     const uint32_t N = c->N, nt = level + c->K, beta = (level + c->alpha - 1) / c->alpha;
-    bool aligned = aligned16(w.ext) && aligned16(w.u) && (term_stride & 1) == 0 && (c0_stride & 1) == 0 && aligned16(w.d);
-    for (uint32_t t = 0; t < nterm; t++) aligned = aligned && aligned16(terms.evk[t]) && aligned16(terms.c0[t]);
-    if (beta <= IP_TERMS_MAX_BETA && aligned) {
-        const dim3 grid(N / (2 * IP_THREADS), (nb + IP_BCH - 1) / IP_BCH, nt);
-        auto *k = beta == 1 ? inner_product_terms_kernel<1> : beta == 2 ? inner_product_terms_kernel<2> : beta == 3 ? inner_product_terms_kernel<3> : inner_product_terms_kernel<4>;
-        launch(k, grid, IP_THREADS, 0, s, c->dev, w.ext, term_stride, w.d.base, w.d.stride, terms, nterm, c0_stride, w.u, level, nb, acc_u ? 1 : 0);
+    if (w.mid) {
+        MidArgs a{};
+        a.ext = w.ext; a.d = w.d; a.u = w.u;
+        a.nterm = nterm; a.nb = nb; a.level = level; a.inv_from = nt;
+        a.term_stride = term_stride; a.c0_stride = c0_stride; a.acc_u = acc_u ? 1 : 0;
+        for (uint32_t t = 0; t < nterm; t++) { a.evk[t] = terms.evk[t]; a.galois[t] = terms.galois[t]; a.c0[t] = terms.c0[t]; }
+        launch_mid_rows(c, a, beta, s);
         return;
     }
     // any number of digits, any alignment: one term at a time through the generic kernel, then its P c0
