@@ -1,5 +1,5 @@
-// Butterflies of the negacyclic transform on registers, shared by the transform kernels (ntt.cu) and by the kernel that joins row passes
-// with the inner product between them (mid_rows.cu).
+// Butterflies of the negacyclic transform on registers, shared by the transform kernels (ntt.cu) and by the kernel that runs an
+// inverse column pass, a basis conversion and a forward column pass in one (conv_ntt.cu).
 #pragma once
 #include "common.cuh"
 

@@ -405,6 +405,14 @@ void launch_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const LimbM
 enum NttPart { NTT_ROWS = 1, NTT_COLS = 2, NTT_BOTH = 3 };
 void launch_ntt_part(const ckks_ctx *c, NttPart part, u64 *base, uint32_t nlimbs_total, const LimbMap &map, bool inverse, cudaStream_t s, const NttEpilogue *ep = nullptr,
                      const NttPrologue *pro = nullptr, const NttSource *src = nullptr, const double2 *inv_scale = nullptr);
+// What lies between an inverse and a forward row pass (conv_ntt.cu): the sources' inverse column pass, a basis conversion, the targets'
+// forward column pass.  CONV_UP: ModUp of one digit (an item: entry * digits + digit; src [entry][level], dst [item][level + K]);
+// CONV_DOWN: ModDown of one component (item: entry * 2 + component; src [item][level + K], dst [item][targets]);
+// CONV_DOWN_RS: that of a ModDown which a rescale follows.  targets: of a ModUp the largest number of a digit.
+enum { CONV_UP = 0, CONV_DOWN = 1, CONV_DOWN_RS = 2 };
+cudaError_t conv_strip_prepare(const ckks_ctx *c);          // once per context
+bool conv_strip(const ckks_ctx *c, int mode, uint32_t level, uint32_t items, bool alone = false);     // alone: see launch_ntt
+void launch_conv_strip(const ckks_ctx *c, int mode, const u64 *src, u64 *dst, uint32_t level, uint32_t items, uint32_t targets, cudaStream_t s);
 void launch_ntt_int(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, bool inverse, const NttSource &src, cudaStream_t s);
 
 void launch_mul_plain_acc(const ckks_ctx *c, const u64 *const *cts, u64 *const *accs, uint32_t ncts, const u64 *pt,

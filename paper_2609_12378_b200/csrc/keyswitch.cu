@@ -420,6 +420,12 @@ void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, 
     w.d = d;
     NttSource src;
     src.ptr = d; src.lpitch = 1;
+    if (conv_strip(c, CONV_UP, level, nb * beta, w.alone)) {
+        launch_ntt_part(c, NTT_ROWS, w.dcoef, nb * level, plain_map(0, level), true, s, nullptr, nullptr, &src);
+        launch_conv_strip(c, CONV_UP, w.dcoef, w.ext, level, nb * beta, nt - (level - (beta - 1) * c->alpha), s);
+        if (!w.mid) launch_ntt_part(c, NTT_ROWS, w.ext, nb * beta * nt, ext_map(level, c->K, c->L, c->alpha, beta), false, s);
+        return;
+    }
     launch_ntt(c, w.dcoef, nb * level, plain_map(0, level), true, s, nullptr, nullptr, &src,
                conv_tensor(c) ? nullptr : c->dev.inv_scale_up + (size_t)level * c->L * 2, w.alone);
     if (conv_tensor(c)) {
@@ -537,9 +543,18 @@ static NttEpilogue moddown_epilogue(const ckks_ctx *c, uint32_t level, const KsW
 static void moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, NttEpilogue ep, cudaStream_t s, uint32_t nb) {
     const uint32_t N = c->N, nt = level + c->K, K = c->K;
     // the K special limbs of every (batch, component): groups of K limbs, nt limbs apart
+    const bool strip = conv_strip(c, CONV_DOWN, level, 2 * nb);
+    const NttPart first = NttPart((w.mid ? 0 : NTT_ROWS) | (strip ? 0 : NTT_COLS));
     const double2 *scale = conv_tensor(c) ? nullptr : c->dev.inv_scale_dn;
-    if (w.mid) launch_ntt_part(c, NTT_COLS, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, nullptr, nullptr, nullptr, scale);
-    else launch_ntt(c, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, ep.mode == 3 ? &ep : nullptr, nullptr, nullptr, scale, w.alone);
+    if (first == NTT_BOTH)
+        launch_ntt(c, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, ep.mode == 3 ? &ep : nullptr, nullptr, nullptr, scale, w.alone);
+    else if (first)
+        launch_ntt_part(c, first, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, ep.mode == 3 ? &ep : nullptr, nullptr, nullptr, scale);
+    if (strip) {
+        launch_conv_strip(c, CONV_DOWN, w.u, w.conv, level, 2 * nb, level, s);
+        launch_ntt_part(c, NTT_ROWS, w.conv, nb * 2 * level, plain_map(0, level), false, s, &ep);
+        return;
+    }
     if (conv_tensor(c)) {
         launch_moddown_conv_mma(c, w.u, w.conv, level, nb, s);
     } else {
@@ -580,11 +595,19 @@ void ks_apply_rescale(const ckks_ctx *c, const u64 *evk, uint32_t level, const K
     ep.out = out;
     ep.pinv = c->dev.rs_p_inv_d + (size_t)m * c->L;
     ep.ncomp = 2; ep.level = m; ep.nt = nt; ep.galois = 1;
+    const bool strip = conv_strip(c, CONV_DOWN_RS, level, 2 * nb);
     if (w.mid) mid_inner(c, evk, level, 1, w, m, s, nb, nullptr, &add);
     else ks_inner(c, evk, level, 1, w, s, nb, false, nullptr, &add);
     // the dropped limb and the K special limbs of every (batch, component), nt limbs apart
-    launch_ntt_part(c, w.mid ? NTT_COLS : NTT_BOTH, w.u + (size_t)m * N, nb * 2 * (K + 1), tail_map(m, level, K, c->L), true, s, nullptr, nullptr, nullptr,
-                    c->dev.inv_scale_rs + (size_t)m * (K + 1) * 2);
+    const NttPart first = NttPart((w.mid ? 0 : NTT_ROWS) | (strip ? 0 : NTT_COLS));
+    if (first)
+        launch_ntt_part(c, first, w.u + (size_t)m * N, nb * 2 * (K + 1), tail_map(m, level, K, c->L), true, s, nullptr, nullptr, nullptr,
+                        c->dev.inv_scale_rs + (size_t)m * (K + 1) * 2);
+    if (strip) {
+        launch_conv_strip(c, CONV_DOWN_RS, w.u, w.conv, level, 2 * nb, m, s);
+        launch_ntt_part(c, NTT_ROWS, w.conv, nb * 2 * m, plain_map(0, m), false, s, &ep);
+        return;
+    }
 #define CALL_DN(A) launch_moddown_conv<A, true>(c, w.u, w.conv, level, nb, s)
     DISPATCH_POW2(K, CALL_DN);
 #undef CALL_DN

@@ -377,3 +377,49 @@ def test_transforms_that_leave_out_every_limb_of_one_path(share):
     finally:
         ctx.set_option(binding.OPT_CONV_KERNEL, binding.CONV_FP64)
         ctx.set_option(binding.OPT_NTT_FP_SHARE, 8)
+
+
+@pytest.mark.parametrize("log_n,L,K,dnum,level", [
+    (12, 3, 1, 3, 3), (12, 8, 8, 1, 8), (12, 9, 9, 1, 9), (12, 7, 4, 3, 5), (12, 12, 3, 4, 12), (12, 10, 2, 5, 10), (12, 16, 8, 2, 11),
+    (13, 12, 6, 2, 12), (14, 6, 2, 3, 5), (14, 16, 8, 2, 16), (15, 12, 4, 3, 9), (15, 8, 8, 1, 8), (16, 3, 3, 1, 3), (16, 10, 5, 2, 6)])
+def test_key_switches_of_every_ring_and_digit_size(log_n, L, K, dnum, level):
+    """One to nine sources per conversion (eight are the most that stay in registers), full and partial digits, one to five digits (four
+    are the most whose row pass forms the inner product), rings from the smallest that runs a strip of columns through conversion and
+    both transforms: a rotation whose sources lie at the ends of the residues, a sum of rotations over two groups of terms, a product
+    that drops a limb and a rescale, all of it on one ciphertext and on several."""
+    from tests.gpu_util import context, ct_dev, host, key_dev
+    P, ctx = params(log_n, L, K, dnum), context(log_n, L, K, dnum)
+    o, g = P.oracle, inputs.rng(800, level + 100 * L + 10000 * log_n)
+    alpha = -(-L // dnum)
+    d = np.empty((1, level, P.N), dtype=np.uint64)
+    for i in range(level):
+        q, lo = int(P.q[i]), i // alpha * alpha
+        hat = 1
+        for b in range(lo, min(lo + alpha, level)):
+            hat = hat * (int(P.q[b]) if b != i else 1) % q
+        ends = np.array([y * hat % q for y in (0, 1, q - 1, q // 2, q // 2 + 1)], dtype=np.uint64)
+        d[0, i] = ends[g.integers(0, 5, P.N)]
+        d[0, i, :64] = ends[3 + np.arange(64) % 2]          # all sources at q / 2 together
+    ct = np.concatenate([inputs.uniform_residues(g, P.q[:level], P.N, 1), o.ntt(d)])
+    more = [inputs.uniform_residues(g, P.q[:level], P.N, 2) for _ in range(4)]
+    keys = [inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, dnum * 2).reshape(dnum, 2, L + K, P.N) for _ in range(3)]
+    gals = [o.galois_element(r) for r in (3, 64, P.n - 1)]
+    dk = [key_dev(k, e) for k, e in zip(keys, gals)]
+    assert np.array_equal(host(ctx.rotate(ct_dev(ct, 1.0), dk[0]).data), o.rotate(ct, keys[0], gals[0]))
+    batch = ctx.rotate_batch([ct_dev(x, 1.0) for x in [ct] + more], dk[1])
+    for got, x in zip(batch, [ct] + more):
+        assert np.array_equal(host(got.data), o.rotate(x, keys[1], gals[1]))
+    pick = [0, 1, 2, 0, 1]
+    got = ctx.rotate_sum([ct_dev(x, 1.0) for x in [ct] + more], [dk[j] for j in pick])
+    assert np.array_equal(host(got.data), o.rotate_sum(np.stack([ct] + more), [keys[j] for j in pick], [gals[j] for j in pick]))
+    if level < 3:
+        return
+    coeffs = [0.25, -0.5, 0.75]
+    for xs in ([ct], [ct] + more[:2]):
+        outs = [ctx.poly_eval(ct_dev(x, 2.0 ** 50), coeffs, key_dev(keys[0], 0)) for x in xs]
+        for got, x in zip(outs, xs):
+            assert np.array_equal(host(got.data), o.poly_eval(x, 2.0 ** 50, coeffs, keys[0])[0])
+    prod = ctx.mul_relin(ct_dev(ct, 1.0), ct_dev(more[0], 1.0), key_dev(keys[2], 0))
+    want = o.mul_relin(ct, more[0], keys[2])
+    assert np.array_equal(host(prod.data), want)
+    assert np.array_equal(host(ctx.rescale(prod).data), o.rescale(want))
