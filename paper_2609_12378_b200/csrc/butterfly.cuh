@@ -38,7 +38,8 @@ __device__ __forceinline__ void load_tw(const double *p, double (&v)[ML]) {
 //   1.63 2.33 3.12 4.01 | 5.51c 7.20c | u reduced: 2.40c 3.20,
 // the row pass goes on with 4.10 5.61c 7.31c | u reduced: 2.42c | 3.22 4.12 5.64c 7.35c and one exact reduction at the end:
 // two half reductions on the way for sixteen stages.  Smaller rings reduce u in their last column stage instead, which
-// keeps the row pass's input at or below 3.20 for every N.
+// keeps the row pass's input at or below 3.20 for every N.  From 1.25 q, which the conversions of conv_ntt.cu hand over, it is
+//   1.91 2.64 3.48 4.41 | 5.96c 7.71c | 2.46c 3.27 and 4.18 5.70c 7.42c | 2.43c | 3.23 4.13 5.65c 7.36c.
 
 // Stage s (1 .. LOGR) of the forward column pass.
 __host__ __device__ constexpr bool col_coarse(uint32_t s) { return s >= 5 && s <= 7; }
@@ -232,5 +233,83 @@ struct ColShape {
 __device__ __forceinline__ uint32_t padded(uint32_t i) { return i + 2 * (i >> 4); }
 constexpr uint32_t ROW_PAD = 256 + 32, ROW_CTA = 4;
 
+
+// ---- a row by a warp: eight coefficients per lane, stages in groups of 3, 3 and 2 -----------------------------------------------
+// Half the chain of dependent operations and twice the warps of sixteen lanes per row, for more exchanges: where a launch is bound by
+// latency (mid_rows.cu, the row passes of few limbs).  The exchange row has four spare words behind every 32.
+constexpr uint32_t WROW_PAD = 256 + 32;
+__device__ __forceinline__ uint32_t wrow_at(uint32_t i) { return i + 4 * (i >> 5); }
+// words t + 32 k of the row in v (3.27 q) -> the row's results at s, in order, at most half a prime; base: R + row
+__device__ __forceinline__ void wrow_forward(double (&v)[8], double *s, uint32_t t, const double *__restrict__ tw, uint32_t base, double q, double qinv) {
+    const uint32_t b32 = wrow_at(t / 4 * 32) + t % 4;              // word 32 b + s, the lane's place in the middle group
+    fwd_stage<1, 8, false, false>(v, 0, tw, base, q, qinv);
+    fwd_stage<2, 8, true, false>(v, 0, tw, base, q, qinv);
+    fwd_stage<4, 8, true, false>(v, 0, tw, base, q, qinv);
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) s[t + 36 * k] = v[k];
+    __syncwarp();
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) v[k] = s[b32 + 4 * k];
+    fwd_stage<1, 8, true, true>(v, 0, tw, 8 * base + t / 4, q, qinv);
+    fwd_stage<2, 8, false, false>(v, 0, tw, 8 * base + t / 4, q, qinv);
+    fwd_stage<4, 8, false, false>(v, 0, tw, 8 * base + t / 4, q, qinv);
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) s[b32 + 4 * k] = v[k];
+    __syncwarp();
+    // words 4 t .. and 128 + 4 t ..
+#pragma unroll
+    for (uint32_t h = 0; h < 2; h++) {
+        double *blk = s + wrow_at(4 * t) + 144 * h;
+#pragma unroll
+        for (uint32_t k = 0; k < 4; k += 2) {
+            const double2 w = *reinterpret_cast<const double2 *>(blk + k);
+            v[4 * h + k] = w.x; v[4 * h + k + 1] = w.y;
+        }
+        fwd_stage<1, 4, true, false>(v, 4 * h, tw, 64 * base + 32 * h + t, q, qinv);
+        fwd_stage<2, 4, true, false>(v, 4 * h, tw, 64 * base + 32 * h + t, q, qinv);
+#pragma unroll
+        for (uint32_t k = 0; k < 4; k += 2)
+            *reinterpret_cast<double2 *>(blk + k) = make_double2(reduce_d(v[4 * h + k], q, qinv), reduce_d(v[4 * h + k + 1], q, qinv));
+    }
+}
+// Bounds of the inverse row pass in groups of 2, 3 and 3 stages from canonical residues; it ends below inv_in(3) (see gs_plan)
+constexpr double WROW_IN0 = 1.0, WROW_T0 = 1.5, WROW_IN1 = gs_out(2, WROW_IN0, WROW_T0), WROW_T1 = 1.44, WROW_IN2 = gs_out(3, WROW_IN1, WROW_T1), WROW_T2 = 1.8;
+static_assert(gs_out(3, WROW_IN2, WROW_T2) <= inv_in(3), "the column pass takes these values");
+#define WROW_INV(S, G, IN, THR, X0, BASE) inv_stage<S, G, gs_pre(G, IN, THR, false, S), gs_coarse(G, IN, THR, false, S), false>(v, X0, tw, BASE, q, qinv)
+// the row at s, in order -> words t + 32 k in v
+__device__ __forceinline__ void wrow_inverse(double (&v)[8], double *s, uint32_t t, const double *__restrict__ tw, uint32_t base, double q, double qinv) {
+    const uint32_t b32 = wrow_at(t / 4 * 32) + t % 4;
+#pragma unroll
+    for (uint32_t h = 0; h < 2; h++) {
+        double *blk = s + wrow_at(4 * t) + 144 * h;
+#pragma unroll
+        for (uint32_t k = 0; k < 4; k += 2) {
+            const double2 w = *reinterpret_cast<const double2 *>(blk + k);
+            v[4 * h + k] = w.x; v[4 * h + k + 1] = w.y;
+        }
+        WROW_INV(0, 2, WROW_IN0, WROW_T0, 4 * h, 64 * base + 32 * h + t);
+        WROW_INV(1, 2, WROW_IN0, WROW_T0, 4 * h, 64 * base + 32 * h + t);
+        reduce_masked<gs_post(2, WROW_IN0, WROW_T0, false), 4>(v, 4 * h, q, qinv);
+#pragma unroll
+        for (uint32_t k = 0; k < 4; k += 2) *reinterpret_cast<double2 *>(blk + k) = make_double2(v[4 * h + k], v[4 * h + k + 1]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) v[k] = s[b32 + 4 * k];
+    WROW_INV(0, 3, WROW_IN1, WROW_T1, 0, 8 * base + t / 4);
+    WROW_INV(1, 3, WROW_IN1, WROW_T1, 0, 8 * base + t / 4);
+    WROW_INV(2, 3, WROW_IN1, WROW_T1, 0, 8 * base + t / 4);
+    reduce_masked<gs_post(3, WROW_IN1, WROW_T1, false), 8>(v, 0, q, qinv);
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) s[b32 + 4 * k] = v[k];
+    __syncwarp();
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) v[k] = s[t + 36 * k];
+    WROW_INV(0, 3, WROW_IN2, WROW_T2, 0, base);
+    WROW_INV(1, 3, WROW_IN2, WROW_T2, 0, base);
+    WROW_INV(2, 3, WROW_IN2, WROW_T2, 0, base);
+    reduce_masked<gs_post(3, WROW_IN2, WROW_T2, false), 8>(v, 0, q, qinv);
+}
+#undef WROW_INV
 
 }  // namespace

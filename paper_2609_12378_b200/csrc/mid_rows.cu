@@ -12,22 +12,15 @@ namespace {
 // A warp per row, eight coefficients per lane (stages in groups of 3, 3 and 2), so that the sums of both components fit 64 registers:
 // the kernel waits for its key words and digits, and 32 warps per SM wait for more of them at a time (16 lanes per row with
 // sixteen coefficients and 128 registers: 54 us for one ciphertext at N = 2^16, level 24).
-constexpr uint32_t MID_ROWS = 4, MID_PAD = 256 + 32;
-__device__ __forceinline__ uint32_t mid_at(uint32_t i) { return i + 4 * (i >> 5); }
-
-// bounds of the inverse row pass in groups of 2, 3 and 3 stages from sums of half a prime; it ends below inv_in(3) (see gs_plan)
-constexpr double MID_IN0 = 0.5, MID_T0 = 1.26, MID_IN1 = gs_out(2, MID_IN0, MID_T0), MID_T1 = 0.92, MID_IN2 = gs_out(3, MID_IN1, MID_T1), MID_T2 = 1.92;
-static_assert(gs_out(3, MID_IN2, MID_T2) <= inv_in(3), "the column pass takes these values");
-#define MID_INV(S, G, IN, THR, X0, BASE) inv_stage<S, G, gs_pre(G, IN, THR, false, S), gs_coarse(G, IN, THR, false, S), false>(v, X0, twi, BASE, q, qinv)
+constexpr uint32_t MID_ROWS = 4;
 
 template <uint32_t BETA, bool TERMS>
 __global__ void __launch_bounds__(32 * MID_ROWS, TERMS ? 5 : 8) mid_rows(DevTables c, const __grid_constant__ MidArgs a) {
-    __shared__ __align__(16) double sm[BETA][MID_ROWS][MID_PAD];
+    __shared__ __align__(16) double sm[BETA][MID_ROWS][WROW_PAD];
     const uint32_t t = threadIdx.x & 31, rl = threadIdx.x >> 5, row = blockIdx.x * MID_ROWS + rl, R = c.N >> 8;
     const uint32_t bz = blockIdx.y, x = blockIdx.z, nt = a.level + c.K, kt = x < a.level ? x : c.L + (x - a.level);
     const double q = c.modd[kt].x, qinv = c.modd[kt].y;
     const uint32_t p0 = row * 256 + 2 * t, own = x < a.level ? x / c.alpha : BETA;       // own: the digit that has x among its own limbs
-    const uint32_t b32 = mid_at(t / 4 * 32) + t % 4;                                     // word 32 b + s, the lane's place in the middle group
     const size_t limb = (size_t)1 << c.log_n;
     double s0[8], s1[8];               // sums of words p0 + 64 k, p0 + 64 k + 1 of both components
     if (TERMS)
@@ -48,7 +41,7 @@ __global__ void __launch_bounds__(32 * MID_ROWS, TERMS ? 5 : 8) mid_rows(DevTabl
 #pragma unroll
                 for (uint32_t k = 0; k < 4; k++) w[k] = ld_pair<true>(d + 64 * k);
 #pragma unroll
-                for (uint32_t k = 0; k < 4; k++) *reinterpret_cast<double2 *>(s + mid_at(2 * t) + 72 * k) = make_double2(u64_to_d(w[k].x), u64_to_d(w[k].y));
+                for (uint32_t k = 0; k < 4; k++) *reinterpret_cast<double2 *>(s + wrow_at(2 * t) + 72 * k) = make_double2(u64_to_d(w[k].x), u64_to_d(w[k].y));
                 continue;
             }
             const double *tw = c.twd_fwd + ((size_t)kt << c.log_n);
@@ -56,36 +49,7 @@ __global__ void __launch_bounds__(32 * MID_ROWS, TERMS ? 5 : 8) mid_rows(DevTabl
             double v[8];
 #pragma unroll
             for (uint32_t k = 0; k < 8; k++) v[k] = g[32 * k];
-            // 3.30 q in (see butterfly.cuh)
-            fwd_stage<1, 8, false, false>(v, 0, tw, R + srow, q, qinv);
-            fwd_stage<2, 8, true, false>(v, 0, tw, R + srow, q, qinv);
-            fwd_stage<4, 8, true, false>(v, 0, tw, R + srow, q, qinv);
-#pragma unroll
-            for (uint32_t k = 0; k < 8; k++) s[t + 36 * k] = v[k];
-            __syncwarp();
-#pragma unroll
-            for (uint32_t k = 0; k < 8; k++) v[k] = s[b32 + 4 * k];
-            fwd_stage<1, 8, true, true>(v, 0, tw, 8 * (R + srow) + t / 4, q, qinv);
-            fwd_stage<2, 8, false, false>(v, 0, tw, 8 * (R + srow) + t / 4, q, qinv);
-            fwd_stage<4, 8, false, false>(v, 0, tw, 8 * (R + srow) + t / 4, q, qinv);
-#pragma unroll
-            for (uint32_t k = 0; k < 8; k++) s[b32 + 4 * k] = v[k];
-            __syncwarp();
-            // words 4 t .. and 128 + 4 t ..
-#pragma unroll
-            for (uint32_t h = 0; h < 2; h++) {
-                double *blk = s + mid_at(4 * t) + 144 * h;
-#pragma unroll
-                for (uint32_t k = 0; k < 4; k += 2) {
-                    const double2 w = *reinterpret_cast<const double2 *>(blk + k);
-                    v[4 * h + k] = w.x; v[4 * h + k + 1] = w.y;
-                }
-                fwd_stage<1, 4, true, false>(v, 4 * h, tw, 64 * (R + srow) + 32 * h + t, q, qinv);
-                fwd_stage<2, 4, true, false>(v, 4 * h, tw, 64 * (R + srow) + 32 * h + t, q, qinv);
-#pragma unroll
-                for (uint32_t k = 0; k < 4; k += 2)
-                    *reinterpret_cast<double2 *>(blk + k) = make_double2(reduce_d(v[4 * h + k], q, qinv), reduce_d(v[4 * h + k + 1], q, qinv));
-            }
+            wrow_forward(v, s, t, tw, R + srow, q, qinv);
         }
         __syncwarp();
         const u64 *c0 = TERMS && x < a.level && a.c0[term] ? a.c0[term] + bz * a.c0_stride + x * limb + srow * 256 : nullptr;
@@ -110,7 +74,7 @@ __global__ void __launch_bounds__(32 * MID_ROWS, TERMS ? 5 : 8) mid_rows(DevTabl
             }
 #pragma unroll
             for (uint32_t j = 0; j < BETA; j++) {
-                const double2 e = *reinterpret_cast<const double2 *>(sm[j][rl] + mid_at(so));
+                const double2 e = *reinterpret_cast<const double2 *>(sm[j][rl] + wrow_at(so));
                 const double e0 = odd ? e.y : e.x, e1 = odd ? e.x : e.y;
                 s0[2 * k] = __dadd_rn(s0[2 * k], mulmod_dd(e0, u64_to_d(kv[j][0].x), q, qinv));
                 s0[2 * k + 1] = __dadd_rn(s0[2 * k + 1], mulmod_dd(e1, u64_to_d(kv[j][0].y), q, qinv));
@@ -148,45 +112,15 @@ __global__ void __launch_bounds__(32 * MID_ROWS, TERMS ? 5 : 8) mid_rows(DevTabl
         }
         double *s = sm[0][rl];
 #pragma unroll
-        for (uint32_t k = 0; k < 4; k++) *reinterpret_cast<double2 *>(s + mid_at(2 * t) + 72 * k) = make_double2(v[2 * k], v[2 * k + 1]);
+        for (uint32_t k = 0; k < 4; k++) *reinterpret_cast<double2 *>(s + wrow_at(2 * t) + 72 * k) = make_double2(v[2 * k], v[2 * k + 1]);
         __syncwarp();
-#pragma unroll
-        for (uint32_t h = 0; h < 2; h++) {
-            double *blk = s + mid_at(4 * t) + 144 * h;
-#pragma unroll
-            for (uint32_t k = 0; k < 4; k += 2) {
-                const double2 w = *reinterpret_cast<const double2 *>(blk + k);
-                v[4 * h + k] = w.x; v[4 * h + k + 1] = w.y;
-            }
-            MID_INV(0, 2, MID_IN0, MID_T0, 4 * h, 64 * (R + row) + 32 * h + t);
-            MID_INV(1, 2, MID_IN0, MID_T0, 4 * h, 64 * (R + row) + 32 * h + t);
-            reduce_masked<gs_post(2, MID_IN0, MID_T0, false), 4>(v, 4 * h, q, qinv);
-#pragma unroll
-            for (uint32_t k = 0; k < 4; k += 2) *reinterpret_cast<double2 *>(blk + k) = make_double2(v[4 * h + k], v[4 * h + k + 1]);
-        }
-        __syncwarp();
-#pragma unroll
-        for (uint32_t k = 0; k < 8; k++) v[k] = s[b32 + 4 * k];
-        MID_INV(0, 3, MID_IN1, MID_T1, 0, 8 * (R + row) + t / 4);
-        MID_INV(1, 3, MID_IN1, MID_T1, 0, 8 * (R + row) + t / 4);
-        MID_INV(2, 3, MID_IN1, MID_T1, 0, 8 * (R + row) + t / 4);
-        reduce_masked<gs_post(3, MID_IN1, MID_T1, false), 8>(v, 0, q, qinv);
-#pragma unroll
-        for (uint32_t k = 0; k < 8; k++) s[b32 + 4 * k] = v[k];
-        __syncwarp();
-#pragma unroll
-        for (uint32_t k = 0; k < 8; k++) v[k] = s[t + 36 * k];
-        MID_INV(0, 3, MID_IN2, MID_T2, 0, R + row);
-        MID_INV(1, 3, MID_IN2, MID_T2, 0, R + row);
-        MID_INV(2, 3, MID_IN2, MID_T2, 0, R + row);
-        reduce_masked<gs_post(3, MID_IN2, MID_T2, false), 8>(v, 0, q, qinv);
+        wrow_inverse(v, s, t, twi, R + row, q, qinv);
         double *g = reinterpret_cast<double *>(u) - t;
 #pragma unroll
         for (uint32_t k = 0; k < 8; k++) g[32 * k] = v[k];
         __syncwarp();
     }
 }
-#undef MID_INV
 
 }  // namespace
 

@@ -382,6 +382,102 @@ __global__ void __launch_bounds__(16 * ROW_CTA, 48 / ROW_CTA) ntt_inv_rows(DevTa
     for (uint32_t k = 0; k < 16; k++) reinterpret_cast<double *>(g)[t + 16 * k] = x[k];
 }
 
+// ---- row passes of few limbs: a row by a warp -----------------------------------------------------------------------------
+// forward, EP 0 and 1 as in ntt_fwd_rows; the other operands are on their way while the row is transformed
+template <int EP, bool WIDE>
+__global__ void __launch_bounds__(32 * ROW_CTA, 6) ntt_fwd_wrows(DevTables c, u64 *base, LimbMap map, uint32_t fp_share, const __grid_constant__ NttEpilogue ep) {
+    __shared__ __align__(16) double sm[ROW_CTA][WROW_PAD];
+    const int prime = limb_prime(map, blockIdx.y);
+    if (prime < 0 || (blockIdx.y & 7) >= fp_share) return leave_out(fp_share);
+    const double q = c.modd[prime].x, qinv = c.modd[prime].y;
+    const double *tw = c.twd_fwd + ((size_t)prime << c.log_n);
+    const uint32_t t = threadIdx.x & 31, rl = threadIdx.x >> 5, row = blockIdx.x * ROW_CTA + rl, R = c.N >> 8;
+    u64 *g = base + (limb_index(map, blockIdx.y) << c.log_n) + (size_t)row * 256;
+    double *s = sm[rl], v[8];
+    grid_dep_sync();
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) v[k] = reinterpret_cast<const double *>(g)[t + 32 * k];
+    const double *sp = s + wrow_at(2 * t);                // word 2 t + 64 k is 72 k further
+    if (EP == 0) {
+        __syncwarp();
+        wrow_forward(v, s, t, tw, R + row, q, qinv);
+        __syncwarp();
+#pragma unroll
+        for (uint32_t k = 0; k < 4; k++) {
+            const double2 w = *reinterpret_cast<const double2 *>(sp + 72 * k);
+            st_pair<WIDE>(g + 2 * t + 64 * k, make_ulonglong2(canonical_d(w.x, q), canonical_d(w.y, q)));
+        }
+        return;
+    }
+    const uint32_t y = blockIdx.y + ep.y0, i = y % ep.level, comp = (y / ep.level) % ep.ncomp, bz = y / (ep.ncomp * ep.level);
+    const double2 pinv = ep.pinv[i];
+    const uint32_t p0 = row * 256 + 2 * t;
+    // grouped: entry bz is key bz / group applied to member bz % group (own: to the entry itself)
+    const uint32_t rot = ep.group ? bz / ep.group : bz, mem = ep.group ? bz % ep.group : bz;
+    const uint32_t gal = (uint32_t)(ep.multi ? ep.mgalois[rot] : ep.galois);
+    const u64 *add = (ep.add_comps >> comp & 1) ? ep.add.at(ep.own ? bz : mem) + (((size_t)comp * ep.level + i) << c.log_n) : nullptr;
+    const u64 *acc = ep.accumulate ? ep.acc.at(bz) + (((size_t)comp * ep.level + i) << c.log_n) + p0 : nullptr;
+    const uint32_t bstep = ep.tl.R ? ep.tl.R * 64 : 64;        // words from one 64-word block of the destination to the next
+    u64 *dst = ep.tl.R ? const_cast<u64 *>(ep.out.base) + tiled_index(ep.tl.R, c.N, ep.tl.row0 + rot * ep.rot_rows + (ep.group ? mem : bz) * ep.tl.row_stride + comp, i, row * 256) + 2 * t
+                       : const_cast<u64 *>(ep.group ? ep.out.base + rot * ep.rot_stride + mem * ep.out.stride : ep.out.at(bz)) + (((size_t)comp * ep.level + i) << c.log_n) + p0;
+    const u64 *up = ep.u.at(bz) + (((size_t)comp * ep.nt + i) << c.log_n) + p0;
+    ulonglong2 ua[4], aa[4];
+    uint32_t sr[4];
+#pragma unroll
+    for (uint32_t k = 0; k < 4; k++) {
+        ua[k] = ld_pair<WIDE>(up + 64 * k);
+        if (add) {      // the permutation maps the pair onto a pair, possibly swapped
+            sr[k] = galois_src(p0 + 64 * k, gal, c.log_n);
+            aa[k] = ld_pair<WIDE>(add + (sr[k] & ~1u));
+        }
+    }
+    __syncwarp();
+    wrow_forward(v, s, t, tw, R + row, q, qinv);
+    __syncwarp();
+#pragma unroll
+    for (uint32_t k = 0; k < 4; k++) {
+        const double2 w = *reinterpret_cast<const double2 *>(sp + 72 * k);
+        // |u - v| < 1.5 q, times P^-1 -> |.| < 0.9 q, plus up to two residues, reduced once
+        double r0 = mulmod_d<0>(__dsub_rn(u64_to_d(ua[k].x), w.x), pinv, q);
+        double r1 = mulmod_d<0>(__dsub_rn(u64_to_d(ua[k].y), w.y), pinv, q);
+        if (add) {
+            const bool odd = sr[k] & 1;
+            r0 = __dadd_rn(r0, u64_to_d(odd ? aa[k].y : aa[k].x));
+            r1 = __dadd_rn(r1, u64_to_d(odd ? aa[k].x : aa[k].y));
+        }
+        if (ep.accumulate) {
+            const ulonglong2 o = ld_pair<WIDE>(acc + 64 * k);
+            r0 = __dadd_rn(r0, u64_to_d(o.x));
+            r1 = __dadd_rn(r1, u64_to_d(o.y));
+        }
+        st_pair<WIDE>(dst + k * bstep, make_ulonglong2(canonical_d(reduce_d(r0, q, qinv), q), canonical_d(reduce_d(r1, q, qinv), q)));
+    }
+}
+
+// inverse; src as in ntt_inv_rows
+template <bool WIDE>
+__global__ void __launch_bounds__(32 * ROW_CTA, 8) ntt_inv_wrows(DevTables c, u64 *base, LimbMap map, uint32_t fp_share, const __grid_constant__ NttSource src) {
+    __shared__ __align__(16) double sm[ROW_CTA][WROW_PAD];
+    const int prime = limb_prime(map, blockIdx.y);
+    if (prime < 0 || (blockIdx.y & 7) >= fp_share) return leave_out(fp_share);
+    const double q = c.modd[prime].x, qinv = c.modd[prime].y;
+    const double *tw = c.twd_inv + ((size_t)prime << c.log_n);
+    const uint32_t t = threadIdx.x & 31, rl = threadIdx.x >> 5, row = blockIdx.x * ROW_CTA + rl, R = c.N >> 8;
+    u64 *g = base + (limb_index(map, blockIdx.y) << c.log_n) + (size_t)row * 256;
+    const u64 *gs = src.lpitch ? src.ptr.at(blockIdx.y / map.period) + (((size_t)(blockIdx.y % map.period) * src.lpitch) << c.log_n) + (size_t)row * 256 : g;
+    double *s = sm[rl], v[8];
+    grid_dep_sync();
+    ulonglong2 w[4];
+#pragma unroll
+    for (uint32_t k = 0; k < 4; k++) w[k] = ld_pair<WIDE>(gs + 2 * t + 64 * k);
+#pragma unroll
+    for (uint32_t k = 0; k < 4; k++) *reinterpret_cast<double2 *>(s + wrow_at(2 * t) + 72 * k) = make_double2(u64_to_d(w[k].x), u64_to_d(w[k].y));
+    __syncwarp();
+    wrow_inverse(v, s, t, tw, R + row, q, qinv);
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) reinterpret_cast<double *>(g)[t + 32 * k] = v[k];
+}
+
 // ---- both passes in one kernel: a cluster of CTAs per limb --------------------------------------------------------------
 // CL CTAs hold a limb in shared memory: CTA c does the column stages of 256 / CL columns, the values cross to the CTAs that
 // own their rows through distributed shared memory, and CTA d does the row stages of R / CL rows (inverse: the other way
@@ -607,6 +703,10 @@ static void run_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const L
             }
         };
         const dim3 grid(R / ROW_CTA, ny);
+        // A row by a warp where the launch is bound by latency: up to six CTAs of four rows per SM.  (Rotation at N = 2^14, 192 CTAs,
+        // 28.8 -> 27.3 us; at N = 2^15, 768 CTAs, 44.1 -> 43.4; the 64 x 64 projection at N = 2^13 175.4 -> 168.7; from there on the
+        // additional exchanges cost more: rotation at N = 2^16, level 9, 1152 CTAs, 72.0 -> 74.0.)
+        const bool few = (uint64_t)grid.x * ny <= 6 * (uint64_t)c->sms;
         if (share > 0 && !inverse) {
             if (part & NTT_COLS) cols();
             if (!(part & NTT_ROWS)) continue;
@@ -621,7 +721,10 @@ static void run_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const L
                     : mode == 1 ? (wide ? ntt_fwd_rows<1, true> : ntt_fwd_rows<1, false>)
                     : mode == 2 ? (wide ? ntt_fwd_rows<2, true> : ntt_fwd_rows<2, false>)
                                 : (wide ? ntt_fwd_rows<0, true> : ntt_fwd_rows<0, false>);
-            launch(k, grid, 16 * ROW_CTA, 0, s, c->dev, b, map, share, e);
+            if (mode < 2 && few)
+                launch(mode ? (wide ? ntt_fwd_wrows<1, true> : ntt_fwd_wrows<1, false>) : (wide ? ntt_fwd_wrows<0, true> : ntt_fwd_wrows<0, false>), grid, 32 * ROW_CTA, 0, s, c->dev, b, map,
+                       share, e);
+            else launch(k, grid, 16 * ROW_CTA, 0, s, c->dev, b, map, share, e);
         } else if (share > 0) {
             const NttSource none{};
             const bool wide = src ? aligned16(src->ptr) : aligned16(b);
@@ -630,6 +733,8 @@ static void run_ntt(const ckks_ctx *c, u64 *base, uint32_t nlimbs_total, const L
             if (!(part & NTT_ROWS)) {
             } else if (ep) {
                 launch(inner[ep->beta - 1], grid, 16 * ROW_CTA, 0, s, c->dev, b, map, share, *ep);
+            } else if (few) {
+                launch(wide ? ntt_inv_wrows<true> : ntt_inv_wrows<false>, grid, 32 * ROW_CTA, 0, s, c->dev, b, map, share, src ? sr : none);
             } else {
                 launch(wide ? ntt_inv_rows<true> : ntt_inv_rows<false>, grid, 16 * ROW_CTA, 0, s, c->dev, b, map, share, src ? sr : none);
             }

@@ -423,3 +423,23 @@ def test_key_switches_of_every_ring_and_digit_size(log_n, L, K, dnum, level):
     want = o.mul_relin(ct, more[0], keys[2])
     assert np.array_equal(host(prod.data), want)
     assert np.array_equal(host(ctx.rescale(prod).data), o.rescale(want))
+
+
+@pytest.mark.parametrize("log_n,batch,limbs", [(10, 1, 1), (12, 74, 3), (12, 75, 3), (15, 9, 3), (15, 14, 2), (16, 13, 1), (16, 7, 2)])
+def test_transforms_on_either_side_of_a_row_per_warp(log_n, batch, limbs):
+    """Both directions with the most limbs whose rows are taken by a warp each (six CTAs of four rows per SM of 148) and the fewest
+    that are taken by half a warp each, in a buffer that is 16-byte aligned and in one that is not."""
+    import torch
+    from tests.gpu_util import context, host
+    P, ctx = params(log_n, 3, 1, 3), context(log_n, 3, 1, 3)
+    o, g = P.oracle, inputs.rng(810, log_n + 100 * batch)
+    x = inputs.uniform_residues(g, P.q[:limbs], P.N, batch)
+    x[0] = np.array([int(q) - 1 for q in P.q[:limbs]], dtype=np.uint64)[:, None]
+    fwd, inv = o.ntt(x), o.intt(x)
+    for offset in (0, 1):
+        buf = torch.zeros(x.size + 1, dtype=torch.int64, device="cuda").view(torch.uint64)
+        y = buf[offset:offset + x.size].view(batch, limbs, P.N)
+        y.copy_(torch.from_numpy(x))
+        assert np.array_equal(host(ctx.ntt(y)), fwd)
+        y.copy_(torch.from_numpy(x))
+        assert np.array_equal(host(ctx.intt(y)), inv)
