@@ -268,7 +268,7 @@ inline void count_launches(unsigned n = 1) { g_kernel_launches += n; }
 // Launches are programmatic dependent launches: a kernel's CTAs may become resident as soon as every CTA of the kernel before
 // it on the stream has exited, and grid_dep_sync waits until that kernel's writes are visible.  Until then a kernel may only
 // read the context's tables.  Between dependent kernels of a few microseconds this hides the launch latency and the table
-// fetches (a rotation of one ciphertext, 11 launches at the time, ten now: 208 -> 186 us).  No kernel triggers its dependents earlier: CTAs that
+// fetches (a rotation of one ciphertext, 11 launches at the time, nine now: 208 -> 186 us).  No kernel triggers its dependents earlier: CTAs that
 // wait for the last wave of a large launch take the slots and the issue cycles it needs (64 hoisted rotations 1 % slower,
 // the 4096 x 4096 projection 3 %; for grids of at most one wave alone, one rotation 156 -> 160 us).
 __device__ __forceinline__ void grid_dep_sync() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
