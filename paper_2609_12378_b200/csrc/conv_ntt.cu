@@ -39,21 +39,23 @@ struct StripShape {
     static __device__ __forceinline__ uint32_t at(uint32_t row, uint32_t cc) { return (COLS == 8 ? row ^ (row >> 4 & 1) : row) * COLS + cc; }
 };
 constexpr uint32_t STRIP_CHUNK = 32, STRIP_NS = 8;         // targets and sources of a CTA at most
-// registers per thread of the two roles: 256 x (160 + 96) is what the CTA is launched with
+// Registers per thread of the two roles.  256 (176 + 80) = 512 x 128, which is what the CTA is launched with (every instance is compiled
+// to 128): more in sum would wait for registers that nobody gives back.
 constexpr uint32_t CONV_REGS = 176, NTT_REGS = 80;
+static_assert(CONV_REGS + NTT_REGS == 256, "the two halves of the CTA share the registers of its launch");
 
 __device__ __forceinline__ void group_sync(uint32_t id, uint32_t threads) { asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory"); }
-
 __device__ __forceinline__ void group_arrive(uint32_t id, uint32_t threads) { asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(threads) : "memory"); }
 
 // out[p] (+)= sum_a y[p][a] w[a] mod t.  The quotient of the whole sum is formed in two roundings, k = round(lo / t + round(hi / t)),
 // hi / t below 2^51: |out| <= (1/2 + 1/4 + 1/2) t = 1.25 t.
-template <bool FIRST, uint32_t NS, uint32_t CPT>
+// FULL: ns = NS, without a branch per source, so that the constants' fetches run ahead of the products.
+template <bool FIRST, bool FULL, uint32_t NS, uint32_t CPT>
 __device__ __forceinline__ void strip_dot(const double (&y)[CPT][NS], const double *w, uint32_t ns, double t, double tinv, double (&out)[CPT]) {
     double H[CPT];
 #pragma unroll
     for (uint32_t a = 0; a < NS; a++) {
-        if (a >= ns) break;
+        if (!FULL && a >= ns) break;
         const double wa = w[a];
 #pragma unroll
         for (uint32_t p = 0; p < CPT; p++) {
@@ -150,7 +152,7 @@ __global__ void __launch_bounds__(StripShape<LOGR>::THREADS, 1) conv_cols(DevTab
             // each remaining limb, where ModDown and rescale after each other take two
             const double2 md = c.modd[targets], pinv = c.dn_p_inv_d[targets];
             double v[CPT];
-            strip_dot<true, NS, CPT>(y, s_w + (x1 - x0) * NS, nd, md.x, md.y, v);
+            strip_dot<true, false, NS, CPT>(y, s_w + (x1 - x0) * NS, nd, md.x, md.y, v);
 #pragma unroll
             for (uint32_t p = 0; p < CPT; p++) {
                 double *d = dropped + threadIdx.x + p * S::CONV;
@@ -158,22 +160,26 @@ __global__ void __launch_bounds__(StripShape<LOGR>::THREADS, 1) conv_cols(DevTab
             }
         }
         group_sync(1, S::CONV);                               // the sources have been read
+        auto convert = [&](auto full) {
 #pragma unroll 1
-        for (uint32_t xt = x0; xt < x1; xt++) {
-            const uint32_t b = (xt - x0) % S::BUFFERS;
-            const double2 md = s_m[xt - x0];
-            double v[CPT];
-            if (RESC) {
-                const double pq = c.dn_p_mod_d[xt];
+            for (uint32_t xt = x0; xt < x1; xt++) {
+                const uint32_t b = (xt - x0) % S::BUFFERS;
+                const double2 md = s_m[xt - x0];
+                double v[CPT];
+                if (RESC) {
+                    const double pq = c.dn_p_mod_d[xt];
 #pragma unroll
-                for (uint32_t p = 0; p < CPT; p++) v[p] = mulmod_dd(dropped[threadIdx.x + p * S::CONV], pq, md.x, md.y);
+                    for (uint32_t p = 0; p < CPT; p++) v[p] = mulmod_dd(dropped[threadIdx.x + p * S::CONV], pq, md.x, md.y);
+                }
+                strip_dot<!RESC, decltype(full)::value, NS, CPT>(y, s_w + (xt - x0) * NS, nd, md.x, md.y, v);
+                if (xt - x0 >= S::BUFFERS) group_sync(EMPTY + b, PASS);
+#pragma unroll
+                for (uint32_t p = 0; p < CPT; p++) bufs[b * LIMB + threadIdx.x + p * S::CONV] = v[p];
+                group_arrive(FULL + b, PASS);
             }
-            strip_dot<!RESC, NS, CPT>(y, s_w + (xt - x0) * NS, nd, md.x, md.y, v);
-            if (xt - x0 >= S::BUFFERS) group_sync(EMPTY + b, PASS);
-#pragma unroll
-            for (uint32_t p = 0; p < CPT; p++) bufs[b * LIMB + threadIdx.x + p * S::CONV] = v[p];
-            group_arrive(FULL + b, PASS);
-        }
+        };
+        if (nd == NS) convert(std::true_type());
+        else convert(std::false_type());
     } else {
         // ---- forward column passes (see ntt_fwd_cols), every other target
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(NTT_REGS));
@@ -251,9 +257,14 @@ cudaError_t conv_strip_prepare(const ckks_ctx *c) {
     return for_ring(c, [](auto logr) {
         cudaError_t e = cudaSuccess;
         for (int mode = 0; mode < 3; mode++)
-            for (uint32_t i = 0; i < 4 && e == cudaSuccess; i++)
-                e = cudaFuncSetAttribute(strip_kernels<decltype(logr)::value>[mode][i], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)strip_smem<decltype(logr)::value>(mode, 1u << i));
+            for (uint32_t i = 0; i < 4 && e == cudaSuccess; i++) {
+                StripKernel k = strip_kernels<decltype(logr)::value>[mode][i];
+                cudaFuncAttributes fa;
+                e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)strip_smem<decltype(logr)::value>(mode, 1u << i));
+                if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
+                // the registers that the roles share out have to be there: a kernel compiled to fewer must not be launched
+                if (e == cudaSuccess && (fa.numRegs + 7) / 8 * 8 * 2 != (int)(CONV_REGS + NTT_REGS)) e = cudaErrorInvalidKernelImage;
+            }
         return e;
     });
 }
