@@ -637,7 +637,7 @@ extern "C" int32_t ckks_rotate_sum(ckks_ctx *c, const ckks_ct *in, const ckks_ev
         const uint32_t m = std::min(MRB_CHUNK, n - i0);
         for (uint32_t i = 0; i < m; i++)
             cudaMemcpyAsync(xin + (size_t)i * ctl, in[i0 + i].data, ctl * sizeof(u64), cudaMemcpyDeviceToDevice, s);
-        w.mid = true;
+        w.mid = ks_mid_sum(c, level, n, 1);
         for (uint32_t i = 0; i < m; i++) {
             const u64 *evk = (const u64 *)keys[i0 + i].data;
             w.mid = w.mid && ks_mid(c, level, w, Ptrs(xin + ptl, ctl), &evk, 1);
@@ -888,7 +888,7 @@ static int32_t run_projections(ckks_ctx *c, const ckks_proj_desc *descs, uint32_
                     const uint32_t nup = std::min(lazy_giants(S), ng - gl);
                     u64 *ag = acc + (size_t)gl * S * ctl;
                     std::vector<IpTerms> tms((nup + IP_TERMS - 1) / IP_TERMS);
-                    kx.mid = true;
+                    kx.mid = ks_mid_sum(c, level, ng, S);
                     for (uint32_t t = 0; t < nup; t++) {
                         IpTerms &tm = tms[t / IP_TERMS];
                         const u64 ge = ckks_galois_element(c, (int64_t)(g0 + gl + t) * B * T);

@@ -476,6 +476,8 @@ struct KsOut {
 void ks_moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb = 1, const KsMulti *multi = nullptr);
 // Whether launch_mid_rows takes the digits d of key switches, which serve one key each (nkeys keys in all)
 bool ks_mid(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const Ptrs &d, const u64 *const *evk, uint32_t nkeys);
+// and whether it is to take a sum of nterm terms of nb entries each
+bool ks_mid_sum(const ckks_ctx *c, uint32_t level, uint32_t nterm, uint32_t nb);
 // Both together: out = ModDown(<digits, key>) and the final combination, digits read through the permutation of o.galois
 void ks_apply(const ckks_ctx *c, const u64 *evk, uint32_t level, const KsWorkspace &w, const KsOut &o, cudaStream_t s, uint32_t nb = 1, const KsMulti *multi = nullptr);
 // out = rescale(ModDown(<digits, key>) + add), level - 1 limbs per component, without the tensor-core conversions (see ks_fused_rescale)

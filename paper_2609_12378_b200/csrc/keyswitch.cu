@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(THREADS) inner_product_generic_kernel(DevTable
 // pair (s, s ^ 1), so digits and key words both move as 16-byte loads.  Without `multi` a thread walks `bch` batch
 // entries (blockIdx.y picks the chunk) with the key words of its pair held in registers; with it, an entry is one
 // of up to KS_MULTI keys applied to the same digits.
-constexpr uint32_t IP_MAX_BETA = 8;
+constexpr uint32_t IP_MAX_BETA = 8, IP_TERMS_MAX_BETA = 4;
 template <uint32_t BETA, bool ADD>
 __global__ void __launch_bounds__(IP_THREADS) inner_product_kernel(DevTables c, const u64 *ext, const __grid_constant__ Ptrs d, const u64 *evk, u64 g, u64 *u,
                                                                 uint32_t level, uint32_t nb, uint32_t bch, int has_multi, const __grid_constant__ KsMulti multi,
@@ -269,6 +269,94 @@ __global__ void __launch_bounds__(IP_THREADS) inner_product_kernel(DevTables c, 
             if (acc_u) {
                 const ulonglong2 old = *reinterpret_cast<const ulonglong2 *>(o + cm * js);
                 const u64 m = c.mod[kt];
+                r.x = add_mod(r.x, old.x, m);
+                r.y = add_mod(r.y, old.y, m);
+            }
+            *reinterpret_cast<ulonglong2 *>(o + cm * js) = r;
+        }
+    }
+}
+
+// The inner product of several terms at once (see ks_inner_terms): like inner_product_kernel, but every term has its
+// own digits, key, permutation and first component, and the running sums of a chunk of IP_BCH batch entries stay in
+// registers over the terms.
+// Two entries per thread at 64 registers and 32 warps per SM: four entries at 85 registers kept too few loads in flight (the
+// 4096 x 4096 projection's share: 20.2 -> 17.4 ms; one entry 19.9, two at 48 registers 21.3).
+constexpr uint32_t IP_BCH = 2;
+template <uint32_t BETA>
+__global__ void __launch_bounds__(IP_THREADS, 8) inner_product_terms_kernel(DevTables c, const u64 *ext, size_t term_stride, const u64 *d, size_t d_stride,
+                                                                         const __grid_constant__ IpTerms tm, uint32_t nterm, size_t c0_stride,
+                                                                         u64 *u, uint32_t level, uint32_t nb, int acc_u) {
+    const uint32_t p = (blockIdx.x * IP_THREADS + threadIdx.x) * 2;
+    const uint32_t x = blockIdx.z, b0 = blockIdx.y * IP_BCH;
+    const uint32_t nt = level + c.K;
+    const uint32_t kt = x < level ? x : c.L + (x - level);
+    const double2 md = c.modd[kt];
+    const size_t js = (size_t)nt * c.N, ks = (size_t)c.T * c.N;
+    const double pq = x < level ? c.dn_p_mod_d[x] : 0.0;
+    const uint32_t own = x < level ? x / c.alpha : BETA;       // the digit that has x among its own limbs: it lies in d
+    double acc[IP_BCH][2][2];
+#pragma unroll
+    for (uint32_t bi = 0; bi < IP_BCH; bi++) acc[bi][0][0] = acc[bi][0][1] = acc[bi][1][0] = acc[bi][1][1] = 0.0;
+    grid_dep_sync();
+    for (uint32_t t = 0; t < nterm; t++) {
+        const uint32_t src = galois_src(p, (uint32_t)tm.galois[t], c.log_n);
+        const bool odd = src & 1;
+        const u64 *evk = tm.evk[t];
+        double k[BETA][2][2];
+#pragma unroll
+        for (uint32_t j = 0; j < BETA; j++)
+#pragma unroll
+            for (uint32_t cm = 0; cm < 2; cm++) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(evk + ((size_t)j * 2 + cm) * ks + (size_t)kt * c.N + p);
+                k[j][cm][0] = u64_to_d(v.x);
+                k[j][cm][1] = u64_to_d(v.y);
+            }
+        const uint32_t so = src & ~1u;
+        const u64 *z = (x < level && tm.c0[t]) ? tm.c0[t] + b0 * c0_stride + (size_t)x * c.N : nullptr;
+        // no branch in here, so that the loads of all entries of the chunk are in flight together: an entry past the end
+        // of the batch repeats the last one and is not stored
+#pragma unroll
+        for (uint32_t bi = 0; bi < IP_BCH; bi++) {
+            const uint32_t bc = min(bi, nb - 1 - b0);
+            double sum[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+            for (uint32_t j = 0; j < BETA; j++) {
+                const u64 *ej = (j == own ? d + (size_t)(t * nb + b0 + bc) * d_stride
+                                          : ext + t * term_stride + ((size_t)(b0 + bc) * BETA + j) * js) + (size_t)x * c.N;
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(ej + so);
+                const double d0 = u64_to_d(odd ? v.y : v.x), d1 = u64_to_d(odd ? v.x : v.y);
+#pragma unroll
+                for (uint32_t cm = 0; cm < 2; cm++) {
+                    sum[cm][0] = __dadd_rn(sum[cm][0], mulmod_dd(d0, k[j][cm][0], md.x, md.y));
+                    sum[cm][1] = __dadd_rn(sum[cm][1], mulmod_dd(d1, k[j][cm][1], md.x, md.y));
+                }
+            }
+            if (z) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(z + bc * c0_stride + so);
+                sum[0][0] = __dadd_rn(sum[0][0], mulmod_dd(u64_to_d(odd ? v.y : v.x), pq, md.x, md.y));
+                sum[0][1] = __dadd_rn(sum[0][1], mulmod_dd(u64_to_d(odd ? v.x : v.y), pq, md.x, md.y));
+            }
+            // at most BETA + 1 products of size 0.75 m on top of a reduced sum: far below 2^53
+#pragma unroll
+            for (uint32_t cm = 0; cm < 2; cm++) {
+                acc[bi][cm][0] = reduce_d(__dadd_rn(acc[bi][cm][0], sum[cm][0]), md.x, md.y);
+                acc[bi][cm][1] = reduce_d(__dadd_rn(acc[bi][cm][1], sum[cm][1]), md.x, md.y);
+            }
+        }
+    }
+    const u64 m = c.mod[kt];
+#pragma unroll
+    for (uint32_t bi = 0; bi < IP_BCH; bi++) {
+        if (b0 + bi >= nb) break;
+        u64 *o = u + (size_t)(b0 + bi) * 2 * js + (size_t)x * c.N + p;
+#pragma unroll
+        for (uint32_t cm = 0; cm < 2; cm++) {
+            ulonglong2 r;
+            r.x = canonical_d(acc[bi][cm][0], md.x);
+            r.y = canonical_d(acc[bi][cm][1], md.x);
+            if (acc_u) {
+                const ulonglong2 old = *reinterpret_cast<const ulonglong2 *>(o + cm * js);
                 r.x = add_mod(r.x, old.x, m);
                 r.y = add_mod(r.y, old.y, m);
             }
@@ -488,6 +576,14 @@ bool ks_mid(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const Ptrs 
     for (uint32_t k = 0; k < nkeys; k++) ok = ok && aligned16(evk[k]);
     return ok;
 }
+// Sums of terms: a row's terms follow one another in its CTA, so that few CTAs make a long chain, where separate launches transform all
+// terms' digits side by side.  mid_rows takes them from three CTAs per SM on (sums of sixteen terms: N = 2^15, level 12, 512 CTAs, 459 ->
+// 432 us; level 10, 448 CTAs, 401 -> 386; but level 8, 384 CTAs, 273 -> 282; N = 2^14, level 6, 128 CTAs, 191 -> 252; N = 2^13, level 4, 40
+// CTAs, 149 -> 223; lazy projections of one to three shards there 1.07 to 1.22 times as long), and short chains of two terms
+// everywhere (N = 2^13, level 4, 40.3 -> 39.6 us; of four 48.5 -> 60.4).
+bool ks_mid_sum(const ckks_ctx *c, uint32_t level, uint32_t nterm, uint32_t nb) {
+    return nterm <= 2 || (uint64_t)(c->N >> 10) * nb * (level + c->K) >= 3 * (uint64_t)c->sms;
+}
 static void mid_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 galois, const KsWorkspace &w, uint32_t inv_from, cudaStream_t s, uint32_t nb, const KsMulti *multi,
                       const Ptrs *add) {
     MidArgs a{};
@@ -624,6 +720,14 @@ void ks_inner_terms(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, siz
         a.term_stride = term_stride; a.c0_stride = c0_stride; a.acc_u = acc_u ? 1 : 0;
         for (uint32_t t = 0; t < nterm; t++) { a.evk[t] = terms.evk[t]; a.galois[t] = terms.galois[t]; a.c0[t] = terms.c0[t]; }
         launch_mid_rows(c, a, beta, s);
+        return;
+    }
+    bool aligned = aligned16(w.ext) && aligned16(w.u) && (term_stride & 1) == 0 && (c0_stride & 1) == 0 && aligned16(w.d);
+    for (uint32_t t = 0; t < nterm; t++) aligned = aligned && aligned16(terms.evk[t]) && aligned16(terms.c0[t]);
+    if (beta <= IP_TERMS_MAX_BETA && aligned) {
+        const dim3 grid(N / (2 * IP_THREADS), (nb + IP_BCH - 1) / IP_BCH, nt);
+        auto *k = beta == 1 ? inner_product_terms_kernel<1> : beta == 2 ? inner_product_terms_kernel<2> : beta == 3 ? inner_product_terms_kernel<3> : inner_product_terms_kernel<4>;
+        launch(k, grid, IP_THREADS, 0, s, c->dev, w.ext, term_stride, w.d.base, w.d.stride, terms, nterm, c0_stride, w.u, level, nb, acc_u ? 1 : 0);
         return;
     }
     // any number of digits, any alignment: one term at a time through the generic kernel, then its P c0

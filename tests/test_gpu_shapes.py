@@ -443,3 +443,27 @@ def test_transforms_on_either_side_of_a_row_per_warp(log_n, batch, limbs):
         assert np.array_equal(host(ctx.ntt(y)), fwd)
         y.copy_(torch.from_numpy(x))
         assert np.array_equal(host(ctx.intt(y)), inv)
+
+
+@pytest.mark.parametrize("log_n,L,K,dnum,level", [(12, 4, 4, 1, 4), (13, 6, 1, 6, 4), (14, 8, 2, 4, 8), (15, 16, 4, 4, 13), (15, 16, 4, 4, 12), (15, 12, 4, 3, 10), (15, 12, 4, 3, 9)])
+def test_sums_of_rotations_whose_terms_share_a_row_or_not(log_n, L, K, dnum, level):
+    """Two terms, which follow one another in the kernel between the column passes on every ring, and five, which do so from three CTAs per
+    SM on and otherwise have their digits transformed by a launch before the inner product: one to four digits, a partial one among
+    them, on either side of the line."""
+    import torch
+    from paper_2609_12378_b200 import binding
+    from tests.gpu_util import context, ct_dev, host, key_dev
+    P, ctx = params(log_n, L, K, dnum), context(log_n, L, K, dnum)
+    o, g = P.oracle, inputs.rng(820, level + 100 * L + 10000 * log_n)
+    cts = [inputs.uniform_residues(g, P.q[:level], P.N, 2) for _ in range(5)]
+    keys = [inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, dnum * 2).reshape(dnum, 2, L + K, P.N) for _ in range(5)]
+    gals = [o.galois_element(r) for r in (1, 5, 64, 3, P.n - 1)]
+    dcts, dkeys = [ct_dev(x, 1.0) for x in cts], [key_dev(k, e) for k, e in zip(keys, gals)]
+    launches = []
+    for n in (2, 5):
+        before = binding.kernel_launches()
+        got = ctx.rotate_sum(dcts[:n], dkeys[:n])
+        launches.append(binding.kernel_launches() - before)
+        assert np.array_equal(host(got.data), o.rotate_sum(np.stack(cts[:n]), keys[:n], gals[:n]))
+    one_kernel = (P.N >> 10) * (level + K) >= 3 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert launches[1] - launches[0] == (1 if one_kernel else 2)      # five terms take two passes
