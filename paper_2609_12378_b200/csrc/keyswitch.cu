@@ -572,6 +572,8 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
 // mid_rows takes up to IP_FUSED_BETA digits and 16-byte accesses (one rotation at N = 2^16, level 24: 153 -> 149.4 us, at N = 2^14 32.8 ->
 // 29.4; the degree-63 polynomial 2139 -> 2091; projections of 24 tokens, which sum their giant steps, 32.1 -> 31.7 ms)
 bool ks_mid(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const Ptrs &d, const u64 *const *evk, uint32_t nkeys) {
+    // plain transforms around the tensor cores' conversions: a share of their limbs may be on the integer pipe, which runs whole transforms
+    if (conv_tensor(c) && c->ntt_fp_share < 8 && c->log_n == 16) return false;
     bool ok = (level + c->alpha - 1) / c->alpha <= IP_FUSED_BETA && aligned16(w.ext) && aligned16(w.u) && aligned16(d);
     for (uint32_t k = 0; k < nkeys; k++) ok = ok && aligned16(evk[k]);
     return ok;

@@ -379,6 +379,31 @@ def test_transforms_that_leave_out_every_limb_of_one_path(share):
         ctx.set_option(binding.OPT_NTT_FP_SHARE, 8)
 
 
+def test_key_switches_of_one_key_take_the_integer_share():
+    """With the tensor-core conversions a rotation's transforms are plain ones, so that the share of limbs on the integer transform applies
+    to them as it does in a hoisted rotation: the same number of launches."""
+    from paper_2609_12378_b200 import binding
+    from tests.gpu_util import context, ct_dev, host, key_dev
+    P, ctx = params(16, 3, 1, 3), context(16, 3, 1, 3)
+    o, g = P.oracle, inputs.rng(815, 0)
+    x = inputs.uniform_residues(g, P.q[:2], P.N, 2)
+    key = inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, 6).reshape(3, 2, 4, P.N)
+    gal = o.galois_element(5)
+    want, count = o.rotate(x, key, gal), []
+    ctx.set_option(binding.OPT_CONV_KERNEL, binding.CONV_TENSOR)
+    ctx.set_option(binding.OPT_NTT_FP_SHARE, 4)
+    try:
+        for call in (lambda: ctx.rotate_hoisted(ct_dev(x, 1.0), [key_dev(key, gal)])[0], lambda: ctx.rotate(ct_dev(x, 1.0), key_dev(key, gal))):
+            before = binding.kernel_launches()
+            got = call()
+            count.append(binding.kernel_launches() - before)
+            assert np.array_equal(host(got.data), want)
+    finally:
+        ctx.set_option(binding.OPT_CONV_KERNEL, binding.CONV_FP64)
+        ctx.set_option(binding.OPT_NTT_FP_SHARE, 8)
+    assert count[0] == count[1]
+
+
 @pytest.mark.parametrize("log_n,L,K,dnum,level", [
     (12, 3, 1, 3, 3), (12, 8, 8, 1, 8), (12, 9, 9, 1, 9), (12, 7, 4, 3, 5), (12, 12, 3, 4, 12), (12, 10, 2, 5, 10), (12, 16, 8, 2, 11),
     (13, 12, 6, 2, 12), (14, 6, 2, 3, 5), (14, 16, 8, 2, 16), (15, 12, 4, 3, 9), (15, 8, 8, 1, 8), (16, 3, 3, 1, 3), (16, 10, 5, 2, 6)])
