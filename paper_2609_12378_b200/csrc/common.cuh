@@ -77,6 +77,7 @@ struct ckks_ctx {
     int ntt_bulk_store = 1;                  // kept for get and set; selects nothing
     int conv_kernel = 0;                     // basis conversions: 0 = FP64 pipe, 1 = tensor cores (conv_mma.cu)
     int mac_kernel = 82;                     // projection multiply-accumulate kernel (see launch_mac_mma)
+    bool strips = false;                     // conversions may run in strips (conv_strip_prepare)
     long long wait_cycles = 2000000000ll;    // clock bound of every device-side wait (about a second)
     // Streams of the context.  ckks_attention_pack, whose work is many independent single-ciphertext chains, spreads them over
     // `lanes` streams, lane 0 being the caller's: a single ciphertext's kernels fill the GPU for at most one wave, so
@@ -410,7 +411,9 @@ void launch_ntt_part(const ckks_ctx *c, NttPart part, u64 *base, uint32_t nlimbs
 // CONV_DOWN: ModDown of one component (item: entry * 2 + component; src [item][level + K], dst [item][targets]);
 // CONV_DOWN_RS: that of a ModDown which a rescale follows.  targets: of a ModUp the largest number of a digit.
 enum { CONV_UP = 0, CONV_DOWN = 1, CONV_DOWN_RS = 2 };
-cudaError_t conv_strip_prepare(const ckks_ctx *c);          // once per context
+// Once per context: whether it can run, i.e. the ring has an instance, and the compiler gave the kernels the registers that their roles
+// share out (with fewer they would wait for ones that nobody gives back).  Without it the conversions take their separate kernels.
+bool conv_strip_prepare(const ckks_ctx *c);
 bool conv_strip(const ckks_ctx *c, int mode, uint32_t level, uint32_t items, bool alone = false);     // alone: see launch_ntt
 void launch_conv_strip(const ckks_ctx *c, int mode, const u64 *src, u64 *dst, uint32_t level, uint32_t items, uint32_t targets, cudaStream_t s);
 void launch_ntt_int(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, bool inverse, const NttSource &src, cudaStream_t s);

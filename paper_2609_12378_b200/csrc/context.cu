@@ -443,11 +443,12 @@ extern "C" int32_t ckks_context_create(const ckks_params *prm, ckks_ctx **out) {
     bool lanes_ok = true;
     for (cudaStream_t &ls : c->lane_stream) lanes_ok = lanes_ok && cudaStreamCreateWithFlags(&ls, cudaStreamNonBlocking) == cudaSuccess;
     for (cudaEvent_t &le : c->lane_event) lanes_ok = lanes_ok && cudaEventCreateWithFlags(&le, cudaEventDisableTiming) == cudaSuccess;
-    if (!lanes_ok || conv_strip_prepare(c) != cudaSuccess) {
+    if (!lanes_ok) {
         cudaSetDevice(prev);
         ckks_context_destroy(c);
         return CKKS_ERR_CUDA;
     }
+    c->strips = conv_strip_prepare(c);
     cudaSetDevice(prev);
     *out = c;
     return CKKS_OK;

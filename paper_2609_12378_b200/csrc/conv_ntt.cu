@@ -252,20 +252,19 @@ uint32_t strip_sources(const ckks_ctx *c, int mode, uint32_t level) { return mod
 
 }  // namespace
 
-cudaError_t conv_strip_prepare(const ckks_ctx *c) {
-    if (c->log_n < 12) return cudaSuccess;
+bool conv_strip_prepare(const ckks_ctx *c) {
+    if (c->log_n < 12) return false;
     return for_ring(c, [](auto logr) {
-        cudaError_t e = cudaSuccess;
+        bool ok = true;
         for (int mode = 0; mode < 3; mode++)
-            for (uint32_t i = 0; i < 4 && e == cudaSuccess; i++) {
+            for (uint32_t i = 0; i < 4 && ok; i++) {
                 StripKernel k = strip_kernels<decltype(logr)::value>[mode][i];
                 cudaFuncAttributes fa;
-                e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)strip_smem<decltype(logr)::value>(mode, 1u << i));
-                if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
-                // the registers that the roles share out have to be there: a kernel compiled to fewer must not be launched
-                if (e == cudaSuccess && (fa.numRegs + 7) / 8 * 8 * 2 != (int)(CONV_REGS + NTT_REGS)) e = cudaErrorInvalidKernelImage;
+                ok = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)strip_smem<decltype(logr)::value>(mode, 1u << i)) == cudaSuccess &&
+                     cudaFuncGetAttributes(&fa, k) == cudaSuccess && (fa.numRegs + 7) / 8 * 8 * 2 == (int)(CONV_REGS + NTT_REGS);
             }
-        return e;
+        if (!ok) cudaGetLastError();
+        return ok;
     });
 }
 
@@ -277,7 +276,7 @@ cudaError_t conv_strip_prepare(const ckks_ctx *c) {
 // product and rescale 71.7 -> 66.3; N = 2^14: ModUp 29.3 -> 28.4), but for ModDowns of a few strips (29.3 -> 30.7) and, at N = 2^13, for ModUps inside longer calls (a
 // 64 x 64 projection 172.4 -> 175.3; a rotation of its own 30.7 -> 29.2).
 bool conv_strip(const ckks_ctx *c, int mode, uint32_t level, uint32_t items, bool alone) {
-    if (c->conv_kernel == CKKS_CONV_TENSOR || c->log_n < 12 || items > 65535 || strip_sources(c, mode, level) > STRIP_NS) return false;
+    if (!c->strips || c->conv_kernel == CKKS_CONV_TENSOR || items > 65535 || strip_sources(c, mode, level) > STRIP_NS) return false;
     const uint64_t strips = (uint64_t)(c->N >> 11) * items;
     return strips >= 3 * (uint64_t)c->sms || (c->log_n < 16 && (mode == CONV_UP ? alone || c->log_n > 13 : strips >= 32));
 }

@@ -492,3 +492,44 @@ def test_sums_of_rotations_whose_terms_share_a_row_or_not(log_n, L, K, dnum, lev
         assert np.array_equal(host(got.data), o.rotate_sum(np.stack(cts[:n]), keys[:n], gals[:n]))
     one_kernel = (P.N >> 10) * (level + K) >= 3 * torch.cuda.get_device_properties(0).multi_processor_count
     assert launches[1] - launches[0] == (1 if one_kernel else 2)      # five terms take two passes
+
+
+FEWER_REGISTERS = r"""
+#define _GNU_SOURCE
+#include <dlfcn.h>
+#include <cuda_runtime_api.h>
+cudaError_t cudaFuncGetAttributes(struct cudaFuncAttributes *a, const void *f) {
+    cudaError_t (*real)(struct cudaFuncAttributes *, const void *) = dlsym(dlopen("libcudart.so.12", RTLD_LAZY | RTLD_NOLOAD), "cudaFuncGetAttributes");
+    cudaError_t e = real(a, f);
+    a->numRegs -= 32;
+    return e;
+}
+"""
+ROTATE_ONCE = """
+import numpy as np
+from paper_2609_12378_b200 import binding, inputs
+from tests.gpu_util import context, ct_dev, host, key_dev
+from tests.harness import params
+P, ctx = params(15, 4, 2, 2), context(15, 4, 2, 2)
+g = inputs.rng(830, 0)
+x = inputs.uniform_residues(g, P.q, P.N, 2)
+key = inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, 4).reshape(2, 2, 6, P.N)
+before = binding.kernel_launches()
+y = host(ctx.rotate(ct_dev(x, 1.0), key_dev(key, P.oracle.galois_element(3))).data)
+assert np.array_equal(y, P.oracle.rotate(x, key, P.oracle.galois_element(3)))
+print(binding.kernel_launches() - before)
+"""
+
+
+def test_context_without_the_registers_of_the_strip_kernel(tmp_path):
+    """A library whose strip kernels were compiled to other registers than their roles share out (here: whose runtime says so) makes
+    contexts all the same and takes the separate kernels: the same rotation in more launches."""
+    import os
+    import subprocess
+    import sys
+    src, lib, root = tmp_path / "regs.c", tmp_path / "regs.so", os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    src.write_text(FEWER_REGISTERS)
+    subprocess.run(["gcc", "-shared", "-fPIC", "-I/usr/local/cuda/include", str(src), "-o", str(lib), "-ldl"], check=True)
+    count = [int(subprocess.run([sys.executable, "-c", ROTATE_ONCE], cwd=root, env={**os.environ, **env}, check=True, stdout=subprocess.PIPE, timeout=300).stdout)
+             for env in ({}, {"LD_PRELOAD": " ".join([str(lib), os.environ.get("LD_PRELOAD", "")]).strip()})]
+    assert count[0] == 5 and count[1] > 5
