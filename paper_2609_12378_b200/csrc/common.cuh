@@ -409,13 +409,13 @@ void launch_ntt_part(const ckks_ctx *c, NttPart part, u64 *base, uint32_t nlimbs
 // What lies between an inverse and a forward row pass (conv_ntt.cu): the sources' inverse column pass, a basis conversion, the targets'
 // forward column pass.  CONV_UP: ModUp of one digit (an item: entry * digits + digit; src [entry][level], dst [item][level + K]);
 // CONV_DOWN: ModDown of one component (item: entry * 2 + component; src [item][level + K], dst [item][targets]);
-// CONV_DOWN_RS: that of a ModDown which a rescale follows.  targets: of a ModUp the largest number of a digit.
+// CONV_DOWN_RS: that of a ModDown which a rescale follows.
 enum { CONV_UP = 0, CONV_DOWN = 1, CONV_DOWN_RS = 2 };
 // Once per context: whether it can run, i.e. the ring has an instance, and the compiler gave the kernels the registers that their roles
 // share out (with fewer they would wait for ones that nobody gives back).  Without it the conversions take their separate kernels.
 bool conv_strip_prepare(const ckks_ctx *c);
 bool conv_strip(const ckks_ctx *c, int mode, uint32_t level, uint32_t items, bool alone = false);     // alone: see launch_ntt
-void launch_conv_strip(const ckks_ctx *c, int mode, const u64 *src, u64 *dst, uint32_t level, uint32_t items, uint32_t targets, cudaStream_t s);
+void launch_conv_strip(const ckks_ctx *c, int mode, const u64 *src, u64 *dst, uint32_t level, uint32_t items, cudaStream_t s);
 void launch_ntt_int(const ckks_ctx *c, u64 *b, uint32_t ny, const LimbMap &map, bool inverse, const NttSource &src, cudaStream_t s);
 
 void launch_mul_plain_acc(const ckks_ctx *c, const u64 *const *cts, u64 *const *accs, uint32_t ncts, const u64 *pt,

@@ -73,25 +73,31 @@ __device__ __forceinline__ void strip_dot(const double (&y)[CPT][NS], const doub
     }
 }
 
+// The CTAs of a launch: the first `whole` take a strip of an item with all its targets, the others one of `split` strips with `chunk` targets
+struct StripGrid { uint32_t whole, split, chunk; };
+
 // src: limbs after the inverse row pass (signed doubles); dst: limbs for the forward row pass.  NS: sources at most
 template <uint32_t LOGR, int MODE, uint32_t NS>
-__global__ void __launch_bounds__(StripShape<LOGR>::THREADS, 1) conv_cols(DevTables c, const double *src, double *dst, uint32_t level, uint32_t targets, uint32_t chunk) {
+__global__ void __launch_bounds__(StripShape<LOGR>::THREADS, 1) conv_cols(DevTables c, const double *src, double *dst, uint32_t level, uint32_t targets, StripGrid grid) {
     using S = StripShape<LOGR>;
     constexpr uint32_t E = S::E, R = S::R, RS = S::RS, LIMB = S::LIMB, COLS = S::COLS, TG = S::TG, GROUPS = S::GROUPS, CPT = S::CPT;
     constexpr bool RESC = MODE == CONV_DOWN_RS;
     extern __shared__ __align__(16) double ssm[];
-    const uint32_t grp = threadIdx.x / TG, tid = threadIdx.x % TG, cc = tid % COLS, r = tid / COLS, col = blockIdx.x * COLS + cc;
+    const uint32_t grp = threadIdx.x / TG, tid = threadIdx.x % TG, cc = tid % COLS, r = tid / COLS;
+    constexpr uint32_t STRIPS = 256 / COLS;                   // of an item
+    const bool whole = blockIdx.x < grid.whole;
+    const uint32_t slot = blockIdx.x - (whole ? 0 : grid.whole), strip = whole ? slot : grid.whole + slot % grid.split, col = strip % STRIPS * COLS + cc;
     double *bufs = ssm;                                       // [sources][LIMB] (the dropped limb last); the first BUFFERS pass targets later
     double *stw = bufs + (NS > S::BUFFERS ? NS : S::BUFFERS) * LIMB + (RESC ? LIMB : 0);       // [GROUPS][R] twiddles
     double2 *s_m = reinterpret_cast<double2 *>(stw + GROUPS * R);       // the targets' primes and inverses
     double *s_w = reinterpret_cast<double *>(s_m + STRIP_CHUNK);        // [targets of the chunk (+ the dropped limb)][NS] constants
     double *dropped = bufs + (NS > S::BUFFERS ? NS : S::BUFFERS) * LIMB;
     // the conversion's sources and targets
-    const uint32_t item = blockIdx.z;
+    const uint32_t item = strip / STRIPS;
     const uint32_t beta = MODE == CONV_UP ? (level + c.alpha - 1) / c.alpha : 1, j = MODE == CONV_UP ? item % beta : 0, bz = item / beta;
     const uint32_t lo = j * c.alpha, nd = MODE == CONV_UP ? min(c.alpha, level - lo) : c.K;
     const uint32_t nt = level + c.K;
-    const uint32_t x0 = blockIdx.y * chunk, x1 = min(x0 + chunk, MODE == CONV_UP ? nt - nd : targets);      // ModUp: counted without the digit's own limbs
+    const uint32_t x0 = whole ? 0 : slot / grid.split * grid.chunk, x1 = min(whole ? targets : x0 + grid.chunk, MODE == CONV_UP ? nt - nd : targets);      // ModUp: counted without the digit's own limbs
     if (x0 >= x1) return;
     auto target_limb = [&](uint32_t xt) { return MODE == CONV_UP && xt >= lo ? xt + nd : xt; };
     auto target_prime = [&](uint32_t xt) { const uint32_t x = target_limb(xt); return MODE == CONV_UP && x >= level ? c.L + (x - level) : x; };
@@ -249,6 +255,34 @@ auto for_ring(const ckks_ctx *c, F f) {
     }
 }
 uint32_t strip_sources(const ckks_ctx *c, int mode, uint32_t level) { return mode == CONV_UP ? std::min(c->alpha, level) : c->K; }
+// (of a ModUp the most that a digit has: the last one's)
+uint32_t strip_targets(const ckks_ctx *c, int mode, uint32_t level) {
+    return mode == CONV_UP ? (level + c->alpha - 1) / c->alpha * c->alpha - c->alpha + c->K : mode == CONV_DOWN ? level : level - 1;
+}
+
+// The cheapest grid for `strips` strips, one CTA per SM at a time.  A CTA's time is its targets in groups of four and half as much per
+// round of sources, which every chunk of the same strip repeats.  As many strips as fill whole waves can go by one CTA each; cut into
+// chunks, the others share out the last wave.  (N = 2^16, level 24, in a burst and back to back under the power limit: eight hoisted
+// rotations, 512 strips, 3.46 waves, by the separate kernels 576 and 566 us, by a CTA per strip 588 and 559, so 575 and 545; fourteen, 6.05
+// waves, 910 and 924, 931 and 918, 911 and 878.)
+struct StripPlan { StripGrid grid; uint32_t ctas, cost, full; };        // full: the cost if all SMs were busy throughout, times their number
+StripPlan strip_plan(const ckks_ctx *c, int mode, uint32_t level, uint32_t strips) {
+    const uint32_t targets = strip_targets(c, mode, level), sms = (uint32_t)c->sms, rounds = (strip_sources(c, mode, level) + (mode == CONV_DOWN_RS) + 3) / 4;
+    auto cta = [&](uint32_t n) { return (std::min(n, targets) + 3) / 4 * 2 + rounds; };
+    StripPlan p{};
+    p.full = strips * cta(targets);
+    p.cost = ~0u;
+    const uint32_t waves = targets <= STRIP_CHUNK ? strips / sms : 0;
+    for (uint32_t w = 0;; w = waves) {
+        const uint32_t whole = w * sms, split = strips - whole;
+        for (uint32_t ch = 4; ch <= STRIP_CHUNK && ch < targets + 4; ch += 4) {
+            const uint32_t n = (targets + ch - 1) / ch, cost = w * cta(targets) + (split * n + sms - 1) / sms * cta(ch);
+            if (cost <= p.cost) p = {{whole, std::max(split, 1u), ch}, whole + split * n, cost, p.full};
+        }
+        if (w == waves) break;
+    }
+    return p;
+}
 
 }  // namespace
 
@@ -269,33 +303,31 @@ bool conv_strip_prepare(const ckks_ctx *c) {
 }
 
 // Whether a conversion of `items` items runs here.  It can from N = 2^12 on with at most eight sources, whose coefficients fit the
-// registers.  A CTA has an SM to itself, so that at N = 2^16 the few CTAs of one ciphertext (96 for ModUp, 64 for ModDown) leave a third
-// of the GPU idle or repeat their sources' transforms: there it takes batches of three strips per SM and more (64 hoisted rotations
-// 3810 -> 3680 us, the attention of 128 tokens with 32 channels 61.1 -> 57.9 ms; one rotation would go from 149 to 156).  The separate
-// kernels of smaller rings are bound by latency, and fewer launches win from the first ciphertext on (N = 2^15: rotation 49.5 -> 43.9,
-// product and rescale 71.7 -> 66.3; N = 2^14: ModUp 29.3 -> 28.4), but for ModDowns of a few strips (29.3 -> 30.7) and, at N = 2^13, for ModUps inside longer calls (a
-// 64 x 64 projection 172.4 -> 175.3; a rotation of its own 30.7 -> 29.2).
+// registers.  At N = 2^16 a strip takes an SM as long as the separate kernels do, and what it saves is traffic: batches of four strips
+// per SM and more, and of three with eight targets and more where the last wave is nearly full, take the same time in a burst (0.98 to
+// 1.02 of it) and under the power limit 0.91 to 1.01 of it, most of them 0.96 and less (64 hoisted rotations at level 24 3952 -> 3750 us,
+// sixteen products 2056 -> 1950).  Seven hoisted rotations at level 5, 3.03 waves, would go from 205 to 216 us and from 152 to 164, eight
+// from 171 to 175.  The few strips of one ciphertext (96 for ModUp, 64 for ModDown) leave a third of the GPU idle or repeat their sources'
+// transforms (a rotation 149 -> 156).
+// The separate kernels of smaller rings are bound by latency, and fewer launches win from the first ciphertext on (N = 2^15: rotation
+// 49.5 -> 43.9, product and rescale 71.7 -> 66.3; N = 2^14: ModUp 29.3 -> 28.4), but for ModDowns of a few strips (29.3 -> 30.7) and, at
+// N = 2^13, for ModUps inside longer calls (a 64 x 64 projection 172.4 -> 175.3; a rotation of its own 30.7 -> 29.2).
 bool conv_strip(const ckks_ctx *c, int mode, uint32_t level, uint32_t items, bool alone) {
     if (!c->strips || c->conv_kernel == CKKS_CONV_TENSOR || items > 65535 || strip_sources(c, mode, level) > STRIP_NS) return false;
-    const uint64_t strips = (uint64_t)(c->N >> 11) * items;
-    return strips >= 3 * (uint64_t)c->sms || (c->log_n < 16 && (mode == CONV_UP ? alone || c->log_n > 13 : strips >= 32));
+    const uint32_t strips = (c->N >> 11) * items, sms = (uint32_t)c->sms;
+    if (strips >= 4 * sms || (c->log_n < 16 && (mode == CONV_UP ? alone || c->log_n > 13 : strips >= 32))) return true;
+    if (strips < 3 * sms || strip_targets(c, mode, level) < 8) return false;
+    const StripPlan p = strip_plan(c, mode, level, strips);
+    return 10 * p.full >= 9 * sms * p.cost;
 }
 
-void launch_conv_strip(const ckks_ctx *c, int mode, const u64 *src, u64 *dst, uint32_t level, uint32_t items, uint32_t targets, cudaStream_t s) {
+void launch_conv_strip(const ckks_ctx *c, int mode, const u64 *src, u64 *dst, uint32_t level, uint32_t items, cudaStream_t s) {
     const uint32_t ns = strip_sources(c, mode, level), i = ns <= 1 ? 0 : ns <= 2 ? 1 : ns <= 4 ? 2 : 3;
     for_ring(c, [&](auto logr) {
         constexpr uint32_t LOGR = decltype(logr)::value;
         using S = StripShape<LOGR>;
-        const uint32_t strips = 256 / S::COLS, rounds0 = (ns + S::GROUPS - 1) / S::GROUPS;
-        // Targets per CTA.  A CTA's time is its batches of targets and half as much per round of sources, which every chunk of the
-        // same strip repeats; the smallest product with the number of waves wins (one CTA per SM).
-        uint32_t chunk = S::GROUPS;
-        uint64_t best = ~0ull;
-        for (uint32_t ch = S::GROUPS; ch <= STRIP_CHUNK && ch < targets + S::GROUPS; ch += S::GROUPS) {
-            const uint64_t ctas = (uint64_t)strips * items * ((targets + ch - 1) / ch), cost = (ctas + c->sms - 1) / c->sms * (2 * ch / S::GROUPS + rounds0);
-            if (cost <= best) { best = cost; chunk = ch; }
-        }
-        launch(strip_kernels<LOGR>[mode][i], dim3(strips, (targets + chunk - 1) / chunk, items), S::THREADS, strip_smem<LOGR>(mode, 1u << i), s, c->dev,
-               reinterpret_cast<const double *>(src), reinterpret_cast<double *>(dst), level, targets, chunk);
+        const StripPlan p = strip_plan(c, mode, level, 256 / S::COLS * items);
+        launch(strip_kernels<LOGR>[mode][i], p.ctas, S::THREADS, strip_smem<LOGR>(mode, 1u << i), s, c->dev, reinterpret_cast<const double *>(src), reinterpret_cast<double *>(dst),
+               level, strip_targets(c, mode, level), p.grid);
     });
 }

@@ -510,7 +510,7 @@ void ks_modup(const ckks_ctx *c, const Ptrs &d, uint32_t level, KsWorkspace &w, 
     src.ptr = d; src.lpitch = 1;
     if (conv_strip(c, CONV_UP, level, nb * beta, w.alone)) {
         launch_ntt_part(c, NTT_ROWS, w.dcoef, nb * level, plain_map(0, level), true, s, nullptr, nullptr, &src);
-        launch_conv_strip(c, CONV_UP, w.dcoef, w.ext, level, nb * beta, nt - (level - (beta - 1) * c->alpha), s);
+        launch_conv_strip(c, CONV_UP, w.dcoef, w.ext, level, nb * beta, s);
         if (!w.mid) launch_ntt_part(c, NTT_ROWS, w.ext, nb * beta * nt, ext_map(level, c->K, c->L, c->alpha, beta), false, s);
         return;
     }
@@ -649,7 +649,7 @@ static void moddown(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, Ntt
     else if (first)
         launch_ntt_part(c, first, w.u + (size_t)level * N, nb * 2 * K, pitched_map(c->L, K, nt), true, s, ep.mode == 3 ? &ep : nullptr, nullptr, nullptr, scale);
     if (strip) {
-        launch_conv_strip(c, CONV_DOWN, w.u, w.conv, level, 2 * nb, level, s);
+        launch_conv_strip(c, CONV_DOWN, w.u, w.conv, level, 2 * nb, s);
         launch_ntt_part(c, NTT_ROWS, w.conv, nb * 2 * level, plain_map(0, level), false, s, &ep);
         return;
     }
@@ -702,7 +702,7 @@ void ks_apply_rescale(const ckks_ctx *c, const u64 *evk, uint32_t level, const K
         launch_ntt_part(c, first, w.u + (size_t)m * N, nb * 2 * (K + 1), tail_map(m, level, K, c->L), true, s, nullptr, nullptr, nullptr,
                         c->dev.inv_scale_rs + (size_t)m * (K + 1) * 2);
     if (strip) {
-        launch_conv_strip(c, CONV_DOWN_RS, w.u, w.conv, level, 2 * nb, m, s);
+        launch_conv_strip(c, CONV_DOWN_RS, w.u, w.conv, level, 2 * nb, s);
         launch_ntt_part(c, NTT_ROWS, w.conv, nb * 2 * m, plain_map(0, m), false, s, &ep);
         return;
     }

@@ -494,6 +494,31 @@ def test_sums_of_rotations_whose_terms_share_a_row_or_not(log_n, L, K, dnum, lev
     assert launches[1] - launches[0] == (1 if one_kernel else 2)      # five terms take two passes
 
 
+@pytest.mark.parametrize("L,K,dnum,level,separate", [(3, 1, 3, 3, (7, 8, 9)), (10, 8, 2, 9, (7,)), (24, 8, 3, 24, ())])
+def test_last_wave_of_the_strips(L, K, dnum, level, separate):
+    """Hoisted rotations at N = 2^16 whose strips (64 per rotation, on 148 SMs) fill three waves and a bit to six waves and a bit: whole strips
+    and strips cut into chunks in one grid.  Where most of the last wave would be idle the separate kernels run, two launches more."""
+    import torch
+    from paper_2609_12378_b200 import binding
+    from tests.gpu_util import context, ct_dev, host, key_dev
+    P, ctx = params(16, L, K, dnum), context(16, L, K, dnum)
+    o, g = P.oracle, inputs.rng(840, level)
+    ct = inputs.uniform_residues(g, P.q[:level], P.N, 2)
+    keys = [inputs.uniform_residues(g, list(P.q) + list(P.p), P.N, dnum * 2).reshape(dnum, 2, L + K, P.N) for _ in range(3)] * 5
+    gals = [o.galois_element(r) for r in range(1, 16)]
+    want = o.rotate_hoisted(ct, keys[:14], gals[:14])
+    data, count = [key_dev(k, 0).data for k in keys[:3]], {}
+    dkeys = [binding.SwitchKey(data[i % 3], e) for i, e in enumerate(gals)]
+    for n in (6, 7, 8, 9, 14):
+        before = binding.kernel_launches()
+        got = ctx.rotate_hoisted(ct_dev(ct, 1.0), dkeys[:n])
+        count[n] = binding.kernel_launches() - before
+        for x, w in zip(got, want):
+            assert np.array_equal(host(x.data), w)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert [n for n in (7, 8, 9, 14) if count[n] == count[14] + 2] == list(separate), count
+
+
 FEWER_REGISTERS = r"""
 #define _GNU_SOURCE
 #include <dlfcn.h>
