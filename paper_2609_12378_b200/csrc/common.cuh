@@ -375,11 +375,10 @@ struct NttEpilogue {
     // tl.row0 + r * rot_rows + m * tl.row_stride + comp, or to out.base + r * rot_stride + m * out.stride
     uint32_t group, own, rot_rows;
     size_t rot_stride;
-    // mode 3: extended digits [entry][beta][nt][N] and the digits' own limbs (shared: entry 0 for all), the key (multi: one per
-    // rotation), the batch
-    const u64 *ext, *evk, *mevk[KS_MULTI];
+    // mode 3: extended digits [member][beta][nt][N] and the digits' own limbs (not grouped: one member's), a key per rotation, the batch
+    const u64 *ext, *mevk[KS_MULTI];
     Ptrs d;
-    uint32_t beta, shared, nb;
+    uint32_t beta, nb;
     uint32_t y0;           // (filled in) first limb of the launch
 };
 // Prologue of the forward transform: the first pass reads one buffer [batch][N] (batch = limb index / map.period) instead of

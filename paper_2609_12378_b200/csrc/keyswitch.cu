@@ -536,7 +536,7 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
     const uint32_t nkeys = multi ? (multi->group ? nb / multi->group : nb) : 0;
     for (uint32_t b = 0; b < nkeys; b++) aligned = aligned && aligned16(multi->evk[b]);
     if (add) aligned = aligned && aligned16(*add);
-    const bool fast = beta <= IP_MAX_BETA && aligned;
+    const bool fast = beta <= IP_MAX_BETA && aligned && (!add || beta > IP_FUSED_BETA);       // (mid_rows adds to fewer digits' products)
     const Ptrs pa = add ? *add : Ptrs();
     if (multi && multi->group && !fast) {       // grouped entries without the fast kernel: one key at a time
         for (uint32_t r = 0; r < nkeys; r++) {
@@ -560,9 +560,8 @@ void ks_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 ext_galois,
         using K = decltype(&inner_product_kernel<1, false>);
         static constexpr K plain[IP_MAX_BETA] = {inner_product_kernel<1, false>, inner_product_kernel<2, false>, inner_product_kernel<3, false>, inner_product_kernel<4, false>,
                                                  inner_product_kernel<5, false>, inner_product_kernel<6, false>, inner_product_kernel<7, false>, inner_product_kernel<8, false>};
-        static constexpr K adding[IP_MAX_BETA] = {inner_product_kernel<1, true>, inner_product_kernel<2, true>, inner_product_kernel<3, true>, inner_product_kernel<4, true>,
-                                                  inner_product_kernel<5, true>, inner_product_kernel<6, true>, inner_product_kernel<7, true>, inner_product_kernel<8, true>};
-        launch((add ? adding : plain)[beta - 1], grid, IP_THREADS, 0, s, c->dev, w.ext, w.d, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au, pa);
+        static constexpr K adding[IP_MAX_BETA - IP_FUSED_BETA] = {inner_product_kernel<5, true>, inner_product_kernel<6, true>, inner_product_kernel<7, true>, inner_product_kernel<8, true>};
+        launch(add ? adding[beta - 1 - IP_FUSED_BETA] : plain[beta - 1], grid, IP_THREADS, 0, s, c->dev, w.ext, w.d, evk, ext_galois, w.u, level, nb, bch, multi ? 1 : 0, m, au, pa);
     } else {
         launch(inner_product_generic_kernel, dim3(N / THREADS, nb, nt), THREADS, 0, s, c->dev, w.ext, w.d, 0u, evk, ext_galois, w.u, level, multi ? 1 : 0, m, au,
                add ? 1 : 0, pa);
@@ -601,24 +600,25 @@ static void mid_inner(const ckks_ctx *c, const u64 *evk, uint32_t level, u64 gal
 }
 
 // Whether the row pass that ends a ModDown forms the inner product's q-limbs itself (mode 3 of the epilogue), so that the sum u
-// is written and read back for the special limbs only.  It does where a key word serves fewer than four entries (four or more share
-// it from registers in inner_product_kernel, where this form would read it from L2 for each) and the pass fills the GPU once:
-// below that its eight steps of dependent reads cost more than the traffic (64 hoisted rotations at N = 2^16, level 24:
-// 4550 -> 4110 us; the key/value projections of 24 tokens 35.9 -> 34.3 ms).  Digits that serve one key go through mid_rows instead.  Operands have to take 16-byte accesses.
-static bool inner_fused(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const u64 *evk, uint32_t nb, const KsMulti *multi) {
-    const uint32_t beta = (level + c->alpha - 1) / c->alpha, nkeys = multi ? (multi->group ? nb / multi->group : nb) : 0, per = multi ? multi->group : nb;
-    bool ok = per < 4 && beta <= IP_FUSED_BETA && nb * 2 * level <= 32768 && (uint64_t)nb * 2 * level * (c->N >> 10) >= 16 * (uint64_t)c->sms &&
-              aligned16(w.ext) && aligned16(w.d) && (multi || aligned16(evk));
+// is written and read back for the special limbs only.  It does where keys share digits (digits of one key go through mid_rows), a key
+// word serves fewer than four entries (four or more share it from registers in inner_product_kernel, where this form would read it from
+// L2 for each) and the pass fills the GPU once: below that its eight steps of dependent reads cost more than the traffic (64 hoisted
+// rotations at N = 2^16, level 24: 4550 -> 4110 us; the key/value projections of 24 tokens 35.9 -> 34.3 ms).  Operands have to take
+// 16-byte accesses.
+static bool inner_fused(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, uint32_t nb, const KsMulti *multi) {
+    if (!multi || multi->own) return false;
+    const uint32_t beta = (level + c->alpha - 1) / c->alpha, nkeys = multi->group ? nb / multi->group : nb;
+    bool ok = multi->group < 4 && beta <= IP_FUSED_BETA && nb * 2 * level <= 32768 && (uint64_t)nb * 2 * level * (c->N >> 10) >= 16 * (uint64_t)c->sms &&
+              aligned16(w.ext) && aligned16(w.d);
     for (uint32_t b = 0; b < nkeys; b++) ok = ok && aligned16(multi->evk[b]);
     return ok;
 }
 // the part of the epilogue that describes the inner product
-static void fuse_inner(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, const u64 *evk, uint32_t nb, const KsMulti *multi, NttEpilogue &ep) {
+static void fuse_inner(const ckks_ctx *c, uint32_t level, const KsWorkspace &w, uint32_t nb, const KsMulti &multi, NttEpilogue &ep) {
     ep.mode = 3;
-    ep.ext = w.ext; ep.d = w.d; ep.evk = evk; ep.nb = nb;
+    ep.ext = w.ext; ep.d = w.d; ep.nb = nb;
     ep.beta = (level + c->alpha - 1) / c->alpha;
-    ep.shared = multi && !multi->group;
-    if (multi) for (uint32_t b = 0; b < KS_MULTI; b++) ep.mevk[b] = multi->evk[b];
+    for (uint32_t b = 0; b < KS_MULTI; b++) ep.mevk[b] = multi.evk[b];
 }
 static bool out_aligned(const NttEpilogue &ep) { return aligned16(ep.add) && aligned16(ep.acc) && aligned16(ep.out) && (ep.rot_stride & 1) == 0; }
 
@@ -674,8 +674,7 @@ void ks_apply(const ckks_ctx *c, const u64 *evk, uint32_t level, const KsWorkspa
         moddown(c, level, w, ep, s, nb);
         return;
     }
-    const bool fused = inner_fused(c, level, w, evk, nb, multi) && out_aligned(ep);
-    if (fused) fuse_inner(c, level, w, evk, nb, multi, ep);
+    if (inner_fused(c, level, w, nb, multi) && out_aligned(ep)) fuse_inner(c, level, w, nb, *multi, ep);
     else ks_inner(c, evk, level, o.galois, w, s, nb, false, multi);
     moddown(c, level, w, ep, s, nb);
 }

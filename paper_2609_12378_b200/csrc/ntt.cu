@@ -219,8 +219,8 @@ __global__ void __launch_bounds__(16 * ROW_CTA, 64 / ROW_CTA) ntt_fwd_rows(DevTa
         if (EP == 3) {
             // u = sum_j digit_j key_j
             const size_t ks = (size_t)2 * c.T << c.log_n;
-            const uint32_t de = ep.shared ? 0 : ep.group && !ep.own ? mem : bz, own = i / c.alpha;
-            const u64 *kp = (ep.multi ? ep.mevk[rot] : ep.evk) + (((size_t)comp * c.T + i) << c.log_n) + p0;
+            const uint32_t de = ep.group ? mem : 0, own = i / c.alpha;
+            const u64 *kp = ep.mevk[rot] + (((size_t)comp * c.T + i) << c.log_n) + p0;
             const u64 *eb = ep.ext + (((size_t)de * BETA * ep.nt + i) << c.log_n), *od = ep.d.at(de) + ((size_t)i << c.log_n);
 #pragma unroll
             for (uint32_t k = 0; k < 8; k++) {
@@ -333,9 +333,9 @@ __global__ void __launch_bounds__(16 * ROW_CTA, 48 / ROW_CTA) ntt_inv_rows(DevTa
     if constexpr (BETA > 0) {
         const uint32_t e = blockIdx.y / map.period, comp = e & 1, bz = e >> 1, xl = src.nt - map.period + blockIdx.y % map.period, p0 = row * 256 + 2 * t;
         const uint32_t rot = src.group ? bz / src.group : bz, mem = src.group ? bz % src.group : bz;
-        const uint32_t gal = (uint32_t)(src.multi ? src.mgalois[rot] : src.galois), de = src.shared ? 0 : src.group && !src.own ? mem : bz;
+        const uint32_t gal = (uint32_t)src.mgalois[rot], de = src.group ? mem : 0;
         const size_t ks = (size_t)2 * c.T << c.log_n;
-        const u64 *kp = (src.multi ? src.mevk[rot] : src.evk) + (((size_t)comp * c.T + prime) << c.log_n) + p0;
+        const u64 *kp = src.mevk[rot] + (((size_t)comp * c.T + prime) << c.log_n) + p0;
         const u64 *eb = src.ext + (((size_t)de * BETA * src.nt + xl) << c.log_n);
 #pragma unroll
         for (uint32_t k = 0; k < 8; k++) {

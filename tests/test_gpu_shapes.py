@@ -307,9 +307,10 @@ def test_hoisted_rotations_with_and_without_a_stored_inner_product(dnum, level):
         assert np.array_equal(host(x.data), want)
 
 
-@pytest.mark.parametrize("dnum,level", [(1, 21), (3, 22), (4, 22), (3, 19)])
+@pytest.mark.parametrize("dnum,level", [(1, 21), (3, 22), (4, 22), (3, 19), (5, 22), (5, 19)])
 def test_large_product_with_and_without_a_stored_inner_product(dnum, level):
-    """x^2 at N = 2^16 on either side of the size from which the last row pass forms the inner product."""
+    """x^2 at N = 2^16 with one to four digits, whose inner product is formed between the row passes and never stored for the limbs that
+    ModDown converts, and with five, whose sum is."""
     from tests.gpu_util import context, ct_dev, host, key_dev
     K = -(-22 // dnum)
     P, ctx = params(16, 22, K, dnum), context(16, 22, K, dnum)
@@ -408,10 +409,10 @@ def test_key_switches_of_one_key_take_the_integer_share():
     (12, 3, 1, 3, 3), (12, 8, 8, 1, 8), (12, 9, 9, 1, 9), (12, 7, 4, 3, 5), (12, 12, 3, 4, 12), (12, 10, 2, 5, 10), (12, 16, 8, 2, 11),
     (13, 12, 6, 2, 12), (14, 6, 2, 3, 5), (14, 16, 8, 2, 16), (15, 12, 4, 3, 9), (15, 8, 8, 1, 8), (16, 3, 3, 1, 3), (16, 10, 5, 2, 6)])
 def test_key_switches_of_every_ring_and_digit_size(log_n, L, K, dnum, level):
-    """One to nine sources per conversion (eight are the most that stay in registers), full and partial digits, one to five digits (four
-    are the most whose row pass forms the inner product), rings from the smallest that runs a strip of columns through conversion and
-    both transforms: a rotation whose sources lie at the ends of the residues, a sum of rotations over two groups of terms, a product
-    that drops a limb and a rescale, all of it on one ciphertext and on several."""
+    """One to nine sources per conversion, full and partial digits, one to five digits (four are the most whose row pass forms the inner
+    product): a rotation whose sources lie at the ends of the residues, a sum of rotations over two groups of terms, a product that drops a
+    limb and a rescale, all of it on one ciphertext and on several.  At N = 2^14 and 2^15 the ModUps run in strips, at 2^15 the ModDowns
+    too; test_gpu_strips.py has the batches that do so on the other rings."""
     from tests.gpu_util import context, ct_dev, host, key_dev
     P, ctx = params(log_n, L, K, dnum), context(log_n, L, K, dnum)
     o, g = P.oracle, inputs.rng(800, level + 100 * L + 10000 * log_n)
