@@ -86,7 +86,10 @@ __global__ void __launch_bounds__(StripShape<LOGR>::THREADS, 1) conv_cols(DevTab
     const uint32_t grp = threadIdx.x / TG, tid = threadIdx.x % TG, cc = tid % COLS, r = tid / COLS;
     constexpr uint32_t STRIPS = 256 / COLS;                   // of an item
     const bool whole = blockIdx.x < grid.whole;
-    const uint32_t slot = blockIdx.x - (whole ? 0 : grid.whole), strip = whole ? slot : grid.whole + slot % grid.split, col = strip % STRIPS * COLS + cc;
+    uint32_t slot = blockIdx.x - (whole ? 0 : grid.whole), x0 = 0;
+    if (!whole)                                               // (few steps: a division is in the way of short launches)
+        for (; slot >= grid.split; slot -= grid.split) x0 += grid.chunk;
+    const uint32_t strip = whole ? slot : grid.whole + slot, col = strip % STRIPS * COLS + cc;
     double *bufs = ssm;                                       // [sources][LIMB] (the dropped limb last); the first BUFFERS pass targets later
     double *stw = bufs + (NS > S::BUFFERS ? NS : S::BUFFERS) * LIMB + (RESC ? LIMB : 0);       // [GROUPS][R] twiddles
     double2 *s_m = reinterpret_cast<double2 *>(stw + GROUPS * R);       // the targets' primes and inverses
@@ -97,7 +100,7 @@ __global__ void __launch_bounds__(StripShape<LOGR>::THREADS, 1) conv_cols(DevTab
     const uint32_t beta = MODE == CONV_UP ? (level + c.alpha - 1) / c.alpha : 1, j = MODE == CONV_UP ? item % beta : 0, bz = item / beta;
     const uint32_t lo = j * c.alpha, nd = MODE == CONV_UP ? min(c.alpha, level - lo) : c.K;
     const uint32_t nt = level + c.K;
-    const uint32_t x0 = whole ? 0 : slot / grid.split * grid.chunk, x1 = min(whole ? targets : x0 + grid.chunk, MODE == CONV_UP ? nt - nd : targets);      // ModUp: counted without the digit's own limbs
+    const uint32_t x1 = min(whole ? targets : x0 + grid.chunk, MODE == CONV_UP ? nt - nd : targets);      // ModUp: counted without the digit's own limbs
     if (x0 >= x1) return;
     auto target_limb = [&](uint32_t xt) { return MODE == CONV_UP && xt >= lo ? xt + nd : xt; };
     auto target_prime = [&](uint32_t xt) { const uint32_t x = target_limb(xt); return MODE == CONV_UP && x >= level ? c.L + (x - level) : x; };
