@@ -124,6 +124,8 @@ const char *ckks_last_cuda_error(const ckks_ctx *ctx);
 /* Options of a context: host-side state, read whenever a call is made (set them between calls, not while another
  * thread is inside one).  None of them changes a result: every kernel variant is bit-identical.
  *   CKKS_OPT_NTT_FP_SHARE   N = 2^16 transform: of every 8 limbs, how many run on the FP64 pipe (0..8, default 8).
+ *                           Plain transforms only: those fused with what comes before or after them (all of a key switch
+ *                           with CKKS_CONV_FP64) take the FP64 pipe throughout.
  *   CKKS_OPT_CONV_KERNEL    ModUp / ModDown basis conversions: CKKS_CONV_FP64 (default) or CKKS_CONV_TENSOR.
  *   CKKS_OPT_MAC_KERNEL     the projection's multiply-accumulate: CKKS_MAC_MMA (default: mma.sync, 8 coefficients per
  *                           CTA, a warp per coefficient), CKKS_MAC_MMA_ASYNC (the same joined by mbarriers instead of

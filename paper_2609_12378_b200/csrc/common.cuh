@@ -217,6 +217,13 @@ __device__ __forceinline__ u64 centred_to(u64 y, u64 src, u64 dst) {
 constexpr double MAGIC0 = 6755399441055744.0;    // 1.5 * 2^52: rounds |v| < 2^51 to the nearest integer
 constexpr double MAGIC1 = 13510798882111488.0;   // 1.5 * 2^53: rounds |v| < 2^52 to the nearest even integer
 constexpr double TWO52 = 4503599627370496.0;
+// Basis conversions: out[t] = sum_a y_a C[a][t] mod t with centred sources |y_a| <= q_a / 2 and centred constants |C| <= t / 2 (a dense
+// contraction, bound by the FP64 pipe).  The exact 100-bit products of up to eight sources are summed as they are:
+//   H' = fma(y, C, H) starting from H = 1.5 * 2^102 rounds the running sum to multiples of 2^50 (|sum| <= 8 * 2^98 =
+//   2^101 keeps H inside [2^102, 2^103)); h = H' - H is exact, l = fma(y, C, -h) is the exact rest, |l| <= 2^49,
+// so the sum is (H - 1.5 * 2^102) + sum l, four instructions per (source, target) pair where a reduction of every product took seven.
+// The high part is below 2 q t, its quotient by t below 2^51; the low parts are at most 8 * 2^49.
+constexpr double CONV_SIGMA = 0x1.8p+102;
 
 template <int COARSE>
 __device__ __forceinline__ double mulmod_d(double y, double2 w, double q) {

@@ -5,22 +5,11 @@
 // targets starts with their column pass.  A CTA takes a strip of columns of all sources of one conversion, keeps their
 // coefficients in shared memory and walks a chunk of the targets, so that neither the sources' coefficients nor the converted
 // limbs make a trip through memory between these steps, and three launches are one.
-//
-// Arithmetic of a conversion: out[t] = sum_a y_a C[a][t] mod t with centred sources |y_a| <= q_a / 2 and centred constants
-// |C| <= t / 2 (a dense contraction, bound by the FP64 pipe).  The exact 100-bit products are summed as they are and reduced
-// once per eight sources:
-//   H' = fma(y, C, H) starting from H = 1.5 * 2^102 rounds the running sum to multiples of 2^50 (|sum| <= 8 * 2^98 =
-//   2^101 keeps H inside [2^102, 2^103)); h = H' - H is exact, l = fma(y, C, -h) is the exact rest, |l| <= 2^49,
-// so the sum is (H - 1.5 * 2^102) + sum l, four instructions per (source, target) pair where a reduction of every product
-// took seven.  The high part is below 2 q t, so its quotient by t is below 2^51 (nearest rounding) and leaves |r| <= 1.1 t;
-// with the low parts (<= 8 * 2^49, plus a reduced carry of the previous eight sources) the sum stays below 2^53.
 #include <type_traits>
 
 #include "butterfly.cuh"
 
 namespace {
-
-constexpr double CONV_SIGMA = 0x1.8p+102;
 
 // Shape for R = 2^LOGR rows: strips of 2048 words (eight columns at N = 2^16), one CTA of 16 warps per SM, four groups of TG = 128
 // threads.  A transform of a limb's strip is a group's, sixteen coefficients per thread, as in the column passes of ntt.cu: radix 16,
@@ -28,7 +17,7 @@ constexpr double CONV_SIGMA = 0x1.8p+102;
 // kinds and none waits for the other's loads: two convert, CPT = 8 coefficients per thread with all their sources in registers, and
 // pass one target after the other through BUFFERS buffers to the two that transform them.  (All groups doing both in turn, with the
 // sources in shared memory: 395 us for the ModDowns of sixteen hoisted rotations at N = 2^16, level 24; with the sources in registers
-// and a barrier of the CTA per batch of targets: 416; in this form 369, the FP64 pipe busy 67 % of it.  The three kernels this
+// and a barrier of the CTA per batch of targets: 416; in this form 354, the FP64 pipe busy 71 % of its cycles.  The three kernels this
 // replaces take 344 one by one, but move another 64 MiB per rotation, which under the power limit costs more than they save.)
 template <uint32_t LOGR>
 struct StripShape {
@@ -40,15 +29,16 @@ struct StripShape {
 };
 constexpr uint32_t STRIP_CHUNK = 32, STRIP_NS = 8;         // targets and sources of a CTA at most
 // Registers per thread of the two roles.  256 (176 + 80) = 512 x 128, which is what the CTA is launched with (every instance is compiled
-// to 128): more in sum would wait for registers that nobody gives back.
+// to 128): more in sum would wait for registers that nobody gives back.  Eight sources spill: 36 to 96 bytes per thread stored, 64 to 144
+// read, more of them the larger the ring.
 constexpr uint32_t CONV_REGS = 176, NTT_REGS = 80;
 static_assert(CONV_REGS + NTT_REGS == 256, "the two halves of the CTA share the registers of its launch");
 
 __device__ __forceinline__ void group_sync(uint32_t id, uint32_t threads) { asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory"); }
 __device__ __forceinline__ void group_arrive(uint32_t id, uint32_t threads) { asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(threads) : "memory"); }
 
-// out[p] (+)= sum_a y[p][a] w[a] mod t.  The quotient of the whole sum is formed in two roundings, k = round(lo / t + round(hi / t)),
-// hi / t below 2^51: |out| <= (1/2 + 1/4 + 1/2) t = 1.25 t.
+// out[p] (+)= sum_a y[p][a] w[a] mod t (see CONV_SIGMA; out enters below t).  The quotient of the whole sum is formed in two roundings,
+// k = round(lo / t + round(hi / t)), hi / t below 2^51 and the low parts with out below 2^53: |out| <= (1/2 + 1/4 + 1/2) t = 1.25 t.
 // FULL: ns = NS, without a branch per source, so that the constants' fetches run ahead of the products.
 template <bool FIRST, bool FULL, uint32_t NS, uint32_t CPT>
 __device__ __forceinline__ void strip_dot(const double (&y)[CPT][NS], const double *w, uint32_t ns, double t, double tinv, double (&out)[CPT]) {

@@ -19,19 +19,9 @@ constexpr uint32_t THREADS = 256, IP_THREADS = 128;
 // hoisted rotations' 615 -> 601; 64 threads fetch their constants too often, 618)
 constexpr uint32_t CONV_THREADS = 128;
 
-// ---------------------------------------------------------------------------
-// Basis conversions: out[x] = sum_a y_a C[a][x] mod t_x with centred sources |y_a| <= q_a / 2 and centred constants
-// |C| <= t / 2 (a dense contraction, bound by the FP64 pipe).  The exact 100-bit products are summed as they are and
-// reduced once per eight sources:
-//   H' = fma(y, C, H) starting from H = 1.5 * 2^102 rounds the running sum to multiples of 2^50 (|sum| <= 8 * 2^98 =
-//   2^101 keeps H inside [2^102, 2^103)); h = H' - H is exact, l = fma(y, C, -h) is the exact rest, |l| <= 2^49,
-// so the sum is (H - 1.5 * 2^102) + sum l, four instructions per (source, target) pair where a reduction of every product
-// took seven.  The high part is below 2 q t, so its quotient by t is below 2^51 (nearest rounding) and leaves |r| <= 1.1 t;
-// with the low parts (<= 8 * 2^49, plus a reduced carry of the previous eight sources) the sum stays below 2^53.
+// ---- basis conversions (see CONV_SIGMA), any number of sources, reduced once per eight: the quotient of the high part, rounded to nearest,
+// leaves |r| <= 1.1 t, and with the low parts and a reduced carry of the previous eight sources the sum stays below 2^53.
 // A thread takes CPT adjacent coefficients, so that a pair of constants from shared memory serves 2 CPT pairs.
-// ---------------------------------------------------------------------------
-constexpr double CONV_SIGMA = 0x1.8p+102;
-
 // out enters holding a further summand below t (FIRST: nothing)
 template <bool FIRST, uint32_t NS, uint32_t CPT>
 __device__ __forceinline__ void conv_dot(const double (&y)[CPT][NS], const double *w, double t, double tinv, double (&out)[CPT]) {

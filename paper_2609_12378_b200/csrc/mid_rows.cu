@@ -11,7 +11,8 @@ namespace {
 
 // A warp per row, eight coefficients per lane (stages in groups of 3, 3 and 2), so that the sums of both components fit 64 registers:
 // the kernel waits for its key words and digits, and 32 warps per SM wait for more of them at a time (16 lanes per row with
-// sixteen coefficients and 128 registers: 54 us for one ciphertext at N = 2^16, level 24).
+// sixteen coefficients and 128 registers: 54 us for one ciphertext at N = 2^16, level 24).  Sums over terms hold theirs throughout, and at
+// five CTAs per SM those of three and four digits spill (144 and 220 bytes per thread stored).
 constexpr uint32_t MID_ROWS = 4;
 
 template <uint32_t BETA, bool TERMS>
