@@ -63,7 +63,9 @@ __device__ __forceinline__ void strip_dot(const double (&y)[CPT][NS], const doub
     }
 }
 
-// The CTAs of a launch: the first `whole` take a strip of an item with all its targets, the others one of `split` strips with `chunk` targets
+// The CTAs of a launch: strips by chunks of targets (x, y), or, with `whole`, in one row: the first `whole` take a strip with all its
+// targets, the others one of the `split` remaining ones with `chunk` targets.  (The short launches are of the first kind, which has no
+// arithmetic in the way of their start: a rotation at N = 2^15, level 4 30.4 us, with one row for both and two divisions 31.0.)
 struct StripGrid { uint32_t whole, split, chunk; };
 
 // src: limbs after the inverse row pass (signed doubles); dst: limbs for the forward row pass.  NS: sources at most
@@ -75,11 +77,14 @@ __global__ void __launch_bounds__(StripShape<LOGR>::THREADS, 1) conv_cols(DevTab
     extern __shared__ __align__(16) double ssm[];
     const uint32_t grp = threadIdx.x / TG, tid = threadIdx.x % TG, cc = tid % COLS, r = tid / COLS;
     constexpr uint32_t STRIPS = 256 / COLS;                   // of an item
-    const bool whole = blockIdx.x < grid.whole;
-    uint32_t slot = blockIdx.x - (whole ? 0 : grid.whole), x0 = 0;
-    if (!whole)                                               // (few steps: a division is in the way of short launches)
-        for (; slot >= grid.split; slot -= grid.split) x0 += grid.chunk;
-    const uint32_t strip = whole ? slot : grid.whole + slot, col = strip % STRIPS * COLS + cc;
+    uint32_t strip = blockIdx.x, x0 = blockIdx.y * grid.chunk, take = grid.chunk;
+    if (grid.whole) {
+        if (strip < grid.whole) take = targets;
+        else
+#pragma unroll 1
+            for (; strip >= grid.whole + grid.split; strip -= grid.split) x0 += grid.chunk;
+    }
+    const uint32_t col = strip % STRIPS * COLS + cc;
     double *bufs = ssm;                                       // [sources][LIMB] (the dropped limb last); the first BUFFERS pass targets later
     double *stw = bufs + (NS > S::BUFFERS ? NS : S::BUFFERS) * LIMB + (RESC ? LIMB : 0);       // [GROUPS][R] twiddles
     double2 *s_m = reinterpret_cast<double2 *>(stw + GROUPS * R);       // the targets' primes and inverses
@@ -90,7 +95,7 @@ __global__ void __launch_bounds__(StripShape<LOGR>::THREADS, 1) conv_cols(DevTab
     const uint32_t beta = MODE == CONV_UP ? (level + c.alpha - 1) / c.alpha : 1, j = MODE == CONV_UP ? item % beta : 0, bz = item / beta;
     const uint32_t lo = j * c.alpha, nd = MODE == CONV_UP ? min(c.alpha, level - lo) : c.K;
     const uint32_t nt = level + c.K;
-    const uint32_t x1 = min(whole ? targets : x0 + grid.chunk, MODE == CONV_UP ? nt - nd : targets);      // ModUp: counted without the digit's own limbs
+    const uint32_t x1 = min(x0 + take, MODE == CONV_UP ? nt - nd : targets);      // ModUp: counted without the digit's own limbs
     if (x0 >= x1) return;
     auto target_limb = [&](uint32_t xt) { return MODE == CONV_UP && xt >= lo ? xt + nd : xt; };
     auto target_prime = [&](uint32_t xt) { const uint32_t x = target_limb(xt); return MODE == CONV_UP && x >= level ? c.L + (x - level) : x; };
@@ -258,7 +263,7 @@ uint32_t strip_targets(const ckks_ctx *c, int mode, uint32_t level) {
 // chunks, the others share out the last wave.  (N = 2^16, level 24, in a burst and back to back under the power limit: eight hoisted
 // rotations, 512 strips, 3.46 waves, by the separate kernels 576 and 566 us, by a CTA per strip 588 and 559, so 575 and 545; fourteen, 6.05
 // waves, 910 and 924, 931 and 918, 911 and 878.)
-struct StripPlan { StripGrid grid; uint32_t ctas, cost, full; };        // full: the cost if all SMs were busy throughout, times their number
+struct StripPlan { StripGrid grid; dim3 ctas; uint32_t cost, full; };        // full: the cost if all SMs were busy throughout, times their number
 StripPlan strip_plan(const ckks_ctx *c, int mode, uint32_t level, uint32_t strips) {
     const uint32_t targets = strip_targets(c, mode, level), sms = (uint32_t)c->sms, rounds = (strip_sources(c, mode, level) + (mode == CONV_DOWN_RS) + 3) / 4;
     auto cta = [&](uint32_t n) { return (std::min(n, targets) + 3) / 4 * 2 + rounds; };
@@ -270,7 +275,7 @@ StripPlan strip_plan(const ckks_ctx *c, int mode, uint32_t level, uint32_t strip
         const uint32_t whole = w * sms, split = strips - whole;
         for (uint32_t ch = 4; ch <= STRIP_CHUNK && ch < targets + 4; ch += 4) {
             const uint32_t n = (targets + ch - 1) / ch, cost = w * cta(targets) + (split * n + sms - 1) / sms * cta(ch);
-            if (cost <= p.cost) p = {{whole, std::max(split, 1u), ch}, whole + split * n, cost, p.full};
+            if (cost <= p.cost) p = {{whole, split, ch}, whole ? dim3(whole + split * n) : dim3(split, n), cost, p.full};
         }
         if (w == waves) break;
     }
